@@ -232,7 +232,7 @@ gp_status gpi::launch(gp_ctx* c, const void* x, void* y, int add, cudaStream_t s
   a.zruns = c->d_zruns;
   a.nzruns = add ? 0 : (int32_t)p.num_zero_runs();
   a.g = p.jumps.data();
-  a.m = p.mass.data();
+  a.m = p.lump.data();
   a.s = p.scale.data();
   cudaEvent_t* ev = nullptr;
   if (c->prof && trace) {
@@ -855,7 +855,7 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
                           b->cap);
       if (e == cudaSuccess)
         e = g.ops.run(g.k, g.d_fsegs, g.d_lsegs, g.d_ptrs[i], (int)g.prob.size(), g.face_blocks, g.lift_blocks,
-                      pl0.jumps.data(), pl0.mass.data(), g.tiles, b->cap);
+                      pl0.jumps.data(), pl0.lump.data(), g.tiles, b->cap);
     }
     cudaGraph_t graph = nullptr;
     const cudaError_t e2 = cudaStreamEndCapture(b->cap, &graph);

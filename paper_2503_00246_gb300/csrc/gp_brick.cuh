@@ -125,8 +125,9 @@ template <int D, int K, class A, int AX>
 __device__ __forceinline__ void brick_chunk(const uint32_t* __restrict__ bface, const int f0, const int f1,
                                             const int fl, const int tau, const int fb, const typename A::V* xs,
                                             Sum<typename A::V>* ys,
-                                            typename A::V (*buf)[K][Shape<D, K>::L],
-                                            typename A::V (*sb2)[K][Shape<D, K>::L],
+                                            typename A::V (*buf)[K][TanShape<D, K>::LP],
+                                            typename A::V (*dots)[K][K + 1],
+                                            const TanTable<D, K, typename A::V>& tab,
                                             const Consts<typename A::V, K>& c) {
   using V = typename A::V;
   constexpr int L = Shape<D, K>::L, NN = 2 * K + 1, K1 = K + 1;
@@ -150,11 +151,10 @@ __device__ __forceinline__ void brick_chunk(const uint32_t* __restrict__ bface, 
     V tj[K];
     line_jumps<K, V>(v, FoldScale<V>::value ? c.gs : c.g, tj);
 #pragma unroll
-    for (int j = 0; j < K; ++j) buf[fl][j][tau] = tj[j];
+    for (int j = 0; j < K; ++j) buf[fl][j][TanShape<D, K>::at(tau)] = tj[j];
   }
-  __syncthreads();
   V out[K];
-  line_tangential_eo<D, K, V, L>(buf, sb2, fb, c, fl, tau, out);
+  tangential_mass<D, K, V>(buf, dots, fb, c, tab, fl, tau, out);
   V w[NN];
   if (valid) {
     if constexpr (!FoldScale<V>::value) {
@@ -183,7 +183,9 @@ brick_kernel(const typename A::IO* __restrict__ x, typename A::IO* __restrict__ 
   using IO = typename A::IO;
   constexpr int L = Shape<D, K>::L, K1 = K + 1;
   constexpr int NB = (D == 3) ? K1 * K1 * K1 : K1 * K1;
-  typedef V Plane[K][L];
+  typedef V Plane[K][TanShape<D, K>::LP];
+  typedef V Dots[K][K1];
+  __shared__ TanTable<D, K, V> tab;
   const int t = threadIdx.x, nt = (int)blockDim.x;
   // the plane fixup may take its prologue while the bricks run (it waits for this grid)
   asm volatile("griddepcontrol.launch_dependents;");
@@ -219,8 +221,9 @@ brick_kernel(const typename A::IO* __restrict__ x, typename A::IO* __restrict__ 
   p0 += align16((size_t)ba.maxown * sizeof(int32_t));
   int32_t* srow = reinterpret_cast<int32_t*>(p0);          // region: row starts ...
   Plane* buf = reinterpret_cast<Plane*>(p0);               // ... or jump planes
-  Plane* sb2 = buf + fb;
+  Dots* dots = reinterpret_cast<Dots*>(buf + fb);
 
+  fill_tan_table<D, K, V>(tab, c, t);
   // ---- own-cell map and coordinates, zero accumulators, row starts, staged x blocks
   for (int i = t; i < nown; i += nt) {
     const int cc = __ldg(ba.bccoord + cell_off + i);
@@ -256,11 +259,11 @@ brick_kernel(const typename A::IO* __restrict__ x, typename A::IO* __restrict__ 
     const int fl = t / L, tau = t - fl * L;
     const uint32_t* bf = ba.bface + face_off;
     const int a1 = sd[8], a2 = (D == 3) ? sd[9] : nface;
-    for (int f0 = 0; f0 < a1; f0 += fb) brick_chunk<D, K, A, 0>(bf, f0, a1, fl, tau, fb, xs, ys, buf, sb2, c);
-    for (int f0 = a1; f0 < a2; f0 += fb) brick_chunk<D, K, A, 1>(bf, f0, a2, fl, tau, fb, xs, ys, buf, sb2, c);
+    for (int f0 = 0; f0 < a1; f0 += fb) brick_chunk<D, K, A, 0>(bf, f0, a1, fl, tau, fb, xs, ys, buf, dots, tab, c);
+    for (int f0 = a1; f0 < a2; f0 += fb) brick_chunk<D, K, A, 1>(bf, f0, a2, fl, tau, fb, xs, ys, buf, dots, tab, c);
     if constexpr (D == 3) {
       for (int f0 = a2; f0 < nface; f0 += fb)
-        brick_chunk<D, K, A, 2>(bf, f0, nface, fl, tau, fb, xs, ys, buf, sb2, c);
+        brick_chunk<D, K, A, 2>(bf, f0, nface, fl, tau, fb, xs, ys, buf, dots, tab, c);
     }
   }
 

@@ -45,8 +45,8 @@ struct Tiles {
 constexpr int MAX_CTA_THREADS = 512;
 constexpr size_t MAX_DYN_SMEM = 46 * 1024;   // plus < 2 KB of static shared memory: under the 48 KB default
 
-// dynamic shared memory of the face kernel: the k jump planes (and the first
-// tangential pass in 3D) of fb faces
+// dynamic shared memory of the face kernel: the k jump planes of fb faces, twice in 3D (room for
+// the padded planes and the second direction's sums, see TanShape)
 template <int D, int K, typename V>
 __host__ __device__ constexpr size_t face_smem(int fb) {
   return (size_t)((D == 3) ? 2 : 1) * fb * K * Shape<D, K>::L * sizeof(V);
@@ -66,24 +66,21 @@ struct Consts {
   V g[K][2 * K + 1];   // jump of the j-th derivative of patch basis b (row j-1)
   V gs[K][2 * K + 1];  // s_j g_j[b], the jump vectors of the first step (FP64, float-float)
   V s[K];              // s_j (FP32)
-  V m[K + 1][K + 1];   // reference mass matrix
-  // even and odd halves of the centrosymmetric mass matrix (M^[N-1-p][N-1-i] = M^[p][i], N = k+1):
-  // me[p][i] = (M^[p][i] + M^[p][N-1-i]) / 2 (M^[p][i] for the middle i), mo[p][i] = (M^[p][i] - M^[p][N-1-i]) / 2
-  V me[(K + 2) / 2][(K + 2) / 2];
-  V mo[(K + 1) / 2][(K + 1) / 2];
+  // reference mass M^ = diag(mw) (I + mc ma^T) (see tangential_mass)
+  V ma[K + 1];
+  V mc[K + 1];
+  V mw[K + 1];
 };
 
-// Fills the even / odd halves of the mass matrix m (row-major, (k+1)^2) into c.
+// Fills the lumped form of the reference mass from p = (ma, mc, mw), 3 (k+1) values.
 template <typename V, int K>
-void mass_halves(const double* m, Consts<V, K>& c) {
-  constexpr int N = K + 1, NE = (K + 2) / 2, H = (K + 1) / 2;
-  for (int p = 0; p < NE; ++p)
-    for (int i = 0; i < NE; ++i) {
-      const bool mid = 2 * i == N - 1;
-      c.me[p][i] = from_host<V>(mid ? m[p * N + i] : 0.5 * (m[p * N + i] + m[p * N + N - 1 - i]));
-    }
-  for (int p = 0; p < H; ++p)
-    for (int i = 0; i < H; ++i) c.mo[p][i] = from_host<V>(0.5 * (m[p * N + i] - m[p * N + N - 1 - i]));
+void mass_consts(const double* p, Consts<V, K>& c) {
+  constexpr int N = K + 1;
+  for (int i = 0; i < N; ++i) {
+    c.ma[i] = from_host<V>(p[i]);
+    c.mc[i] = from_host<V>(p[N + i]);
+    c.mw[i] = from_host<V>(p[2 * N + i]);
+  }
 }
 
 struct FaceArgs {
@@ -136,79 +133,105 @@ __device__ __forceinline__ void line_jumps(const V (&v)[2 * K + 1], const V (*g)
   }
 }
 
-// The mass matrix applied to one line of N = k+1 values u through its even and odd halves:
-// y[p] = E_p + O_p and y[N-1-p] = E_p - O_p, E_p = sum_i me[p][i] (u[i] + u[N-1-i]) (the middle
-// value once), O_p = sum_i mo[p][i] (u[i] - u[N-1-i]): (N/2)^2 + (N/2 rounded up)^2 terms and
-// 2 (N/2) folds and merges instead of N^2 terms.
-template <int K, typename V>
-__device__ __forceinline__ void mass_line_eo(const Consts<V, K>& c, const V (&u)[K + 1], V (&y)[K + 1]) {
-  constexpr int N = K + 1, NE = (K + 2) / 2, H = (K + 1) / 2;
-  V e[NE], o[H > 0 ? H : 1];
-#pragma unroll
-  for (int i = 0; i < H; ++i) {
-    e[i] = vadd_loose(u[i], u[N - 1 - i]);
-    o[i] = vsub_loose(u[i], u[N - 1 - i]);
-  }
-  if (N % 2 == 1) e[NE - 1] = u[NE - 1];
-#pragma unroll
-  for (int p = 0; p < NE; ++p) {
-    Dot<V> ev = dot_first(c.me[p][0], e[0]);
-#pragma unroll
-    for (int i = 1; i < NE; ++i) dot_fma(ev, c.me[p][i], e[i]);
-    if (p < H) {
-      Dot<V> ov = dot_first(c.mo[p][0], o[0]);
-#pragma unroll
-      for (int i = 1; i < H; ++i) dot_fma(ov, c.mo[p][i], o[i]);
-      y[p] = dot_merge<false>(ev, ov);
-      y[N - 1 - p] = dot_merge<true>(ev, ov);
-    } else {
-      y[p] = dot_value(ev);
-    }
-  }
+// ------------------------------------------------------ tangential masses --
+// Gauss-Lobatto quadrature with N = k+1 points is exact up to degree 2k - 1, and the product of
+// two nodal polynomials has degree 2k, so the exact mass matrix differs from the lumped one by the
+// quadrature error of x^(2k), a rank-one term in the leading coefficients a_i of the l_i:
+//   M^ = diag(w) - E a a^T = diag(mw) (I + mc ma^T),   ma = a / max|a|,  mc = -E max|a| a / w
+// (k = 1: diag(1/6) (I + 1 1^T), which has no cancellation).  One line costs 2 N multiply-adds
+// and the N factors mw, which both directions share as one product per normal line: 2 (d-1) k + k
+// multiply-adds per line.  The even / odd halves of M^ took (N^2 / 2 + 2 N) (d-1) k / N, i.e. 20
+// against 34 at d = 3, k = 4 and 40 against 101 at k = 8.  Bound by the FP64 pipe: the native
+// FP64 apply of the 128^3 gyroid at k = 4 went from 1780 to 1519 us and that of the 64^3 ball at
+// k = 3 from 77.2 to 68.7 us; float-float 96^3 ball at k = 5 277 to 270 us; FP32 unchanged.
+//
+// Shared-memory layout of the tangential pass: a plane of the k jump values of a face's L lines
+// (3D: line (t1, t2) at t1 + pitch t2 with an odd pitch, so that walking t1 or t2 in neighbouring
+// lanes meets distinct banks; k = 3, 5, 7 had 2- to 8-way conflicts) and in 3D the N sums per
+// order of the second direction.  In 3D both fit the two planes that the launch reserves.
+template <int D, int K>
+struct TanShape {
+  static constexpr int N = K + 1;
+  static constexpr int PITCH = (D == 3) ? (N | 1) : N;
+  static constexpr int LP = (D == 3) ? PITCH * N : N;   // one order of one face
+  __host__ __device__ static constexpr int at(int tau) { return (D == 3) ? tau % N + PITCH * (tau / N) : tau; }
+};
+
+// The factors a line's thread needs at its own tangential index (lane-dependent, so not in the
+// constant bank): mw of the line (the product of both directions) and mc.
+template <int D, int K, typename V>
+struct TanTable {
+  V w[Shape<D, K>::L];
+  V c[K + 1];
+};
+template <int D, int K, typename V>
+__device__ __forceinline__ void fill_tan_table(TanTable<D, K, V>& tab, const Consts<V, K>& c, const int t) {
+  constexpr int N = K + 1;
+  if (t < Shape<D, K>::L) tab.w[t] = (D == 3) ? vmul(c.mw[t % N], c.mw[t / N]) : c.mw[t];
+  if (t < N) tab.c[t] = c.mc[t];
 }
 
-// The tangential masses applied line by line through the even / odd halves of M^: a task is
-// one (face, order j, tangential line of k+1 values); the tasks of the CTA's fb faces are
-// spread over its threads in order (task u on thread u), so the busy threads fill whole warps
-// and the rest of the CTA idles at the barriers.  Each task moves 2 (k+1) shared-memory values
-// instead of the (k+1)^2 of one output per thread, and does (k+1)^2 / 2 + O(k) instead of
-// (k+1)^2 multiply-adds.  3D: pass 1 along t1 from `plane` into `plane2`, pass 2 along t2 back
-// into `plane`; 2D: one pass, in place (the 2D kernels hold one plane per face).  Thread
-// (fl, tau) then reads out[j] = plane[fl][j][tau].  Every thread of the CTA must call it (it
-// synchronises); nt >= fb L.
-template <int D, int K, typename V, int L>
-__device__ __forceinline__ void line_tangential_eo(V (*plane)[K][L], V (*plane2)[K][L], const int fb,
-                                                   const Consts<V, K>& c, const int fl, const int tau,
-                                                   V (&out)[K]) {
+// out[j] = ((M^ x M^) u_j)(tau) for the k jump values u_j of every line in `plane`.  A task is one
+// (face, order j, tangential line of N values); the tasks of the CTA's fb faces are packed onto its
+// first threads.  3D: pass 1 along t2 (neighbouring lanes on neighbouring t1) in place; pass 2
+// along t1 only takes the dot product ma . u of each line, and every line's thread adds its own
+// mc and multiplies by mw (FP32, bound by shared-memory accesses and not by arithmetic: pass 2 in
+// place too, one access less per value).  2D: pass 1 in place.  Every thread of the CTA calls it
+// (it synchronises, also before its first read: the caller has only written plane and tab).
+template <int D, int K, typename V>
+__device__ __forceinline__ void tangential_mass(V (*plane)[K][TanShape<D, K>::LP], V (*dots)[K][K + 1], const int fb,
+                                                const Consts<V, K>& c, const TanTable<D, K, V>& tab, const int fl,
+                                                const int tau, V (&out)[K]) {
+  using T = TanShape<D, K>;
   constexpr int N = K + 1;
-  constexpr int T = (D == 3) ? K * N : K;     // tasks per face and pass
+  constexpr int TASKS = (D == 3) ? K * N : K;     // per face and pass
+  constexpr int ST = (D == 3) ? T::PITCH : 1;     // stride of pass 1
+  constexpr bool DOTS = D == 3 && !std::is_same<V, float>::value;
   const int u = threadIdx.x;
-  const bool task = u < fb * T;
-  const int tf = u / T, w = u - tf * T;
+  const bool task = u < fb * TASKS;
+  const int tf = u / TASKS, w = u - tf * TASKS;
   const int j = (D == 3) ? w / N : w, tr = (D == 3) ? w % N : 0;
-  if (task) {       // first pass: along t1 within the line t2 = tr (2D: the only pass)
-    V uu[N], yv[N];
+  __syncthreads();
+  if (task) {
+    V* p = &plane[tf][j][tr];
+    V uu[N];
 #pragma unroll
-    for (int q = 0; q < N; ++q) uu[q] = plane[tf][j][q + N * tr];
-    mass_line_eo<K, V>(c, uu, yv);
-    V (*dst)[K][L] = (D == 3) ? plane2 : plane;   // 2D: the task owns row j of its face's plane
+    for (int q = 0; q < N; ++q) uu[q] = p[ST * q];
+    Dot<V> acc = dot_first(c.ma[0], uu[0]);
 #pragma unroll
-    for (int i = 0; i < N; ++i) dst[tf][j][i + N * tr] = yv[i];
+    for (int q = 1; q < N; ++q) dot_fma(acc, c.ma[q], uu[q]);
+    const V s = dot_value(acc);
+#pragma unroll
+    for (int q = 0; q < N; ++q) p[ST * q] = vfma(c.mc[q], s, uu[q]);
   }
   __syncthreads();
   if constexpr (D == 3) {
-    if (task) {     // second pass: along t2 within the line t1 = tr
-      V uu[N], yv[N];
+    if (task) {
+      V* p = &plane[tf][j][T::PITCH * tr];
+      V uu[N];
 #pragma unroll
-      for (int q = 0; q < N; ++q) uu[q] = plane2[tf][j][tr + N * q];
-      mass_line_eo<K, V>(c, uu, yv);
+      for (int q = 0; q < N; ++q) uu[q] = p[q];
+      Dot<V> acc = dot_first(c.ma[0], uu[0]);
 #pragma unroll
-      for (int i = 0; i < N; ++i) plane[tf][j][tr + N * i] = yv[i];
+      for (int q = 1; q < N; ++q) dot_fma(acc, c.ma[q], uu[q]);
+      const V s = dot_value(acc);
+      if constexpr (DOTS) {
+        dots[tf][j][tr] = s;
+      } else {
+#pragma unroll
+        for (int q = 0; q < N; ++q) p[q] = vfma(c.mc[q], s, uu[q]);
+      }
     }
     __syncthreads();
   }
+  const V wt = tab.w[tau];
+  const V ct = DOTS ? tab.c[tau % N] : vzero<V>();
 #pragma unroll
-  for (int jj = 0; jj < K; ++jj) out[jj] = plane[fl][jj][tau];
+  for (int jj = 0; jj < K; ++jj) {
+    V v = plane[fl][jj][T::at(tau)];
+    if constexpr (DOTS) v = vfma(ct, dots[fl][jj][tau / N], v);
+    out[jj] = vmul(wt, v);
+  }
 }
 
 // Normal expansion w[b] = sum_j g_j[b] sj[j] (sj: the tangential results of the line):
@@ -251,9 +274,12 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
   using V = typename A::V;
   using IO = typename A::IO;
   constexpr int L = S::L, NN = S::NN, K1 = K + 1;
-  typedef V Plane[K][L];
-  Plane* buf = reinterpret_cast<Plane*>(dsm);            // [fb][K][L]
-  Plane* sb2 = buf + fb;                                  // [fb][K][L], 3D only
+  using T = TanShape<D, K>;
+  typedef V Plane[K][T::LP];
+  typedef V Dots[K][K1];
+  Plane* buf = reinterpret_cast<Plane*>(dsm);            // [fb][K][LP]
+  Dots* dots = reinterpret_cast<Dots*>(buf + fb);         // [fb][K][N], 3D only
+  __shared__ TanTable<D, K, V> tab;
   const int nt = (int)blockDim.x;
   // the lift may start its prologue as soon as every face CTA is running (programmatic
   // dependent launch; it waits for this grid's completion before it reads W)
@@ -288,6 +314,7 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
   const int fl = t / L, tau = t - fl * L;
   const int f = f0 + fl;
   const bool valid = f < fend;
+  fill_tan_table<D, K, V>(tab, c, t);
 
   // ---- gather this thread's normal line (2k+1 values)
   V v[NN];
@@ -314,11 +341,10 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
     V t[K];
     line_jumps<K, V>(v, gs, t);
 #pragma unroll
-    for (int j = 0; j < K; ++j) buf[fl][j][tau] = t[j];
+    for (int j = 0; j < K; ++j) buf[fl][j][T::at(tau)] = t[j];
   }
-  __syncthreads();
   V out[K];
-  line_tangential_eo<D, K, V, L>(buf, sb2, fb, c, fl, tau, out);
+  tangential_mass<D, K, V>(buf, dots, fb, c, tab, fl, tau, out);
 
   // ---- normal expansion W_F[b, tau] = sum_j g_j[b] s_j out[j], stored at tau + L b (the
   // lanes of a face store neighbouring values)

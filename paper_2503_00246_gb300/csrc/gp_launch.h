@@ -25,7 +25,7 @@ struct ApplyArgs {
   const int2* zruns = nullptr;
   int32_t nzruns = 0;        // zero runs to fill (0 for the add form)
   const double* g = nullptr; // host FP64: k x (2k+1)
-  const double* m = nullptr; // host FP64: (k+1)^2
+  const double* m = nullptr; // host FP64: the lumped mass, 3 (k+1) values (Plan::lump)
   const double* s = nullptr; // host FP64: k
   cudaEvent_t* ev = nullptr;  // optional: 3 events recorded around the two kernels
   Tiles tiles{};              // 0 fields: the defaults of default_tiles
@@ -277,9 +277,7 @@ cudaError_t run_apply(const ApplyArgs& Ar, cudaStream_t st) {
     c.s[j] = from_host<V>(Ar.s[j]);
     for (int b = 0; b < 2 * K + 1; ++b) c.gs[j][b] = from_host<V>(Ar.s[j] * Ar.g[j * (2 * K + 1) + b]);
   }
-  for (int p = 0; p < K + 1; ++p)
-    for (int q = 0; q < K + 1; ++q) c.m[p][q] = from_host<V>(Ar.m[p * (K + 1) + q]);
-  mass_halves<V, K>(Ar.m, c);
+  mass_consts<V, K>(Ar.m, c);
   if (Ar.brick) return run_brick<D, K, A>(Ar, c, st);
   Tiles t = Ar.tiles;
   if (!resolve_tiles<D, K, V>(t)) return cudaErrorInvalidConfiguration;
@@ -390,9 +388,7 @@ cudaError_t run_batch(const void* fsegs, const void* lsegs, const void* ptrs, in
   Consts<V, K> c;
   for (int j = 0; j < K; ++j)
     for (int b = 0; b < 2 * K + 1; ++b) c.g[j][b] = from_host<V>(g[j * (2 * K + 1) + b]);
-  for (int p = 0; p < K + 1; ++p)
-    for (int q = 0; q < K + 1; ++q) c.m[p][q] = from_host<V>(m[p * (K + 1) + q]);
-  mass_halves<V, K>(m, c);
+  mass_consts<V, K>(m, c);
   for (int j = 0; j < K; ++j) {
     c.s[j] = vzero<V>();                                          // per segment: FaceSeg::s
     for (int b = 0; b < 2 * K + 1; ++b) c.gs[j][b] = vzero<V>();  // per segment: FaceSeg::gs

@@ -148,6 +148,48 @@ void reference_1d(int k, const std::vector<double>& /*gl*/, std::vector<double>&
     }
 }
 
+// Gauss-Lobatto quadrature with weights w integrates l_a l_b up to the error of its x^(2k) term:
+//   M^ = diag(w) - E a a^T,  a_i = prod_{j != i} 1 / (x_i - x_j) the leading coefficients,
+// with E the error for x^(2k) on [0, 1].  For the Legendre polynomial P_k on [-1, 1] the rule gives
+// 2/k for the integral of P_k^2 and the integral is 2/(2k+1), and P_k has the leading coefficient
+// c = (2k)! / (2^k k!^2), so E = (2/k - 2/(2k+1)) / c^2 / 2 / 4^k.  k = 1 has the equal form
+// diag(1/6) (I + 1 1^T), whose terms are all positive.
+bool lumped_mass(int k, const std::vector<double>& mass, std::vector<double>& lump) {
+  const int N = k + 1;
+  std::vector<R> gl, a(N, R(1)), w(N);
+  gauss_lobatto_01_r(k, gl);
+  R E = 0, amax = 0;
+  if (k == 1) {
+    w[0] = w[1] = R(1) / 6;
+    E = -R(1) / 6;
+    amax = 1;
+  } else {
+    R c = 1;
+    for (int i = 1; i <= k; ++i) c *= R(k + i) / (2 * R(i));
+    E = (R(2) / k - R(2) / (2 * k + 1)) / (c * c) / 2;
+    for (int i = 0; i < k; ++i) E /= 4;
+    for (int i = 0; i < N; ++i) {
+      R p, dp;
+      legendre(k, 2 * gl[i] - 1, p, dp);
+      w[i] = 1 / (R(k) * (k + 1) * p * p);
+      for (int j = 0; j < N; ++j)
+        if (j != i) a[i] /= (gl[i] - gl[j]);
+      amax = std::max(amax, std::fabs(a[i]));
+    }
+  }
+  lump.assign(3 * N, 0.0);
+  for (int i = 0; i < N; ++i) {
+    lump[i] = (double)(a[i] / amax);
+    lump[N + i] = (double)(-E * a[i] * amax / w[i]);
+    lump[2 * N + i] = (double)w[i];
+  }
+  R dev = 0;
+  for (int i = 0; i < N; ++i)
+    for (int j = 0; j < N; ++j)
+      dev = std::max(dev, std::fabs((i == j ? w[i] : R(0)) - E * a[i] * a[j] - R(mass[i * N + j])));
+  return dev <= R(1e-15);
+}
+
 // Macro-patch stabilisation (the alternative named in Sec. 2.2): on the two-cell patch
 // [0,1] u [1,2] of a face, the difference between the polynomial on one cell and the
 // extension of the neighbour's polynomial into it, squared and integrated over both cells:
@@ -1088,6 +1130,7 @@ gp_status build_plan(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* 
   // ---- 1D reference data and the per-order scale c_j h^(d-2)
   gauss_lobatto_01(k, p.gl);
   reference_1d(k, p.gl, p.mass, p.jumps);
+  if (!lumped_mass(k, p.mass, p.lump)) { err = "internal: the lumped form misses the reference mass"; return GP_EINVAL; }
   reference_stiffness(k, p.stiff);
   p.scale.resize(k);
   p.stabilization = opts->stabilization;

@@ -113,6 +113,7 @@ struct Plan {
   std::vector<double> gl;         // k+1 Gauss-Lobatto points on [0,1]
   std::vector<double> stiff;      // (k+1)^2: int_0^1 l_a' l_b' 
   std::vector<double> mass;       // (k+1)^2
+  std::vector<double> lump;       // 3 (k+1): ma, mc, mw with mass = diag(mw) (I + mc ma^T)
   std::vector<double> jumps;      // k x (2k+1)
   std::vector<double> scale;      // k: c_j h^(dim-2) (macro patch: gamma lambda_j h^dim)
   int stabilization = GP_STAB_GHOST;
@@ -139,6 +140,8 @@ gp_status partition_slabs(const gp_mesh* mesh, const gp_levelset* ls, const gp_o
 void gauss_lobatto_01(int k, std::vector<double>& x);
 void reference_1d(int k, const std::vector<double>& gl, std::vector<double>& mass,
                   std::vector<double>& jumps);
+// The lumped form of the mass matrix (see Plan::lump); false if it does not reproduce `mass`.
+bool lumped_mass(int k, const std::vector<double>& mass, std::vector<double>& lump);
 void reference_stiffness(int k, std::vector<double>& stiff);
 // Macro-patch 1D data: k mirror-(anti)symmetric vectors (k x (2k+1)) and weights lambda_j;
 // false if the matrix is not of rank k with the expected parities.
