@@ -171,12 +171,12 @@ cudaError_t upload(T** dst, const std::vector<T>& src) {
 }
 
 void free_device(gp_ctx* c) {
-  void* ptrs[] = {c->d_frows, c->d_lwin, c->d_lrow, c->d_zruns, c->d_tp, c->d_xh, c->d_yh, c->d_truns,
+  void* ptrs[] = {c->d_frows, c->d_lwin, c->d_lrow, c->d_lmask, c->d_zruns, c->d_tp, c->d_xh, c->d_yh, c->d_truns,
                   c->d_bdesc, c->d_bcell, c->d_bccoord, c->d_bface, c->d_rowtab,
                   c->d_pnode, c->d_poff, c->d_pslot, c->d_part};
   for (void* p : ptrs)
     if (p) cudaFree(p);
-  c->d_frows = c->d_lwin = c->d_lrow = nullptr;
+  c->d_frows = c->d_lwin = c->d_lrow = c->d_lmask = nullptr;
   c->d_zruns = nullptr;
   c->d_tp = c->d_xh = c->d_yh = nullptr;
   c->d_truns = nullptr;
@@ -208,7 +208,7 @@ void free_device(gp_ctx* c) {
 }  // namespace
 
 gp_status gpi::launch(gp_ctx* c, const void* x, void* y, int add, cudaStream_t st, void* scratch, bool trace,
-                      const gp::Tiles* tiles, int which, const SlabRun* run) {
+                      const gp::Tiles* tiles, int which, const SlabRun* run, bool full_outputs) {
   const gp::Plan& p = c->plan;
   const bool brick = c->use_brick && which == 3;
   if (!scratch && p.num_faces() > 0 && (brick ? (!c->d_part && p.num_plane_nodes() > 0) : !c->d_tp))
@@ -227,6 +227,7 @@ gp_status gpi::launch(gp_ctx* c, const void* x, void* y, int add, cudaStream_t s
   for (int i = 0; i < 4; ++i) a.fstart[i] = p.fstart[i];
   a.la.lwin = c->d_lwin;
   a.la.lrow = c->d_lrow;
+  a.la.lmask = c->d_lmask;
   a.la.nlift = (int32_t)p.num_lift_cells();
   a.la.n_active = (int32_t)p.n_active;
   a.zruns = c->d_zruns;
@@ -248,6 +249,7 @@ gp_status gpi::launch(gp_ctx* c, const void* x, void* y, int add, cudaStream_t s
   a.ev = ev;
   a.tiles = tiles ? *tiles : c->tiles;
   a.which = which;
+  a.full_outputs = full_outputs;
   a.slabs = run ? run->table : p.slabs.data();
   a.nslab = run ? run->n : p.num_slabs();
   a.slab_events = run ? run->events : nullptr;
@@ -386,6 +388,7 @@ gp_status gp_setup(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* op
     if (e == cudaSuccess) e = upload(&c->d_frows, p.frows);
     if (e == cudaSuccess) e = upload(&c->d_lwin, p.lwin);
     if (e == cudaSuccess) e = upload(&c->d_lrow, p.lrow);
+    if (e == cudaSuccess) e = upload(&c->d_lmask, p.lmask);
     if (e == cudaSuccess) e = upload(&c->d_zruns, zruns);
     const size_t vbytes = p.precision == GP_FP32 ? 4 : 8;
     if (c->use_brick) {
@@ -824,6 +827,7 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
       sp.fa.nzruns = (int32_t)pl.num_zero_runs();
       sp.la.lwin = c->d_lwin;
       sp.la.lrow = c->d_lrow;
+      sp.la.lmask = c->d_lmask;
       sp.la.nlift = (int32_t)pl.num_lift_cells();
       sp.la.n_active = (int32_t)pl.n_active;
       sp.wp = (char*)b->d_w + woff[gi][i];

@@ -16,6 +16,7 @@ struct gp_ctx {
   int32_t* d_frows = nullptr;
   int32_t* d_lwin = nullptr;
   int32_t* d_lrow = nullptr;
+  int32_t* d_lmask = nullptr;
   int2* d_zruns = nullptr;
   void* d_tp = nullptr;          // per-face outputs W_F (scratch of the face + lift path)
   // brick path (gp_brick.cuh): tables and the partial grids of the plane nodes (scratch)
@@ -76,7 +77,8 @@ gp_status fail(const gp_ctx* c, gp_status s, const std::string& m);
 // Enqueues y = G x (add = 0) or y += G x (add = 1) for context c; `scratch` replaces the
 // context's face-output buffer when given; `trace` = false never records events.
 // `tiles` overrides the context's tile shape; `which` (bit 0 face, bit 1 lift) drops a
-// kernel (the autotuner times them apart).
+// kernel (the autotuner times them apart); `full_outputs` makes a face launch store W_F in every
+// arithmetic (the model system's gather reads it).
 // A slab pipeline for one launch: a slab table (SLAB ints per slab) and an event per slab.
 struct SlabRun {
   const int32_t* table = nullptr;
@@ -85,7 +87,8 @@ struct SlabRun {
   cudaEvent_t* inputs = nullptr;   // waited for before each slab's face launch (or nullptr)
 };
 gp_status launch(gp_ctx* c, const void* x, void* y, int add, cudaStream_t st, void* scratch = nullptr,
-                 bool trace = true, const gp::Tiles* tiles = nullptr, int which = 3, const SlabRun* run = nullptr);
+                 bool trace = true, const gp::Tiles* tiles = nullptr, int which = 3, const SlabRun* run = nullptr,
+                 bool full_outputs = false);
 
 // Slab pipeline of the face + lift path (gp_opts.slabs): at most MAX_SLABS slabs.
 static_assert(gp::SLAB == gp::SLAB_INTS, "the plan's and the launcher's slab records differ");

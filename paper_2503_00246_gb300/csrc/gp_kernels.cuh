@@ -101,6 +101,7 @@ constexpr int ZGROUP = 16;  // zero runs per zero-fill CTA
 struct LiftArgs {
   const int32_t* lwin;    // [nlift][NW] candidate face ids of each owner cell (-1 if none)
   const int32_t* lrow;    // [nlift][KR] compact index of node (ci k, cj k + q, cl k + r)
+  const int32_t* lmask;   // [nlift] which nodes a ghost face reaches (see Plan::lmask)
   int32_t nlift;
   int32_t n_active;
 };
@@ -259,13 +260,38 @@ __device__ __forceinline__ void line_expand(const Consts<V, K>& c, const V (&sj)
   }
 }
 
+// ------------------------------------------------------- compact face outputs --
+// The face kernel stores either the (2k+1) L values W_F[b][tau] of every face or only the k L
+// tangential results T_F[tau][j] behind them (k padded to KP for vector accesses), which the lift
+// then expands along the normal for k nodes at once (lift_lines_body): 2.25 times fewer bytes at
+// k = 4 and one vector access per line instead of 2k + 1.
+template <int K, typename V>
+struct Compact {
+  static constexpr int KP = (K == 3) ? 4 : (K == 5) ? 6 : (K == 7) ? 8 : K;
+  static constexpr int VW = (sizeof(V) == 4 && KP % 4 == 0) ? 4 : (KP % 2 == 0) ? 2 : 1;   // values per access
+  static_assert(KP <= 2 * K + 1, "compact outputs must fit the face-output buffer");
+};
+template <int VW, typename V>
+struct alignas(VW * sizeof(V)) Chunk {
+  V v[VW];
+};
+// FP32 stores T_F: both of its kernels were bound by L1 wavefronts (68% and 65% of their peak) and
+// moved 1.11 GB per apply of the 128^3 gyroid at k = 4, 0.79 GB now: apply 306 -> 256 us (face kernel
+// 187 -> 158 us, lift 117 -> 104 us).
+// FP64 stores W_F: the expansion and its FP64 adds cost the same operations either way, and W_F
+// hides under the FP64 pipe.
+template <typename V>
+struct StoreCompact {
+  static constexpr bool value = std::is_same<V, float>::value;
+};
+
 // ----------------------------------------------------------------- face --
 // One thread per (face, normal line tau); fb faces per CTA (blockDim.x = fb L).
 // `blk` is the CTA's index within its problem; `gs` holds the jump vectors of the first step
 // (FP64, float-float: the scaled s_j g_j, c.gs or a batch segment's copy in shared memory;
 // FP32: the plain c.g) and `sc` the k factors s_j (FP32 only); `dsm` is the
-// face_smem<D, K, V>(fb) bytes of dynamic shared memory.
-template <int D, int K, class A>
+// face_smem<D, K, V>(fb) bytes of dynamic shared memory.  COMPACT: store T_F instead of W_F.
+template <int D, int K, class A, bool COMPACT>
 __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, typename A::V* __restrict__ wp,
                                           typename A::IO* __restrict__ y, const FaceArgs& fa,
                                           const Consts<typename A::V, K>& c, const typename A::V (*gs)[2 * K + 1],
@@ -346,14 +372,29 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
   V out[K];
   tangential_mass<D, K, V>(buf, dots, fb, c, tab, fl, tau, out);
 
-  // ---- normal expansion W_F[b, tau] = sum_j g_j[b] s_j out[j], stored at tau + L b (the
-  // lanes of a face store neighbouring values)
-  if (valid) {
-    V* dst = wp + (size_t)f * S::P + tau;
-    if constexpr (!FoldScale<V>::value) {
+  if (!valid) return;
+  if constexpr (!FoldScale<V>::value) {
 #pragma unroll
-      for (int j = 0; j < K; ++j) out[j] = vmul(sc[j], out[j]);
+    for (int j = 0; j < K; ++j) out[j] = vmul(sc[j], out[j]);
+  }
+  if constexpr (COMPACT) {
+    using CP = Compact<K, V>;
+    using Ch = Chunk<CP::VW, V>;
+    Ch* dst = reinterpret_cast<Ch*>(wp + ((size_t)f * L + tau) * CP::KP);
+#pragma unroll
+    for (int i = 0; i < CP::KP / CP::VW; ++i) {
+      Ch ch;
+#pragma unroll
+      for (int e = 0; e < CP::VW; ++e) {
+        const int j = i * CP::VW + e;
+        ch.v[e] = j < K ? out[j < K ? j : 0] : vzero<V>();
+      }
+      dst[i] = ch;
     }
+  } else {
+    // ---- normal expansion W_F[b, tau] = sum_j g_j[b] s_j out[j], stored at tau + L b (the
+    // lanes of a face store neighbouring values)
+    V* dst = wp + (size_t)f * S::P + tau;
     V w[NN];
     line_expand<K, V>(c, out, w);
 #pragma unroll
@@ -363,12 +404,12 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
 
 extern __shared__ __align__(16) unsigned char gp_dyn_smem[];
 
-template <int D, int K, class A>
+template <int D, int K, class A, bool COMPACT>
 __global__ void __launch_bounds__(MAX_CTA_THREADS)
 face_kernel(const typename A::IO* __restrict__ x, typename A::V* __restrict__ wp,
             typename A::IO* __restrict__ y, const FaceArgs fa, const int fb,
             const __grid_constant__ Consts<typename A::V, K> c) {
-  face_body<D, K, A>(x, wp, y, fa, c, FoldScale<typename A::V>::value ? c.gs : c.g, c.s, blockIdx.x, fb, gp_dyn_smem);
+  face_body<D, K, A, COMPACT>(x, wp, y, fa, c, FoldScale<typename A::V>::value ? c.gs : c.g, c.s, blockIdx.x, fb, gp_dyn_smem);
   if (fa.tail_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
@@ -426,9 +467,9 @@ face_kernel_batched(const FaceSeg<typename A::V, K>* __restrict__ segs, const in
   if constexpr (FoldScale<V>::value) {
     for (int i = threadIdx.x; i < K * (2 * K + 1); i += blockDim.x) sg[i / (2 * K + 1)][i % (2 * K + 1)] = seg.gs[i];
     __syncthreads();
-    face_body<D, K, A>(sp.x, seg.wp, sp.y, seg.fa, c, sg, seg.s, (int)blockIdx.x - seg.block0, fb, gp_dyn_smem);
+    face_body<D, K, A, StoreCompact<V>::value>(sp.x, seg.wp, sp.y, seg.fa, c, sg, seg.s, (int)blockIdx.x - seg.block0, fb, gp_dyn_smem);
   } else {
-    face_body<D, K, A>(sp.x, seg.wp, sp.y, seg.fa, c, c.g, seg.s, (int)blockIdx.x - seg.block0, fb, gp_dyn_smem);
+    face_body<D, K, A, StoreCompact<V>::value>(sp.x, seg.wp, sp.y, seg.fa, c, c.g, seg.s, (int)blockIdx.x - seg.block0, fb, gp_dyn_smem);
   }
 }
 
@@ -647,6 +688,224 @@ __device__ __forceinline__ void lift_body(const typename A::V* __restrict__ wp, 
       y[idx] = to_io(outv, (IO*)nullptr);
     }
   }
+}
+
+// ------------------------------------------------------- lift of compact outputs --
+// With T_F stored, a node needs sum_j g_j[b] T_F[tau][j] of every face that holds it: k values per
+// contribution, unless the k nodes of a normal line share them.  So the lift walks the owner cell's
+// lines along each axis in turn: phase a gives every line (p_t1, p_t2) along a to one thread, which
+// adds the T_F of the faces that share the line (up to four where p_t1 or p_t2 is 0), for the owner
+// as K- (s_a = 2, b = p), K+ (s_a = 1, b = p + k) and end node (s_a = 0, b = 2k, p = 0 only), and
+// expands them onto its k nodes.  The nodes' sums pass from phase to phase through shared memory;
+// the last phase writes y with x-contiguous lanes.  One vector load (k = 4: 16 bytes per lane, the
+// lanes of a face contiguous) replaces k loads of W_F.  Each node sums its contributions in one
+// fixed order, whatever the tile shape.
+template <int D, int K>
+struct LineShape {
+  static constexpr int KR = LiftShape<D, K>::KR;            // lines per owner and axis
+  // node (p, q, r) at p + K q + PZ r: a padded plane stride keeps the lanes of a y line apart
+  static constexpr int PZ = K * K + (K % 2 == 0 ? K : 0);
+  static constexpr int OS = (D == 3) ? PZ * K : K * K;      // nodes' sums per owner
+  // resident CTAs of 512 threads to compile for: k = 4 is held to 32 registers (0: the compiler's
+  // own choice, 40 to 64 registers; holding those too makes it spill)
+  static constexpr int CTAS = (K == 4) ? 4 : 0;
+};
+template <int D, int K, typename V>
+__host__ __device__ constexpr size_t lift_lines_smem(int cb) {
+  return (size_t)cb * (LiftShape<D, K>::NW + LineShape<D, K>::KR + 1) * sizeof(int) +
+         (size_t)cb * LineShape<D, K>::OS * sizeof(Sum<V>);
+}
+// Owner cells per CTA that fit the dynamic shared memory (a tile may ask for more).
+template <int D, int K, typename V>
+constexpr int lift_lines_cells(int cb) {
+  constexpr size_t per = (LiftShape<D, K>::NW + LineShape<D, K>::KR + 1) * sizeof(int) +
+                         LineShape<D, K>::OS * sizeof(Sum<V>);
+  constexpr int most = (int)(MAX_DYN_SMEM / per);
+  return cb < most ? cb : most;
+}
+
+// acc[p] += the faces of normal AX on a line of an owner cell.  The line's type M (bit 0: t1 == 0,
+// bit 1: t2 == 0; 3D) fixes at compile time which of the up to four candidate faces per s_a can
+// share it.  `line` points at the T_F of tangential index (t1, t2) of face 0.
+template <int D, int K, typename V, int AX, int M>
+__device__ __forceinline__ void lift_line(const V* __restrict__ line, const int* win, const Consts<V, K>& c,
+                                          Sum<V> (&acc)[K]) {
+  using CP = Compact<K, V>;
+  using Ch = Chunk<CP::VW, V>;
+  constexpr int K1 = K + 1, L = Shape<D, K>::L, NS = (D == 3) ? 4 : 2, NCH = (K + CP::VW - 1) / CP::VW;
+  // the sums over the faces that share the line, for the owner as K- (s_a = 2), K+ and end node.
+  // AHEAD: every load before the first use of one (96^3 ball at k = 5: 52.6 -> 49.4 us); for small
+  // k the registers of that cost more resident warps than it gains (k = 4: 104 against 108 us, with
+  // the kernel held to 32 registers).
+  constexpr bool AHEAD = K >= 5;
+  V s[3][K];
+  bool any[3];
+  auto expand = [&](const int sa) {
+    if (!any[sa]) return;
+#pragma unroll
+    for (int j = 0; j < K; ++j)
+#pragma unroll
+      for (int p = 0; p < (sa == 0 ? 1 : K); ++p) dot_fma(acc[p], c.g[j][p + (2 - sa) * K], s[sa][j]);
+  };
+#pragma unroll
+  for (int sa = 2; sa >= 0; --sa) {
+    // the window's order (s_1, s_2): (0,0) (0,1) (1,0) (1,1); 2D: s_1 = 0, 1
+    any[sa] = false;
+#pragma unroll
+    for (int u = NS - 1; u >= 0; --u) {
+      const int s1 = (D == 3) ? u >> 1 : u, s2 = (D == 3) ? u & 1 : 1;
+      if ((s1 == 0 && !(M & 1)) || (s2 == 0 && !(M & 2))) continue;
+      const int f = win[AX * 3 * NS + sa * NS + u];
+      const bool ok = f >= 0;
+      any[sa] = any[sa] || ok;
+      const Ch* src = reinterpret_cast<const Ch*>(line + (int64_t)f * (L * CP::KP) +
+                                                  ((1 - s1) * K + (1 - s2) * K * K1) * CP::KP);
+      Ch ch[NCH];
+#pragma unroll
+      for (int i = 0; i < NCH; ++i) {
+#pragma unroll
+        for (int e = 0; e < CP::VW; ++e) ch[i].v[e] = vzero<V>();
+        if (ok) ch[i] = src[i];
+      }
+#pragma unroll
+      for (int j = 0; j < K; ++j) {
+        const V v = ch[j / CP::VW].v[j % CP::VW];
+        s[sa][j] = (u == NS - 1) ? v : vadd(s[sa][j], v);
+      }
+    }
+    if constexpr (!AHEAD) expand(sa);
+  }
+  if constexpr (AHEAD) {
+#pragma unroll
+    for (int sa = 2; sa >= 0; --sa) expand(sa);
+  }
+}
+
+// Walks the lines of type M along AX of the CTA's nc owner cells, from item g (the nc count(M) items
+// of the type start at `first`) in steps of blockDim.x.  The nodes' sums are read from acc (unless
+// AX == 0, the first phase) and written back, or handed to out(ci, t1, t2, sums) in the last phase.
+template <int D, int K, class A, int AX, int M, class Out>
+__device__ __forceinline__ void lift_lines(int& g, const int first, const typename A::V* __restrict__ tp, const int* win,
+                                           const Consts<typename A::V, K>& c, Sum<typename A::V>* acc, const int nc,
+                                           Out out) {
+  using S = LiftShape<D, K>;
+  using LS = LineShape<D, K>;
+  using V = typename A::V;
+  constexpr int PZ = LS::PZ, KP = Compact<K, V>::KP, CNT = S::count(M);
+  // strides of the sums along the line and along its two tangential axes
+  constexpr int ST = (AX == 0) ? 1 : (AX == 1) ? K : PZ;
+  constexpr int S1 = (AX == 0) ? K : 1, S2 = (AX == 2) ? K : PZ;
+  if constexpr (CNT > 0) {
+    for (; g < first + nc * CNT; g += (int)blockDim.x) {
+      const unsigned local = (unsigned)(g - first);
+      const int ci = (int)(local / CNT);
+      const unsigned rem = local - (unsigned)ci * CNT;
+      constexpr unsigned K0 = K > 1 ? K - 1 : 1;
+      const int t1 = (M & 1) ? 0 : 1 + (int)(rem % K0);
+      const int t2 = (D == 2 || (M & 2)) ? 0 : 1 + (int)((M & 1) ? rem : rem / K0);
+      Sum<V>* a = acc + ci * LS::OS + S1 * t1 + ((D == 3) ? S2 * t2 : 0);
+      Sum<V> s[K];
+#pragma unroll
+      for (int p = 0; p < K; ++p) s[p] = (AX == 0) ? sum_zero<V>() : a[p * ST];
+      lift_line<D, K, V, AX, M>(tp + (t1 + ((D == 3) ? (K + 1) * t2 : 0)) * KP, win + ci * S::NW, c, s);
+      if constexpr (AX == D - 1) {
+        out(ci, t1, t2, s);
+      } else {
+#pragma unroll
+        for (int p = 0; p < K; ++p) a[p * ST] = s[p];
+      }
+    }
+  }
+}
+
+// One phase: the lines along AX ordered by type, so that a warp's lanes mostly take one path (whole
+// owners per warp, with the warp's own barriers, took 125 us against 104: each warp ran every path).
+template <int D, int K, class A, int AX, class Out>
+__device__ __forceinline__ void lift_phase(const typename A::V* __restrict__ tp, const int* win,
+                                           const Consts<typename A::V, K>& c, Sum<typename A::V>* acc, const int nc,
+                                           Out out) {
+  using S = LiftShape<D, K>;
+  int g = (int)threadIdx.x, first = 0;
+  lift_lines<D, K, A, AX, 0>(g, first, tp, win, c, acc, nc, out);
+  first += nc * S::count(0);
+  lift_lines<D, K, A, AX, 1>(g, first, tp, win, c, acc, nc, out);
+  if constexpr (D == 3) {
+    first += nc * S::count(1);
+    lift_lines<D, K, A, AX, 2>(g, first, tp, win, c, acc, nc, out);
+    first += nc * S::count(2);
+    lift_lines<D, K, A, AX, 3>(g, first, tp, win, c, acc, nc, out);
+  }
+}
+
+template <int D, int K, class A>
+__device__ __forceinline__ void lift_lines_body(const typename A::V* __restrict__ tp, typename A::IO* __restrict__ y,
+                                                const int add, const LiftArgs& la, const Consts<typename A::V, K>& c,
+                                                const int blk, const int cb, unsigned char* dsm) {
+  using LS = LineShape<D, K>;
+  using V = typename A::V;
+  using IO = typename A::IO;
+  constexpr int NW = LiftShape<D, K>::NW, KR = LS::KR, OS = LS::OS;
+  Sum<V>* acc = reinterpret_cast<Sum<V>*>(dsm);                     // [cb][OS]
+  int* win = reinterpret_cast<int*>(dsm + (size_t)cb * OS * sizeof(Sum<V>));   // [cb][NW]
+  int* row = win + cb * NW;                                         // [cb][KR]
+  int* mask = row + cb * KR;                                        // [cb]
+  const int cell0 = blk * cb;
+  const int nc = min(cb, la.nlift - cell0);
+  const int t = threadIdx.x, nt = (int)blockDim.x;
+  for (int i = t; i < nc * NW; i += nt) win[i] = __ldg(la.lwin + (size_t)cell0 * NW + i);
+  for (int i = t; i < nc * KR; i += nt) row[i] = __ldg(la.lrow + (size_t)cell0 * KR + i);
+  for (int i = t; i < nc; i += nt) mask[i] = __ldg(la.lmask + cell0 + i);
+  __syncthreads();
+  // wait for the face kernel (a no-op unless launched as its programmatic dependent), and let a
+  // programmatic dependent of this grid start
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;");
+  auto none = [](int, int, int, const Sum<V>(&)[K]) {};
+  lift_phase<D, K, A, 0>(tp, win, c, acc, nc, none);
+  __syncthreads();
+  if constexpr (D == 3) {
+    lift_phase<D, K, A, 1>(tp, win, c, acc, nc, none);
+    __syncthreads();
+  }
+  // the last axis: line (p, q) in 3D, p in 2D; its k nodes are complete
+  lift_phase<D, K, A, D - 1>(tp, win, c, acc, nc, [&](const int ci, const int p, const int q, const Sum<V>(&s)[K]) {
+    // bit (p > 0) + 2 (q > 0) + 4 (r > 0) of the owner's mask: a face reaches the nodes of that kind
+    const int m = mask[ci] >> ((p > 0 ? 1 : 0) + ((D == 3 && q > 0) ? 2 : 0));
+    constexpr int UP = (D == 3) ? 4 : 2, SR = (D == 3) ? K : 1;
+    const int* rw = row + ci * KR + q;
+#pragma unroll
+    for (int r = 0; r < K; ++r) {
+      if (!((m >> (r > 0 ? UP : 0)) & 1)) continue;
+      IO* dst = y + (rw[SR * r] + p);
+      const V sv = dot_value(s[r]);
+      *dst = to_io(add ? vadd(from_io(*dst, (V*)nullptr), sv) : sv, (IO*)nullptr);
+    }
+  });
+}
+
+template <int D, int K, class A>
+__global__ void __launch_bounds__(MAX_CTA_THREADS, LineShape<D, K>::CTAS)
+lift_lines_kernel(const typename A::V* __restrict__ tp, typename A::IO* __restrict__ y, const int add,
+                  const LiftArgs la, const int cb, const __grid_constant__ Consts<typename A::V, K> c) {
+  lift_lines_body<D, K, A>(tp, y, add, la, c, blockIdx.x, cb, gp_dyn_smem);
+}
+
+template <int D, int K, class A>
+__global__ void __launch_bounds__(MAX_CTA_THREADS, LineShape<D, K>::CTAS)
+lift_lines_kernel_batched(const LiftSeg* __restrict__ segs, const FaceSeg<typename A::V, K>* __restrict__ fsegs,
+                          const int nseg, const SegPtrs<typename A::IO>* __restrict__ ptrs, const int cb,
+                          const __grid_constant__ Consts<typename A::V, K> c) {
+  __shared__ LiftSeg seg;
+  __shared__ typename A::V* tp;
+  __shared__ typename A::IO* y;
+  if (threadIdx.x == 0) {
+    const int s = find_segment(segs, nseg, (int)blockIdx.x);
+    seg = segs[s];
+    tp = fsegs[s].wp;
+    y = ptrs[s].y;
+  }
+  __syncthreads();
+  lift_lines_body<D, K, A>(tp, y, 0, seg.la, c, (int)blockIdx.x - seg.block0, cb, gp_dyn_smem);
 }
 
 template <int D, int K, class A>

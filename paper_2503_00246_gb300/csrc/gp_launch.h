@@ -30,6 +30,8 @@ struct ApplyArgs {
   cudaEvent_t* ev = nullptr;  // optional: 3 events recorded around the two kernels
   Tiles tiles{};              // 0 fields: the defaults of default_tiles
   int which = 3;              // bit 0: face kernel, bit 1: lift kernel (the autotuner times them apart)
+  bool full_outputs = false;  // the face kernel stores W_F whatever its arithmetic (the model system's gather
+                              // reads it); only with which = 1
   const int32_t* slabs = nullptr;  // host: SLAB ints per slab (see Plan::slabs); nslab > 1: slab pipeline
   int nslab = 0;
   cudaEvent_t* slab_events = nullptr;  // host, nslab events: recorded after each slab's lift (the
@@ -41,13 +43,24 @@ struct ApplyArgs {
   PlaneArgs pa{};             // plane-fixup tables
 };
 
-// Default tile shape: about 256 threads per CTA, one item per thread.
-template <int D, int K>
+// Default tile shape: about 256 threads per CTA, one item per thread.  Compact outputs in 3D: face
+// CTAs of about 160 threads (more CTAs per SM to run while one waits at a barrier; 128^3 gyroid,
+// k = 4, face kernel with 2 / 5 / 6 / 10 / 20 faces: 238 / 162 / 159 / 164 / 199 us), and from
+// k = 4 on two to four lines per lift thread (inner lines first, then edge lines with more faces, so
+// that the warps meet at the barriers; 128^3 gyroid with 1 / 2 / 4 lines: 152 / 104 / 150 us; 49^3
+// ball at k = 8, 128 threads, with 1 / 2 / 4 / 8: 102 / 56 / 49 / 61 us).
+template <int D, int K, typename V>
 Tiles default_tiles_t() {
+  constexpr bool CO = StoreCompact<V>::value && D == 3;
   Tiles t;
-  t.fb = Shape<D, K>::FB;
+  t.fb = CO ? (160 / Shape<D, K>::L > 0 ? 160 / Shape<D, K>::L : 1) : Shape<D, K>::FB;
   t.lcb = LiftShape<D, K>::CB;
   t.lnt = LiftShape<D, K>::NT;
+  if (CO && K == 4) t.lcb = 32;
+  if (CO && K >= 5) {
+    t.lcb = K <= 6 ? 16 : 8;
+    t.lnt = 128;
+  }
   return t;
 }
 
@@ -56,7 +69,7 @@ Tiles default_tiles_t() {
 // shared memory <= MAX_DYN_SMEM).  Returns false if t is out of range.
 template <int D, int K, typename V>
 bool resolve_tiles(Tiles& t) {
-  const Tiles d = default_tiles_t<D, K>();
+  const Tiles d = default_tiles_t<D, K, V>();
   if (t.fb == 0) t.fb = d.fb;
   if (t.lcb == 0) t.lcb = d.lcb;
   if (t.lnt == 0) t.lnt = d.lnt;
@@ -84,14 +97,14 @@ TileOps tile_ops_ff_d3();
   TileOps ops;                                                                                \
   ops.defaults = [](int k) -> Tiles {                                                         \
     switch (k) {                                                                              \
-      case 1: return default_tiles_t<D, 1>();                                                 \
-      case 2: return default_tiles_t<D, 2>();                                                 \
-      case 3: return default_tiles_t<D, 3>();                                                 \
-      case 4: return default_tiles_t<D, 4>();                                                 \
-      case 5: return default_tiles_t<D, 5>();                                                 \
-      case 6: return default_tiles_t<D, 6>();                                                 \
-      case 7: return default_tiles_t<D, 7>();                                                 \
-      default: return default_tiles_t<D, 8>();                                                \
+      case 1: return default_tiles_t<D, 1, typename A::V>();                                                 \
+      case 2: return default_tiles_t<D, 2, typename A::V>();                                                 \
+      case 3: return default_tiles_t<D, 3, typename A::V>();                                                 \
+      case 4: return default_tiles_t<D, 4, typename A::V>();                                                 \
+      case 5: return default_tiles_t<D, 5, typename A::V>();                                                 \
+      case 6: return default_tiles_t<D, 6, typename A::V>();                                                 \
+      case 7: return default_tiles_t<D, 7, typename A::V>();                                                 \
+      default: return default_tiles_t<D, 8, typename A::V>();                                                \
     }                                                                                         \
   };                                                                                          \
   ops.resolve = [](int k, Tiles& t) -> bool {                                                 \
@@ -191,6 +204,37 @@ cudaError_t launch_pdl(void (*kernel)(P...), int grid, int threads, size_t smem,
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// Owner cells per lift CTA and dynamic shared memory of the lift kernel of this arithmetic.
+template <int D, int K, typename V>
+int lift_cells(const Tiles& t) {
+  if constexpr (StoreCompact<V>::value) return lift_lines_cells<D, K, V>(t.lcb);
+  else return t.lcb;
+}
+template <int D, int K, typename V>
+size_t lift_dyn_smem(int cb) {
+  if constexpr (StoreCompact<V>::value) return lift_lines_smem<D, K, V>(cb);
+  else return lift_smem<D, K>(cb);
+}
+
+// Launches the lift of the owners la, as a programmatic dependent of the kernel before it (pdl)
+// or in plain stream order.
+template <int D, int K, class A>
+cudaError_t launch_lift(bool pdl, const Tiles& t, const typename A::V* w, typename A::IO* y, int add,
+                        const LiftArgs& la, const Consts<typename A::V, K>& c, cudaStream_t st) {
+  using V = typename A::V;
+  const int cb = lift_cells<D, K, V>(t);
+  const int nlb = (la.nlift + cb - 1) / cb;
+  const size_t smem = lift_dyn_smem<D, K, V>(cb);
+  if constexpr (StoreCompact<V>::value) {
+    if (pdl) return launch_pdl(lift_lines_kernel<D, K, A>, nlb, t.lnt, smem, st, w, y, add, la, cb, c);
+    lift_lines_kernel<D, K, A><<<nlb, t.lnt, smem, st>>>(w, y, add, la, cb, c);
+  } else {
+    if (pdl) return launch_pdl(lift_kernel<D, K, A>, nlb, t.lnt, smem, st, w, y, add, la, cb);
+    lift_kernel<D, K, A><<<nlb, t.lnt, smem, st>>>(w, y, add, la, cb);
+  }
+  return cudaGetLastError();
+}
+
 // The face + lift path as a pipeline of slabs along the last axis, so that the face outputs of a
 // slab are still in L2 when its lift reads them: face(0), lift(0), face(1), lift(1), ...  Slab s
 // holds a range of owner cells and the faces that range needs and no earlier range needed.
@@ -231,30 +275,26 @@ cudaError_t run_slabs(const ApplyArgs& Ar, const Consts<typename A::V, K>& c, co
       const cudaError_t e = cudaStreamWaitEvent(st, Ar.slab_inputs[s], 0);
       if (e != cudaSuccess) return e;
     }
+    constexpr bool COMPACT = StoreCompact<V>::value;
     if (nb > 0) {
       const cudaError_t e =
           (s == 0 || Ar.slab_events)
-              ? (face_kernel<D, K, A><<<nb, t.fb * S::L, face_smem<D, K, V>(t.fb), st>>>((const IO*)Ar.x, (V*)Ar.tp,
-                                                                                     (IO*)Ar.y, fa, t.fb, c),
+              ? (face_kernel<D, K, A, COMPACT><<<nb, t.fb * S::L, face_smem<D, K, V>(t.fb), st>>>(
+                     (const IO*)Ar.x, (V*)Ar.tp, (IO*)Ar.y, fa, t.fb, c),
                  cudaGetLastError())
-              : launch_pdl(face_kernel<D, K, A>, nb, t.fb * S::L, face_smem<D, K, V>(t.fb), st, (const IO*)Ar.x,
-                           (V*)Ar.tp, (IO*)Ar.y, fa, (int)t.fb, c);
+              : launch_pdl(face_kernel<D, K, A, COMPACT>, nb, t.fb * S::L, face_smem<D, K, V>(t.fb), st,
+                           (const IO*)Ar.x, (V*)Ar.tp, (IO*)Ar.y, fa, (int)t.fb, c);
       if (e != cudaSuccess) return e;
     }
     LiftArgs la = Ar.la;
     la.lwin = Ar.la.lwin + (size_t)sl[0] * NW;
     la.lrow = Ar.la.lrow + (size_t)sl[0] * KR;
+    la.lmask = Ar.la.lmask + sl[0];
     la.nlift = sl[1] - sl[0];
-    const int32_t nlb = (la.nlift + t.lcb - 1) / t.lcb;
-    if (nlb > 0) {
+    if (la.nlift > 0) {
       // programmatic dependent of this slab's face launch (a plain launch after an event)
       const cudaError_t e =
-          (nb > 0 || !Ar.slab_events)
-              ? launch_pdl(lift_kernel<D, K, A>, nlb, t.lnt, lift_smem<D, K>(t.lcb), st, (const V*)Ar.tp, (IO*)Ar.y,
-                           Ar.add, la, (int)t.lcb)
-              : (lift_kernel<D, K, A><<<nlb, t.lnt, lift_smem<D, K>(t.lcb), st>>>((const V*)Ar.tp, (IO*)Ar.y, Ar.add, la,
-                                                                                 t.lcb),
-                 cudaGetLastError());
+          launch_lift<D, K, A>(nb > 0 || !Ar.slab_events, t, (const V*)Ar.tp, (IO*)Ar.y, Ar.add, la, c, st);
       if (e != cudaSuccess) return e;
     }
     if (Ar.slab_events) {
@@ -298,32 +338,21 @@ cudaError_t run_apply(const ApplyArgs& Ar, cudaStream_t st) {
   }
   for (int a = D; a < 4; ++a) fa.bstart[a] = nb;
   const bool faces = Ar.fstart[D] > 0;
-  const int32_t nlb = (Ar.la.nlift + t.lcb - 1) / t.lcb;
   if (Ar.ev) cudaEventRecord(Ar.ev[0], st);
-  if (nb > 0 && (Ar.which & 1))
-    face_kernel<D, K, A><<<nb, t.fb * S::L, face_smem<D, K, V>(t.fb), st>>>((const IO*)Ar.x, (V*)Ar.tp,
-                                                                          (IO*)Ar.y, fa, t.fb, c);
+  if (nb > 0 && (Ar.which & 1)) {
+    if (StoreCompact<V>::value && Ar.full_outputs)
+      face_kernel<D, K, A, false><<<nb, t.fb * S::L, face_smem<D, K, V>(t.fb), st>>>((const IO*)Ar.x, (V*)Ar.tp,
+                                                                                   (IO*)Ar.y, fa, t.fb, c);
+    else
+      face_kernel<D, K, A, StoreCompact<V>::value><<<nb, t.fb * S::L, face_smem<D, K, V>(t.fb), st>>>(
+          (const IO*)Ar.x, (V*)Ar.tp, (IO*)Ar.y, fa, t.fb, c);
+  }
   if (Ar.ev) cudaEventRecord(Ar.ev[1], st);
-  if (nlb > 0 && faces && (Ar.which & 2)) {
-    if (Ar.ev || !(Ar.which & 1)) {
-      lift_kernel<D, K, A><<<nlb, t.lnt, lift_smem<D, K>(t.lcb), st>>>((const V*)Ar.tp, (IO*)Ar.y, Ar.add, Ar.la,
-                                                                       t.lcb);
-    } else {
-      // programmatic dependent launch: the lift's CTAs start while the face grid drains
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)nlb);
-      cfg.blockDim = dim3((unsigned)t.lnt);
-      cfg.dynamicSmemBytes = lift_smem<D, K>(t.lcb);
-      cfg.stream = st;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-      attr[0].val.programmaticStreamSerializationAllowed = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      const cudaError_t e = cudaLaunchKernelEx(&cfg, lift_kernel<D, K, A>, (const V*)Ar.tp, (IO*)Ar.y, Ar.add, Ar.la,
-                                               (int)t.lcb);
-      if (e != cudaSuccess) return e;
-    }
+  if (Ar.la.nlift > 0 && faces && (Ar.which & 2)) {
+    // programmatic dependent launch: the lift's CTAs start while the face grid drains
+    const cudaError_t e = launch_lift<D, K, A>(!Ar.ev && (Ar.which & 1), t, (const V*)Ar.tp, (IO*)Ar.y, Ar.add,
+                                               Ar.la, c, st);
+    if (e != cudaSuccess) return e;
   }
   if (Ar.ev) cudaEventRecord(Ar.ev[2], st);
   return cudaGetLastError();
@@ -369,7 +398,8 @@ bool pack_batch(const std::vector<SegSpec>& in, Tiles& t, std::vector<unsigned c
     LiftSeg ls;
     ls.la = in[i].la;
     ls.block0 = lb;
-    if (fs.fa.fstart[D] > 0) lb += (ls.la.nlift + t.lcb - 1) / t.lcb;
+    const int cb = lift_cells<D, K, V>(t);
+    if (fs.fa.fstart[D] > 0) lb += (ls.la.nlift + cb - 1) / cb;
     std::memcpy(&fsegs[i * sizeof(FaceSeg<V, K>)], &fs, sizeof(fs));
     std::memcpy(&lsegs[i * sizeof(LiftSeg)], &ls, sizeof(ls));
   }
@@ -396,9 +426,16 @@ cudaError_t run_batch(const void* fsegs, const void* lsegs, const void* ptrs, in
   if (face_blocks > 0)
     face_kernel_batched<D, K, A><<<face_blocks, t.fb * S::L, face_smem<D, K, V>(t.fb), st>>>(
         (const FaceSeg<V, K>*)fsegs, nseg, (const SegPtrs<IO>*)ptrs, t.fb, c);
-  if (lift_blocks > 0)
-    lift_kernel_batched<D, K, A><<<lift_blocks, t.lnt, lift_smem<D, K>(t.lcb), st>>>(
-        (const LiftSeg*)lsegs, (const FaceSeg<V, K>*)fsegs, nseg, (const SegPtrs<IO>*)ptrs, t.lcb);
+  if (lift_blocks > 0) {
+    const int cb = lift_cells<D, K, V>(t);
+    const size_t smem = lift_dyn_smem<D, K, V>(cb);
+    if constexpr (StoreCompact<V>::value)
+      lift_lines_kernel_batched<D, K, A><<<lift_blocks, t.lnt, smem, st>>>(
+          (const LiftSeg*)lsegs, (const FaceSeg<V, K>*)fsegs, nseg, (const SegPtrs<IO>*)ptrs, cb, c);
+    else
+      lift_kernel_batched<D, K, A><<<lift_blocks, t.lnt, smem, st>>>(
+          (const LiftSeg*)lsegs, (const FaceSeg<V, K>*)fsegs, nseg, (const SegPtrs<IO>*)ptrs, cb);
+  }
   return cudaGetLastError();
 }
 

@@ -1083,6 +1083,19 @@ gp_status build_plan(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* 
     p.lcell.assign(4 * nlift, 0);
     p.lrow.assign((size_t)KR * nlift, -1);
     p.lwin.assign((size_t)p.lwin_width * nlift, -1);
+    p.lmask.assign(nlift, 0);
+    // the kinds of nodes that candidate face w reaches (see Plan::lmask)
+    int32_t reach[36] = {};
+    for (int w = 0; w < d * nw; ++w) {
+      const int a = w / nw, v = w % nw, t1 = a == 0 ? 1 : 0, t2 = a == 2 ? 1 : 2;
+      const int sa = d == 3 ? v / 4 : v / 2, s1 = d == 3 ? (v % 4) / 2 : v % 2, s2 = d == 3 ? v % 2 : 1;
+      bool all[3] = {true, true, true};           // the face reaches the nodes beyond 0 along each axis
+      all[a] = sa != 0;
+      all[t1] = s1 != 0;
+      if (d == 3) all[t2] = s2 != 0;
+      for (int m = 0; m < (1 << d); ++m)
+        if (((m & 1) == 0 || all[0]) && ((m & 2) == 0 || all[1]) && ((m & 4) == 0 || all[2])) reach[w] |= 1 << m;
+    }
     for (int64_t i = 0; i < nlift; ++i) {
       int64_t o = order[i].second;
       int ci = (int)(o % n1), cj = (int)((o / n1) % n1), cl = d == 3 ? (int)(o / ((int64_t)n1 * n1)) : 0;
@@ -1091,6 +1104,8 @@ gp_status build_plan(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* 
       p.lcell[4 * i + 2] = cl;
       const int co[3] = {ci, cj, cl};
       window(co, &p.lwin[(size_t)p.lwin_width * i]);
+      for (int w = 0; w < d * nw; ++w)
+        if (p.lwin[(size_t)p.lwin_width * i + w] >= 0) p.lmask[i] |= reach[w];
       for (int t = 0; t < KR; ++t) {
         int q = t % k, r = t / k;
         int Y = cj * k + q, Z = cl * k + r, X = ci * k;
@@ -1120,6 +1135,22 @@ gp_status build_plan(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* 
       if (f < -1 || f >= (int32_t)nf) { err = "internal: lift window outside the face list"; return GP_EINVAL; }
     for (int32_t r : p.lrow)
       if (r < -1 || r >= na) { err = "internal: lift row outside the active DoFs"; return GP_EINVAL; }
+    // every node that the lift writes for the owner's mask
+    const int KR = (int)ipow(k, d - 1);
+    for (int64_t i = 0; i < p.num_lift_cells(); ++i) {
+      const int m = p.lmask[i];
+      int last[4];                                  // by row kind (q > 0) + 2 (r > 0)
+      for (int kind = 0; kind < 4; ++kind) last[kind] = (m >> (2 * kind + 1)) & 1 ? k - 1 : (m >> (2 * kind)) & 1 ? 0 : -1;
+      const int32_t* row = &p.lrow[(size_t)i * KR];
+      for (int r = 0; r < KR / k; ++r)
+        for (int q = 0; q < k; ++q, ++row) {
+          const int l = last[(q > 0 ? 1 : 0) + (r > 0 ? 2 : 0)];
+          if (l >= 0 && (*row < 0 || *row + l >= na)) {
+            err = "internal: lift node outside the active DoFs";
+            return GP_EINVAL;
+          }
+        }
+    }
     for (size_t i = 0; i + 1 < p.zruns.size(); i += 2)
       if (p.zruns[i] < 0 || p.zruns[i + 1] < 1 || p.zruns[i + 1] > ZRUN_MAX || p.zruns[i] + p.zruns[i + 1] > na) {
         err = "internal: zero run outside the active DoFs";

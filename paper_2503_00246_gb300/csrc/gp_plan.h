@@ -56,6 +56,10 @@ struct Plan {
   std::vector<int32_t> lrow;
   std::vector<int32_t> lwin;      // nlift x (3*12 | 2*6): candidate face ids (-1 if none)
   int lwin_width = 0;
+  // per owner cell: bit (p > 0) + 2 (q > 0) + 4 (r > 0) set when some ghost face reaches its nodes
+  // (p, q, r) of that kind (a face reaches the nodes with p_a = 0 only where the owner is its patch's
+  // far end along a, and all others otherwise)
+  std::vector<int32_t> lmask;
   // zero fill of the active DoFs outside every face patch: runs (c0, len <= 256)
   std::vector<int32_t> zruns;
   int64_t num_lift_cells() const { return (int64_t)lcell.size() / 4; }

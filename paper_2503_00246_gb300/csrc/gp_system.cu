@@ -138,7 +138,7 @@ cudaError_t dot(gp_system* s, const T* a, const T* b, double* out) {
 // partial sums of dotp . y (one per gather CTA, s->nparts of them) in s->part.
 gp_status sys_apply(gp_system* s, gp_ctx* c, gp::CellsFn cells, const void* x, void* y, cudaStream_t st,
                     const void* dotp = nullptr) {
-  gp_status g = gpi::launch(c, x, y, 1, st, nullptr, false, nullptr, 1);   // face kernel alone
+  gp_status g = gpi::launch(c, x, y, 1, st, nullptr, false, nullptr, 1, nullptr, true);   // face kernel alone, W_F
   if (g != GP_OK) return g;
   const gp::Plan& p = c->plan;
   gp::CellTabs ct = s->ct;

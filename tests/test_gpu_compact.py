@@ -1,0 +1,33 @@
+"""GPU: the FP32 lift over compact face outputs at the sizes where it can go wrong: every degree,
+owner cells with every candidate face (a full box) and with few (a ball), lift tiles of one owner,
+of more lines than threads, and larger than the shared memory (the kernel then takes fewer owners).
+Against the oracle at the FP32 bound of the library (1e-5), and bitwise equal over the tiles."""
+import numpy as np
+import pytest
+
+from oracle.ghost_penalty import Oracle
+from paper_2503_00246_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("box", [False, True])
+@pytest.mark.parametrize("dim,n,k", [(2, 9, k) for k in range(1, 9)] + [(3, 5, 1), (3, 5, 2), (3, 4, 5), (3, 3, 7), (3, 3, 8)])
+def test_compact_lift(gplib, cuda, dim, n, k, box):
+    pr = W.box_problem(dim, n, k, hi=1.0) if box else W.small_ball(dim, 2 * n, k, seed=70 + k)
+    ctx = gplib.setup_problem(pr, precision=1)
+    x = W.x_vectors(pr, ctx.n_active)[0].astype(np.float32)
+    ref = Oracle(pr).apply(x.astype(np.float64))
+    xd = cuda.tensor(x, device="cuda")
+    first = None
+    for cells, threads in ((0, 0), (1, 32), (3, 64), (46 * 1024 // (4 * (37 if dim == 3 else 13)), 256)):
+        gplib.gp_set_tiles(ctx, {"faces_per_cta": 0, "lift_cells_per_cta": cells, "lift_threads": threads})
+        for add in (False, True):
+            yd = cuda.ones_like(xd) if add else cuda.full_like(xd, float("nan"))
+            (gplib.gp_apply_add if add else gplib.gp_apply)(ctx, xd, yd)
+            cuda.cuda.synchronize()
+            y = yd.double().cpu().numpy() - (1.0 if add else 0.0)
+            assert np.abs(y - ref).max() <= 1e-5 * max(np.abs(ref).max(), 1.0 if add else 0.0)
+            if not add:
+                first = yd if first is None else first
+                assert cuda.equal(yd, first), (cells, threads)
