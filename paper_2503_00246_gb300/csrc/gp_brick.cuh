@@ -192,15 +192,7 @@ brick_kernel(const typename A::IO* __restrict__ x, typename A::IO* __restrict__ 
 
   if ((int)blockIdx.x < ba.nzblocks) {
     // zero fill of the active DoFs outside every face patch (overwrite form only)
-    __shared__ int2 zr[ZGROUP];
-    const int r0 = blockIdx.x * ZGROUP;
-    const int nr = min(ZGROUP, ba.nzruns - r0);
-    for (int i = t; i < nr; i += nt) zr[i] = __ldg(ba.zruns + r0 + i);
-    __syncthreads();
-    for (int r = 0; r < nr; ++r) {
-      const int2 run = zr[r];
-      for (int i = t; i < run.y; i += nt) __stcs(y + run.x + i, IO(0));   // not read again: streaming
-    }
+    zero_fill(y, ba.zruns, ba.nzruns, (int)blockIdx.x);
     return;
   }
   const int brick = (int)blockIdx.x - ba.nzblocks;

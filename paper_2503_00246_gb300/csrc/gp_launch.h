@@ -259,7 +259,7 @@ cudaError_t run_slabs(const ApplyArgs& Ar, const Consts<typename A::V, K>& c, co
     fa.nzruns = s == 0 ? Ar.nzruns : 0;
     fa.nzblocks = (fa.nzruns + ZGROUP - 1) / ZGROUP;
     fa.tail_wait = s > 0 && !Ar.slab_events;
-    int32_t nb = fa.nzblocks;
+    int32_t nb = 0;
     for (int a = 0; a < 4; ++a) {
       const bool in = a < D;
       fa.fstart[a] = in ? sl[2 + 2 * a] : 0;
@@ -271,6 +271,8 @@ cudaError_t run_slabs(const ApplyArgs& Ar, const Consts<typename A::V, K>& c, co
       nb += (fa.fend[a] - fa.fstart[a] + t.fb - 1) / t.fb;
     }
     for (int a = D; a < 4; ++a) fa.bstart[a] = nb;
+    nb += fa.nzblocks;
+    set_zero_step(fa, nb);
     if (Ar.slab_inputs) {
       const cudaError_t e = cudaStreamWaitEvent(st, Ar.slab_inputs[s], 0);
       if (e != cudaSuccess) return e;
@@ -329,7 +331,7 @@ cudaError_t run_apply(const ApplyArgs& Ar, cudaStream_t st) {
   fa.nzruns = Ar.nzruns;
   fa.nzblocks = (Ar.nzruns + ZGROUP - 1) / ZGROUP;
   fa.tail_wait = 0;
-  int32_t nb = fa.nzblocks;
+  int32_t nb = 0;
   for (int a = 0; a < 4; ++a) fa.fstart[a] = Ar.fstart[a];
   for (int a = 0; a < 4; ++a) fa.fend[a] = a < D ? Ar.fstart[a + 1] : Ar.fstart[D];
   for (int a = 0; a < D; ++a) {
@@ -337,6 +339,8 @@ cudaError_t run_apply(const ApplyArgs& Ar, cudaStream_t st) {
     nb += (Ar.fstart[a + 1] - Ar.fstart[a] + t.fb - 1) / t.fb;
   }
   for (int a = D; a < 4; ++a) fa.bstart[a] = nb;
+  nb += fa.nzblocks;
+  set_zero_step(fa, nb);
   const bool faces = Ar.fstart[D] > 0;
   if (Ar.ev) cudaEventRecord(Ar.ev[0], st);
   if (nb > 0 && (Ar.which & 1)) {
@@ -384,12 +388,14 @@ bool pack_batch(const std::vector<SegSpec>& in, Tiles& t, std::vector<unsigned c
     fs.fa.nzblocks = (fs.fa.nzruns + ZGROUP - 1) / ZGROUP;
     fs.fa.tail_wait = 0;
     for (int a = 0; a < 4; ++a) fs.fa.fend[a] = a < D ? fs.fa.fstart[a + 1] : fs.fa.fstart[D];
-    int32_t nb = fs.fa.nzblocks;
+    int32_t nb = 0;
     for (int a = 0; a < D; ++a) {
       fs.fa.bstart[a] = nb;
       nb += (fs.fa.fstart[a + 1] - fs.fa.fstart[a] + t.fb - 1) / t.fb;
     }
     for (int a = D; a < 4; ++a) fs.fa.bstart[a] = nb;
+    nb += fs.fa.nzblocks;
+    set_zero_step(fs.fa, nb);
     fs.wp = (V*)in[i].wp;
     fs.gs = (const V*)in[i].gs;
     for (int j = 0; j < K; ++j) fs.s[j] = from_host<V>(in[i].s[j]);
