@@ -33,8 +33,8 @@ struct gp_system {
   int32_t* d_o2l_lo = nullptr;
   gp::CellTabs ct{};
   int nparts = 0;           // CTAs of the cell gather (fused inner-product partials)
-  int nblk = 0;             // CTAs of the vector reductions: 4 per SM
-  int nvec = 0;             // CTAs of the element-wise vector kernels: 8 per SM
+  int nblk = 0;             // CTAs of the vector reductions: at most 4 per SM, one quad per thread at least
+  int nvec = 0;             // CTAs of the element-wise vector kernels: at most 8 per SM
   gp::CellsFn cells_hi = nullptr, cells_lo = nullptr;
   // solver vectors
   double *r = nullptr, *p = nullptr, *q = nullptr, *dd = nullptr, *z = nullptr, *ri = nullptr;
@@ -42,6 +42,7 @@ struct gp_system {
   double* dinv = nullptr;   // 1 / diag(A) (Jacobi)
   float* dinv32 = nullptr;
   double* part = nullptr;   // dot partials + result
+  double* part_pq = nullptr;  // p . q partials of the gather, then their sum
   double* h_res = nullptr;  // pinned copy of the dot result
   void* d_cg = nullptr;     // CgScalars of the running CG (device)
   void* h_cg = nullptr;     // pinned copy
@@ -135,19 +136,22 @@ cudaError_t dot(gp_system* s, const T* a, const T* b, double* out) {
 // kernel (face outputs only), the cell kernel (cell outputs; it overlaps the face kernel
 // as its programmatic dependent), and one gather that adds, per node, the face outputs
 // and then the cell outputs and writes y once.  With dotp, the gather also leaves the
-// partial sums of dotp . y (one per gather CTA, s->nparts of them) in s->part.
+// partial sums of dotp . y (one per gather CTA, s->nparts of them) in s->part_pq.
 gp_status sys_apply(gp_system* s, gp_ctx* c, gp::CellsFn cells, const void* x, void* y, cudaStream_t st,
                     const void* dotp = nullptr) {
-  gp_status g = gpi::launch(c, x, y, 1, st, nullptr, false, nullptr, 1, nullptr, true);   // face kernel alone, W_F
+  // the face kernel alone, storing W_F
+  gp_status g = gpi::launch(c, x, y, 1, st, nullptr, false, nullptr, 1, nullptr, true);
   if (g != GP_OK) return g;
   const gp::Plan& p = c->plan;
   gp::CellTabs ct = s->ct;
   ct.dotp = dotp;
-  ct.dotpart = dotp ? s->part : nullptr;
+  ct.dotpart = dotp ? s->part_pq : nullptr;
   ct.wf = c->d_tp;
   ct.fwin = c->d_lwin;
   ct.own2lift = c == s->hi ? s->d_o2l_hi : s->d_o2l_lo;
-  const cudaError_t e = cells(p.k, x, y, ct, p.mass.data(), p.stiff.data(), p.h, 1.0, 1.0, 0, 0, st);
+  // without a face launch before it the cell kernel is the first of the call
+  const int first = p.num_faces() == 0 ? 1 : 0;
+  const cudaError_t e = cells(p.k, x, y, ct, p.mass.data(), p.stiff.data(), p.h, 1.0, 1.0, 0, first, st);
   if (e != cudaSuccess) return fail(c, GP_ECUDA, std::string("cell kernels: ") + cudaGetErrorString(e));
   return GP_OK;
 }
@@ -161,7 +165,7 @@ gp::CellsFn cells_for(const gp::Plan& p) {
 void sys_free(gp_system* s) {
   void* ptrs[] = {s->d_crow, s->d_cwin, s->d_corow, s->d_wc, s->d_o2l_hi, s->d_o2l_lo, s->r, s->p, s->q, s->dd,
                   s->z, s->ri, s->r32,
-                  s->d32, s->ri32, s->p32, s->q32, s->z32, s->dinv, s->dinv32, s->part, s->d_cg};
+                  s->d32, s->ri32, s->p32, s->q32, s->z32, s->dinv, s->dinv32, s->part, s->part_pq, s->d_cg};
   for (void* v : ptrs)
     if (v) cudaFree(v);
   if (s->h_res) cudaFreeHost(s->h_res);
@@ -179,18 +183,37 @@ void sys_free(gp_system* s) {
   } while (0)
 
 // ---- CG with its scalars on the device --------------------------------------------
-// One iteration is enqueued without a host round trip: q = A p; alpha = rz / (p.q);
-// d += alpha p, r -= alpha q, z = D^-1 r together with the partial sums of r.r and r.z;
-// beta = rz' / rz; p = z + beta p.  A block of kCgBlock iterations is captured once as a
-// CUDA graph and replayed; the host reads the scalars (converged, iterations) after
-// each replay.  Iterations after convergence leave d and r unchanged (alpha = 0).
-// Every reduction has a fixed grid and tree: bitwise reproducible.
+// One iteration is enqueued without a host round trip: q = A p (face, cell and gather kernel, with
+// the partial sums of p.q); cg_update: alpha = rz / (p.q), d += alpha p, r -= alpha q, z = D^-1 r
+// and the partial sums of r.r and r.z; cg_direction: beta = rz' / rz, p = z + beta p.  Up to
+// kDirectSums partials, every CTA of the last two sums them for itself, in one fixed order: five
+// kernels per iteration (24^3 ball at k = 2, 29 thousand DoFs, where launches count: 28.1 -> 21.3 us
+// per FP32 iteration of seven kernels before, vector grids cut to the vectors' size included).  More
+// partials are first added up by one CTA (64^3 ball at k = 3: 80 us when all 608 and 1216 CTAs sum
+// 1900 and 1216 doubles, 65 us so).  Programmatic launches of these kernels measured no gain.
+// The scalars are double buffered: iteration i reads sc[i % 2] and one thread of cg_direction writes
+// sc[(i + 1) % 2].  A block of kCgBlock iterations (even) is captured once as a CUDA graph and
+// replayed; the host reads the scalars (converged, iterations) after each replay.  Iterations
+// after convergence leave d, r and p unchanged.  Every reduction has a fixed grid and tree: bitwise
+// reproducible.
 struct CgScalars {
-  double rz, rr, stop, alpha, beta;
+  double rz, rr, stop;
   int done, iters, maxit, breakdown;
 };
 
 constexpr int kCgBlock = 16;
+static_assert(kCgBlock % 2 == 0, "a block must end on the buffer it began with");
+constexpr int kDirectSums = 512;
+
+__device__ __forceinline__ double block_sum(const double v, double* sh) {
+  sh[threadIdx.x] = v;
+  __syncthreads();
+  for (int o = kThreads / 2; o > 0; o >>= 1) {
+    if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
+    __syncthreads();
+  }
+  return sh[0];
+}
 
 __global__ void __launch_bounds__(kThreads) cg_init_final(const double* __restrict__ part, const int nblk,
                                                           CgScalars* sc, double tol, int maxit) {
@@ -218,32 +241,19 @@ __global__ void __launch_bounds__(kThreads) cg_init_final(const double* __restri
     sc->iters = 0;
     sc->maxit = maxit;
     sc->breakdown = 0;
-    sc->alpha = sc->beta = 0.0;
     sc->done = (maxit <= 0 || !(rr0 > sc->stop) || !(rr0 > 0.0)) ? 1 : 0;
   }
 }
 
-// alpha = rz / (p.q) from the nparts partial sums of p.q
-__global__ void __launch_bounds__(kThreads) cg_alpha(const double* __restrict__ part, const int nparts,
-                                                     CgScalars* sc) {
+// out[k] = the sum of part[k n .. (k + 1) n), k < gridDim.x
+__global__ void __launch_bounds__(kThreads) cg_sums(const double* __restrict__ part, const int n,
+                                                    double* __restrict__ out) {
   __shared__ double sh[kThreads];
+  const double* p = part + (size_t)blockIdx.x * n;
   double a = 0.0;
-  for (int i = threadIdx.x; i < nparts; i += kThreads) a += part[i];
-  sh[threadIdx.x] = a;
-  __syncthreads();
-  for (int o = kThreads / 2; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    const double pq = sh[0];
-    double alpha = 0.0;
-    if (!sc->done) {
-      if (pq > 0.0) alpha = sc->rz / pq;
-      else { sc->done = 1; sc->breakdown = 1; }
-    }
-    sc->alpha = alpha;
-  }
+  for (int i = threadIdx.x; i < n; i += kThreads) a += p[i];
+  const double t = block_sum(a, sh);
+  if (threadIdx.x == 0) out[blockIdx.x] = t;
 }
 
 // Four consecutive vector elements, loaded and stored as one 16-byte (FP32) or
@@ -274,14 +284,33 @@ __device__ __forceinline__ void block_sums2(double a, double b, double* __restri
   }
 }
 
-// d += alpha p, r -= alpha q, z = dinv r (when dinv), and the partial sums of r.r, r.z
+// alpha = rz / (p.q) from the npq partial sums of p.q; d += alpha p, r -= alpha q, z = dinv r (when
+// dinv), and the partial sums of r.r, r.z
 template <typename T>
 __global__ void __launch_bounds__(kThreads) cg_update(T* __restrict__ d, T* __restrict__ r, const T* __restrict__ p,
                                                       const T* __restrict__ q, T* __restrict__ z,
-                                                      const T* __restrict__ dinv, const CgScalars* __restrict__ sc,
+                                                      const T* __restrict__ dinv, CgScalars* sc,
+                                                      const double* __restrict__ pqp, const int npq,
                                                       int64_t n, double* __restrict__ part) {
+  __shared__ double sh[kThreads];
+  __shared__ T s_alpha;
+  __shared__ int s_go;
   if (sc->done) return;
-  const T a = (T)sc->alpha;
+  double pq = 0.0;
+  if (npq > 1) {
+    for (int i = threadIdx.x; i < npq; i += kThreads) pq += pqp[i];
+    pq = block_sum(pq, sh);
+  }
+  if (threadIdx.x == 0) {   // (one thread divides: an FP64 division by every thread took 3 us)
+    if (npq == 1) pq = pqp[0];
+    s_go = pq > 0.0 ? 1 : 0;
+    s_alpha = s_go ? (T)(sc->rz / pq) : (T)0;
+    // breakdown: nothing changes, and cg_direction stops the iteration
+    if (!s_go && blockIdx.x == 0) sc->breakdown = 1;
+  }
+  __syncthreads();
+  if (!s_go) return;
+  const T a = s_alpha;
   gp::IoDot<T> rr, rz;
   const int64_t tid = (int64_t)blockIdx.x * kThreads + threadIdx.x, stride = (int64_t)gridDim.x * kThreads;
   const int64_t n4 = n >> 2;
@@ -321,45 +350,47 @@ __global__ void __launch_bounds__(kThreads) cg_update(T* __restrict__ d, T* __re
   block_sums2(rr.value(), rz.value(), part);
 }
 
-// beta = rz' / rz, the convergence test and the iteration count
-__global__ void __launch_bounds__(kThreads) cg_beta(const double* __restrict__ part, const int nblk,
-                                                    CgScalars* sc) {
-  __shared__ double sa[kThreads], sb[kThreads];
-  __shared__ int done;
-  if (threadIdx.x == 0) done = sc->done;
-  __syncthreads();
-  if (done) return;
-  double a = 0.0, b = 0.0;
-  for (int i = threadIdx.x; i < nblk; i += kThreads) {
-    a += part[i];
-    b += part[nblk + i];
-  }
-  sa[threadIdx.x] = a;
-  sb[threadIdx.x] = b;
-  __syncthreads();
-  for (int o = kThreads / 2; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o) {
-      sa[threadIdx.x] += sa[threadIdx.x + o];
-      sb[threadIdx.x] += sb[threadIdx.x + o];
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    const double rr = sa[0], rz1 = sb[0];
-    sc->beta = rz1 / sc->rz;
-    sc->rz = rz1;
-    sc->rr = rr;
-    sc->iters += 1;
-    if (!(rr > sc->stop) || !(rr > 0.0) || sc->iters >= sc->maxit) sc->done = 1;
-  }
-}
-
-// p = z + beta p
+// beta = rz' / rz from the nsum partial sums of r.r and of r.z, the convergence test and the iteration
+// count (into next); p = z + beta p unless this was the last iteration
 template <typename T>
 __global__ void __launch_bounds__(kThreads, kVecPerSm)
-cg_direction(T* __restrict__ p, const T* __restrict__ z, const CgScalars* __restrict__ sc, int64_t n) {
-  if (sc->done) return;
-  const T bt = (T)sc->beta;
+cg_direction(T* __restrict__ p, const T* __restrict__ z, const CgScalars* __restrict__ sc, CgScalars* __restrict__ next,
+             const double* __restrict__ part, const int nsum, int64_t n) {
+  __shared__ double sh[kThreads];
+  __shared__ T s_beta;
+  __shared__ int s_go;
+  const bool stop = sc->done || sc->breakdown;
+  double rr = 0.0, rz1 = 0.0;
+  if (!stop && nsum > 1) {
+    for (int i = threadIdx.x; i < nsum; i += kThreads) {
+      rr += part[i];
+      rz1 += part[nsum + i];
+    }
+    rr = block_sum(rr, sh);
+    __syncthreads();
+    rz1 = block_sum(rz1, sh);
+  }
+  if (threadIdx.x == 0) {
+    bool done = stop;
+    CgScalars nx = *sc;
+    if (!stop) {
+      if (nsum == 1) {
+        rr = part[0];
+        rz1 = part[1];
+      }
+      s_beta = (T)(rz1 / nx.rz);
+      nx.rz = rz1;
+      nx.rr = rr;
+      nx.iters += 1;
+      done = !(rr > nx.stop) || !(rr > 0.0) || nx.iters >= nx.maxit;
+    }
+    nx.done = done ? 1 : 0;
+    s_go = !done;
+    if (blockIdx.x == 0) *next = nx;
+  }
+  __syncthreads();
+  if (!s_go) return;
+  const T bt = s_beta;
   const int64_t tid = (int64_t)blockIdx.x * kThreads + threadIdx.x, stride = (int64_t)gridDim.x * kThreads;
   const int64_t n4 = n >> 2;
   for (int64_t j = tid; j < n4; j += stride) {
@@ -407,12 +438,25 @@ gp_status cg(gp_system* s, gp_ctx* c, gp::CellsFn cells, const T* rhs, T* d, T* 
   SYS_CUDA(cudaStreamBeginCapture(s->st, cudaStreamCaptureModeThreadLocal));
   gp_status g = GP_OK;
   for (int i = 0; i < kCgBlock && g == GP_OK; ++i) {
+    CgScalars *cur = sc + (i & 1), *next = sc + ((i + 1) & 1);
     g = sys_apply(s, c, cells, p, q, s->st, p);   // q = A p and the partial sums of p . q
     if (g != GP_OK) break;
-    cg_alpha<<<1, kThreads, 0, s->st>>>(s->part, s->nparts, sc);
-    cg_update<T><<<s->nblk, kThreads, 0, s->st>>>(d, r, p, q, z, dinv, sc, n, s->part);
-    cg_beta<<<1, kThreads, 0, s->st>>>(s->part, s->nblk, sc);
-    cg_direction<T><<<s->nvec, kThreads, 0, s->st>>>(p, zz, sc, n);
+    const double* pq = s->part_pq;
+    int npq = s->nparts;
+    if (npq > kDirectSums) {
+      cg_sums<<<1, kThreads, 0, s->st>>>(s->part_pq, npq, s->part_pq + npq);
+      pq += npq;
+      npq = 1;
+    }
+    cg_update<T><<<s->nblk, kThreads, 0, s->st>>>(d, r, p, q, z, dinv, cur, pq, npq, n, s->part);
+    const double* rr = s->part;
+    int nsum = s->nblk;
+    if (nsum > kDirectSums) {
+      cg_sums<<<2, kThreads, 0, s->st>>>(s->part, nsum, s->part + 2 * nsum);
+      rr += 2 * nsum;
+      nsum = 1;
+    }
+    cg_direction<T><<<s->nvec, kThreads, 0, s->st>>>(p, zz, cur, next, rr, nsum, n);
   }
   const cudaError_t ec = cudaStreamEndCapture(s->st, &graph);
   if (g != GP_OK) {
@@ -501,8 +545,10 @@ gp_status gp_system_create(gp_ctx* hi, gp_ctx* lo, gp_system** out) {
   cudaError_t e = cudaStreamCreateWithFlags(&s->st, cudaStreamNonBlocking);
   int sms = 0;
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, s->device);
-  s->nblk = kDotPerSm * std::max(sms, 1);
-  s->nvec = kVecPerSm * std::max(sms, 1);
+  // one quad of elements per thread is the least: 608 CTAs for 29 thousand DoFs left 580 of them empty
+  const int quads = (int)std::min<int64_t>((s->n / 4 + kThreads - 1) / kThreads + 1, 1 << 20);
+  s->nblk = std::min(kDotPerSm * std::max(sms, 1), quads);
+  s->nvec = std::min(kVecPerSm * std::max(sms, 1), quads);
   auto upload = [](int32_t** dst, const std::vector<int32_t>& v) -> cudaError_t {
     if (v.empty()) return cudaSuccess;
     cudaError_t r = cudaMalloc((void**)dst, v.size() * sizeof(int32_t));
@@ -552,10 +598,10 @@ gp_status gp_system_create(gp_ctx* hi, gp_ctx* lo, gp_system** out) {
   if (e == cudaSuccess && lo) e = cudaMalloc(&s->p32, n4);
   if (e == cudaSuccess && lo) e = cudaMalloc(&s->q32, n4);
   s->nparts = (int)gp::gather_ctas(p.dim, p.k, p.ncown);
-  if (e == cudaSuccess)
-    e = cudaMalloc(&s->part, (size_t)std::max<int64_t>(2 * s->nblk + 1, s->nparts) * sizeof(double));
+  if (e == cudaSuccess) e = cudaMalloc(&s->part, (size_t)(2 * s->nblk + 2) * sizeof(double));
+  if (e == cudaSuccess) e = cudaMalloc(&s->part_pq, (size_t)(s->nparts + 1) * sizeof(double));
   if (e == cudaSuccess) e = cudaMallocHost(&s->h_res, sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&s->d_cg, sizeof(CgScalars));
+  if (e == cudaSuccess) e = cudaMalloc(&s->d_cg, 2 * sizeof(CgScalars));
   if (e == cudaSuccess) e = cudaMallocHost(&s->h_cg, sizeof(CgScalars));
   if (e != cudaSuccess) return cleanup(e);
   *out = s;
