@@ -31,6 +31,7 @@ struct Shape {
   static constexpr int L = (D == 2) ? (K + 1) : (K + 1) * (K + 1);  // tangential nodes per face
   static constexpr int NN = 2 * K + 1;                               // nodes on a normal line
   static constexpr int P = NN * L;                                   // patch nodes per face
+  static constexpr int NP = (NN + 3) / 4 * 4;                        // row-start entries per patch column
   static constexpr int FB = (256 / L) > 0 ? (256 / L) : 1;           // default faces per CTA
 };
 
@@ -46,10 +47,21 @@ constexpr int MAX_CTA_THREADS = 512;
 constexpr size_t MAX_DYN_SMEM = 46 * 1024;   // plus < 2 KB of static shared memory: under the 48 KB default
 
 // dynamic shared memory of the face kernel: the k jump planes of fb faces, twice in 3D (room for
-// the padded planes and the second direction's sums, see TanShape)
+// the padded planes and the second direction's sums, see TanShape); FP32 also stages the patches of
+// faces of normal x there (below 36 KB for every CTA of at most MAX_CTA_THREADS lines)
+template <int D, int K, typename V>
+__host__ __device__ constexpr size_t face_planes(int fb) {
+  return (size_t)((D == 3) ? 2 : 1) * fb * K * Shape<D, K>::L * sizeof(V);
+}
+template <typename V>
+struct StagePatch {
+    static constexpr bool value = std::is_same<V, float>::value;
+};
 template <int D, int K, typename V>
 __host__ __device__ constexpr size_t face_smem(int fb) {
-  return (size_t)((D == 3) ? 2 : 1) * fb * K * Shape<D, K>::L * sizeof(V);
+  const size_t stage = StagePatch<V>::value ? (size_t)fb * Shape<D, K>::P * sizeof(V) : 0;
+  const size_t planes = face_planes<D, K, V>(fb);
+  return planes > stage ? planes : stage;
 }
 
 // Kernel constants (passed by value; they sit in the constant bank).  In FP64 and float-float
@@ -88,30 +100,47 @@ struct FaceArgs {
   int64_t rbase[4];       // row entry of face fstart[a] of each axis
   int32_t fstart[4];      // first face of each axis in this launch
   int32_t fend[4];        // one past the last face of each axis in this launch
-  int32_t bstart[4];      // first CTA of each axis among the face CTAs; bstart[D] = face CTAs
   const int2* zruns;      // (c0, len <= 256) runs of untouched active DoFs
   int32_t nzruns;         // 0 for the add form
-  int32_t nzblocks;       // zero-fill CTAs, spread evenly over the grid (see zero_block)
-  uint64_t zstep;         // nzblocks / grid in units of 2^-32, rounded up
+  int32_t nzblocks;       // zero-fill CTAs
+  uint64_t zstep;         // shares that spread() takes: zero-fill CTAs of the grid,
+  uint64_t xstep, ystep;  // normal-x CTAs of the face CTAs, normal-y CTAs of the others
   int32_t tail_wait;      // 1: before exiting, wait for the grid this launch programmatically
                           // depends on (slab pipeline: so that this grid completes after it)
 };
 
 constexpr int ZGROUP = 16;  // zero runs per zero-fill CTA
 
-// The zero fill writes to HBM while the face CTAs compute, so its CTAs are spread over the grid:
-// CTA blk is zero-fill CTA floor(blk nz / grid) where that count steps at blk, and a face CTA
-// otherwise.  Returns the zero-fill index, or -1 - the index among the face CTAs.  At the front of
-// the grid they ran alone, 382 MB of zeros in an FP64 apply of the 128^3 gyroid (k = 4) with the FP64
-// pipe idle; spread, with the vector stores of zero_fill, that apply went from 1519 to 1450 us, the
-// FP32 one from 261 to 240 us, and the FP32 1023^2 disc (k = 4, almost all zeros) from 12.3 to 11.0.
-inline void set_zero_step(FaceArgs& fa, const int grid) {
-  fa.zstep = grid > 0 ? (((uint64_t)fa.nzblocks << 32) + (uint64_t)grid - 1) / (uint64_t)grid : 0;
+// The kinds of CTA of a face launch are spread evenly over its grid: CTA i of n, of which m are of a
+// kind, is CTA floor(i m / n) of that kind where that count steps at i, and otherwise one of the rest.
+// Zero-fill CTAs write to HBM while the face CTAs compute: at the front of the grid they ran alone,
+// 382 MB of zeros in an FP64 apply of the 128^3 gyroid (k = 4) with the FP64 pipe idle; spread, with
+// the vector stores of zero_fill, that apply went from 1519 to 1450 us, the FP32 one from 261 to
+// 240 us, and the FP32 1023^2 disc (k = 4, almost all zeros) from 12.3 to 11.0.
+// The faces of each axis follow the lexicographic order of their cells, so that spread axes work on
+// one region of the mesh at a time and read its x from HBM once instead of once per axis (face
+// kernel of the 128^3 gyroid at k = 4: FP32 132 -> 127 us, float-float 365 -> 355 us).
+inline uint64_t spread_step(const int64_t m, const int64_t n) {   // m / n in units of 2^-32, rounded up
+  return n > 0 ? (((uint64_t)m << 32) + (uint64_t)n - 1) / (uint64_t)n : 0;
 }
-__device__ __forceinline__ int zero_block(const int blk, const uint64_t zstep) {
-  const int zi = (int)(((uint64_t)blk * zstep) >> 32);
-  const int zn = (int)(((uint64_t)(blk + 1) * zstep) >> 32);
-  return zn > zi ? zi : -1 - (blk - zi);
+// the index of CTA i within its kind, or -1 - (its index among the rest)
+__device__ __forceinline__ int spread(const int i, const uint64_t step) {
+  const int k0 = (int)(((uint64_t)i * step) >> 32);
+  const int k1 = (int)(((uint64_t)(i + 1) * step) >> 32);
+  return k1 > k0 ? k0 : -1 - (i - k0);
+}
+// Fills the shares for fb faces per CTA; returns the CTAs of the launch.
+inline int face_grid(FaceArgs& fa, const int dim, const int fb) {
+  fa.nzblocks = (fa.nzruns + ZGROUP - 1) / ZGROUP;
+  int nb[3] = {0, 0, 0}, faces = 0;
+  for (int a = 0; a < dim; ++a) {
+    nb[a] = (fa.fend[a] - fa.fstart[a] + fb - 1) / fb;
+    faces += nb[a];
+  }
+  fa.zstep = spread_step(fa.nzblocks, fa.nzblocks + faces);
+  fa.xstep = spread_step(nb[0], faces);
+  fa.ystep = spread_step(nb[1], faces - nb[0]);
+  return fa.nzblocks + faces;
 }
 
 // Zeros of the runs [ZGROUP zi, ZGROUP (zi + 1)): a warp per run, 16-byte streaming stores between
@@ -350,23 +379,24 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
   // dependent launch; it waits for this grid's completion before it reads W)
   asm volatile("griddepcontrol.launch_dependents;");
 
-  const int zb = zero_block(blk, fa.zstep);
+  const int zb = spread(blk, fa.zstep);
   if (zb >= 0) {
     // zero fill of the active DoFs outside every face patch (overwrite form only)
     zero_fill(y, fa.zruns, fa.nzruns, zb);
     return;
   }
-  const int fblk = -1 - zb;
   // axis of this CTA's faces (constant indices only: no local-memory copy of fa)
-  int axis = 0, fbase = fa.fstart[0], fend = fa.fend[0], bbase = fa.bstart[0];
+  int axis = 0, fbase = fa.fstart[0], fend = fa.fend[0], ib = spread(-1 - zb, fa.xstep);
   int64_t rbase = fa.rbase[0];
-  if (D >= 2 && fblk >= fa.bstart[1]) {
-    axis = 1; fbase = fa.fstart[1]; fend = fa.fend[1]; bbase = fa.bstart[1]; rbase = fa.rbase[1];
+  if (ib < 0) {
+    ib = spread(-1 - ib, fa.ystep);
+    axis = 1; fbase = fa.fstart[1]; fend = fa.fend[1]; rbase = fa.rbase[1];
+    if (D == 3 && ib < 0) {
+      ib = -1 - ib;
+      axis = 2; fbase = fa.fstart[2]; fend = fa.fend[2]; rbase = fa.rbase[2];
+    }
   }
-  if (D >= 3 && fblk >= fa.bstart[2]) {
-    axis = 2; fbase = fa.fstart[2]; fend = fa.fend[2]; bbase = fa.bstart[2]; rbase = fa.rbase[2];
-  }
-  const int f0 = fbase + (fblk - bbase) * fb;
+  const int f0 = fbase + ib * fb;
   const int t = threadIdx.x;
   const int fl = t / L, tau = t - fl * L;
   const int f = f0 + fl;
@@ -375,19 +405,53 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
 
   // ---- gather this thread's normal line (2k+1 values)
   V v[NN];
-  if (valid) {
+  if (StagePatch<V>::value && axis == 0) {
+    // Normal x: a line is 2k+1 consecutive values, and a lane per line would touch a cache line per
+    // lane in each of its 2k+1 loads (FP32's kernel is bound by L1 wavefronts).  The CTA loads the
+    // patches value by value, lanes along the lines, and passes them on through shared memory (an
+    // odd pitch of 2k+1: no bank conflicts).  128^3 gyroid, k = 4: face kernel 132.5 -> 127 us.
+    if constexpr (StagePatch<V>::value) {
+      V* st = reinterpret_cast<V*>(dsm);
+      const int32_t* rows = fa.frows + rbase + (int64_t)(f0 - fbase) * L;
+      const int items = min(fb, fend - f0) * S::P;
+      int32_t at[NN];
+#pragma unroll
+      for (int u = 0; u < NN; ++u) {
+        const int i = t + u * nt;
+        const int line = i / NN;
+        at[u] = i < items ? __ldg(rows + line) + (i - line * NN) : -1;
+      }
+#pragma unroll
+      for (int u = 0; u < NN; ++u)
+        if (at[u] >= 0) st[t + u * nt] = __ldg(x + at[u]);
+      __syncthreads();
+#pragma unroll
+      for (int b = 0; b < NN; ++b) v[b] = valid ? st[t * NN + b] : vzero<V>();
+      __syncthreads();
+    }
+  } else if (valid) {
     if (axis == 0) {
       const int32_t base = __ldg(fa.frows + rbase + (int64_t)(f - fbase) * L + tau);
 #pragma unroll
       for (int b = 0; b < NN; ++b) v[b] = from_io(__ldg(x + base + b), (V*)nullptr);
     } else {
-      // tau = tx + (K+1) tr; row b of the patch at outer tangential index tr
-      constexpr int R = (D == 3) ? NN * K1 : NN;
+      // tau = tx + (K+1) tr; row b of the patch at outer tangential index tr, four starts per load
+      // (one load per start: float-float apply of the 128^3 gyroid at k = 4 713 us, so 666 us)
+      constexpr int NP = S::NP, R = (D == 3) ? NP * K1 : NP;
       const int tx = (D == 3) ? tau % K1 : tau;
       const int tr = (D == 3) ? tau / K1 : 0;
-      const int32_t* rows = fa.frows + rbase + (int64_t)(f - fbase) * R + NN * tr;
+      const int4* rows = reinterpret_cast<const int4*>(fa.frows + rbase + (int64_t)(f - fbase) * R + NP * tr);
+      int32_t at[NP];
 #pragma unroll
-      for (int b = 0; b < NN; ++b) v[b] = from_io(__ldg(x + __ldg(rows + b) + tx), (V*)nullptr);
+      for (int u = 0; u < NP / 4; ++u) {
+        const int4 r4 = __ldg(rows + u);
+        at[4 * u] = r4.x;
+        at[4 * u + 1] = r4.y;
+        at[4 * u + 2] = r4.z;
+        at[4 * u + 3] = r4.w;
+      }
+#pragma unroll
+      for (int b = 0; b < NN; ++b) v[b] = from_io(__ldg(x + at[b] + tx), (V*)nullptr);
     }
   } else {
 #pragma unroll
@@ -435,8 +499,15 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
 
 extern __shared__ __align__(16) unsigned char gp_dyn_smem[];
 
+// resident CTAs of MAX_CTA_THREADS threads to compile for: FP32 is held to 32 registers, every warp
+// slot of the SM (128^3 gyroid, k = 4, with 38 registers: 154 against 135 us); 0: the compiler's choice
+template <typename V>
+struct FaceCtas {
+  static constexpr int value = std::is_same<V, float>::value ? 4 : 0;
+};
+
 template <int D, int K, class A, bool COMPACT>
-__global__ void __launch_bounds__(MAX_CTA_THREADS)
+__global__ void __launch_bounds__(MAX_CTA_THREADS, FaceCtas<typename A::V>::value)
 face_kernel(const typename A::IO* __restrict__ x, typename A::V* __restrict__ wp,
             typename A::IO* __restrict__ y, const FaceArgs fa, const int fb,
             const __grid_constant__ Consts<typename A::V, K> c) {
@@ -481,7 +552,7 @@ __device__ __forceinline__ int find_segment(const Seg* segs, const int nseg, con
 }
 
 template <int D, int K, class A>
-__global__ void __launch_bounds__(MAX_CTA_THREADS)
+__global__ void __launch_bounds__(MAX_CTA_THREADS, FaceCtas<typename A::V>::value)
 face_kernel_batched(const FaceSeg<typename A::V, K>* __restrict__ segs, const int nseg,
                     const SegPtrs<typename A::IO>* __restrict__ ptrs, const int fb,
                     const __grid_constant__ Consts<typename A::V, K> c) {

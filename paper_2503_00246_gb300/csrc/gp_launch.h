@@ -44,8 +44,8 @@ struct ApplyArgs {
 };
 
 // Default tile shape: about 256 threads per CTA, one item per thread.  Compact outputs in 3D: face
-// CTAs of about 160 threads (more CTAs per SM to run while one waits at a barrier; 128^3 gyroid,
-// k = 4, face kernel with 2 / 5 / 6 / 10 / 20 faces: 238 / 162 / 159 / 164 / 199 us), and from
+// CTAs of about 130 threads (more CTAs per SM to run while one waits at a barrier; 128^3 gyroid,
+// k = 4, face kernel with 2 / 5 / 6 / 10 / 20 faces: 193 / 127 / 132 / 136 / 158 us), and from
 // k = 4 on two to four lines per lift thread (inner lines first, then edge lines with more faces, so
 // that the warps meet at the barriers; 128^3 gyroid with 1 / 2 / 4 lines: 152 / 104 / 150 us; 49^3
 // ball at k = 8, 128 threads, with 1 / 2 / 4 / 8: 102 / 56 / 49 / 61 us).
@@ -53,7 +53,7 @@ template <int D, int K, typename V>
 Tiles default_tiles_t() {
   constexpr bool CO = StoreCompact<V>::value && D == 3;
   Tiles t;
-  t.fb = CO ? (160 / Shape<D, K>::L > 0 ? 160 / Shape<D, K>::L : 1) : Shape<D, K>::FB;
+  t.fb = CO ? (130 / Shape<D, K>::L > 0 ? 130 / Shape<D, K>::L : 1) : Shape<D, K>::FB;
   t.lcb = LiftShape<D, K>::CB;
   t.lnt = LiftShape<D, K>::NT;
   if (CO && K == 4) t.lcb = 32;
@@ -73,7 +73,7 @@ bool resolve_tiles(Tiles& t) {
   if (t.fb == 0) t.fb = d.fb;
   if (t.lcb == 0) t.lcb = d.lcb;
   if (t.lnt == 0) t.lnt = d.lnt;
-  if (t.fb < 1 || t.fb * Shape<D, K>::L > MAX_CTA_THREADS || face_smem<D, K, V>(t.fb) > MAX_DYN_SMEM) return false;
+  if (t.fb < 1 || t.fb * Shape<D, K>::L > MAX_CTA_THREADS || face_planes<D, K, V>(t.fb) > MAX_DYN_SMEM) return false;
   if (t.lnt < 32 || t.lnt > MAX_CTA_THREADS || t.lnt % 32 != 0) return false;
   if (t.lcb < 1 || lift_smem<D, K>(t.lcb) > MAX_DYN_SMEM) return false;
   return true;
@@ -249,7 +249,7 @@ cudaError_t run_slabs(const ApplyArgs& Ar, const Consts<typename A::V, K>& c, co
   using S = Shape<D, K>;
   using V = typename A::V;
   using IO = typename A::IO;
-  const int R[3] = {S::L, (D == 3) ? S::NN * (K + 1) : S::NN, S::NN * (K + 1)};   // row entries per face
+  const int R[3] = {S::L, S::NP * ((D == 3) ? K + 1 : 1), S::NP * (K + 1)};   // row entries per face
   constexpr int KR = LiftShape<D, K>::KR, NW = LiftShape<D, K>::NW;
   for (int s = 0; s < Ar.nslab; ++s) {
     const int32_t* sl = Ar.slabs + (size_t)s * SLAB_INTS;
@@ -257,22 +257,14 @@ cudaError_t run_slabs(const ApplyArgs& Ar, const Consts<typename A::V, K>& c, co
     fa.frows = Ar.frows;
     fa.zruns = Ar.zruns;
     fa.nzruns = s == 0 ? Ar.nzruns : 0;
-    fa.nzblocks = (fa.nzruns + ZGROUP - 1) / ZGROUP;
     fa.tail_wait = s > 0 && !Ar.slab_events;
-    int32_t nb = 0;
     for (int a = 0; a < 4; ++a) {
       const bool in = a < D;
       fa.fstart[a] = in ? sl[2 + 2 * a] : 0;
       fa.fend[a] = in ? sl[3 + 2 * a] : 0;
       fa.rbase[a] = in ? Ar.rbase[a] + (int64_t)(fa.fstart[a] - Ar.fstart[a]) * R[a] : 0;
     }
-    for (int a = 0; a < D; ++a) {
-      fa.bstart[a] = nb;
-      nb += (fa.fend[a] - fa.fstart[a] + t.fb - 1) / t.fb;
-    }
-    for (int a = D; a < 4; ++a) fa.bstart[a] = nb;
-    nb += fa.nzblocks;
-    set_zero_step(fa, nb);
+    const int nb = face_grid(fa, D, t.fb);
     if (Ar.slab_inputs) {
       const cudaError_t e = cudaStreamWaitEvent(st, Ar.slab_inputs[s], 0);
       if (e != cudaSuccess) return e;
@@ -329,18 +321,10 @@ cudaError_t run_apply(const ApplyArgs& Ar, cudaStream_t st) {
   for (int a = 0; a < 4; ++a) fa.rbase[a] = Ar.rbase[a];
   fa.zruns = Ar.zruns;
   fa.nzruns = Ar.nzruns;
-  fa.nzblocks = (Ar.nzruns + ZGROUP - 1) / ZGROUP;
   fa.tail_wait = 0;
-  int32_t nb = 0;
   for (int a = 0; a < 4; ++a) fa.fstart[a] = Ar.fstart[a];
   for (int a = 0; a < 4; ++a) fa.fend[a] = a < D ? Ar.fstart[a + 1] : Ar.fstart[D];
-  for (int a = 0; a < D; ++a) {
-    fa.bstart[a] = nb;
-    nb += (Ar.fstart[a + 1] - Ar.fstart[a] + t.fb - 1) / t.fb;
-  }
-  for (int a = D; a < 4; ++a) fa.bstart[a] = nb;
-  nb += fa.nzblocks;
-  set_zero_step(fa, nb);
+  const int nb = face_grid(fa, D, t.fb);
   const bool faces = Ar.fstart[D] > 0;
   if (Ar.ev) cudaEventRecord(Ar.ev[0], st);
   if (nb > 0 && (Ar.which & 1)) {
@@ -385,17 +369,9 @@ bool pack_batch(const std::vector<SegSpec>& in, Tiles& t, std::vector<unsigned c
   for (size_t i = 0; i < in.size(); ++i) {
     FaceSeg<V, K> fs;
     fs.fa = in[i].fa;
-    fs.fa.nzblocks = (fs.fa.nzruns + ZGROUP - 1) / ZGROUP;
     fs.fa.tail_wait = 0;
     for (int a = 0; a < 4; ++a) fs.fa.fend[a] = a < D ? fs.fa.fstart[a + 1] : fs.fa.fstart[D];
-    int32_t nb = 0;
-    for (int a = 0; a < D; ++a) {
-      fs.fa.bstart[a] = nb;
-      nb += (fs.fa.fstart[a + 1] - fs.fa.fstart[a] + t.fb - 1) / t.fb;
-    }
-    for (int a = D; a < 4; ++a) fs.fa.bstart[a] = nb;
-    nb += fs.fa.nzblocks;
-    set_zero_step(fs.fa, nb);
+    const int nb = face_grid(fs.fa, D, t.fb);
     fs.wp = (V*)in[i].wp;
     fs.gs = (const V*)in[i].gs;
     for (int j = 0; j < K; ++j) fs.s[j] = from_host<V>(in[i].s[j]);

@@ -445,7 +445,7 @@ void build_diagonal(const Plan& p, std::vector<double>& diag) {
   std::vector<double> gb(NN, 0.0);  // sum_j s_j g_j[b]^2
   for (int b = 0; b < NN; ++b)
     for (int j = 0; j < k; ++j) gb[b] += p.scale[j] * p.jumps[j * NN + b] * p.jumps[j * NN + b];
-  const int L = p.L, R = d == 3 ? NN * K1 : NN;
+  const int L = p.L, NP = p.row_pitch(), R = d == 3 ? NP * K1 : NP;
   for (int a = 0; a < d; ++a)
     for (int64_t f = p.fstart[a]; f < p.fstart[a + 1]; ++f)
       for (int tau = 0; tau < L; ++tau) {
@@ -454,7 +454,7 @@ void build_diagonal(const Plan& p, std::vector<double>& diag) {
         for (int b = 0; b < NN; ++b) {
           int64_t idx;
           if (a == 0) idx = p.frows[p.rbase[0] + (f - p.fstart[0]) * L + tau] + b;
-          else idx = p.frows[p.rbase[a] + (f - p.fstart[a]) * R + b + NN * t2] + t1;
+          else idx = p.frows[p.rbase[a] + (f - p.fstart[a]) * R + b + NP * t2] + t1;
           diag[idx] += gb[b] * mt;
         }
       }
@@ -584,7 +584,7 @@ std::vector<int64_t> slab_y_bounds(const Plan& p, const std::vector<int32_t>& ta
 std::vector<int64_t> slab_x_bounds(const Plan& p, const std::vector<int32_t>& table) {
   const int ns = (int)(table.size() / SLAB);
   const int k = p.k, d = p.dim, L = p.L, NN = 2 * k + 1, K1 = k + 1;
-  const int R1 = d == 3 ? NN * K1 : NN;
+  const int R1 = p.row_pitch() * (d == 3 ? K1 : 1);
   std::vector<int64_t> b(ns, 0);
   int64_t hi = 0;
   for (int s = 0; s < ns; ++s) {
@@ -938,9 +938,10 @@ gp_status build_plan(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* 
   // ---- per-face row starts (the gather reads them with one coalesced load per face)
   {
     const int K1 = k + 1, NN = 2 * k + 1;
-    const int R0 = L, R1 = d == 3 ? NN * K1 : NN;
+    const int NP = p.row_pitch(), R0 = L, R1 = NP * (d == 3 ? K1 : 1);
     int64_t off = 0;
     for (int a = 0; a < d; ++a) {
+      off = (off + 3) / 4 * 4;
       p.rbase[a] = off;
       off += (int64_t)(p.fstart[a + 1] - p.fstart[a]) * (a == 0 ? R0 : R1);
     }
@@ -962,8 +963,10 @@ gp_status build_plan(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* 
               const int bc = b <= k ? b : b - k;
               // a = 1: rows (b, tz) -> b + K1 tz ; a = 2: rows (ty, b) -> ty + K1 b
               const int ri = d == 2 ? bc : (a == 1 ? bc + K1 * tr : tr + K1 * bc);
-              dst[b + NN * tr] = rt[ri];
+              dst[b + NP * tr] = rt[ri];
             }
+          for (int tr = 0; tr < outer; ++tr)
+            for (int b = NN; b < NP; ++b) dst[b + NP * tr] = dst[NN - 1 + NP * tr];
         }
       }
   }
@@ -1122,7 +1125,7 @@ gp_status build_plan(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* 
   // ---- bounds of every index the kernels read or write (the GPU has no bounds checker here)
   {
     const int64_t na = p.n_active, K1 = k + 1, NN = 2 * k + 1;
-    const int R1 = d == 3 ? (int)(NN * K1) : (int)NN;
+    const int R1 = p.row_pitch() * (d == 3 ? (int)K1 : 1);
     for (int a = 0; a < d; ++a) {
       const int64_t rows = (int64_t)(p.fstart[a + 1] - p.fstart[a]) * (a == 0 ? L : R1);
       const int64_t span = a == 0 ? NN : K1;          // contiguous values read from each row start

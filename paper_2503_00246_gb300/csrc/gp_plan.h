@@ -38,8 +38,10 @@ struct Plan {
   std::vector<int64_t> inv_cells; // involved cells (sorted)
   std::vector<int32_t> rowtab;    // ninv x L: compact index of (ci*k, row tau) per involved cell
   // per-face row starts of the patch: axis 0: L rows (one per normal line, 2k+1 long);
-  // axis a > 0: (2k+1)*(k+1)^(d-2) rows (normal index b, outer tangential index), k+1 long
+  // axis a > 0: per outer tangential index (k+1 in 3D, one in 2D) the 2k+1 rows of normal index b,
+  // k+1 long, padded to row_pitch() entries (copies of the last row): 16-byte loads
   std::vector<int32_t> frows;
+  int row_pitch() const { return (2 * k + 4) / 4 * 4; }
   int64_t rbase[4] = {0, 0, 0, 0};
   std::vector<int32_t> face_of;   // dim x ncell: face id of (axis, lower cell), -1 if none
 
