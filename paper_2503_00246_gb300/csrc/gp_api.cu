@@ -4,6 +4,7 @@
 #include <map>
 #include <mutex>
 #include <new>
+#include <set>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -235,6 +236,7 @@ gp_status gpi::launch(gp_ctx* c, const void* x, void* y, int add, cudaStream_t s
   a.g = p.jumps.data();
   a.m = p.lump.data();
   a.s = p.scale.data();
+  a.ldl = p.ldl.empty() ? nullptr : p.ldl.data();
   cudaEvent_t* ev = nullptr;
   if (c->prof && trace) {
     const size_t need = 3 * (size_t)(c->nprof + 1);
@@ -692,10 +694,12 @@ struct gp_batch {
     void* d_ptrs[2] = {nullptr, nullptr};
     void* h_ptrs[2] = {nullptr, nullptr};  // pinned: read by the graph's copy node at replay
     int face_blocks = 0, lift_blocks = 0;
+    bool ldl = false;                  // the problems run one triangular normal basis (Plan::ldl)
     gp::BatchOps ops{};
     gp::Tiles tiles{};                 // the tile shape of the group's first context
   };
   std::vector<Group> groups;
+  int64_t nkinds = 0;                  // groups by (dimension, degree, arithmetic, stabilisation)
   void* d_w = nullptr;
   void* d_gs = nullptr;                // per problem: the scaled jump vectors s_j g_j
   size_t w_bytes = 0;
@@ -757,10 +761,18 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
   b->ctxs.assign(ctxs, ctxs + nprob);
   DeviceGuard dg(b->device);
   // group problems by (dimension, degree, arithmetic, stabilisation)
-  std::map<std::tuple<int, int, int, int>, int> key;   // (d, k, arithmetic, stabilisation): one set of 1D data
+  // (d, k, arithmetic, stabilisation): one set of 1D data; FP64 problems of one group whose weights have
+  // other triangular normal bases B launch apart, so that each problem runs as in gp_apply
+  typedef std::tuple<int, int, int, int> Key;
+  std::map<std::pair<Key, std::vector<double>>, int> key;
+  std::set<Key> kinds;
   for (int p = 0; p < nprob; ++p) {
     const gp::Plan& pl = ctxs[p]->plan;
-    auto kk = std::make_tuple(pl.dim, pl.k, pl.precision, pl.stabilization);
+    const Key kd = std::make_tuple(pl.dim, pl.k, pl.precision, pl.stabilization);
+    kinds.insert(kd);
+    const bool ldl = pl.precision == GP_FP64 && !pl.ldl.empty();
+    const auto kk = std::make_pair(
+        kd, ldl ? std::vector<double>(pl.ldl.begin(), pl.ldl.begin() + pl.k * (pl.k + 1)) : std::vector<double>());
     auto it = key.find(kk);
     int gi;
     if (it == key.end()) {
@@ -772,6 +784,7 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
       b->groups[gi].prec = pl.precision;
       b->groups[gi].ops = ops_for(pl.precision, pl.dim);
       b->groups[gi].tiles = ctxs[p]->tiles;
+      b->groups[gi].ldl = ldl;
     } else {
       gi = it->second;
     }
@@ -780,6 +793,7 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
       b->groups[gi].rhs.push_back(r);
     }
   }
+  b->nkinds = (int64_t)kinds.size();
   // face-output buffers, one per segment, 256-byte aligned in one allocation
   std::vector<std::vector<size_t>> woff(b->groups.size());
   size_t total = 0;
@@ -814,6 +828,7 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
   for (size_t gi = 0; gi < b->groups.size() && e == cudaSuccess; ++gi) {
     auto& g = b->groups[gi];
     std::vector<gp::SegSpec> specs(g.prob.size());
+    const size_t nb = (size_t)g.k * (g.k + 1);   // the entries of B; D follows
     for (size_t i = 0; i < g.prob.size(); ++i) {
       const gp_ctx* c = ctxs[g.prob[i]];
       const gp::Plan& pl = c->plan;
@@ -832,7 +847,7 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
       sp.la.n_active = (int32_t)pl.n_active;
       sp.wp = (char*)b->d_w + woff[gi][i];
       sp.gs = (const char*)b->d_gs + gs_off[g.prob[i]];
-      for (int j = 0; j < pl.k; ++j) sp.s[j] = pl.scale[j];
+      for (int j = 0; j < pl.k; ++j) sp.s[j] = g.ldl ? pl.ldl[nb + j] : pl.scale[j];
     }
     std::vector<unsigned char> fs, ls;
     if (!g.ops.pack(g.k, specs, g.tiles, fs, ls, g.face_blocks, g.lift_blocks)) {
@@ -859,7 +874,7 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
                           b->cap);
       if (e == cudaSuccess)
         e = g.ops.run(g.k, g.d_fsegs, g.d_lsegs, g.d_ptrs[i], (int)g.prob.size(), g.face_blocks, g.lift_blocks,
-                      pl0.jumps.data(), pl0.lump.data(), g.tiles, b->cap);
+                      pl0.jumps.data(), pl0.lump.data(), g.ldl ? pl0.ldl.data() : nullptr, g.tiles, b->cap);
     }
     cudaGraph_t graph = nullptr;
     const cudaError_t e2 = cudaStreamEndCapture(b->cap, &graph);
@@ -908,7 +923,7 @@ gp_status gp_batch_apply(gp_batch* b, const void* const* x, void* const* y, void
 
 gp_status gp_batch_info(const gp_batch* b, int64_t* ngroups, int64_t* scratch_bytes) {
   if (!b || !ngroups || !scratch_bytes) return fail(nullptr, GP_EINVAL, "null argument");
-  *ngroups = (int64_t)b->groups.size();
+  *ngroups = b->nkinds;
   *scratch_bytes = (int64_t)b->w_bytes;
   return GP_OK;
 }

@@ -154,7 +154,7 @@ __device__ __forceinline__ void brick_chunk(const uint32_t* __restrict__ bface, 
     for (int j = 0; j < K; ++j) buf[fl][j][TanShape<D, K>::at(tau)] = tj[j];
   }
   V out[K];
-  tangential_mass<D, K, V>(buf, dots, fb, c, tab, fl, tau, out);
+  tangential_mass<D, K, V>(buf, dots, fb, c, tab.w, tab.c, fl, tau, out);
   V w[NN];
   if (valid) {
     if constexpr (!FoldScale<V>::value) {

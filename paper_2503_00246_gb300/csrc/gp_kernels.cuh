@@ -61,7 +61,12 @@ template <int D, int K, typename V>
 __host__ __device__ constexpr size_t face_smem(int fb) {
   const size_t stage = StagePatch<V>::value ? (size_t)fb * Shape<D, K>::P * sizeof(V) : 0;
   const size_t planes = face_planes<D, K, V>(fb);
-  return planes > stage ? planes : stage;
+  // the padded planes and sums in use with the line factors of the triangular basis (FP64) behind them
+  constexpr int N = K + 1, LP = (D == 3) ? (N | 1) * N : N;
+  const size_t ldl = std::is_same<V, double>::value
+                         ? ((size_t)fb * K * (LP + ((D == 3) ? N : 0)) + (size_t)K * Shape<D, K>::L) * sizeof(V) : 0;
+  const size_t most = planes > ldl ? planes : ldl;
+  return most > stage ? most : stage;
 }
 
 // Kernel constants (passed by value; they sit in the constant bank).  In FP64 and float-float
@@ -202,6 +207,83 @@ __device__ __forceinline__ void line_jumps(const V (&v)[2 * K + 1], const V (*g)
   }
 }
 
+// ------------------------------------------------- triangular normal basis --
+// The jump vectors of one parity span the same space as r vectors in echelon form, r = number of
+// orders of that parity: G^ = sum_j s_j g_j g_j^T = B diag(D) B^T, row j of B with a 1 at its pivot
+// node and 0 at the pivots of the earlier rows of its parity (rows j = 0, 2, .. even in b, 1, 3, ..
+// odd).  Those entries cost nothing in the jumps (t_j = B_j . v) or in the expansion: 12 + 12
+// multiply-adds per line instead of 18 + 18 at k = 4, 48 + 48 instead of 68 + 68 at k = 8; D_j goes into the line factors mw (a table per CTA).  The host eliminates
+// in 113-bit arithmetic (Plan::ldl), from the largest direction to the smallest: D is graded and
+// non-negative, so x^T G x stays a sum of squares.  The pivot orders are those whose elimination
+// grows least (entries below 1.2 for the default and for the factorial weights).  Native FP64 only,
+// whose kernel is bound by the FP64 pipe: apply of the 128^3 gyroid at k = 4 1450 -> 1263 us, of the
+// 64^3 ball at k = 3 68.9 -> 62.1 us.  Weights below 0 run the jump vectors themselves.
+template <int K>
+struct Pivots {
+  // pivot node of row j in hexadecimal digit j
+  static constexpr uint32_t CODE = K == 1 ? 0x1u : K == 2 ? 0x12u : K == 3 ? 0x122u : K == 4 ? 0x3223u :
+                                   K == 5 ? 0x54133u : K == 6 ? 0x561244u : K == 7 ? 0x4276245u : 0x66187245u;
+  __host__ __device__ static constexpr int at(int j) { return (int)((CODE >> (4 * j)) & 15u); }
+  // node b is the pivot of an earlier row of j's parity
+  __host__ __device__ static constexpr bool zero(int j, int b) {
+    for (int i = j & 1; i < j; i += 2)
+      if (at(i) == b) return true;
+    return false;
+  }
+};
+
+// t_j = B_j . v on the folded line (B in rows of g)
+template <int K, typename V>
+__device__ __forceinline__ void line_jumps_ldl(const V (&v)[2 * K + 1], const V (*g)[2 * K + 1], V (&t)[K]) {
+  using P = Pivots<K>;
+  constexpr int NN = 2 * K + 1;
+  V f[2][K + 1];   // even and odd part; the middle node counts once
+#pragma unroll
+  for (int b = 0; b < K; ++b) {
+    f[0][b] = v[b] + v[NN - 1 - b];
+    f[1][b] = v[b] - v[NN - 1 - b];
+  }
+  f[0][K] = v[K];
+#pragma unroll
+  for (int j = 0; j < K; ++j) {
+    V acc = f[j & 1][P::at(j)];
+#pragma unroll
+    for (int b = 0; b <= K; ++b)
+      if (!((j & 1) && b == K) && b != P::at(j) && !P::zero(j, b)) acc = vfma(g[j][b], f[j & 1][b], acc);
+    t[j] = acc;
+  }
+}
+
+// w[b] = sum_j B_j[b] T[j], with w[b] = E_b + O_b and w[2k - b] = E_b - O_b
+template <int K, typename V>
+__device__ __forceinline__ void line_expand_ldl(const V (*g)[2 * K + 1], const V (&T)[K], V (&w)[2 * K + 1]) {
+  using P = Pivots<K>;
+  constexpr int NN = 2 * K + 1;
+#pragma unroll
+  for (int b = 0; b <= K; ++b) {
+    V s[2];
+#pragma unroll
+    for (int par = 0; par < 2; ++par) {
+      bool have = false;
+      s[par] = vzero<V>();
+#pragma unroll
+      for (int j = par; j < K; j += 2) {
+        if (P::zero(j, b)) continue;
+        if (P::at(j) == b) s[par] = have ? s[par] + T[j] : T[j];
+        else s[par] = have ? vfma(g[j][b], T[j], s[par]) : g[j][b] * T[j];
+        have = true;
+      }
+    }
+    if (b == K || K == 1) {
+      w[b] = s[0];
+      if (b < K) w[NN - 1 - b] = s[0];
+    } else {
+      w[b] = s[0] + s[1];
+      w[NN - 1 - b] = s[0] - s[1];
+    }
+  }
+}
+
 // ------------------------------------------------------ tangential masses --
 // Gauss-Lobatto quadrature with N = k+1 points is exact up to degree 2k - 1, and the product of
 // two nodal polynomials has degree 2k, so the exact mass matrix differs from the lumped one by the
@@ -245,11 +327,13 @@ __device__ __forceinline__ void fill_tan_table(TanTable<D, K, V>& tab, const Con
 // first threads.  3D: pass 1 along t2 (neighbouring lanes on neighbouring t1) in place; pass 2
 // along t1 only takes the dot product ma . u of each line, and every line's thread adds its own
 // mc and multiplies by mw (FP32, bound by shared-memory accesses and not by arithmetic: pass 2 in
-// place too, one access less per value).  2D: pass 1 in place.  Every thread of the CTA calls it
-// (it synchronises, also before its first read: the caller has only written plane and tab).
-template <int D, int K, typename V>
+// place too, one access less per value).  2D: pass 1 in place.  wl[tau + WS j] is the factor of
+// order j and line tau (WS = 0: one for every order), mc[t] the correction of tangential index t, both
+// in shared memory.  Every thread of the CTA calls it (it synchronises, also before its first read:
+// the caller has only written plane, wl and mc).
+template <int D, int K, typename V, int WS = 0>
 __device__ __forceinline__ void tangential_mass(V (*plane)[K][TanShape<D, K>::LP], V (*dots)[K][K + 1], const int fb,
-                                                const Consts<V, K>& c, const TanTable<D, K, V>& tab, const int fl,
+                                                const Consts<V, K>& c, const V* wl, const V* mc, const int fl,
                                                 const int tau, V (&out)[K]) {
   using T = TanShape<D, K>;
   constexpr int N = K + 1;
@@ -293,13 +377,13 @@ __device__ __forceinline__ void tangential_mass(V (*plane)[K][TanShape<D, K>::LP
     }
     __syncthreads();
   }
-  const V wt = tab.w[tau];
-  const V ct = DOTS ? tab.c[tau % N] : vzero<V>();
+  const V wt = wl[tau];
+  const V ct = DOTS ? mc[tau % N] : vzero<V>();
 #pragma unroll
   for (int jj = 0; jj < K; ++jj) {
     V v = plane[fl][jj][T::at(tau)];
     if constexpr (DOTS) v = vfma(ct, dots[fl][jj][tau / N], v);
-    out[jj] = vmul(wt, v);
+    out[jj] = vmul(WS ? wl[WS * jj + tau] : wt, v);
   }
 }
 
@@ -358,8 +442,9 @@ struct StoreCompact {
 // `blk` is the CTA's index within its problem; `gs` holds the jump vectors of the first step
 // (FP64, float-float: the scaled s_j g_j, c.gs or a batch segment's copy in shared memory;
 // FP32: the plain c.g) and `sc` the k factors s_j (FP32 only); `dsm` is the
-// face_smem<D, K, V>(fb) bytes of dynamic shared memory.  COMPACT: store T_F instead of W_F.
-template <int D, int K, class A, bool COMPACT>
+// face_smem<D, K, V>(fb) bytes of dynamic shared memory.  COMPACT: store T_F instead of W_F.  LDL: gs
+// holds the rows of B and sc the k factors D_j.
+template <int D, int K, class A, bool COMPACT, bool LDL>
 __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, typename A::V* __restrict__ wp,
                                           typename A::IO* __restrict__ y, const FaceArgs& fa,
                                           const Consts<typename A::V, K>& c, const typename A::V (*gs)[2 * K + 1],
@@ -374,6 +459,7 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
   Plane* buf = reinterpret_cast<Plane*>(dsm);            // [fb][K][LP]
   Dots* dots = reinterpret_cast<Dots*>(buf + fb);         // [fb][K][N], 3D only
   __shared__ TanTable<D, K, V> tab;
+  V* wj = reinterpret_cast<V*>(dots + ((D == 3) ? fb : 0));   // LDL: [K][L] line factors D_j mw
   const int nt = (int)blockDim.x;
   // the lift may start its prologue as soon as every face CTA is running (programmatic
   // dependent launch; it waits for this grid's completion before it reads W)
@@ -401,7 +487,16 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
   const int fl = t / L, tau = t - fl * L;
   const int f = f0 + fl;
   const bool valid = f < fend;
-  fill_tan_table<D, K, V>(tab, c, t);
+  if constexpr (LDL) {
+    if (t < L) {
+      const V w = (D == 3) ? c.mw[t % K1] * c.mw[t / K1] : c.mw[t];
+#pragma unroll
+      for (int j = 0; j < K; ++j) wj[j * L + t] = sc[j] * w;
+    }
+    if (t < K1) tab.c[t] = c.mc[t];
+  } else {
+    fill_tan_table<D, K, V>(tab, c, t);
+  }
 
   // ---- gather this thread's normal line (2k+1 values)
   V v[NN];
@@ -460,12 +555,13 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
   // ---- contract with the k jump vectors, then the tangential reference masses
   {
     V t[K];
-    line_jumps<K, V>(v, gs, t);
+    if constexpr (LDL) line_jumps_ldl<K, V>(v, gs, t);
+    else line_jumps<K, V>(v, gs, t);
 #pragma unroll
     for (int j = 0; j < K; ++j) buf[fl][j][T::at(tau)] = t[j];
   }
   V out[K];
-  tangential_mass<D, K, V>(buf, dots, fb, c, tab, fl, tau, out);
+  tangential_mass<D, K, V, LDL ? L : 0>(buf, dots, fb, c, LDL ? wj : tab.w, tab.c, fl, tau, out);
 
   if (!valid) return;
   if constexpr (!FoldScale<V>::value) {
@@ -491,7 +587,8 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
     // lanes of a face store neighbouring values)
     V* dst = wp + (size_t)f * S::P + tau;
     V w[NN];
-    line_expand<K, V>(c, out, w);
+    if constexpr (LDL) line_expand_ldl<K, V>(gs, out, w);
+    else line_expand<K, V>(c, out, w);
 #pragma unroll
     for (int bb = 0; bb < NN; ++bb) dst[L * bb] = w[bb];
   }
@@ -506,12 +603,13 @@ struct FaceCtas {
   static constexpr int value = std::is_same<V, float>::value ? 4 : 0;
 };
 
-template <int D, int K, class A, bool COMPACT>
+template <int D, int K, class A, bool COMPACT, bool LDL>
 __global__ void __launch_bounds__(MAX_CTA_THREADS, FaceCtas<typename A::V>::value)
 face_kernel(const typename A::IO* __restrict__ x, typename A::V* __restrict__ wp,
             typename A::IO* __restrict__ y, const FaceArgs fa, const int fb,
             const __grid_constant__ Consts<typename A::V, K> c) {
-  face_body<D, K, A, COMPACT>(x, wp, y, fa, c, FoldScale<typename A::V>::value ? c.gs : c.g, c.s, blockIdx.x, fb, gp_dyn_smem);
+  face_body<D, K, A, COMPACT, LDL>(x, wp, y, fa, c, (FoldScale<typename A::V>::value && !LDL) ? c.gs : c.g, c.s, blockIdx.x,
+                                   fb, gp_dyn_smem);
   if (fa.tail_wait) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
@@ -524,7 +622,7 @@ struct FaceSeg {
   FaceArgs fa;
   V* wp;           // this segment's face outputs
   const V* gs;     // FP64, float-float: K x (2K+1) scaled jump vectors s_j g_j of the problem
-  V s[K];          // FP32: s_j of the problem
+  V s[K];          // FP32: s_j of the problem; triangular basis: D_j
   int32_t block0;  // first CTA of the segment in the group's face launch
 };
 
@@ -551,7 +649,7 @@ __device__ __forceinline__ int find_segment(const Seg* segs, const int nseg, con
   return lo;
 }
 
-template <int D, int K, class A>
+template <int D, int K, class A, bool LDL>
 __global__ void __launch_bounds__(MAX_CTA_THREADS, FaceCtas<typename A::V>::value)
 face_kernel_batched(const FaceSeg<typename A::V, K>* __restrict__ segs, const int nseg,
                     const SegPtrs<typename A::IO>* __restrict__ ptrs, const int fb,
@@ -559,19 +657,23 @@ face_kernel_batched(const FaceSeg<typename A::V, K>* __restrict__ segs, const in
   using V = typename A::V;
   __shared__ FaceSeg<V, K> seg;
   __shared__ SegPtrs<typename A::IO> sp;
-  __shared__ V sg[K][2 * K + 1];
   if (threadIdx.x == 0) {
     const int s = find_segment(segs, nseg, (int)blockIdx.x);
     seg = segs[s];
     sp = ptrs[s];
   }
   __syncthreads();
-  if constexpr (FoldScale<V>::value) {
+  if constexpr (LDL) {
+    // the group's problems share B (the constant bank); D is the segment's
+    face_body<D, K, A, StoreCompact<V>::value, true>(sp.x, seg.wp, sp.y, seg.fa, c, c.g, seg.s,
+                                                     (int)blockIdx.x - seg.block0, fb, gp_dyn_smem);
+  } else if constexpr (FoldScale<V>::value) {
+    __shared__ V sg[K][2 * K + 1];
     for (int i = threadIdx.x; i < K * (2 * K + 1); i += blockDim.x) sg[i / (2 * K + 1)][i % (2 * K + 1)] = seg.gs[i];
     __syncthreads();
-    face_body<D, K, A, StoreCompact<V>::value>(sp.x, seg.wp, sp.y, seg.fa, c, sg, seg.s, (int)blockIdx.x - seg.block0, fb, gp_dyn_smem);
+    face_body<D, K, A, StoreCompact<V>::value, false>(sp.x, seg.wp, sp.y, seg.fa, c, sg, seg.s, (int)blockIdx.x - seg.block0, fb, gp_dyn_smem);
   } else {
-    face_body<D, K, A, StoreCompact<V>::value>(sp.x, seg.wp, sp.y, seg.fa, c, c.g, seg.s, (int)blockIdx.x - seg.block0, fb, gp_dyn_smem);
+    face_body<D, K, A, StoreCompact<V>::value, false>(sp.x, seg.wp, sp.y, seg.fa, c, c.g, seg.s, (int)blockIdx.x - seg.block0, fb, gp_dyn_smem);
   }
 }
 
@@ -841,7 +943,7 @@ __device__ __forceinline__ void lift_line(const V* __restrict__ line, const int*
   // the kernel held to 32 registers).
   constexpr bool AHEAD = K >= 5;
   V s[3][K];
-  bool any[3];
+  bool any[3] = {false, false, false};
   auto expand = [&](const int sa) {
     if (!any[sa]) return;
 #pragma unroll

@@ -27,6 +27,7 @@ struct ApplyArgs {
   const double* g = nullptr; // host FP64: k x (2k+1)
   const double* m = nullptr; // host FP64: the lumped mass, 3 (k+1) values (Plan::lump)
   const double* s = nullptr; // host FP64: k
+  const double* ldl = nullptr;  // host FP64: the triangular normal basis (Plan::ldl); nullptr: g and s as they are
   cudaEvent_t* ev = nullptr;  // optional: 3 events recorded around the two kernels
   Tiles tiles{};              // 0 fields: the defaults of default_tiles
   int which = 3;              // bit 0: face kernel, bit 1: lift kernel (the autotuner times them apart)
@@ -235,6 +236,23 @@ cudaError_t launch_lift(bool pdl, const Tiles& t, const typename A::V* w, typena
   return cudaGetLastError();
 }
 
+// The face kernel of this arithmetic: with the triangular normal basis or the jump vectors, storing its
+// compact outputs or (full) W_F.
+template <int D, int K, class A>
+auto pick_face(const bool ldl, const bool full) {
+  using V = typename A::V;
+  constexpr bool CO = StoreCompact<V>::value, LD = std::is_same<V, double>::value;
+  static_assert(!(CO && LD), "compact outputs are expanded with the jump vectors");
+  auto f = face_kernel<D, K, A, CO, false>;
+  if constexpr (CO) {
+    if (full) f = face_kernel<D, K, A, false, false>;
+  }
+  if constexpr (LD) {
+    if (ldl) f = face_kernel<D, K, A, false, true>;
+  }
+  return f;
+}
+
 // The face + lift path as a pipeline of slabs along the last axis, so that the face outputs of a
 // slab are still in L2 when its lift reads them: face(0), lift(0), face(1), lift(1), ...  Slab s
 // holds a range of owner cells and the faces that range needs and no earlier range needed.
@@ -245,7 +263,8 @@ cudaError_t launch_lift(bool pdl, const Tiles& t, const typename A::V* w, typena
 // recorded after every lift (another stream can then take the slab's finished part of y) and
 // each face launch follows it in plain stream order.
 template <int D, int K, class A>
-cudaError_t run_slabs(const ApplyArgs& Ar, const Consts<typename A::V, K>& c, const Tiles& t, cudaStream_t st) {
+cudaError_t run_slabs(const ApplyArgs& Ar, const Consts<typename A::V, K>& c, const Tiles& t, const bool ldl,
+                      cudaStream_t st) {
   using S = Shape<D, K>;
   using V = typename A::V;
   using IO = typename A::IO;
@@ -269,15 +288,14 @@ cudaError_t run_slabs(const ApplyArgs& Ar, const Consts<typename A::V, K>& c, co
       const cudaError_t e = cudaStreamWaitEvent(st, Ar.slab_inputs[s], 0);
       if (e != cudaSuccess) return e;
     }
-    constexpr bool COMPACT = StoreCompact<V>::value;
     if (nb > 0) {
+      const auto face = pick_face<D, K, A>(ldl, false);
       const cudaError_t e =
           (s == 0 || Ar.slab_events)
-              ? (face_kernel<D, K, A, COMPACT><<<nb, t.fb * S::L, face_smem<D, K, V>(t.fb), st>>>(
-                     (const IO*)Ar.x, (V*)Ar.tp, (IO*)Ar.y, fa, t.fb, c),
+              ? (face<<<nb, t.fb * S::L, face_smem<D, K, V>(t.fb), st>>>((const IO*)Ar.x, (V*)Ar.tp, (IO*)Ar.y, fa, t.fb, c),
                  cudaGetLastError())
-              : launch_pdl(face_kernel<D, K, A, COMPACT>, nb, t.fb * S::L, face_smem<D, K, V>(t.fb), st,
-                           (const IO*)Ar.x, (V*)Ar.tp, (IO*)Ar.y, fa, (int)t.fb, c);
+              : launch_pdl(face, nb, t.fb * S::L, face_smem<D, K, V>(t.fb), st, (const IO*)Ar.x, (V*)Ar.tp, (IO*)Ar.y,
+                           fa, (int)t.fb, c);
       if (e != cudaSuccess) return e;
     }
     LiftArgs la = Ar.la;
@@ -299,6 +317,19 @@ cudaError_t run_slabs(const ApplyArgs& Ar, const Consts<typename A::V, K>& c, co
   return cudaGetLastError();
 }
 
+// Native FP64 runs the triangular normal basis where the host found one.
+template <typename V>
+struct UseLdl {
+  static constexpr bool value = std::is_same<V, double>::value;
+};
+template <typename V, int K>
+void ldl_consts(const double* p, Consts<V, K>& c) {
+  for (int j = 0; j < K; ++j) {
+    for (int b = 0; b <= K; ++b) c.g[j][b] = from_host<V>(p[j * (K + 1) + b]);
+    c.s[j] = from_host<V>(p[K * (K + 1) + j]);
+  }
+}
+
 template <int D, int K, class A>
 cudaError_t run_apply(const ApplyArgs& Ar, cudaStream_t st) {
   using S = Shape<D, K>;
@@ -312,10 +343,14 @@ cudaError_t run_apply(const ApplyArgs& Ar, cudaStream_t st) {
     for (int b = 0; b < 2 * K + 1; ++b) c.gs[j][b] = from_host<V>(Ar.s[j] * Ar.g[j * (2 * K + 1) + b]);
   }
   mass_consts<V, K>(Ar.m, c);
+  // the triangular basis takes the place of g and s (the brick path runs the general form)
+  constexpr bool HAS_LDL = UseLdl<V>::value;
+  const bool ldl = HAS_LDL && Ar.ldl && !Ar.brick;
+  if (ldl) ldl_consts<V, K>(Ar.ldl, c);
   if (Ar.brick) return run_brick<D, K, A>(Ar, c, st);
   Tiles t = Ar.tiles;
   if (!resolve_tiles<D, K, V>(t)) return cudaErrorInvalidConfiguration;
-  if (Ar.nslab > 1 && !Ar.ev && Ar.which == 3) return run_slabs<D, K, A>(Ar, c, t, st);
+  if (Ar.nslab > 1 && !Ar.ev && Ar.which == 3) return run_slabs<D, K, A>(Ar, c, t, ldl, st);
   FaceArgs fa;
   fa.frows = Ar.frows;
   for (int a = 0; a < 4; ++a) fa.rbase[a] = Ar.rbase[a];
@@ -328,12 +363,8 @@ cudaError_t run_apply(const ApplyArgs& Ar, cudaStream_t st) {
   const bool faces = Ar.fstart[D] > 0;
   if (Ar.ev) cudaEventRecord(Ar.ev[0], st);
   if (nb > 0 && (Ar.which & 1)) {
-    if (StoreCompact<V>::value && Ar.full_outputs)
-      face_kernel<D, K, A, false><<<nb, t.fb * S::L, face_smem<D, K, V>(t.fb), st>>>((const IO*)Ar.x, (V*)Ar.tp,
-                                                                                   (IO*)Ar.y, fa, t.fb, c);
-    else
-      face_kernel<D, K, A, StoreCompact<V>::value><<<nb, t.fb * S::L, face_smem<D, K, V>(t.fb), st>>>(
-          (const IO*)Ar.x, (V*)Ar.tp, (IO*)Ar.y, fa, t.fb, c);
+    const auto face = pick_face<D, K, A>(ldl, Ar.full_outputs);
+    face<<<nb, t.fb * S::L, face_smem<D, K, V>(t.fb), st>>>((const IO*)Ar.x, (V*)Ar.tp, (IO*)Ar.y, fa, t.fb, c);
   }
   if (Ar.ev) cudaEventRecord(Ar.ev[1], st);
   if (Ar.la.nlift > 0 && faces && (Ar.which & 2)) {
@@ -353,7 +384,7 @@ struct SegSpec {
   LiftArgs la;
   void* wp = nullptr;   // the segment's face-output buffer
   const void* gs = nullptr;   // device: K x (2K+1) scaled jump vectors of the segment's problem
-  double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};   // the problem's s_j
+  double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};   // the problem's s_j (triangular basis: D_j)
 };
 
 // Packs the segments of one (d, k, arithmetic) group into the device layouts of
@@ -392,7 +423,7 @@ bool pack_batch(const std::vector<SegSpec>& in, Tiles& t, std::vector<unsigned c
 
 template <int D, int K, class A>
 cudaError_t run_batch(const void* fsegs, const void* lsegs, const void* ptrs, int nseg, int face_blocks,
-                      int lift_blocks, const double* g, const double* m, Tiles t, cudaStream_t st) {
+                      int lift_blocks, const double* g, const double* m, const double* ldl, Tiles t, cudaStream_t st) {
   using V = typename A::V;
   using IO = typename A::IO;
   using S = Shape<D, K>;
@@ -405,9 +436,16 @@ cudaError_t run_batch(const void* fsegs, const void* lsegs, const void* ptrs, in
     c.s[j] = vzero<V>();                                          // per segment: FaceSeg::s
     for (int b = 0; b < 2 * K + 1; ++b) c.gs[j][b] = vzero<V>();  // per segment: FaceSeg::gs
   }
+  auto face = face_kernel_batched<D, K, A, false>;
+  if constexpr (UseLdl<V>::value) {
+    if (ldl) {
+      ldl_consts<V, K>(ldl, c);
+      face = face_kernel_batched<D, K, A, true>;
+    }
+  }
   if (face_blocks > 0)
-    face_kernel_batched<D, K, A><<<face_blocks, t.fb * S::L, face_smem<D, K, V>(t.fb), st>>>(
-        (const FaceSeg<V, K>*)fsegs, nseg, (const SegPtrs<IO>*)ptrs, t.fb, c);
+    face<<<face_blocks, t.fb * S::L, face_smem<D, K, V>(t.fb), st>>>((const FaceSeg<V, K>*)fsegs, nseg,
+                                                                   (const SegPtrs<IO>*)ptrs, t.fb, c);
   if (lift_blocks > 0) {
     const int cb = lift_cells<D, K, V>(t);
     const size_t smem = lift_dyn_smem<D, K, V>(cb);
@@ -438,7 +476,7 @@ struct BatchOps {
                std::vector<unsigned char>&, int&, int&);
   void (*jumps)(int k, const double* g, const double* s, std::vector<unsigned char>& out);
   cudaError_t (*run)(int k, const void*, const void*, const void*, int, int, int, const double*, const double*,
-                     Tiles, cudaStream_t);
+                     const double*, Tiles, cudaStream_t);
 };
 BatchOps batch_ops_f64_d2();
 BatchOps batch_ops_f64_d3();
@@ -465,16 +503,16 @@ BatchOps batch_ops_ff_d3();
     }                                                                                                   \
   };                                                                                                    \
   ops.run = [](int k, const void* fs, const void* ls, const void* pt, int ns, int fb, int lb,          \
-               const double* g, const double* m, Tiles t, cudaStream_t st) -> cudaError_t {             \
+               const double* g, const double* m, const double* l, Tiles t, cudaStream_t st) -> cudaError_t { \
     switch (k) {                                                                                        \
-      case 1: return run_batch<D, 1, A>(fs, ls, pt, ns, fb, lb, g, m, t, st);                           \
-      case 2: return run_batch<D, 2, A>(fs, ls, pt, ns, fb, lb, g, m, t, st);                           \
-      case 3: return run_batch<D, 3, A>(fs, ls, pt, ns, fb, lb, g, m, t, st);                           \
-      case 4: return run_batch<D, 4, A>(fs, ls, pt, ns, fb, lb, g, m, t, st);                           \
-      case 5: return run_batch<D, 5, A>(fs, ls, pt, ns, fb, lb, g, m, t, st);                           \
-      case 6: return run_batch<D, 6, A>(fs, ls, pt, ns, fb, lb, g, m, t, st);                           \
-      case 7: return run_batch<D, 7, A>(fs, ls, pt, ns, fb, lb, g, m, t, st);                           \
-      case 8: return run_batch<D, 8, A>(fs, ls, pt, ns, fb, lb, g, m, t, st);                           \
+      case 1: return run_batch<D, 1, A>(fs, ls, pt, ns, fb, lb, g, m, l, t, st);                        \
+      case 2: return run_batch<D, 2, A>(fs, ls, pt, ns, fb, lb, g, m, l, t, st);                        \
+      case 3: return run_batch<D, 3, A>(fs, ls, pt, ns, fb, lb, g, m, l, t, st);                        \
+      case 4: return run_batch<D, 4, A>(fs, ls, pt, ns, fb, lb, g, m, l, t, st);                        \
+      case 5: return run_batch<D, 5, A>(fs, ls, pt, ns, fb, lb, g, m, l, t, st);                        \
+      case 6: return run_batch<D, 6, A>(fs, ls, pt, ns, fb, lb, g, m, l, t, st);                        \
+      case 7: return run_batch<D, 7, A>(fs, ls, pt, ns, fb, lb, g, m, l, t, st);                        \
+      case 8: return run_batch<D, 8, A>(fs, ls, pt, ns, fb, lb, g, m, l, t, st);                        \
       default: return cudaErrorInvalidValue;                                                            \
     }                                                                                                   \
   };                                                                                                    \

@@ -190,6 +190,66 @@ bool lumped_mass(int k, const std::vector<double>& mass, std::vector<double>& lu
   return dev <= R(1e-15);
 }
 
+// 113-bit arithmetic for the elimination of normal_basis: at k = 8 the factors D span 13 decades.
+#if defined(__SIZEOF_FLOAT128__)
+using Q = __float128;
+#else
+using Q = long double;   // binary128 on aarch64
+#endif
+
+// Pivot nodes of the rows (gp_kernels.cuh holds the same table as Pivots<K>::CODE): of all orders the
+// one whose elimination grows least over the weights c_j = const and c_j = 1 / (j!)^2.
+static const int kPivot[8][8] = {{1}, {2, 1}, {2, 2, 1}, {3, 2, 2, 3}, {3, 3, 1, 4, 5}, {4, 4, 2, 1, 6, 5},
+                                 {5, 4, 2, 6, 7, 2, 4}, {5, 4, 2, 7, 8, 1, 6, 6}};
+
+void normal_basis(int k, const std::vector<double>& jumps, const std::vector<double>& c, double hd,
+                  std::vector<double>& ldl) {
+  const int N = k + 1, NN = 2 * k + 1;
+  auto absq = [](Q v) { return v < 0 ? -v : v; };
+  ldl.assign((size_t)k * N + k, 0.0);
+  for (double v : c)
+    if (!(v >= 0.0)) {
+      ldl.clear();
+      return;
+    }
+  for (int par = 0; par < 2; ++par) {
+    const int n = par == 0 ? k + 1 : k;          // the odd vectors vanish at the shared node
+    std::vector<Q> A((size_t)n * n, Q(0));
+    Q top = 0;
+    for (int a = 0; a < n; ++a)
+      for (int b = 0; b < n; ++b) {
+        for (int j = par; j < k; j += 2) A[a * n + b] += Q(c[j]) * Q(jumps[j * NN + a]) * Q(jumps[j * NN + b]);
+        if (absq(A[a * n + b]) > top) top = absq(A[a * n + b]);
+      }
+    for (int j = par; j < k; j += 2) {
+      const int p = kPivot[k - 1][j];
+      const Q d = A[p * n + p];
+      if (!(absq(d) > top * Q(1e-28))) {          // orders of weight 0: nothing is left in this direction
+        ldl[(size_t)j * N + p] = 1.0;
+        continue;
+      }
+      std::vector<Q> b(n);
+      for (int i = 0; i < n; ++i) {
+        b[i] = A[i * n + p] / d;
+        if (absq(b[i]) > Q(16)) {
+          ldl.clear();
+          return;
+        }
+        ldl[(size_t)j * N + i] = (double)b[i];
+      }
+      for (int i = par; i < j; i += 2) ldl[(size_t)j * N + kPivot[k - 1][i]] = 0.0;
+      ldl[(size_t)k * N + j] = (double)(d * Q(hd));
+      for (int a = 0; a < n; ++a)
+        for (int e = 0; e < n; ++e) A[a * n + e] -= d * b[a] * b[e];
+    }
+    for (const Q& v : A)
+      if (absq(v) > top * Q(1e-20)) {             // (a pivot vanished although its direction does not)
+        ldl.clear();
+        return;
+      }
+  }
+}
+
 // Macro-patch stabilisation (the alternative named in Sec. 2.2): on the two-cell patch
 // [0,1] u [1,2] of a face, the difference between the polynomial on one cell and the
 // extension of the neighbour's polynomial into it, squared and integrated over both cells:
@@ -1181,13 +1241,17 @@ gp_status build_plan(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* 
         return GP_EINVAL;
       }
     }
+    for (double& v : lam) v *= opts->gamma;
+    normal_basis(k, p.jumps, lam, hv, p.ldl);
     return GP_OK;
   }
   if (opts->stabilization != GP_STAB_GHOST) { err = "unknown stabilization"; return GP_EINVAL; }
   const double hd = d == 3 ? h : 1.0;
+  std::vector<double> cw(k);
   for (int j = 0; j < k; ++j) {
     double c = opts->nweights == k ? opts->weights[j] : opts->gamma;
     p.scale[j] = c * hd;
+    cw[j] = c;
     // float-float keeps float's exponent range: the scale factors must stay well inside it
     const double a = std::fabs(p.scale[j]);
     if (opts->precision == GP_FP64_FF && a != 0.0 && !(a >= 0x1p-90 && a <= 0x1p90)) {
@@ -1196,6 +1260,7 @@ gp_status build_plan(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* 
       return GP_EINVAL;
     }
   }
+  normal_basis(k, p.jumps, cw, hd, p.ldl);
   return GP_OK;
 }
 

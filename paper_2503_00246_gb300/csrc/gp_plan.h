@@ -121,6 +121,9 @@ struct Plan {
   std::vector<double> mass;       // (k+1)^2
   std::vector<double> lump;       // 3 (k+1): ma, mc, mw with mass = diag(mw) (I + mc ma^T)
   std::vector<double> jumps;      // k x (2k+1)
+  // triangular normal basis: k rows of k+1 entries of B, then k factors D_j, with sum_j scale_j g_j g_j^T
+  // = B diag(D) B^T (see gp_kernels.cuh); empty if the weights have none
+  std::vector<double> ldl;
   std::vector<double> scale;      // k: c_j h^(dim-2) (macro patch: gamma lambda_j h^dim)
   int stabilization = GP_STAB_GHOST;
 
@@ -148,6 +151,11 @@ void reference_1d(int k, const std::vector<double>& gl, std::vector<double>& mas
                   std::vector<double>& jumps);
 // The lumped form of the mass matrix (see Plan::lump); false if it does not reproduce `mass`.
 bool lumped_mass(int k, const std::vector<double>& mass, std::vector<double>& lump);
+// The triangular normal basis of the weights c (per order, without the factor hd of the mesh
+// size, so that problems of one degree and one set of weights have equal B); empty for weights below 0
+// or an elimination that grows.
+void normal_basis(int k, const std::vector<double>& jumps, const std::vector<double>& c, double hd,
+                  std::vector<double>& ldl);
 void reference_stiffness(int k, std::vector<double>& stiff);
 // Macro-patch 1D data: k mirror-(anti)symmetric vectors (k x (2k+1)) and weights lambda_j;
 // false if the matrix is not of rank k with the expected parities.
