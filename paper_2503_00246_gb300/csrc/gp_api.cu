@@ -21,8 +21,13 @@ cudaError_t noalloc_scratch(int device, void** out);
 namespace {
 thread_local std::string g_err;
 
-// dst[c0 + i] = src[c0 + i] over the runs (c0, len): one warp per run, consecutive lanes on
-// consecutive elements (src: a device view of page-locked host memory)
+constexpr int32_t kRunMax = 256;   // elements per touched run: one batch of loads of a warp
+
+// dst[c0 + i] = src[c0 + i] over the runs (c0, len <= kRunMax): one warp per run, consecutive lanes on
+// consecutive elements (src: a device view of page-locked host memory).  Bound by the latency of the
+// host link: all of a run's loads are issued before the first store (runs of up to 1024 elements
+// with one load in flight per lane took 33 us for any 1.2 MB slab, 500 of the 914 us of a host apply of
+// the 96^3 ball at k = 4 in FP64).
 template <typename T>
 __global__ void __launch_bounds__(256) gather_runs_kernel(const T* __restrict__ src, T* __restrict__ dst,
                                                          const int2* __restrict__ runs, const int nruns) {
@@ -30,7 +35,13 @@ __global__ void __launch_bounds__(256) gather_runs_kernel(const T* __restrict__ 
   const int w0 = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nw = (int)((gridDim.x * blockDim.x) >> 5);
   for (int r = w0; r < nruns; r += nw) {
     const int2 run = __ldg(runs + r);
-    for (int i = lane; i < run.y; i += 32) dst[run.x + i] = src[run.x + i];
+    T v[kRunMax / 32];
+#pragma unroll
+    for (int u = 0; u < kRunMax / 32; ++u)
+      if (lane + 32 * u < run.y) v[u] = src[run.x + lane + 32 * u];
+#pragma unroll
+    for (int u = 0; u < kRunMax / 32; ++u)
+      if (lane + 32 * u < run.y) dst[run.x + lane + 32 * u] = v[u];
   }
 }
 }  // namespace
@@ -70,11 +81,10 @@ const void* device_view(const void* host) {
 cudaError_t ensure_touched_runs(gp_ctx* c) {
   if (c->ntruns >= 0) return cudaSuccess;
   // the touched DoFs are the active DoFs outside the zero runs (which are sorted and disjoint)
-  constexpr int32_t RUN_MAX = 1024;
   const gp::Plan& p = c->plan;
   std::vector<int2> runs;
   auto emit = [&](int64_t a, int64_t b) {
-    for (; a < b; a += RUN_MAX) runs.push_back(make_int2((int)a, (int)std::min<int64_t>(RUN_MAX, b - a)));
+    for (; a < b; a += kRunMax) runs.push_back(make_int2((int)a, (int)std::min<int64_t>(kRunMax, b - a)));
   };
   int64_t pos = 0;
   for (int64_t r = 0; r < p.num_zero_runs(); ++r) {
@@ -99,7 +109,7 @@ cudaError_t ensure_host_pipeline(gp_ctx* c) {
   cudaError_t e = ensure_touched_runs(c);
   if (e != cudaSuccess) return e;
   if (!c->use_brick) {
-    c->hslabs = gp::slab_table(c->plan, host_slabs(c->plan.precision));
+    c->hslabs = gp::slab_table(c->plan, host_slabs((double)c->plan.n_active * c->elem));
     c->hbounds = gp::slab_y_bounds(c->plan, c->hslabs);
     // the touched runs slab s gathers: those that start below the x its face launch reads and
     // were not gathered for an earlier slab (the last slab takes the rest)

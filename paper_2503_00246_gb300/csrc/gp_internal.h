@@ -1,6 +1,8 @@
 // Internal declarations shared by the C-ABI translation units.
 #pragma once
 
+#include <algorithm>
+#include <cmath>
 #include <string>
 #include <vector>
 
@@ -97,10 +99,15 @@ constexpr int MAX_SLABS = 64;
 // the runs of touched DoFs (built on first use), and the copy of those runs of x.
 const void* device_view(const void* host);
 cudaError_t ensure_touched_runs(gp_ctx* c);
-// The host-apply slab pipeline of c (host_slabs slabs; none when the plan has too few owners):
-// 8 for FP32, 16 for the FP64 forms (measured best on the 128^3 gyroid at k = 4: FP32 35.7 /
-// 38.3 / 37.6 GDoF/s end to end with 16 / 8 / 4 slabs, FP64 19.7 / 19.1 / 17.4).
-inline int host_slabs(int precision) { return precision == GP_FP32 ? 8 : 16; }
+// The host-apply slab pipeline of c (host_slabs slabs; none when the plan has too few owners).  The
+// first copy of y starts after one slab's launches, and each slab adds about 40 us of launches that are
+// too small for the GPU, so that the best count grows like the square root of y's bytes: measured best
+// (us at 1 / 2 / 4 / 8 / 16 slabs) for y of 4 MB 1 (72 / 77 / 99), 21 MB 2 to 3 (374 / 329 / 341 /
+// 488 / 729), 88 MB 4 to 8 (842 / 703 / 650 / 664 / 767), 235 MB 8 to 12 (1733 / 1656 / 1546 / 1471 /
+// 1494), 470 MB 12 (4203 / 3561 / 3137 / 2966 / 3174).
+inline int host_slabs(double y_bytes) {
+  return std::min(16, std::max(1, (int)(std::sqrt(y_bytes / (4 << 20)) + 0.5)));
+}
 cudaError_t ensure_host_pipeline(gp_ctx* c);
 cudaError_t gather_runs(const void* src, void* dst, const int2* runs, int nruns, int elem, cudaStream_t st);
 // Default faces per chunk of the brick kernel (about 256 threads).

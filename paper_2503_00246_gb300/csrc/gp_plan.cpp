@@ -644,15 +644,16 @@ std::vector<int64_t> slab_y_bounds(const Plan& p, const std::vector<int32_t>& ta
 std::vector<int64_t> slab_x_bounds(const Plan& p, const std::vector<int32_t>& table) {
   const int ns = (int)(table.size() / SLAB);
   const int k = p.k, d = p.dim, L = p.L, NN = 2 * k + 1, K1 = k + 1;
-  const int R1 = p.row_pitch() * (d == 3 ? K1 : 1);
+  const int NP = p.row_pitch(), outer = d == 3 ? K1 : 1, R1 = NP * outer;
   std::vector<int64_t> b(ns, 0);
   int64_t hi = 0;
   for (int s = 0; s < ns; ++s) {
     for (int a = 0; a < d; ++a) {
       const int rows = a == 0 ? L : R1, span = a == 0 ? NN : K1;
       for (int64_t f = table[(size_t)s * SLAB + 2 + 2 * a]; f < table[(size_t)s * SLAB + 3 + 2 * a]; ++f) {
+        // the numbering is lexicographic: the patch's last row starts last
         const int32_t* r = &p.frows[p.rbase[a] + (f - p.fstart[a]) * rows];
-        for (int i = 0; i < rows; ++i) hi = std::max<int64_t>(hi, (int64_t)r[i] + span);
+        hi = std::max<int64_t>(hi, (int64_t)r[a == 0 ? L - 1 : NN - 1 + NP * (outer - 1)] + span);
       }
     }
     b[s] = hi;
