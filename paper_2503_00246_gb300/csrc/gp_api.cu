@@ -400,7 +400,7 @@ gp_status gp_setup(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* op
     if (e == cudaSuccess) e = upload(&c->d_frows, p.frows);
     if (e == cudaSuccess) e = upload(&c->d_lwin, p.lwin);
     if (e == cudaSuccess) e = upload(&c->d_lrow, p.lrow);
-    if (e == cudaSuccess) e = upload(&c->d_lmask, p.lmask);
+    if (e == cudaSuccess && p.precision == GP_FP32) e = upload(&c->d_lmask, p.lmask);   // compact outputs only
     if (e == cudaSuccess) e = upload(&c->d_zruns, zruns);
     const size_t vbytes = p.precision == GP_FP32 ? 4 : 8;
     if (c->use_brick) {

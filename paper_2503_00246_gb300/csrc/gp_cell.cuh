@@ -10,8 +10,10 @@
 // e = M^ b along y; y_K = M^ (h^3 c + h (d + e)) + S^ (h c) along z (3D), or
 // y_K = M^ (h^2 a + b) + S^ a along y (2D).  One thread per x-line of a cell; the y
 // and z passes go through shared memory.  Every 1D application uses the even / odd
-// halves of the centrosymmetric M^ and S^ (about half the multiply-adds; CellConsts).  The float-float form renormalises after every
-// operation here (the model system's outer residual needs the full accuracy).
+// halves of the centrosymmetric M^ and S^ (about half the multiply-adds; CellConsts).  Bound by
+// instruction issue in float-float (88%): its sums are compensated dot products with one
+// renormalisation each (model system's apply on the 64^3 gyroid at k = 4: 386 -> 362 us against
+// renormalised multiply-adds, error against 64 bits 5.4e-15 both).
 //
 // Two launches, like the face operator: cell_kernel stores every cell's (k+1)^d
 // outputs, and cell_gather adds, for every node, the outputs of the (up to 2^d) active
@@ -62,32 +64,40 @@ struct CellConsts {
   V hs;          // ws h^(d-2)
 };
 
+// Folds and partial sums keep their terms as compensated dot products (gp_arith.cuh: plain FP32 and
+// FP64, for float-float 12 float operations per term and one renormalisation per result, against 15
+// per renormalised multiply-add; the float-float kernel is bound by instruction issue).
 template <int N, class V>
 __device__ __forceinline__ void eo_fold(const V (&x)[N], V (&e)[(N + 1) / 2], V (&o)[N / 2]) {
 #pragma unroll
   for (int i = 0; i < N / 2; ++i) {
-    e[i] = vadd(x[i], x[N - 1 - i]);
-    o[i] = vsub(x[i], x[N - 1 - i]);
+    e[i] = vadd_loose(x[i], x[N - 1 - i]);
+    o[i] = vsub_loose(x[i], x[N - 1 - i]);
   }
   if constexpr (N % 2 == 1) e[N / 2] = x[N / 2];
 }
 
 // the even (E) or odd (O) partial sum of output p: sum_i a[p][i] v[i]
 template <int M, class V>
-__device__ __forceinline__ V eo_row(const V (&a)[M], const V (&v)[M]) {
-  V acc = vmul(a[0], v[0]);
+__device__ __forceinline__ Dot<V> eo_row(const V (&a)[M], const V (&v)[M]) {
+  Dot<V> acc = dot_first(a[0], v[0]);
 #pragma unroll
-  for (int i = 1; i < M; ++i) acc = vfma(a[i], v[i], acc);
+  for (int i = 1; i < M; ++i) dot_fma(acc, a[i], v[i]);
   return acc;
 }
 template <int M, class V>
-__device__ __forceinline__ V eo_row2(const V (&a)[M], const V (&v)[M], const V (&b)[M], const V (&w)[M]) {
-  V acc = vmul(a[0], v[0]);
+__device__ __forceinline__ Dot<V> eo_row2(const V (&a)[M], const V (&v)[M], const V (&b)[M], const V (&w)[M]) {
+  Dot<V> acc = eo_row<M>(a, v);
 #pragma unroll
-  for (int i = 1; i < M; ++i) acc = vfma(a[i], v[i], acc);
-#pragma unroll
-  for (int i = 0; i < M; ++i) acc = vfma(b[i], w[i], acc);
+  for (int i = 0; i < M; ++i) dot_fma(acc, b[i], w[i]);
   return acc;
+}
+// f x + g y
+template <class V>
+__device__ __forceinline__ V dot2(const V f, const V x, const V g, const V y) {
+  Dot<V> acc = dot_first(f, x);
+  dot_fma(acc, g, y);
+  return dot_value(acc);
 }
 
 // Device tables of the cell operator (see Plan::crow, cwin, corow).
@@ -144,13 +154,13 @@ cell_kernel(const typename A::IO* __restrict__ x, typename A::V* __restrict__ wc
     eo_fold<K1>(xl, e, o);
 #pragma unroll
     for (int p = 0; p < NE; ++p) {
-      const V ae = eo_row<NE>(c.me[p], e), be = eo_row<NE>(c.se[p], e);
+      const Dot<V> ae = eo_row<NE>(c.me[p], e), be = eo_row<NE>(c.se[p], e);
       if (p < H) {
-        const V ao = eo_row<H>(c.mo[p], o), bo = eo_row<H>(c.so[p], o);
-        sab[cl][p + K1 * line] = VPair<V>{vadd(ae, ao), vadd(be, bo)};
-        sab[cl][K1 - 1 - p + K1 * line] = VPair<V>{vsub(ae, ao), vsub(be, bo)};
+        const Dot<V> ao = eo_row<H>(c.mo[p], o), bo = eo_row<H>(c.so[p], o);
+        sab[cl][p + K1 * line] = VPair<V>{dot_merge<false>(ae, ao), dot_merge<false>(be, bo)};
+        sab[cl][K1 - 1 - p + K1 * line] = VPair<V>{dot_merge<true>(ae, ao), dot_merge<true>(be, bo)};
       } else {
-        sab[cl][p + K1 * line] = VPair<V>{ae, be};
+        sab[cl][p + K1 * line] = VPair<V>{dot_value(ae), dot_value(be)};
       }
     }
   }
@@ -172,14 +182,16 @@ cell_kernel(const typename A::IO* __restrict__ x, typename A::V* __restrict__ wc
       eo_fold<K1>(by, be, bo);
 #pragma unroll
       for (int p = 0; p < NE; ++p) {
-        const V cE = eo_row<NE>(c.me[p], ae), tE = eo_row2<NE>(c.se[p], ae, c.me[p], be);
+        const Dot<V> cE = eo_row<NE>(c.me[p], ae), tE = eo_row2<NE>(c.se[p], ae, c.me[p], be);
         if (p < H) {
-          const V cO = eo_row<H>(c.mo[p], ao), tO = eo_row2<H>(c.so[p], ao, c.mo[p], bo);
-          const V c0 = vadd(cE, cO), c1 = vsub(cE, cO), t0 = vadd(tE, tO), t1 = vsub(tE, tO);
-          sab[cl][i1 + K1 * (p + K1 * i3)] = VPair<V>{vfma(c.hm, c0, vmul(c.hs, t0)), vmul(c.hs, c0)};
-          sab[cl][i1 + K1 * (K1 - 1 - p + K1 * i3)] = VPair<V>{vfma(c.hm, c1, vmul(c.hs, t1)), vmul(c.hs, c1)};
+          const Dot<V> cO = eo_row<H>(c.mo[p], ao), tO = eo_row2<H>(c.so[p], ao, c.mo[p], bo);
+          const V c0 = dot_merge<false>(cE, cO), c1 = dot_merge<true>(cE, cO);
+          const V t0 = dot_merge<false>(tE, tO), t1 = dot_merge<true>(tE, tO);
+          sab[cl][i1 + K1 * (p + K1 * i3)] = VPair<V>{dot2(c.hs, t0, c.hm, c0), vmul(c.hs, c0)};
+          sab[cl][i1 + K1 * (K1 - 1 - p + K1 * i3)] = VPair<V>{dot2(c.hs, t1, c.hm, c1), vmul(c.hs, c1)};
         } else {
-          sab[cl][i1 + K1 * (p + K1 * i3)] = VPair<V>{vfma(c.hm, cE, vmul(c.hs, tE)), vmul(c.hs, cE)};
+          const V c0 = dot_value(cE), t0 = dot_value(tE);
+          sab[cl][i1 + K1 * (p + K1 * i3)] = VPair<V>{dot2(c.hs, t0, c.hm, c0), vmul(c.hs, c0)};
         }
       }
     }
@@ -198,13 +210,13 @@ cell_kernel(const typename A::IO* __restrict__ x, typename A::V* __restrict__ wc
       eo_fold<K1>(gz, ge, go);
 #pragma unroll
       for (int p = 0; p < NE; ++p) {
-        const V yE = eo_row2<NE>(c.me[p], fe, c.se[p], ge);
+        const Dot<V> yE = eo_row2<NE>(c.me[p], fe, c.se[p], ge);
         if (p < H) {
-          const V yO = eo_row2<H>(c.mo[p], fo, c.so[p], go);
-          yout[p] = vadd(yE, yO);
-          yout[K1 - 1 - p] = vsub(yE, yO);
+          const Dot<V> yO = eo_row2<H>(c.mo[p], fo, c.so[p], go);
+          yout[p] = dot_merge<false>(yE, yO);
+          yout[K1 - 1 - p] = dot_merge<true>(yE, yO);
         } else {
-          yout[p] = yE;
+          yout[p] = dot_value(yE);
         }
       }
       if (valid) {
@@ -222,20 +234,20 @@ cell_kernel(const typename A::IO* __restrict__ x, typename A::V* __restrict__ wc
     for (int q = 0; q < K1; ++q) {
       const VPair<V> v = sab[cl][line + K1 * q];
       const V ay = v.a, by = v.b;
-      f[q] = vfma(c.hm, ay, vmul(c.hs, by));
+      f[q] = dot2(c.hs, by, c.hm, ay);
       g[q] = vmul(c.hs, ay);
     }
     eo_fold<K1>(f, fe, fo);
     eo_fold<K1>(g, ge, go);
 #pragma unroll
     for (int p = 0; p < NE; ++p) {
-      const V yE = eo_row2<NE>(c.me[p], fe, c.se[p], ge);
+      const Dot<V> yE = eo_row2<NE>(c.me[p], fe, c.se[p], ge);
       if (p < H) {
-        const V yO = eo_row2<H>(c.mo[p], fo, c.so[p], go);
-        yout[p] = vadd(yE, yO);
-        yout[K1 - 1 - p] = vsub(yE, yO);
+        const Dot<V> yO = eo_row2<H>(c.mo[p], fo, c.so[p], go);
+        yout[p] = dot_merge<false>(yE, yO);
+        yout[K1 - 1 - p] = dot_merge<true>(yE, yO);
       } else {
-        yout[p] = yE;
+        yout[p] = dot_value(yE);
       }
     }
     if (valid) {

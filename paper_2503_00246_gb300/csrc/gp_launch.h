@@ -301,7 +301,7 @@ cudaError_t run_slabs(const ApplyArgs& Ar, const Consts<typename A::V, K>& c, co
     LiftArgs la = Ar.la;
     la.lwin = Ar.la.lwin + (size_t)sl[0] * NW;
     la.lrow = Ar.la.lrow + (size_t)sl[0] * KR;
-    la.lmask = Ar.la.lmask + sl[0];
+    la.lmask = Ar.la.lmask ? Ar.la.lmask + sl[0] : nullptr;
     la.nlift = sl[1] - sl[0];
     if (la.nlift > 0) {
       // programmatic dependent of this slab's face launch (a plain launch after an event)

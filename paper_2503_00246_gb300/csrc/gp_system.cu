@@ -42,7 +42,7 @@ struct gp_system {
   double* dinv = nullptr;   // 1 / diag(A) (Jacobi)
   float* dinv32 = nullptr;
   double* part = nullptr;   // dot partials + result
-  double* part_pq = nullptr;  // p . q partials of the gather, then their sum
+  double* part_pq = nullptr;  // (behind part) p . q partials of the gather, then their sum
   double* h_res = nullptr;  // pinned copy of the dot result
   void* d_cg = nullptr;     // CgScalars of the running CG (device)
   void* h_cg = nullptr;     // pinned copy
@@ -165,7 +165,7 @@ gp::CellsFn cells_for(const gp::Plan& p) {
 void sys_free(gp_system* s) {
   void* ptrs[] = {s->d_crow, s->d_cwin, s->d_corow, s->d_wc, s->d_o2l_hi, s->d_o2l_lo, s->r, s->p, s->q, s->dd,
                   s->z, s->ri, s->r32,
-                  s->d32, s->ri32, s->p32, s->q32, s->z32, s->dinv, s->dinv32, s->part, s->part_pq, s->d_cg};
+                  s->d32, s->ri32, s->p32, s->q32, s->z32, s->dinv, s->dinv32, s->part, s->d_cg};
   for (void* v : ptrs)
     if (v) cudaFree(v);
   if (s->h_res) cudaFreeHost(s->h_res);
@@ -598,8 +598,8 @@ gp_status gp_system_create(gp_ctx* hi, gp_ctx* lo, gp_system** out) {
   if (e == cudaSuccess && lo) e = cudaMalloc(&s->p32, n4);
   if (e == cudaSuccess && lo) e = cudaMalloc(&s->q32, n4);
   s->nparts = (int)gp::gather_ctas(p.dim, p.k, p.ncown);
-  if (e == cudaSuccess) e = cudaMalloc(&s->part, (size_t)(2 * s->nblk + 2) * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&s->part_pq, (size_t)(s->nparts + 1) * sizeof(double));
+  if (e == cudaSuccess) e = cudaMalloc(&s->part, (size_t)(2 * s->nblk + 2 + s->nparts + 1) * sizeof(double));
+  if (e == cudaSuccess) s->part_pq = s->part + 2 * s->nblk + 2;
   if (e == cudaSuccess) e = cudaMallocHost(&s->h_res, sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&s->d_cg, 2 * sizeof(CgScalars));
   if (e == cudaSuccess) e = cudaMallocHost(&s->h_cg, sizeof(CgScalars));
