@@ -121,7 +121,7 @@ struct CellTabs {
   const int32_t* own2lift = nullptr;
 };
 
-constexpr int GATHER_THREADS = 256;
+constexpr int GATHER_THREADS = 512;   // most threads of a gather CTA (gather_threads)
 
 // the two fields of a pass kept side by side in shared memory, so that one access
 // moves both (half the shared-memory instructions)
@@ -351,13 +351,18 @@ __device__ __forceinline__ void gather_row(const typename A::V* __restrict__ wc,
   }
 }
 
-// A gather CTA takes GATHER_THREADS / KR whole owner cells.  Its threads are ordered
+// A gather CTA takes whole owner cells: 32 of them for k = 3 and 4 in 3D, so that every row type fills
+// whole warps (model-system apply of the 64^3 gyroid at k = 4: float-float 364 -> 361 us, FP32
+// 143 -> 140, FP64 1243 -> 1223), else about 256 threads.  Its threads are ordered
 // by row type (q == 0, r == 0) first, so that a warp's rows take the same path through
 // the row code (the candidate ghost faces and cell windows depend on the type): 3D
 // rows (0, 0), then (0, r > 0), (q > 0, 0), (q > 0, r > 0); 2D rows q = 0, then q > 0.
 // Within a type, owner-major.
 __host__ __device__ constexpr int gather_owners_per_cta(int dim, int k) {
-  return (dim == 3 ? k * k : k) >= GATHER_THREADS ? 1 : GATHER_THREADS / (dim == 3 ? k * k : k);
+  return (dim == 3 && (k == 3 || k == 4)) ? 32 : (dim == 3 ? k * k : k) >= 256 ? 1 : 256 / (dim == 3 ? k * k : k);
+}
+__host__ __device__ constexpr int gather_threads(int dim, int k) {
+  return (dim == 3 && (k == 3 || k == 4)) ? 32 * k * k : 256;
 }
 inline int64_t gather_ctas(int dim, int k, int64_t ncown) {
   const int opc = gather_owners_per_cta(dim, k);
@@ -406,7 +411,7 @@ __host__ __device__ __forceinline__ bool gather_slot(const int u, int& o, int& q
 }
 
 template <int D, int K, class A>
-__global__ void __launch_bounds__(GATHER_THREADS)
+__global__ void __launch_bounds__(gather_threads(D, K))
 cell_gather(const typename A::V* __restrict__ wc, typename A::IO* __restrict__ y, const int add, const CellTabs ct) {
   using S = CellShape<D, K>;
   constexpr int KR = S::KR;
@@ -424,12 +429,12 @@ cell_gather(const typename A::V* __restrict__ wc, typename A::IO* __restrict__ y
     // order, in the accumulator's own arithmetic (no FP64 work for FP32 vectors)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) dot.merge(dot.shfl_down(o));
-    __shared__ IoDot<typename A::IO> wsum[GATHER_THREADS / 32];
+    __shared__ IoDot<typename A::IO> wsum[gather_threads(D, K) / 32];
     if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = dot;
     __syncthreads();
     if (threadIdx.x == 0) {
       IoDot<typename A::IO> tot = wsum[0];
-      for (int w = 1; w < GATHER_THREADS / 32; ++w) tot.merge(wsum[w]);
+      for (int w = 1; w < gather_threads(D, K) / 32; ++w) tot.merge(wsum[w]);
       ct.dotpart[blockIdx.x] = tot.value();
     }
   }
@@ -483,7 +488,7 @@ cudaError_t run_cells(const void* x, void* y, const CellTabs& ct, const double* 
   const int64_t rows = (int64_t)ct.ncown * S::KR;
   if (rows > 0) {
     cfg.gridDim = dim3((unsigned)gather_blocks<D, K>(ct));
-    cfg.blockDim = dim3((unsigned)GATHER_THREADS);
+    cfg.blockDim = dim3((unsigned)gather_threads(D, K));
     e = cudaLaunchKernelEx(&cfg, cell_gather<D, K, A>, (const V*)ct.wc, (IO*)y, add, ct);
     if (e != cudaSuccess) return e;
   }

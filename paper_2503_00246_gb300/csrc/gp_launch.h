@@ -57,6 +57,22 @@ Tiles default_tiles_t() {
   t.fb = CO ? (130 / Shape<D, K>::L > 0 ? 130 / Shape<D, K>::L : 1) : Shape<D, K>::FB;
   t.lcb = LiftShape<D, K>::CB;
   t.lnt = LiftShape<D, K>::NT;
+  // W_F outputs in 3D: with 32 (or 16) owners per CTA every row type fills whole warps, which then take
+  // one path (128^3 gyroid, k = 4, lift with 16 / 32 owners: float-float 283 / 216 us, FP64, whose
+  // warps skip missing faces, 259 / 214 us at one row per thread; 96^3 ball, k = 5: float-float
+  // 118 / 91 us, FP64 112 / 92 us with 16)
+  constexpr bool FF = sizeof(V) == 8 && !std::is_same<V, double>::value && D == 3;
+  constexpr bool F64 = std::is_same<V, double>::value && D == 3;
+  if (FF && K == 3) {
+    t.lcb = 24;
+    t.lnt = 128;
+  }
+  if (FF && K >= 4) t.lcb = 32;
+  if (F64 && K == 3) t.lcb = 16;
+  if (F64 && (K == 4 || K == 5)) {
+    t.lcb = K == 4 ? 32 : 16;
+    t.lnt = 512;
+  }
   if (CO && K == 4) t.lcb = 32;
   if (CO && K >= 5) {
     t.lcb = K <= 6 ? 16 : 8;
