@@ -158,8 +158,9 @@ class Clocks:
 # ---------------------------------------------------------------- GPU arm --
 
 def _flops_face(d, k, nf, prec="fp64", per_output=False):
-    """Flops the face kernel executes (a multiply-add counts 2, a multiply or add 1; an
-    n-term dot product 2n - 1), per normal line: the even-odd split (2k adds), the k
+    """Flops of the factorised face apply with the masses through their even / odd halves, a fixed
+    count of the work per face beside _flops_executed (a multiply-add counts 2, a multiply or add 1;
+    an n-term dot product 2n - 1), per normal line: the even-odd split (2k adds), the k
     jump dot products (k + 1 terms for odd orders, k for even ones), the tangential
     masses, the scaling by s_j (FP32 only: FP64 and float-float fold s_j into the jump
     vectors), and the expansion (per node b <= k one odd-order and, for b < k, one
@@ -184,6 +185,49 @@ def _flops_face(d, k, nf, prec="fp64", per_output=False):
     if k > 1:
         expansion += k * ((2 * n_even - 1) + 2)
     return float(nf) * (L * (contraction + scaling + expansion) + tangential_face)
+
+
+# pivot nodes of the triangular normal basis, row by row (rows 0, 2, .. even, 1, 3, .. odd)
+_PIVOTS = {1: (1,), 2: (2, 1), 3: (2, 2, 1), 4: (3, 2, 2, 3), 5: (3, 3, 1, 4, 5), 6: (4, 4, 2, 1, 6, 5),
+           7: (5, 4, 2, 6, 7, 2, 4), 8: (5, 4, 2, 7, 8, 1, 6, 6)}
+
+
+def _flops_executed(d, k, nf, prec="fp64"):
+    """Flops the face kernel executes, counted as in _flops_face: the even / odd split, the jump values
+    and the expansion of a normal line (FP64: triangular basis, unit and zero entries free; FP32
+    stores compact outputs and does not expand), the lumped masses with their rank-one term
+    line by line, and the scaling."""
+    N, L = k + 1, (k + 1) ** (d - 1)
+    if prec == "fp64":
+        piv = _PIVOTS[k]
+        jumps = expand = 0
+        for par in (0, 1):
+            rows = list(range(par, k, 2))
+            for b in range(k + 1 - par):
+                terms = 0
+                for i, j in enumerate(rows):
+                    if b in [piv[q] for q in rows[:i]]:
+                        continue
+                    unit = piv[j] == b
+                    jumps += 0 if unit else 2
+                    expand += (0 if unit else 1) if terms == 0 else (1 if unit else 2)
+                    terms += 1
+        normal = 2 * k + jumps + expand + (2 * k if k > 1 else 0)
+    else:
+        n_odd, n_even = (k + 1) // 2, k // 2
+        normal = 2 * k + n_odd * (2 * (k + 1) - 1) + n_even * (2 * k - 1)
+        if prec != "fp32":
+            normal += (k + 1) * (2 * n_odd - 1)
+            if k > 1:
+                normal += k * ((2 * n_even - 1) + 2)
+    dot, axpy = 2 * N - 1, 2 * N
+    if d == 3:
+        second = dot + axpy if prec == "fp32" else dot      # per line; else the axpy is per value below
+        tangential = k * N * (dot + axpy + second) + L * k * (1 if prec == "fp32" else 3)
+    else:
+        tangential = k * (dot + axpy) + L * k
+    scaling = k if prec == "fp32" else 0
+    return float(nf) * (L * (normal + scaling) + tangential)
 
 
 def _flops_paper(d, k, nf):
@@ -323,7 +367,7 @@ def run_sweep(args):
             tf = ms_face / calls * 1e-3
             nf = ctx.n_faces
             w = 4 if prec == gp.GP_FP32 else 8
-            fl_exec = _flops_face(pr.dim, k, nf, tags[prec].replace("ff64", "ff"))
+            fl_exec = _flops_executed(pr.dim, k, nf, tags[prec].replace("ff64", "ff"))
             fl_paper = _flops_paper(pr.dim, k, nf)
             r = {"gdofs": ctx.n_active / t / 1e9, "ms": t * 1e3, "face_ms": tf * 1e3, "lift_ms": ms_lift / calls,
                  "gfaces_per_s": nf / t / 1e9,
@@ -561,7 +605,8 @@ def form_summary(rec, pr, prec, gp, hbm, peak_src, ws=1):
     fp32_peak = N_SM * FP32_FLOP_PER_CLK_SM * SM_MAX_MHZ * 1e6 / 1e12
     peak = {gp.GP_FP64: fp64_peak, gp.GP_FP32: fp32_peak, gp.GP_FP64_FF: fp32_peak / FF_OPS_PER_FMA}[prec]
     kname = {gp.GP_FP64: "double", gp.GP_FP32: "float", gp.GP_FP64_FF: "ff64"}[prec]
-    flop_face = _flops_face(d, k, nf, {gp.GP_FP64: "fp64", gp.GP_FP32: "fp32", gp.GP_FP64_FF: "ff"}[prec])
+    form = {gp.GP_FP64: "fp64", gp.GP_FP32: "fp32", gp.GP_FP64_FF: "ff"}[prec]
+    flop_face = _flops_executed(d, k, nf, form)
     brick = rec["kernel_path"]["path"] == gp.GP_PATH_BRICK
     kernels = ("brick_kernel", "plane_fixup_kernel") if brick else ("face_kernel", "lift_kernel")
     roof = {"bound": "alu", "kernel": f"{kernels[0]}<{d},{k},{kname}>",
@@ -572,6 +617,7 @@ def form_summary(rec, pr, prec, gp, hbm, peak_src, ws=1):
                             gp.GP_FP64_FF: "derived: FP32 peak / 12 FP32 ops per compensated float-float "
                                            "multiply-add"}[prec]}
     roof["frac"] = roof["achieved"] / peak if roof["achieved"] else None
+    roof["flops_even_odd_form"] = _flops_face(d, k, nf, form)   # the same work through the even / odd masses
     roof["traffic"] = _traffic(f"face_kernel_{kname}_d{d}k{k}")
     alg = w * (n_touched + n_active)
     out = {"value": ws * n_active / (t * 1e-3) / 1e9, "unit": "GDoF/s", "ms_per_step": t,

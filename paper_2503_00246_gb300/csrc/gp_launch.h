@@ -63,6 +63,10 @@ Tiles default_tiles_t() {
   // 118 / 91 us, FP64 112 / 92 us with 16)
   constexpr bool FF = sizeof(V) == 8 && !std::is_same<V, double>::value && D == 3;
   constexpr bool F64 = std::is_same<V, double>::value && D == 3;
+  // face CTAs at k = 4 (128^3 gyroid, face kernel): float-float 5 faces 355 us, 10 faces 367 us; FP64
+  // 20 faces 992 us, 10 faces 1010 us
+  if (FF && K == 4) t.fb = 5;
+  if (F64 && K == 4) t.fb = 20;
   if (FF && K == 3) {
     t.lcb = 24;
     t.lnt = 128;
