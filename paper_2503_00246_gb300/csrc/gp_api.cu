@@ -261,6 +261,7 @@ gp_status gpi::launch(gp_ctx* c, const void* x, void* y, int add, cudaStream_t s
   a.ev = ev;
   a.tiles = tiles ? *tiles : c->tiles;
   a.which = which;
+  a.form = c->form;
   a.full_outputs = full_outputs;
   a.slabs = run ? run->table : p.slabs.data();
   a.nslab = run ? run->n : p.num_slabs();
@@ -400,9 +401,12 @@ gp_status gp_setup(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* op
     if (e == cudaSuccess) e = upload(&c->d_frows, p.frows);
     if (e == cudaSuccess) e = upload(&c->d_lwin, p.lwin);
     if (e == cudaSuccess) e = upload(&c->d_lrow, p.lrow);
-    if (e == cudaSuccess && p.precision == GP_FP32) e = upload(&c->d_lmask, p.lmask);   // compact outputs only
-    if (e == cudaSuccess) e = upload(&c->d_zruns, zruns);
     const size_t vbytes = p.precision == GP_FP32 ? 4 : 8;
+    // face outputs W_F of the face + lift path: float, double, or a (hi, lo) float pair per value
+    const size_t tp_bytes = (size_t)p.num_faces() * p.L * (2 * p.k + 1) * vbytes;
+    c->form = gp::launch_form(p.precision == GP_FP32, p.dim, p.k, (int64_t)tp_bytes, (int64_t)p.lrow.size());
+    if (e == cudaSuccess && (c->form & gp::FORM_COMPACT)) e = upload(&c->d_lmask, p.lmask);
+    if (e == cudaSuccess) e = upload(&c->d_zruns, zruns);
     if (c->use_brick) {
       if (e == cudaSuccess) e = upload(&c->d_bdesc, p.bdesc);
       if (e == cudaSuccess) e = upload(&c->d_bcell, p.bcell);
@@ -415,8 +419,6 @@ gp_status gp_setup(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* op
       const size_t part_bytes = gpi::brick_scratch_bytes(c);
       if (e == cudaSuccess && part_bytes > 0 && !opts->no_scratch) e = cudaMalloc(&c->d_part, part_bytes);
     }
-    // face outputs W_F of the face + lift path: float, double, or a (hi, lo) float pair per value
-    const size_t tp_bytes = (size_t)p.num_faces() * p.L * (2 * p.k + 1) * vbytes;
     if (e == cudaSuccess && tp_bytes > 0 && !opts->no_scratch && !c->use_brick) e = cudaMalloc(&c->d_tp, tp_bytes);
     if (e != cudaSuccess) {
       std::string m = std::string("device setup: ") + cudaGetErrorString(e);
@@ -704,6 +706,7 @@ struct gp_batch {
     void* d_ptrs[2] = {nullptr, nullptr};
     void* h_ptrs[2] = {nullptr, nullptr};  // pinned: read by the graph's copy node at replay
     int face_blocks = 0, lift_blocks = 0;
+    bool compact = false;              // FP32: the problems store compact face outputs
     bool ldl = false;                  // the problems run one triangular normal basis (Plan::ldl)
     gp::BatchOps ops{};
     gp::Tiles tiles{};                 // the tile shape of the group's first context
@@ -772,17 +775,19 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
   DeviceGuard dg(b->device);
   // group problems by (dimension, degree, arithmetic, stabilisation)
   // (d, k, arithmetic, stabilisation): one set of 1D data; FP64 problems of one group whose weights have
-  // other triangular normal bases B launch apart, so that each problem runs as in gp_apply
+  // other triangular normal bases B, and FP32 problems with other face outputs, launch apart, so that
+  // each problem runs as in gp_apply
   typedef std::tuple<int, int, int, int> Key;
-  std::map<std::pair<Key, std::vector<double>>, int> key;
+  std::map<std::tuple<Key, std::vector<double>, bool>, int> key;
   std::set<Key> kinds;
   for (int p = 0; p < nprob; ++p) {
     const gp::Plan& pl = ctxs[p]->plan;
     const Key kd = std::make_tuple(pl.dim, pl.k, pl.precision, pl.stabilization);
     kinds.insert(kd);
     const bool ldl = pl.precision == GP_FP64 && !pl.ldl.empty();
-    const auto kk = std::make_pair(
-        kd, ldl ? std::vector<double>(pl.ldl.begin(), pl.ldl.begin() + pl.k * (pl.k + 1)) : std::vector<double>());
+    const auto kk = std::make_tuple(
+        kd, ldl ? std::vector<double>(pl.ldl.begin(), pl.ldl.begin() + pl.k * (pl.k + 1)) : std::vector<double>(),
+        (ctxs[p]->form & gp::FORM_COMPACT) != 0);
     auto it = key.find(kk);
     int gi;
     if (it == key.end()) {
@@ -795,6 +800,7 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
       b->groups[gi].ops = ops_for(pl.precision, pl.dim);
       b->groups[gi].tiles = ctxs[p]->tiles;
       b->groups[gi].ldl = ldl;
+      b->groups[gi].compact = (ctxs[p]->form & gp::FORM_COMPACT) != 0;
     } else {
       gi = it->second;
     }
@@ -860,7 +866,7 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
       for (int j = 0; j < pl.k; ++j) sp.s[j] = g.ldl ? pl.ldl[nb + j] : pl.scale[j];
     }
     std::vector<unsigned char> fs, ls;
-    if (!g.ops.pack(g.k, specs, g.tiles, fs, ls, g.face_blocks, g.lift_blocks)) {
+    if (!g.ops.pack(g.k, specs, g.compact, g.tiles, fs, ls, g.face_blocks, g.lift_blocks)) {
       e = cudaErrorInvalidConfiguration;
       break;
     }
@@ -884,7 +890,7 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
                           b->cap);
       if (e == cudaSuccess)
         e = g.ops.run(g.k, g.d_fsegs, g.d_lsegs, g.d_ptrs[i], (int)g.prob.size(), g.face_blocks, g.lift_blocks,
-                      pl0.jumps.data(), pl0.lump.data(), g.ldl ? pl0.ldl.data() : nullptr, g.tiles, b->cap);
+                      pl0.jumps.data(), pl0.lump.data(), g.ldl ? pl0.ldl.data() : nullptr, g.compact, g.tiles, b->cap);
     }
     cudaGraph_t graph = nullptr;
     const cudaError_t e2 = cudaStreamEndCapture(b->cap, &graph);

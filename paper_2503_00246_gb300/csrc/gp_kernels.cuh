@@ -427,11 +427,11 @@ template <int VW, typename V>
 struct alignas(VW * sizeof(V)) Chunk {
   V v[VW];
 };
-// FP32 stores T_F: both of its kernels were bound by L1 wavefronts (68% and 65% of their peak) and
-// moved 1.11 GB per apply of the 128^3 gyroid at k = 4, 0.79 GB now: apply 306 -> 256 us (face kernel
-// 187 -> 158 us, lift 117 -> 104 us).
-// FP64 stores W_F: the expansion and its FP64 adds cost the same operations either way, and W_F
-// hides under the FP64 pipe.
+// FP32 stores T_F where W_F would not stay in L2 (store_compact): both of its kernels were bound by L1
+// wavefronts (68% and 65% of their peak) and moved 1.11 GB per apply of the 128^3 gyroid at k = 4, 0.79 GB
+// so: apply 306 -> 256 us (face kernel 187 -> 158 us, lift 117 -> 104 us).  FP64 stores W_F: the
+// expansion and its FP64 adds cost the same operations either way, and W_F hides under the FP64 pipe;
+// so does float-float (a lift of compact outputs took 385 us there against 283 us).
 template <typename V>
 struct StoreCompact {
   static constexpr bool value = std::is_same<V, float>::value;
@@ -649,7 +649,7 @@ __device__ __forceinline__ int find_segment(const Seg* segs, const int nseg, con
   return lo;
 }
 
-template <int D, int K, class A, bool LDL>
+template <int D, int K, class A, bool COMPACT, bool LDL>
 __global__ void __launch_bounds__(MAX_CTA_THREADS, FaceCtas<typename A::V>::value)
 face_kernel_batched(const FaceSeg<typename A::V, K>* __restrict__ segs, const int nseg,
                     const SegPtrs<typename A::IO>* __restrict__ ptrs, const int fb,
@@ -665,15 +665,15 @@ face_kernel_batched(const FaceSeg<typename A::V, K>* __restrict__ segs, const in
   __syncthreads();
   if constexpr (LDL) {
     // the group's problems share B (the constant bank); D is the segment's
-    face_body<D, K, A, StoreCompact<V>::value, true>(sp.x, seg.wp, sp.y, seg.fa, c, c.g, seg.s,
+    face_body<D, K, A, COMPACT, true>(sp.x, seg.wp, sp.y, seg.fa, c, c.g, seg.s,
                                                      (int)blockIdx.x - seg.block0, fb, gp_dyn_smem);
   } else if constexpr (FoldScale<V>::value) {
     __shared__ V sg[K][2 * K + 1];
     for (int i = threadIdx.x; i < K * (2 * K + 1); i += blockDim.x) sg[i / (2 * K + 1)][i % (2 * K + 1)] = seg.gs[i];
     __syncthreads();
-    face_body<D, K, A, StoreCompact<V>::value, false>(sp.x, seg.wp, sp.y, seg.fa, c, sg, seg.s, (int)blockIdx.x - seg.block0, fb, gp_dyn_smem);
+    face_body<D, K, A, COMPACT, false>(sp.x, seg.wp, sp.y, seg.fa, c, sg, seg.s, (int)blockIdx.x - seg.block0, fb, gp_dyn_smem);
   } else {
-    face_body<D, K, A, StoreCompact<V>::value, false>(sp.x, seg.wp, sp.y, seg.fa, c, c.g, seg.s, (int)blockIdx.x - seg.block0, fb, gp_dyn_smem);
+    face_body<D, K, A, COMPACT, false>(sp.x, seg.wp, sp.y, seg.fa, c, c.g, seg.s, (int)blockIdx.x - seg.block0, fb, gp_dyn_smem);
   }
 }
 

@@ -31,6 +31,7 @@ struct ApplyArgs {
   cudaEvent_t* ev = nullptr;  // optional: 3 events recorded around the two kernels
   Tiles tiles{};              // 0 fields: the defaults of default_tiles
   int which = 3;              // bit 0: face kernel, bit 1: lift kernel (the autotuner times them apart)
+  int form = 0;               // launch_form
   bool full_outputs = false;  // the face kernel stores W_F whatever its arithmetic (the model system's gather
                               // reads it); only with which = 1
   const int32_t* slabs = nullptr;  // host: SLAB ints per slab (see Plan::slabs); nslab > 1: slab pipeline
@@ -44,17 +45,40 @@ struct ApplyArgs {
   PlaneArgs pa{};             // plane-fixup tables
 };
 
-// Default tile shape: about 256 threads per CTA, one item per thread.  Compact outputs in 3D: face
+// Whether an FP32 context stores compact face outputs.  Small W_F stays in L2, where the lift of W_F
+// and its two fewer phases are the faster one for small k (us of an apply, W_F / compact: k = 2, 40^3 ball 6.4 / 7.3; k = 3, 20^3 5.7 /
+// 6.6; k = 4, 12^3 7.7 / 8.7; k = 6, 32^3, 17 MB, 27 / 34); the compact form is from 12 MB of W_F at k = 3
+// (64^3 21.0 / 16.4), 3 MB at k = 4 (24^3 10.2 / 9.7), 24 MB at k = 6 (64^3 81 / 72), and at any size for
+// k = 5, 7 and 8 (10^3: 9.9 / 8.5, k = 7, 11^3 12.9 / 10.4, k = 8, 8^3 13.9 / 11.6) and in 2D (300^2 disc,
+// k = 8: 9.7 / 7.2).
+inline bool store_compact(int dim, int k, int64_t w_bytes) {
+  const int64_t mb = (int64_t)1 << 20;
+  return dim == 2 || k == 5 || k >= 7 || (k == 6 && w_bytes > 24 * mb) || (k == 4 && w_bytes > 3 * mb) ||
+         (k == 3 && w_bytes > 10 * mb);
+}
+// The form of a context's launches: bit 0 compact outputs (FP32), bit 1 so few lift rows that a thread
+// takes one (default tiles): below them the rows of one CTA follow each other on a GPU that is mostly
+// idle (FP32, compact: 16^3 ball, k = 5, 24.2 / 9.5 us, 28^3, k = 8, 40 / 36 us; float-float: 14^3, k = 8,
+// 47 / 35 us; above, 32^3, k = 6, 53 / 62 us).
+constexpr int FORM_COMPACT = 1, FORM_FEW = 2;
+inline int launch_form(bool fp32, int dim, int k, int64_t w_bytes, int64_t rows) {
+  return (fp32 && store_compact(dim, k, w_bytes) ? FORM_COMPACT : 0) |
+         (rows < (fp32 ? 600000 : 100000) ? FORM_FEW : 0);
+}
+
+// Default tile shape: about 256 threads per CTA, one item per thread.  FP32 in 3D: face
 // CTAs of about 130 threads (more CTAs per SM to run while one waits at a barrier; 128^3 gyroid,
-// k = 4, face kernel with 2 / 5 / 6 / 10 / 20 faces: 193 / 127 / 132 / 136 / 158 us), and from
-// k = 4 on two to four lines per lift thread (inner lines first, then edge lines with more faces, so
-// that the warps meet at the barriers; 128^3 gyroid with 1 / 2 / 4 lines: 152 / 104 / 150 us; 49^3
+// k = 4, face kernel with 2 / 5 / 6 / 10 / 20 faces: 193 / 127 / 132 / 136 / 158 us), and,
+// with compact outputs, from k = 4 on two to four lines per lift thread (inner lines first, then edge
+// lines with more faces, so that the warps meet at the barriers; 128^3 gyroid with 1 / 2 / 4 lines: 152 / 104 / 150 us; 49^3
 // ball at k = 8, 128 threads, with 1 / 2 / 4 / 8: 102 / 56 / 49 / 61 us).
 template <int D, int K, typename V>
-Tiles default_tiles_t() {
-  constexpr bool CO = StoreCompact<V>::value && D == 3;
+Tiles default_tiles_t(const int form) {
+  const bool CO = (form & FORM_COMPACT) && StoreCompact<V>::value && D == 3;
+  const bool few = (form & FORM_FEW) != 0;
   Tiles t;
-  t.fb = CO ? (130 / Shape<D, K>::L > 0 ? 130 / Shape<D, K>::L : 1) : Shape<D, K>::FB;
+  constexpr bool F32 = std::is_same<V, float>::value && D == 3;
+  t.fb = F32 ? (130 / Shape<D, K>::L > 0 ? 130 / Shape<D, K>::L : 1) : Shape<D, K>::FB;
   t.lcb = LiftShape<D, K>::CB;
   t.lnt = LiftShape<D, K>::NT;
   // W_F outputs in 3D: with 32 (or 16) owners per CTA every row type fills whole warps, which then take
@@ -67,18 +91,22 @@ Tiles default_tiles_t() {
   // 20 faces 992 us, 10 faces 1010 us
   if (FF && K == 4) t.fb = 5;
   if (F64 && K == 4) t.fb = 20;
-  if (FF && K == 3) {
+  if (FF && K == 3 && !few) {
     t.lcb = 24;
     t.lnt = 128;
   }
-  if (FF && K >= 4) t.lcb = 32;
+  if (FF && (K == 4 || (K > 4 && !few))) t.lcb = 32;
   if (F64 && K == 3) t.lcb = 16;
   if (F64 && (K == 4 || K == 5)) {
     t.lcb = K == 4 ? 32 : 16;
     t.lnt = 512;
   }
-  if (CO && K == 4) t.lcb = 32;
-  if (CO && K >= 5) {
+  if (CO && K == 4) {
+    t.lcb = 32;
+    if (few) t.lnt = 512;
+  }
+  if (CO && few && (K == 5 || K == 7)) t.lcb = K == 5 ? 8 : 4;
+  if (CO && K >= 5 && !few) {
     t.lcb = K <= 6 ? 16 : 8;
     t.lnt = 128;
   }
@@ -89,8 +117,8 @@ Tiles default_tiles_t() {
 // (threads per CTA <= MAX_CTA_THREADS, lift threads a multiple of 32, dynamic
 // shared memory <= MAX_DYN_SMEM).  Returns false if t is out of range.
 template <int D, int K, typename V>
-bool resolve_tiles(Tiles& t) {
-  const Tiles d = default_tiles_t<D, K, V>();
+bool resolve_tiles(Tiles& t, const int form) {
+  const Tiles d = default_tiles_t<D, K, V>(form);
   if (t.fb == 0) t.fb = d.fb;
   if (t.lcb == 0) t.lcb = d.lcb;
   if (t.lnt == 0) t.lnt = d.lnt;
@@ -102,8 +130,8 @@ bool resolve_tiles(Tiles& t) {
 
 // Per (arithmetic, dimension): default tiles and range check for degree k.
 struct TileOps {
-  Tiles (*defaults)(int k);
-  bool (*resolve)(int k, Tiles& t);
+  Tiles (*defaults)(int k, int form);
+  bool (*resolve)(int k, Tiles& t, int form);
 };
 TileOps tile_ops_f64_d2();
 TileOps tile_ops_f64_d3();
@@ -113,22 +141,22 @@ TileOps tile_ops_ff_d2();
 TileOps tile_ops_ff_d3();
 
 #define GP_TILE_CASE(D, A, K) \
-  case K: return resolve_tiles<D, K, typename A::V>(t);
+  case K: return resolve_tiles<D, K, typename A::V>(t, form);
 #define GP_TILE_OPS(D, A)                                                                     \
   TileOps ops;                                                                                \
-  ops.defaults = [](int k) -> Tiles {                                                         \
+  ops.defaults = [](int k, int form) -> Tiles {                                            \
     switch (k) {                                                                              \
-      case 1: return default_tiles_t<D, 1, typename A::V>();                                                 \
-      case 2: return default_tiles_t<D, 2, typename A::V>();                                                 \
-      case 3: return default_tiles_t<D, 3, typename A::V>();                                                 \
-      case 4: return default_tiles_t<D, 4, typename A::V>();                                                 \
-      case 5: return default_tiles_t<D, 5, typename A::V>();                                                 \
-      case 6: return default_tiles_t<D, 6, typename A::V>();                                                 \
-      case 7: return default_tiles_t<D, 7, typename A::V>();                                                 \
-      default: return default_tiles_t<D, 8, typename A::V>();                                                \
+      case 1: return default_tiles_t<D, 1, typename A::V>(form);                                                 \
+      case 2: return default_tiles_t<D, 2, typename A::V>(form);                                                 \
+      case 3: return default_tiles_t<D, 3, typename A::V>(form);                                                 \
+      case 4: return default_tiles_t<D, 4, typename A::V>(form);                                                 \
+      case 5: return default_tiles_t<D, 5, typename A::V>(form);                                                 \
+      case 6: return default_tiles_t<D, 6, typename A::V>(form);                                                 \
+      case 7: return default_tiles_t<D, 7, typename A::V>(form);                                                 \
+      default: return default_tiles_t<D, 8, typename A::V>(form);                                                \
     }                                                                                         \
   };                                                                                          \
-  ops.resolve = [](int k, Tiles& t) -> bool {                                                 \
+  ops.resolve = [](int k, Tiles& t, int form) -> bool {                                    \
     switch (k) {                                                                              \
       GP_TILE_CASE(D, A, 1) GP_TILE_CASE(D, A, 2) GP_TILE_CASE(D, A, 3) GP_TILE_CASE(D, A, 4) \
       GP_TILE_CASE(D, A, 5) GP_TILE_CASE(D, A, 6) GP_TILE_CASE(D, A, 7) GP_TILE_CASE(D, A, 8) \
@@ -225,47 +253,51 @@ cudaError_t launch_pdl(void (*kernel)(P...), int grid, int threads, size_t smem,
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-// Owner cells per lift CTA and dynamic shared memory of the lift kernel of this arithmetic.
+// Owner cells per lift CTA and dynamic shared memory of the lift kernel.
 template <int D, int K, typename V>
-int lift_cells(const Tiles& t) {
-  if constexpr (StoreCompact<V>::value) return lift_lines_cells<D, K, V>(t.lcb);
-  else return t.lcb;
+int lift_cells(const Tiles& t, const bool compact) {
+  if constexpr (StoreCompact<V>::value)
+    if (compact) return lift_lines_cells<D, K, V>(t.lcb);
+  return t.lcb;
 }
 template <int D, int K, typename V>
-size_t lift_dyn_smem(int cb) {
-  if constexpr (StoreCompact<V>::value) return lift_lines_smem<D, K, V>(cb);
-  else return lift_smem<D, K>(cb);
+size_t lift_dyn_smem(int cb, const bool compact) {
+  if constexpr (StoreCompact<V>::value)
+    if (compact) return lift_lines_smem<D, K, V>(cb);
+  return lift_smem<D, K>(cb);
 }
 
 // Launches the lift of the owners la, as a programmatic dependent of the kernel before it (pdl)
 // or in plain stream order.
 template <int D, int K, class A>
-cudaError_t launch_lift(bool pdl, const Tiles& t, const typename A::V* w, typename A::IO* y, int add,
-                        const LiftArgs& la, const Consts<typename A::V, K>& c, cudaStream_t st) {
+cudaError_t launch_lift(bool pdl, const bool compact, const Tiles& t, const typename A::V* w, typename A::IO* y,
+                        int add, const LiftArgs& la, const Consts<typename A::V, K>& c, cudaStream_t st) {
   using V = typename A::V;
-  const int cb = lift_cells<D, K, V>(t);
+  const int cb = lift_cells<D, K, V>(t, compact);
   const int nlb = (la.nlift + cb - 1) / cb;
-  const size_t smem = lift_dyn_smem<D, K, V>(cb);
+  const size_t smem = lift_dyn_smem<D, K, V>(cb, compact);
   if constexpr (StoreCompact<V>::value) {
-    if (pdl) return launch_pdl(lift_lines_kernel<D, K, A>, nlb, t.lnt, smem, st, w, y, add, la, cb, c);
-    lift_lines_kernel<D, K, A><<<nlb, t.lnt, smem, st>>>(w, y, add, la, cb, c);
-  } else {
-    if (pdl) return launch_pdl(lift_kernel<D, K, A>, nlb, t.lnt, smem, st, w, y, add, la, cb);
-    lift_kernel<D, K, A><<<nlb, t.lnt, smem, st>>>(w, y, add, la, cb);
+    if (compact) {
+      if (pdl) return launch_pdl(lift_lines_kernel<D, K, A>, nlb, t.lnt, smem, st, w, y, add, la, cb, c);
+      lift_lines_kernel<D, K, A><<<nlb, t.lnt, smem, st>>>(w, y, add, la, cb, c);
+      return cudaGetLastError();
+    }
   }
+  if (pdl) return launch_pdl(lift_kernel<D, K, A>, nlb, t.lnt, smem, st, w, y, add, la, cb);
+  lift_kernel<D, K, A><<<nlb, t.lnt, smem, st>>>(w, y, add, la, cb);
   return cudaGetLastError();
 }
 
 // The face kernel of this arithmetic: with the triangular normal basis or the jump vectors, storing its
-// compact outputs or (full) W_F.
+// compact outputs or W_F.
 template <int D, int K, class A>
-auto pick_face(const bool ldl, const bool full) {
+auto pick_face(const bool ldl, const bool compact) {
   using V = typename A::V;
   constexpr bool CO = StoreCompact<V>::value, LD = std::is_same<V, double>::value;
   static_assert(!(CO && LD), "compact outputs are expanded with the jump vectors");
-  auto f = face_kernel<D, K, A, CO, false>;
+  auto f = face_kernel<D, K, A, false, false>;
   if constexpr (CO) {
-    if (full) f = face_kernel<D, K, A, false, false>;
+    if (compact) f = face_kernel<D, K, A, true, false>;
   }
   if constexpr (LD) {
     if (ldl) f = face_kernel<D, K, A, false, true>;
@@ -309,7 +341,7 @@ cudaError_t run_slabs(const ApplyArgs& Ar, const Consts<typename A::V, K>& c, co
       if (e != cudaSuccess) return e;
     }
     if (nb > 0) {
-      const auto face = pick_face<D, K, A>(ldl, false);
+      const auto face = pick_face<D, K, A>(ldl, (Ar.form & FORM_COMPACT) != 0);
       const cudaError_t e =
           (s == 0 || Ar.slab_events)
               ? (face<<<nb, t.fb * S::L, face_smem<D, K, V>(t.fb), st>>>((const IO*)Ar.x, (V*)Ar.tp, (IO*)Ar.y, fa, t.fb, c),
@@ -326,7 +358,7 @@ cudaError_t run_slabs(const ApplyArgs& Ar, const Consts<typename A::V, K>& c, co
     if (la.nlift > 0) {
       // programmatic dependent of this slab's face launch (a plain launch after an event)
       const cudaError_t e =
-          launch_lift<D, K, A>(nb > 0 || !Ar.slab_events, t, (const V*)Ar.tp, (IO*)Ar.y, Ar.add, la, c, st);
+          launch_lift<D, K, A>(nb > 0 || !Ar.slab_events, (Ar.form & FORM_COMPACT) != 0, t, (const V*)Ar.tp, (IO*)Ar.y, Ar.add, la, c, st);
       if (e != cudaSuccess) return e;
     }
     if (Ar.slab_events) {
@@ -369,7 +401,7 @@ cudaError_t run_apply(const ApplyArgs& Ar, cudaStream_t st) {
   if (ldl) ldl_consts<V, K>(Ar.ldl, c);
   if (Ar.brick) return run_brick<D, K, A>(Ar, c, st);
   Tiles t = Ar.tiles;
-  if (!resolve_tiles<D, K, V>(t)) return cudaErrorInvalidConfiguration;
+  if (!resolve_tiles<D, K, V>(t, Ar.form)) return cudaErrorInvalidConfiguration;
   if (Ar.nslab > 1 && !Ar.ev && Ar.which == 3) return run_slabs<D, K, A>(Ar, c, t, ldl, st);
   FaceArgs fa;
   fa.frows = Ar.frows;
@@ -383,13 +415,13 @@ cudaError_t run_apply(const ApplyArgs& Ar, cudaStream_t st) {
   const bool faces = Ar.fstart[D] > 0;
   if (Ar.ev) cudaEventRecord(Ar.ev[0], st);
   if (nb > 0 && (Ar.which & 1)) {
-    const auto face = pick_face<D, K, A>(ldl, Ar.full_outputs);
+    const auto face = pick_face<D, K, A>(ldl, (Ar.form & FORM_COMPACT) != 0 && !Ar.full_outputs);
     face<<<nb, t.fb * S::L, face_smem<D, K, V>(t.fb), st>>>((const IO*)Ar.x, (V*)Ar.tp, (IO*)Ar.y, fa, t.fb, c);
   }
   if (Ar.ev) cudaEventRecord(Ar.ev[1], st);
   if (Ar.la.nlift > 0 && faces && (Ar.which & 2)) {
     // programmatic dependent launch: the lift's CTAs start while the face grid drains
-    const cudaError_t e = launch_lift<D, K, A>(!Ar.ev && (Ar.which & 1), t, (const V*)Ar.tp, (IO*)Ar.y, Ar.add,
+    const cudaError_t e = launch_lift<D, K, A>(!Ar.ev && (Ar.which & 1), (Ar.form & FORM_COMPACT) != 0, t, (const V*)Ar.tp, (IO*)Ar.y, Ar.add,
                                                Ar.la, c, st);
     if (e != cudaSuccess) return e;
   }
@@ -410,10 +442,10 @@ struct SegSpec {
 // Packs the segments of one (d, k, arithmetic) group into the device layouts of
 // FaceSeg<V, K> and LiftSeg, with the CTA offsets of both launches.
 template <int D, int K, class A>
-bool pack_batch(const std::vector<SegSpec>& in, Tiles& t, std::vector<unsigned char>& fsegs,
+bool pack_batch(const std::vector<SegSpec>& in, const bool compact, Tiles& t, std::vector<unsigned char>& fsegs,
                 std::vector<unsigned char>& lsegs, int& face_blocks, int& lift_blocks) {
   using V = typename A::V;
-  if (!resolve_tiles<D, K, V>(t)) return false;
+  if (!resolve_tiles<D, K, V>(t, compact)) return false;
   fsegs.assign(in.size() * sizeof(FaceSeg<V, K>), 0);
   lsegs.assign(in.size() * sizeof(LiftSeg), 0);
   int fb = 0, lb = 0;
@@ -431,7 +463,7 @@ bool pack_batch(const std::vector<SegSpec>& in, Tiles& t, std::vector<unsigned c
     LiftSeg ls;
     ls.la = in[i].la;
     ls.block0 = lb;
-    const int cb = lift_cells<D, K, V>(t);
+    const int cb = lift_cells<D, K, V>(t, compact);
     if (fs.fa.fstart[D] > 0) lb += (ls.la.nlift + cb - 1) / cb;
     std::memcpy(&fsegs[i * sizeof(FaceSeg<V, K>)], &fs, sizeof(fs));
     std::memcpy(&lsegs[i * sizeof(LiftSeg)], &ls, sizeof(ls));
@@ -443,11 +475,12 @@ bool pack_batch(const std::vector<SegSpec>& in, Tiles& t, std::vector<unsigned c
 
 template <int D, int K, class A>
 cudaError_t run_batch(const void* fsegs, const void* lsegs, const void* ptrs, int nseg, int face_blocks,
-                      int lift_blocks, const double* g, const double* m, const double* ldl, Tiles t, cudaStream_t st) {
+                      int lift_blocks, const double* g, const double* m, const double* ldl, bool compact, Tiles t,
+                      cudaStream_t st) {
   using V = typename A::V;
   using IO = typename A::IO;
   using S = Shape<D, K>;
-  if (!resolve_tiles<D, K, V>(t)) return cudaErrorInvalidConfiguration;
+  if (!resolve_tiles<D, K, V>(t, compact)) return cudaErrorInvalidConfiguration;
   Consts<V, K> c;
   for (int j = 0; j < K; ++j)
     for (int b = 0; b < 2 * K + 1; ++b) c.g[j][b] = from_host<V>(g[j * (2 * K + 1) + b]);
@@ -456,23 +489,31 @@ cudaError_t run_batch(const void* fsegs, const void* lsegs, const void* ptrs, in
     c.s[j] = vzero<V>();                                          // per segment: FaceSeg::s
     for (int b = 0; b < 2 * K + 1; ++b) c.gs[j][b] = vzero<V>();  // per segment: FaceSeg::gs
   }
-  auto face = face_kernel_batched<D, K, A, false>;
+  auto face = face_kernel_batched<D, K, A, false, false>;
   if constexpr (UseLdl<V>::value) {
     if (ldl) {
       ldl_consts<V, K>(ldl, c);
-      face = face_kernel_batched<D, K, A, true>;
+      face = face_kernel_batched<D, K, A, false, true>;
     }
+  }
+  if constexpr (StoreCompact<V>::value) {
+    if (compact) face = face_kernel_batched<D, K, A, true, false>;
   }
   if (face_blocks > 0)
     face<<<face_blocks, t.fb * S::L, face_smem<D, K, V>(t.fb), st>>>((const FaceSeg<V, K>*)fsegs, nseg,
                                                                    (const SegPtrs<IO>*)ptrs, t.fb, c);
   if (lift_blocks > 0) {
-    const int cb = lift_cells<D, K, V>(t);
-    const size_t smem = lift_dyn_smem<D, K, V>(cb);
-    if constexpr (StoreCompact<V>::value)
-      lift_lines_kernel_batched<D, K, A><<<lift_blocks, t.lnt, smem, st>>>(
-          (const LiftSeg*)lsegs, (const FaceSeg<V, K>*)fsegs, nseg, (const SegPtrs<IO>*)ptrs, cb, c);
-    else
+    const int cb = lift_cells<D, K, V>(t, compact);
+    const size_t smem = lift_dyn_smem<D, K, V>(cb, compact);
+    bool done = false;
+    if constexpr (StoreCompact<V>::value) {
+      if (compact) {
+        lift_lines_kernel_batched<D, K, A><<<lift_blocks, t.lnt, smem, st>>>(
+            (const LiftSeg*)lsegs, (const FaceSeg<V, K>*)fsegs, nseg, (const SegPtrs<IO>*)ptrs, cb, c);
+        done = true;
+      }
+    }
+    if (!done)
       lift_kernel_batched<D, K, A><<<lift_blocks, t.lnt, smem, st>>>(
           (const LiftSeg*)lsegs, (const FaceSeg<V, K>*)fsegs, nseg, (const SegPtrs<IO>*)ptrs, cb);
   }
@@ -492,11 +533,11 @@ void scaled_jumps(int k, const double* g, const double* s, std::vector<unsigned 
 
 // Per translation unit: batch packing and launch for one (arithmetic, dimension).
 struct BatchOps {
-  bool (*pack)(int k, const std::vector<SegSpec>&, Tiles&, std::vector<unsigned char>&,
+  bool (*pack)(int k, const std::vector<SegSpec>&, bool, Tiles&, std::vector<unsigned char>&,
                std::vector<unsigned char>&, int&, int&);
   void (*jumps)(int k, const double* g, const double* s, std::vector<unsigned char>& out);
   cudaError_t (*run)(int k, const void*, const void*, const void*, int, int, int, const double*, const double*,
-                     const double*, Tiles, cudaStream_t);
+                     const double*, bool, Tiles, cudaStream_t);
 };
 BatchOps batch_ops_f64_d2();
 BatchOps batch_ops_f64_d3();
@@ -508,31 +549,32 @@ BatchOps batch_ops_ff_d3();
 #define GP_BATCH_OPS(D, A)                                                                              \
   BatchOps ops;                                                                                         \
   ops.jumps = scaled_jumps<A>;                                                                          \
-  ops.pack = [](int k, const std::vector<SegSpec>& in, Tiles& t, std::vector<unsigned char>& fs,       \
+  ops.pack = [](int k, const std::vector<SegSpec>& in, bool co, Tiles& t, std::vector<unsigned char>& fs,       \
                 std::vector<unsigned char>& ls, int& fb, int& lb) -> bool {                             \
     switch (k) {                                                                                        \
-      case 1: return pack_batch<D, 1, A>(in, t, fs, ls, fb, lb);                                        \
-      case 2: return pack_batch<D, 2, A>(in, t, fs, ls, fb, lb);                                        \
-      case 3: return pack_batch<D, 3, A>(in, t, fs, ls, fb, lb);                                        \
-      case 4: return pack_batch<D, 4, A>(in, t, fs, ls, fb, lb);                                        \
-      case 5: return pack_batch<D, 5, A>(in, t, fs, ls, fb, lb);                                        \
-      case 6: return pack_batch<D, 6, A>(in, t, fs, ls, fb, lb);                                        \
-      case 7: return pack_batch<D, 7, A>(in, t, fs, ls, fb, lb);                                        \
-      case 8: return pack_batch<D, 8, A>(in, t, fs, ls, fb, lb);                                        \
+      case 1: return pack_batch<D, 1, A>(in, co, t, fs, ls, fb, lb);                                        \
+      case 2: return pack_batch<D, 2, A>(in, co, t, fs, ls, fb, lb);                                        \
+      case 3: return pack_batch<D, 3, A>(in, co, t, fs, ls, fb, lb);                                        \
+      case 4: return pack_batch<D, 4, A>(in, co, t, fs, ls, fb, lb);                                        \
+      case 5: return pack_batch<D, 5, A>(in, co, t, fs, ls, fb, lb);                                        \
+      case 6: return pack_batch<D, 6, A>(in, co, t, fs, ls, fb, lb);                                        \
+      case 7: return pack_batch<D, 7, A>(in, co, t, fs, ls, fb, lb);                                        \
+      case 8: return pack_batch<D, 8, A>(in, co, t, fs, ls, fb, lb);                                        \
       default: return false;                                                                            \
     }                                                                                                   \
   };                                                                                                    \
   ops.run = [](int k, const void* fs, const void* ls, const void* pt, int ns, int fb, int lb,          \
-               const double* g, const double* m, const double* l, Tiles t, cudaStream_t st) -> cudaError_t { \
+               const double* g, const double* m, const double* l, bool co, Tiles t,                  \
+               cudaStream_t st) -> cudaError_t {                                                        \
     switch (k) {                                                                                        \
-      case 1: return run_batch<D, 1, A>(fs, ls, pt, ns, fb, lb, g, m, l, t, st);                        \
-      case 2: return run_batch<D, 2, A>(fs, ls, pt, ns, fb, lb, g, m, l, t, st);                        \
-      case 3: return run_batch<D, 3, A>(fs, ls, pt, ns, fb, lb, g, m, l, t, st);                        \
-      case 4: return run_batch<D, 4, A>(fs, ls, pt, ns, fb, lb, g, m, l, t, st);                        \
-      case 5: return run_batch<D, 5, A>(fs, ls, pt, ns, fb, lb, g, m, l, t, st);                        \
-      case 6: return run_batch<D, 6, A>(fs, ls, pt, ns, fb, lb, g, m, l, t, st);                        \
-      case 7: return run_batch<D, 7, A>(fs, ls, pt, ns, fb, lb, g, m, l, t, st);                        \
-      case 8: return run_batch<D, 8, A>(fs, ls, pt, ns, fb, lb, g, m, l, t, st);                        \
+      case 1: return run_batch<D, 1, A>(fs, ls, pt, ns, fb, lb, g, m, l, co, t, st);                        \
+      case 2: return run_batch<D, 2, A>(fs, ls, pt, ns, fb, lb, g, m, l, co, t, st);                        \
+      case 3: return run_batch<D, 3, A>(fs, ls, pt, ns, fb, lb, g, m, l, co, t, st);                        \
+      case 4: return run_batch<D, 4, A>(fs, ls, pt, ns, fb, lb, g, m, l, co, t, st);                        \
+      case 5: return run_batch<D, 5, A>(fs, ls, pt, ns, fb, lb, g, m, l, co, t, st);                        \
+      case 6: return run_batch<D, 6, A>(fs, ls, pt, ns, fb, lb, g, m, l, co, t, st);                        \
+      case 7: return run_batch<D, 7, A>(fs, ls, pt, ns, fb, lb, g, m, l, co, t, st);                        \
+      case 8: return run_batch<D, 8, A>(fs, ls, pt, ns, fb, lb, g, m, l, co, t, st);                        \
       default: return cudaErrorInvalidValue;                                                            \
     }                                                                                                   \
   };                                                                                                    \

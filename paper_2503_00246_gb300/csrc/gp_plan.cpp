@@ -19,6 +19,7 @@
 #include <cmath>
 #include <cstring>
 #include <limits>
+#include <mutex>
 
 namespace gp {
 
@@ -42,7 +43,7 @@ static void legendre(int n, R t, R& p, R& dp) {
   dp = n * (t * p1 - p0) / (t * t - 1);  // P_n' = n (t P_n - P_{n-1}) / (t^2 - 1)
 }
 
-static void gauss_lobatto_01_r(int k, std::vector<R>& x) {
+static void gauss_lobatto_newton(int k, std::vector<R>& x) {
   x.assign(k + 1, R(0));
   x[k] = 1;
   const R pi = 3.141592653589793238462643383279502884L;
@@ -60,6 +61,15 @@ static void gauss_lobatto_01_r(int k, std::vector<R>& x) {
     }
     x[i] = (t + 1) / 2;
   }
+}
+
+// The nodes of each degree, computed once per process: a plan asks for them four times, and binary128
+// arithmetic is done in software.
+static void gauss_lobatto_01_r(int k, std::vector<R>& x) {
+  static std::once_flag once[KMAX + 1];
+  static std::vector<R> nodes[KMAX + 1];
+  std::call_once(once[k], [k] { gauss_lobatto_newton(k, nodes[k]); });
+  x = nodes[k];
 }
 
 void gauss_lobatto_01(int k, std::vector<double>& x) {
@@ -1243,7 +1253,7 @@ gp_status build_plan(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* 
       }
     }
     for (double& v : lam) v *= opts->gamma;
-    normal_basis(k, p.jumps, lam, hv, p.ldl);
+    if (opts->precision == GP_FP64) normal_basis(k, p.jumps, lam, hv, p.ldl);
     return GP_OK;
   }
   if (opts->stabilization != GP_STAB_GHOST) { err = "unknown stabilization"; return GP_EINVAL; }
@@ -1261,7 +1271,7 @@ gp_status build_plan(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* 
       return GP_EINVAL;
     }
   }
-  normal_basis(k, p.jumps, cw, hd, p.ldl);
+  if (opts->precision == GP_FP64) normal_basis(k, p.jumps, cw, hd, p.ldl);
   return GP_OK;
 }
 

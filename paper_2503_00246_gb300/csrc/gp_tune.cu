@@ -85,9 +85,9 @@ int64_t ipow(int64_t b, int e) {
 
 // Candidate shapes: face CTAs of about 64..512 threads; lift CTAs of 64..512 threads
 // with one or two rows per thread.
-void candidates(const gp::Plan& p, const gp::TileOps& ops, std::vector<gp::Tiles>& face,
+void candidates(const gp::Plan& p, const int form, const gp::TileOps& ops, std::vector<gp::Tiles>& face,
                 std::vector<gp::Tiles>& lift) {
-  const gp::Tiles d = ops.defaults(p.k);
+  const gp::Tiles d = ops.defaults(p.k, form);
   const int L = p.L, KR = (int)ipow(p.k, p.dim - 1);
   face.clear();
   lift.clear();
@@ -96,7 +96,7 @@ void candidates(const gp::Plan& p, const gp::TileOps& ops, std::vector<gp::Tiles
     t.fb = std::max(1, T / L);
     bool dup = false;
     for (const auto& u : face) dup = dup || u.fb == t.fb;
-    if (!dup && ops.resolve(p.k, t)) face.push_back(t);
+    if (!dup && ops.resolve(p.k, t, form)) face.push_back(t);
   }
   for (int T : {64, 128, 256, 512})
     for (int depth : {1, 2}) {
@@ -105,7 +105,7 @@ void candidates(const gp::Plan& p, const gp::TileOps& ops, std::vector<gp::Tiles
       t.lcb = std::max(1, depth * T / KR);
       bool dup = false;
       for (const auto& u : lift) dup = dup || (u.lnt == t.lnt && u.lcb == t.lcb);
-      if (!dup && ops.resolve(p.k, t)) lift.push_back(t);
+      if (!dup && ops.resolve(p.k, t, form)) lift.push_back(t);
     }
 }
 
@@ -116,7 +116,7 @@ extern "C" {
 gp_status gp_get_tiles(const gp_ctx* ctx, gp_tiles* out) {
   if (!ctx || !out) return fail(ctx, GP_EINVAL, "null argument");
   gp::Tiles t = ctx->tiles;
-  if (!gpi::tile_ops(ctx->plan.dim, ctx->plan.precision).resolve(ctx->plan.k, t))
+  if (!gpi::tile_ops(ctx->plan.dim, ctx->plan.precision).resolve(ctx->plan.k, t, ctx->form))
     return fail(ctx, GP_EINVAL, "the context holds an invalid tile shape");
   *out = to_abi(t);
   return GP_OK;
@@ -125,7 +125,7 @@ gp_status gp_get_tiles(const gp_ctx* ctx, gp_tiles* out) {
 gp_status gp_set_tiles(gp_ctx* ctx, const gp_tiles* tiles) {
   if (!ctx || !tiles) return fail(ctx, GP_EINVAL, "null argument");
   gp::Tiles t = from_abi(*tiles);
-  if (!gpi::tile_ops(ctx->plan.dim, ctx->plan.precision).resolve(ctx->plan.k, t))
+  if (!gpi::tile_ops(ctx->plan.dim, ctx->plan.precision).resolve(ctx->plan.k, t, ctx->form))
     return fail(ctx, GP_EINVAL, "tile shape out of range (threads per CTA, shared memory or lift threads)");
   ctx->tiles = from_abi(*tiles);
   return GP_OK;
@@ -137,7 +137,7 @@ gp_status gp_tiles_record(int device, int dim, int degree, int precision, const 
       (precision != GP_FP64 && precision != GP_FP32 && precision != GP_FP64_FF))
     return fail(nullptr, GP_EINVAL, "bad (dim, degree, precision)");
   gp::Tiles t = from_abi(*tiles);
-  if (!gpi::tile_ops(dim, precision).resolve(degree, t)) return fail(nullptr, GP_EINVAL, "tile shape out of range");
+  if (!gpi::tile_ops(dim, precision).resolve(degree, t, 0)) return fail(nullptr, GP_EINVAL, "tile shape out of range");
   gpi::tiles_record(device, dim, degree, precision, from_abi(*tiles));
   return GP_OK;
 }
@@ -157,9 +157,9 @@ gp_status gp_autotune(gp_ctx* ctx, int reps, gp_tiles* best, double* ms) {
   const gp::Plan& p = ctx->plan;
   const gp::TileOps ops = gpi::tile_ops(p.dim, p.precision);
   std::vector<gp::Tiles> face, lift;
-  candidates(p, ops, face, lift);
+  candidates(p, ctx->form, ops, face, lift);
   gp::Tiles cur = ctx->tiles;
-  if (!ops.resolve(p.k, cur)) cur = ops.defaults(p.k);
+  if (!ops.resolve(p.k, cur, ctx->form)) cur = ops.defaults(p.k, ctx->form);
   if (p.num_faces() == 0 || face.empty() || lift.empty()) {
     if (best) *best = to_abi(cur);
     if (ms) ms[0] = ms[1] = 0.0;

@@ -11,13 +11,25 @@ from paper_2503_00246_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 
 
+BALL = {3: 100, 4: 84, 5: 54, 6: 44, 7: 34, 8: 28}   # cells per direction of the 3D balls
+
+
+# 3D meshes with more than 24 MB of W_F, above which FP32 stores compact outputs at every k >= 3, and
+# small ones of the degrees that always do, as 2D does
 @pytest.mark.parametrize("box", [False, True])
-@pytest.mark.parametrize("dim,n,k", [(2, 9, k) for k in range(1, 9)] + [(3, 5, 1), (3, 5, 2), (3, 4, 5), (3, 3, 7), (3, 3, 8)])
+@pytest.mark.parametrize("dim,n,k", [(2, 9, k) for k in range(1, 9)] + [(3, 28, 3), (3, 22, 4), (3, 18, 5), (3, 16, 6),
+                                                                       (3, 14, 7), (3, 13, 8), (3, 5, 5), (3, 3, 7),
+                                                                       (3, 3, 8)])
 def test_compact_lift(gplib, cuda, dim, n, k, box):
-    pr = W.box_problem(dim, n, k, hi=1.0) if box else W.small_ball(dim, 2 * n, k, seed=70 + k)
+    pr = W.box_problem(dim, n, k, hi=1.0) if box else W.small_ball(dim, BALL.get(k, n) if dim == 3 and n > 5 else 2 * n, k, seed=70 + k)
     ctx = gplib.setup_problem(pr, precision=1)
+    if dim == 3 and n > 5:
+        assert ctx.n_faces * (2 * k + 1) * (k + 1) ** 2 * 4 > 24 << 20
     x = W.x_vectors(pr, ctx.n_active)[0].astype(np.float32)
-    ref = Oracle(pr).apply(x.astype(np.float64))
+    o = Oracle(pr)
+    rows = np.arange(ctx.n_active) if dim == 2 else np.unique(np.random.default_rng(k).integers(0, ctx.n_active, 1500))
+    ref = o.apply_rows(x.astype(np.float64), rows)
+    scale = np.abs(ref).max()
     xd = cuda.tensor(x, device="cuda")
     first = None
     for cells, threads in ((0, 0), (1, 32), (3, 64), (46 * 1024 // (4 * (37 if dim == 3 else 13)), 256)):
@@ -26,8 +38,8 @@ def test_compact_lift(gplib, cuda, dim, n, k, box):
             yd = cuda.ones_like(xd) if add else cuda.full_like(xd, float("nan"))
             (gplib.gp_apply_add if add else gplib.gp_apply)(ctx, xd, yd)
             cuda.cuda.synchronize()
-            y = yd.double().cpu().numpy() - (1.0 if add else 0.0)
-            assert np.abs(y - ref).max() <= 1e-5 * max(np.abs(ref).max(), 1.0 if add else 0.0)
+            y = yd.double().cpu().numpy()[rows] - (1.0 if add else 0.0)
+            assert np.abs(y - ref).max() <= 1e-5 * max(scale, 1.0 if add else 0.0)
             if not add:
                 first = yd if first is None else first
                 assert cuda.equal(yd, first), (cells, threads)
