@@ -8,10 +8,11 @@
 //   W_F[b, tau] = sum_j g_j[b] T_F[tau, j]             normal expansion
 //
 // i.e. the three-step face apply of Sec. 2.5.1 with the normal step split in
-// two around the tangential masses (G^ has rank k), and stores W_F in the
-// patch's lexicographic order.  The lift kernel then adds, for every touched
-// DoF, the W_F entries of the faces that contain it in a fixed order: a
-// gather, so no atomics and bitwise reproducible.  For the overwrite form,
+// two around the tangential masses (G^ has rank k), and stores W_F as [b][tau]
+// or, compact, T_F as [tau][j].  The lift kernel then adds, for every touched
+// DoF, the W_F entries of the faces that contain it in a fixed order (expanding
+// them from T_F in the compact form): a gather, so no atomics and bitwise
+// reproducible.  For the overwrite form,
 // extra CTAs of the face launch, spread over its grid, write the zeros of the untouched active DoFs.
 //
 // Template parameter A (gp_arith.cuh) picks the arithmetic: FP32, FP64, or
