@@ -1178,8 +1178,7 @@ gp_status build_plan(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* 
       p.lcell[4 * i + 2] = cl;
       const int co[3] = {ci, cj, cl};
       window(co, &p.lwin[(size_t)p.lwin_width * i]);
-      for (int w = 0; w < d * nw; ++w)
-        if (p.lwin[(size_t)p.lwin_width * i + w] >= 0) p.lmask[i] |= reach[w];
+      for (uint64_t m = order[i].first; m != 0; m &= m - 1) p.lmask[i] |= reach[__builtin_ctzll(m)];   // present faces
       for (int t = 0; t < KR; ++t) {
         int q = t % k, r = t / k;
         int Y = cj * k + q, Z = cl * k + r, X = ci * k;
@@ -1209,9 +1208,9 @@ gp_status build_plan(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* 
       if (f < -1 || f >= (int32_t)nf) { err = "internal: lift window outside the face list"; return GP_EINVAL; }
     for (int32_t r : p.lrow)
       if (r < -1 || r >= na) { err = "internal: lift row outside the active DoFs"; return GP_EINVAL; }
-    // every node that the lift writes for the owner's mask
+    // every node that the lift of compact outputs (FP32) writes for the owner's mask
     const int KR = (int)ipow(k, d - 1);
-    for (int64_t i = 0; i < p.num_lift_cells(); ++i) {
+    for (int64_t i = 0; i < p.num_lift_cells() && opts->precision == GP_FP32; ++i) {
       const int m = p.lmask[i];
       int last[4];                                  // by row kind (q > 0) + 2 (r > 0)
       for (int kind = 0; kind < 4; ++kind) last[kind] = (m >> (2 * kind + 1)) & 1 ? k - 1 : (m >> (2 * kind)) & 1 ? 0 : -1;
