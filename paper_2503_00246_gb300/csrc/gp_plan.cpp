@@ -218,7 +218,7 @@ void normal_basis(int k, const std::vector<double>& jumps, const std::vector<dou
   auto absq = [](Q v) { return v < 0 ? -v : v; };
   ldl.assign((size_t)k * N + k, 0.0);
   for (double v : c)
-    if (!(v >= 0.0)) {
+    if (!(v >= 0.0) || std::isinf(v)) {
       ldl.clear();
       return;
     }
@@ -248,7 +248,12 @@ void normal_basis(int k, const std::vector<double>& jumps, const std::vector<dou
         ldl[(size_t)j * N + i] = (double)b[i];
       }
       for (int i = par; i < j; i += 2) ldl[(size_t)j * N + kPivot[k - 1][i]] = 0.0;
-      ldl[(size_t)k * N + j] = (double)(d * Q(hd));
+      const double D = (double)(d * Q(hd));
+      if (!(D >= 0x1p-900 && D <= 0x1p900)) {     // weights at the ends of the range: s_j g_j may still fit
+        ldl.clear();
+        return;
+      }
+      ldl[(size_t)k * N + j] = D;
       for (int a = 0; a < n; ++a)
         for (int e = 0; e < n; ++e) A[a * n + e] -= d * b[a] * b[e];
     }

@@ -152,8 +152,8 @@ void reference_1d(int k, const std::vector<double>& gl, std::vector<double>& mas
 // The lumped form of the mass matrix (see Plan::lump); false if it does not reproduce `mass`.
 bool lumped_mass(int k, const std::vector<double>& mass, std::vector<double>& lump);
 // The triangular normal basis of the weights c (per order, without the factor hd of the mesh
-// size, so that problems of one degree and one set of weights have equal B); empty for weights below 0
-// or an elimination that grows.
+// size, so that problems of one degree and one set of weights have equal B); empty for weights that are
+// negative, infinite or NaN, an elimination that grows, or factors D outside 2^-900 .. 2^900.
 void normal_basis(int k, const std::vector<double>& jumps, const std::vector<double>& c, double hd,
                   std::vector<double>& ldl);
 void reference_stiffness(int k, std::vector<double>& stiff);

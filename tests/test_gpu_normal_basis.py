@@ -47,6 +47,13 @@ def test_fp64_weights(gplib, cuda, dim, n, k, kind):
             assert v @ _apply(gplib, cuda, ctx, v) >= -1e-13 * np.abs(ref).max() * v.size * np.abs(v).max() ** 2
 
 
+@pytest.mark.parametrize("k", [1, 3, 8])
+def test_infinite_weight_is_not_dropped(gplib, cuda, k):
+    pr = W.small_ball(2, 12, k, seed=90 + k, weights=[0.5] * (k - 1) + [float("inf")])
+    ctx = gplib.setup_problem(pr, precision=0, path=gplib.GP_PATH_FACE_LIFT)
+    assert not np.isfinite(_apply(gplib, cuda, ctx, W.x_vectors(pr, ctx.n_active)[0])).all()
+
+
 def test_batch_of_mixed_weights(gplib, cuda):
     probs = [W.small_ball(3, 8, 3, seed=5, weights=_weights(kind, 3)) for kind in ("gamma", "paper", "negative", "gamma")]
     ctxs = [gplib.setup_problem(pr, precision=0) for pr in probs]
