@@ -347,7 +347,9 @@ gp_status gp_profile_read(gp_ctx* ctx, double ms[2], int64_t* calls);
 /* Batched form: several independent problems, nrhs right-hand sides each, replayed
  * as one CUDA graph (the batched workload of many meshes of uneven n, k and
  * geometry).  gp_batch_create groups the problems by (dimension, degree,
- * arithmetic, stabilisation); every (problem, right-hand side) pair gets its own face-output
+ * arithmetic, stabilisation) and by the kernels that gp_apply runs for them (FP32: the form of the
+ * face outputs, which depends on the size; FP64: the normal basis, which depends on the weights);
+ * every (problem, right-hand side) pair gets its own face-output
  * buffer, and one face launch plus one lift launch per group cover all pairs.  The
  * graph also holds the host-to-device copy of the table of x / y pointers, so each
  * gp_batch_apply writes that table (pinned host memory) and launches the graph.
@@ -358,6 +360,7 @@ gp_status gp_profile_read(gp_ctx* ctx, double ms[2], int64_t* calls);
 typedef struct gp_batch gp_batch;
 gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** out);
 gp_status gp_batch_apply(gp_batch* batch, const void* const* x, void* const* y, void* stream);
+/* The launched groups of the batch and the bytes of its face outputs. */
 gp_status gp_batch_info(const gp_batch* batch, int64_t* ngroups, int64_t* scratch_bytes);
 void gp_batch_destroy(gp_batch* batch);
 

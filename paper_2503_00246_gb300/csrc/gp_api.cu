@@ -4,7 +4,6 @@
 #include <map>
 #include <mutex>
 #include <new>
-#include <set>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -712,7 +711,6 @@ struct gp_batch {
     gp::Tiles tiles{};                 // the tile shape of the group's first context
   };
   std::vector<Group> groups;
-  int64_t nkinds = 0;                  // groups by (dimension, degree, arithmetic, stabilisation)
   void* d_w = nullptr;
   void* d_gs = nullptr;                // per problem: the scaled jump vectors s_j g_j
   size_t w_bytes = 0;
@@ -779,11 +777,9 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
   // each problem runs as in gp_apply
   typedef std::tuple<int, int, int, int> Key;
   std::map<std::tuple<Key, std::vector<double>, bool>, int> key;
-  std::set<Key> kinds;
   for (int p = 0; p < nprob; ++p) {
     const gp::Plan& pl = ctxs[p]->plan;
     const Key kd = std::make_tuple(pl.dim, pl.k, pl.precision, pl.stabilization);
-    kinds.insert(kd);
     const bool ldl = pl.precision == GP_FP64 && !pl.ldl.empty();
     const auto kk = std::make_tuple(
         kd, ldl ? std::vector<double>(pl.ldl.begin(), pl.ldl.begin() + pl.k * (pl.k + 1)) : std::vector<double>(),
@@ -809,7 +805,6 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
       b->groups[gi].rhs.push_back(r);
     }
   }
-  b->nkinds = (int64_t)kinds.size();
   // face-output buffers, one per segment, 256-byte aligned in one allocation
   std::vector<std::vector<size_t>> woff(b->groups.size());
   size_t total = 0;
@@ -939,7 +934,7 @@ gp_status gp_batch_apply(gp_batch* b, const void* const* x, void* const* y, void
 
 gp_status gp_batch_info(const gp_batch* b, int64_t* ngroups, int64_t* scratch_bytes) {
   if (!b || !ngroups || !scratch_bytes) return fail(nullptr, GP_EINVAL, "null argument");
-  *ngroups = b->nkinds;
+  *ngroups = (int64_t)b->groups.size();
   *scratch_bytes = (int64_t)b->w_bytes;
   return GP_OK;
 }

@@ -43,3 +43,23 @@ def test_compact_lift(gplib, cuda, dim, n, k, box):
             if not add:
                 first = yd if first is None else first
                 assert cuda.equal(yd, first), (cells, threads)
+
+
+def test_batch_of_both_forms(gplib, cuda):
+    """Large FP32 meshes store compact outputs and small ones W_F: a batch of both runs a pair of launches for
+    each form, and every vector equals gp_apply's bit for bit."""
+    probs = [W.small_ball(3, n, 4, seed=50 + n) for n in (8, 60, 10, 56)]
+    ctxs = [gplib.setup_problem(pr, precision=1, path=gplib.GP_PATH_FACE_LIFT) for pr in probs]
+    xs = [cuda.tensor(W.x_vectors(pr, c.n_active, 2).ravel(), dtype=cuda.float32, device="cuda") for pr, c in zip(probs, ctxs)]
+    ys = [cuda.full_like(x, float("nan")) for x in xs]
+    b = gplib.gp_batch_create(ctxs, 2)
+    assert gplib.gp_batch_info(b)[0] == 2
+    gplib.gp_batch_apply(b, xs, ys)
+    for c, x, y in zip(ctxs, xs, ys):
+        for r in range(2):
+            s = slice(r * c.n_active, (r + 1) * c.n_active)
+            yr = cuda.empty(c.n_active, dtype=cuda.float32, device="cuda")
+            gplib.gp_apply(c, x[s].contiguous(), yr)
+            cuda.cuda.synchronize()
+            assert cuda.equal(y[s], yr)
+    gplib.gp_batch_destroy(b)

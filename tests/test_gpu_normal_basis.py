@@ -60,7 +60,7 @@ def test_batch_of_mixed_weights(gplib, cuda):
     xs = [cuda.tensor(W.x_vectors(pr, c.n_active, 2).ravel(), device="cuda") for pr, c in zip(probs, ctxs)]
     ys = [cuda.full_like(x, float("nan")) for x in xs]
     b = gplib.gp_batch_create(ctxs, 2)
-    assert gplib.gp_batch_info(b)[0] == 1
+    assert gplib.gp_batch_info(b)[0] == 3    # two bases, and the jump vectors of the negative weights
     gplib.gp_batch_apply(b, xs, ys)
     for c, x, y in zip(ctxs, xs, ys):
         for r in range(2):
