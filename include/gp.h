@@ -348,7 +348,7 @@ gp_status gp_profile_read(gp_ctx* ctx, double ms[2], int64_t* calls);
  * as one CUDA graph (the batched workload of many meshes of uneven n, k and
  * geometry).  gp_batch_create groups the problems by (dimension, degree,
  * arithmetic, stabilisation) and by the kernels that gp_apply runs for them (FP32: the form of the
- * face outputs, which depends on the size; FP64: the normal basis, which depends on the weights);
+ * face outputs, which depends on the size; FP64: weights with and without a triangular normal basis);
  * every (problem, right-hand side) pair gets its own face-output
  * buffer, and one face launch plus one lift launch per group cover all pairs.  The
  * graph also holds the host-to-device copy of the table of x / y pointers, so each

@@ -706,13 +706,13 @@ struct gp_batch {
     void* h_ptrs[2] = {nullptr, nullptr};  // pinned: read by the graph's copy node at replay
     int face_blocks = 0, lift_blocks = 0;
     bool compact = false;              // FP32: the problems store compact face outputs
-    bool ldl = false;                  // the problems run one triangular normal basis (Plan::ldl)
+    bool ldl = false;                  // FP64: the problems run their triangular normal bases (Plan::ldl)
     gp::BatchOps ops{};
     gp::Tiles tiles{};                 // the tile shape of the group's first context
   };
   std::vector<Group> groups;
   void* d_w = nullptr;
-  void* d_gs = nullptr;                // per problem: the scaled jump vectors s_j g_j
+  void* d_gs = nullptr;                // per problem: the scaled jump vectors s_j g_j or the basis B
   size_t w_bytes = 0;
   cudaStream_t cap = nullptr;
   cudaGraph_t graph[2] = {nullptr, nullptr};
@@ -771,19 +771,16 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
   b->nrhs = nrhs;
   b->ctxs.assign(ctxs, ctxs + nprob);
   DeviceGuard dg(b->device);
-  // group problems by (dimension, degree, arithmetic, stabilisation)
-  // (d, k, arithmetic, stabilisation): one set of 1D data; FP64 problems of one group whose weights have
-  // other triangular normal bases B, and FP32 problems with other face outputs, launch apart, so that
-  // each problem runs as in gp_apply
+  // one group per (dimension, degree, arithmetic, stabilisation), i.e. set of 1D data, kernel of the normal
+  // step (FP64) and form of the face outputs (FP32): each problem runs as in gp_apply
   typedef std::tuple<int, int, int, int> Key;
-  std::map<std::tuple<Key, std::vector<double>, bool>, int> key;
+  std::map<std::tuple<Key, bool, bool>, int> key;
   for (int p = 0; p < nprob; ++p) {
     const gp::Plan& pl = ctxs[p]->plan;
     const Key kd = std::make_tuple(pl.dim, pl.k, pl.precision, pl.stabilization);
     const bool ldl = pl.precision == GP_FP64 && !pl.ldl.empty();
-    const auto kk = std::make_tuple(
-        kd, ldl ? std::vector<double>(pl.ldl.begin(), pl.ldl.begin() + pl.k * (pl.k + 1)) : std::vector<double>(),
-        (ctxs[p]->form & gp::FORM_COMPACT) != 0);
+    const bool compact = (ctxs[p]->form & gp::FORM_COMPACT) != 0;
+    const auto kk = std::make_tuple(kd, ldl, compact);
     auto it = key.find(kk);
     int gi;
     if (it == key.end()) {
@@ -796,7 +793,7 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
       b->groups[gi].ops = ops_for(pl.precision, pl.dim);
       b->groups[gi].tiles = ctxs[p]->tiles;
       b->groups[gi].ldl = ldl;
-      b->groups[gi].compact = (ctxs[p]->form & gp::FORM_COMPACT) != 0;
+      b->groups[gi].compact = compact;
     } else {
       gi = it->second;
     }
@@ -818,7 +815,7 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
   cudaError_t e = cudaSuccess;
   if (total > 0) e = cudaMalloc(&b->d_w, total);
   b->w_bytes = total;
-  // the scaled jump vectors of every problem, in its group's arithmetic (256-byte aligned)
+  // the scaled jump vectors, or the triangular basis, of every problem, in its group's arithmetic (256-byte aligned)
   std::vector<size_t> gs_off(nprob, 0);
   {
     std::vector<unsigned char> all, one;
@@ -827,7 +824,15 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
         const int pi = b->groups[gi].prob[i];
         if (b->groups[gi].rhs[i] != 0) continue;
         const gp::Plan& pl = ctxs[pi]->plan;
-        b->groups[gi].ops.jumps(pl.k, pl.jumps.data(), pl.scale.data(), one);
+        if (b->groups[gi].ldl) {
+          const int nn = 2 * pl.k + 1;
+          std::vector<double> rows((size_t)pl.k * nn, 0.0), ones(pl.k, 1.0);
+          for (int j = 0; j < pl.k; ++j)
+            for (int i = 0; i <= pl.k; ++i) rows[(size_t)j * nn + i] = pl.ldl[(size_t)j * (pl.k + 1) + i];
+          b->groups[gi].ops.jumps(pl.k, rows.data(), ones.data(), one);
+        } else {
+          b->groups[gi].ops.jumps(pl.k, pl.jumps.data(), pl.scale.data(), one);
+        }
         gs_off[pi] = all.size();
         all.insert(all.end(), one.begin(), one.end());
         all.resize((all.size() + 255) / 256 * 256, 0);
@@ -885,7 +890,7 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
                           b->cap);
       if (e == cudaSuccess)
         e = g.ops.run(g.k, g.d_fsegs, g.d_lsegs, g.d_ptrs[i], (int)g.prob.size(), g.face_blocks, g.lift_blocks,
-                      pl0.jumps.data(), pl0.lump.data(), g.ldl ? pl0.ldl.data() : nullptr, g.compact, g.tiles, b->cap);
+                      pl0.jumps.data(), pl0.lump.data(), g.ldl, g.compact, g.tiles, b->cap);
     }
     cudaGraph_t graph = nullptr;
     const cudaError_t e2 = cudaStreamEndCapture(b->cap, &graph);

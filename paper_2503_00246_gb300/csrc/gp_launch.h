@@ -435,7 +435,7 @@ struct SegSpec {
   FaceArgs fa;          // frows, rbase, fstart, zruns, nzruns of the segment's problem
   LiftArgs la;
   void* wp = nullptr;   // the segment's face-output buffer
-  const void* gs = nullptr;   // device: K x (2K+1) scaled jump vectors of the segment's problem
+  const void* gs = nullptr;   // device: K x (2K+1) scaled jump vectors of the segment's problem, or its B
   double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};   // the problem's s_j (triangular basis: D_j)
 };
 
@@ -475,7 +475,7 @@ bool pack_batch(const std::vector<SegSpec>& in, const bool compact, Tiles& t, st
 
 template <int D, int K, class A>
 cudaError_t run_batch(const void* fsegs, const void* lsegs, const void* ptrs, int nseg, int face_blocks,
-                      int lift_blocks, const double* g, const double* m, const double* ldl, bool compact, Tiles t,
+                      int lift_blocks, const double* g, const double* m, bool ldl, bool compact, Tiles t,
                       cudaStream_t st) {
   using V = typename A::V;
   using IO = typename A::IO;
@@ -491,10 +491,7 @@ cudaError_t run_batch(const void* fsegs, const void* lsegs, const void* ptrs, in
   }
   auto face = face_kernel_batched<D, K, A, false, false>;
   if constexpr (UseLdl<V>::value) {
-    if (ldl) {
-      ldl_consts<V, K>(ldl, c);
-      face = face_kernel_batched<D, K, A, false, true>;
-    }
+    if (ldl) face = face_kernel_batched<D, K, A, false, true>;
   }
   if constexpr (StoreCompact<V>::value) {
     if (compact) face = face_kernel_batched<D, K, A, true, false>;
@@ -537,7 +534,7 @@ struct BatchOps {
                std::vector<unsigned char>&, int&, int&);
   void (*jumps)(int k, const double* g, const double* s, std::vector<unsigned char>& out);
   cudaError_t (*run)(int k, const void*, const void*, const void*, int, int, int, const double*, const double*,
-                     const double*, bool, Tiles, cudaStream_t);
+                     bool, bool, Tiles, cudaStream_t);
 };
 BatchOps batch_ops_f64_d2();
 BatchOps batch_ops_f64_d3();
@@ -564,7 +561,7 @@ BatchOps batch_ops_ff_d3();
     }                                                                                                   \
   };                                                                                                    \
   ops.run = [](int k, const void* fs, const void* ls, const void* pt, int ns, int fb, int lb,          \
-               const double* g, const double* m, const double* l, bool co, Tiles t,                  \
+               const double* g, const double* m, bool l, bool co, Tiles t,                           \
                cudaStream_t st) -> cudaError_t {                                                        \
     switch (k) {                                                                                        \
       case 1: return run_batch<D, 1, A>(fs, ls, pt, ns, fb, lb, g, m, l, co, t, st);                        \

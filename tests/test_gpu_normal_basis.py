@@ -54,13 +54,14 @@ def test_infinite_weight_is_not_dropped(gplib, cuda, k):
     assert not np.isfinite(_apply(gplib, cuda, ctx, W.x_vectors(pr, ctx.n_active)[0])).all()
 
 
-def test_batch_of_mixed_weights(gplib, cuda):
-    probs = [W.small_ball(3, 8, 3, seed=5, weights=_weights(kind, 3)) for kind in ("gamma", "paper", "negative", "gamma")]
+@pytest.mark.parametrize("dim,n,k", [(3, 8, 3), (2, 12, 2), (3, 4, 8)])
+def test_batch_of_mixed_weights(gplib, cuda, dim, n, k):
+    probs = [W.small_ball(dim, n, k, seed=5, weights=_weights(kind, k)) for kind in ("gamma", "paper", "negative", "gamma")]
     ctxs = [gplib.setup_problem(pr, precision=0) for pr in probs]
     xs = [cuda.tensor(W.x_vectors(pr, c.n_active, 2).ravel(), device="cuda") for pr, c in zip(probs, ctxs)]
     ys = [cuda.full_like(x, float("nan")) for x in xs]
     b = gplib.gp_batch_create(ctxs, 2)
-    assert gplib.gp_batch_info(b)[0] == 3    # two bases, and the jump vectors of the negative weights
+    assert gplib.gp_batch_info(b)[0] == 2    # the triangular bases of any weights, and the jump vectors of the negative ones
     gplib.gp_batch_apply(b, xs, ys)
     for c, x, y in zip(ctxs, xs, ys):
         for r in range(2):
