@@ -261,7 +261,7 @@ gp_status gpi::launch(gp_ctx* c, const void* x, void* y, int add, cudaStream_t s
   a.tiles = tiles ? *tiles : c->tiles;
   a.which = which;
   a.form = c->form;
-  a.full_outputs = full_outputs;
+  a.form.system = full_outputs;
   a.slabs = run ? run->table : p.slabs.data();
   a.nslab = run ? run->n : p.num_slabs();
   a.slab_events = run ? run->events : nullptr;
@@ -403,8 +403,8 @@ gp_status gp_setup(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* op
     const size_t vbytes = p.precision == GP_FP32 ? 4 : 8;
     // face outputs W_F of the face + lift path: float, double, or a (hi, lo) float pair per value
     const size_t tp_bytes = (size_t)p.num_faces() * p.L * (2 * p.k + 1) * vbytes;
-    c->form = gp::launch_form(p.precision == GP_FP32, p.dim, p.k, (int64_t)tp_bytes, (int64_t)p.lrow.size());
-    if (e == cudaSuccess && (c->form & gp::FORM_COMPACT)) e = upload(&c->d_lmask, p.lmask);
+    c->form = gp::launch_form(p.precision == GP_FP32, p.dim, p.k, (int64_t)tp_bytes, p.num_faces());
+    if (e == cudaSuccess && c->form.compact) e = upload(&c->d_lmask, p.lmask);
     if (e == cudaSuccess) e = upload(&c->d_zruns, zruns);
     if (c->use_brick) {
       if (e == cudaSuccess) e = upload(&c->d_bdesc, p.bdesc);
@@ -705,7 +705,7 @@ struct gp_batch {
     void* d_ptrs[2] = {nullptr, nullptr};
     void* h_ptrs[2] = {nullptr, nullptr};  // pinned: read by the graph's copy node at replay
     int face_blocks = 0, lift_blocks = 0;
-    bool compact = false;              // FP32: the problems store compact face outputs
+    gp::LaunchForm form{};             // the problems' outputs, the faces of all segments
     bool ldl = false;                  // FP64: the problems run their triangular normal bases (Plan::ldl)
     gp::BatchOps ops{};
     gp::Tiles tiles{};                 // the tile shape of the group's first context
@@ -779,7 +779,7 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
     const gp::Plan& pl = ctxs[p]->plan;
     const Key kd = std::make_tuple(pl.dim, pl.k, pl.precision, pl.stabilization);
     const bool ldl = pl.precision == GP_FP64 && !pl.ldl.empty();
-    const bool compact = (ctxs[p]->form & gp::FORM_COMPACT) != 0;
+    const bool compact = ctxs[p]->form.compact;
     const auto kk = std::make_tuple(kd, ldl, compact);
     auto it = key.find(kk);
     int gi;
@@ -793,10 +793,11 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
       b->groups[gi].ops = ops_for(pl.precision, pl.dim);
       b->groups[gi].tiles = ctxs[p]->tiles;
       b->groups[gi].ldl = ldl;
-      b->groups[gi].compact = compact;
+      b->groups[gi].form.compact = compact;
     } else {
       gi = it->second;
     }
+    b->groups[gi].form.faces += (int64_t)pl.num_faces() * nrhs;
     for (int r = 0; r < nrhs; ++r) {
       b->groups[gi].prob.push_back(p);
       b->groups[gi].rhs.push_back(r);
@@ -866,7 +867,7 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
       for (int j = 0; j < pl.k; ++j) sp.s[j] = g.ldl ? pl.ldl[nb + j] : pl.scale[j];
     }
     std::vector<unsigned char> fs, ls;
-    if (!g.ops.pack(g.k, specs, g.compact, g.tiles, fs, ls, g.face_blocks, g.lift_blocks)) {
+    if (!g.ops.pack(g.k, specs, g.form, g.tiles, fs, ls, g.face_blocks, g.lift_blocks)) {
       e = cudaErrorInvalidConfiguration;
       break;
     }
@@ -890,7 +891,7 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
                           b->cap);
       if (e == cudaSuccess)
         e = g.ops.run(g.k, g.d_fsegs, g.d_lsegs, g.d_ptrs[i], (int)g.prob.size(), g.face_blocks, g.lift_blocks,
-                      pl0.jumps.data(), pl0.lump.data(), g.ldl, g.compact, g.tiles, b->cap);
+                      pl0.jumps.data(), pl0.lump.data(), g.ldl, g.form, g.tiles, b->cap);
     }
     cudaGraph_t graph = nullptr;
     const cudaError_t e2 = cudaStreamEndCapture(b->cap, &graph);

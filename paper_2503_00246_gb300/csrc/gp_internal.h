@@ -19,7 +19,7 @@ struct gp_ctx {
   int32_t* d_lwin = nullptr;
   int32_t* d_lrow = nullptr;
   int32_t* d_lmask = nullptr;
-  int form = 0;                  // gp::launch_form
+  gp::LaunchForm form{};         // gp::launch_form
   int2* d_zruns = nullptr;
   void* d_tp = nullptr;          // per-face outputs W_F (scratch of the face + lift path)
   // brick path (gp_brick.cuh): tables and the partial grids of the plane nodes (scratch)

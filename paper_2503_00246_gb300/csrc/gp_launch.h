@@ -12,6 +12,15 @@
 
 namespace gp {
 
+// What the default tile shapes of a launch depend on: whether FP32 stores compact outputs, the ghost faces
+// of the mesh (of all segments of a batch), and whether the face kernel is the model system's, which stores W_F in
+// every arithmetic (the system's gather reads it).
+struct LaunchForm {
+  bool compact = false;
+  int64_t faces = 0;
+  bool system = false;
+};
+
 struct ApplyArgs {
   int dim = 0, k = 0;
   const void* x = nullptr;   // device, n_active elements
@@ -31,9 +40,7 @@ struct ApplyArgs {
   cudaEvent_t* ev = nullptr;  // optional: 3 events recorded around the two kernels
   Tiles tiles{};              // 0 fields: the defaults of default_tiles
   int which = 3;              // bit 0: face kernel, bit 1: lift kernel (the autotuner times them apart)
-  int form = 0;               // launch_form
-  bool full_outputs = false;  // the face kernel stores W_F whatever its arithmetic (the model system's gather
-                              // reads it); only with which = 1
+  LaunchForm form{};          // launch_form
   const int32_t* slabs = nullptr;  // host: SLAB ints per slab (see Plan::slabs); nslab > 1: slab pipeline
   int nslab = 0;
   cudaEvent_t* slab_events = nullptr;  // host, nslab events: recorded after each slab's lift (the
@@ -47,69 +54,86 @@ struct ApplyArgs {
 
 // Whether an FP32 context stores compact face outputs.  Small W_F stays in L2, where the lift of W_F
 // and its two fewer phases are the faster one for small k (us of an apply, W_F / compact: k = 2, 40^3 ball 6.4 / 7.3; k = 3, 20^3 5.7 /
-// 6.6; k = 4, 12^3 7.7 / 8.7; k = 6, 32^3, 17 MB, 27 / 34); the compact form is from 12 MB of W_F at k = 3
+// 6.6; k = 4, 12^3 7.7 / 8.7; k = 6, 32^3, 17 MB, 27 / 34); the compact form is from 10 MB of W_F at k = 3
 // (64^3 21.0 / 16.4), 3 MB at k = 4 (24^3 10.2 / 9.7), 24 MB at k = 6 (64^3 81 / 72), and at any size for
-// k = 5, 7 and 8 (10^3: 9.9 / 8.5, k = 7, 11^3 12.9 / 10.4, k = 8, 8^3 13.9 / 11.6) and in 2D (300^2 disc,
-// k = 8: 9.7 / 7.2).
+// k = 5, 7 and 8 (10^3: 9.9 / 8.5, k = 7, 11^3 12.9 / 10.4, k = 8, 8^3 13.9 / 11.6).  In 2D, whose W_F is small
+// always, from k = 6 on (64^2 disc, k = 4, 6.9 / 7.3; 600^2, k = 7, 11.3 / 11.0).
 inline bool store_compact(int dim, int k, int64_t w_bytes) {
   const int64_t mb = (int64_t)1 << 20;
-  return dim == 2 || k == 5 || k >= 7 || (k == 6 && w_bytes > 24 * mb) || (k == 4 && w_bytes > 3 * mb) ||
+  if (dim == 2) return k >= 6;
+  return k == 5 || k >= 7 || (k == 6 && w_bytes > 24 * mb) || (k == 4 && w_bytes > 3 * mb) ||
          (k == 3 && w_bytes > 10 * mb);
 }
-// The form of a context's launches: bit 0 compact outputs (FP32), bit 1 so few lift rows that a thread
-// takes one (default tiles): below them the rows of one CTA follow each other on a GPU that is mostly
-// idle (FP32, compact: 16^3 ball, k = 5, 24.2 / 9.5 us, 28^3, k = 8, 40 / 36 us; float-float: 14^3, k = 8,
-// 47 / 35 us; above, 32^3, k = 6, 53 / 62 us).
-constexpr int FORM_COMPACT = 1, FORM_FEW = 2;
-inline int launch_form(bool fp32, int dim, int k, int64_t w_bytes, int64_t rows) {
-  return (fp32 && store_compact(dim, k, w_bytes) ? FORM_COMPACT : 0) |
-         (rows < (fp32 ? 600000 : 100000) ? FORM_FEW : 0);
+inline LaunchForm launch_form(bool fp32, int dim, int k, int64_t w_bytes, int64_t faces) {
+  return LaunchForm{fp32 && store_compact(dim, k, w_bytes), faces};
 }
 
-// Default tile shape: about 256 threads per CTA, one item per thread.  FP32 in 3D: face
-// CTAs of about 130 threads (more CTAs per SM to run while one waits at a barrier; 128^3 gyroid,
-// k = 4, face kernel with 2 / 5 / 6 / 10 / 20 faces: 193 / 127 / 132 / 136 / 158 us), and,
-// with compact outputs, from k = 4 on two to four lines per lift thread (inner lines first, then edge
-// lines with more faces, so that the warps meet at the barriers; 128^3 gyroid with 1 / 2 / 4 lines: 152 / 104 / 150 us; 49^3
-// ball at k = 8, 128 threads, with 1 / 2 / 4 / 8: 102 / 56 / 49 / 61 us).
+// Default tile shapes {faces per face CTA, owners per lift CTA, lift threads}: up to four per degree, by the
+// number of ghost faces.  Small meshes want many small CTAs (few faces each, a row or less per lift thread), or
+// most of the GPU idles while each CTA works through its rows; large ones want what keeps most warps busy:
+// FP64 and float-float face CTAs that fill the SM, lift CTAs with 32 owners, where every row type fills whole
+// warps, and for the compact outputs two to four lines per thread.  Each entry is the fastest of about 30 lift
+// and 10 face shapes, times taken on 15 balls (10^3 .. 96^3) and 5 gyroids per degree and 6 discs in 2D, the
+// limits between them where the fastest shape changes; the same shape at every size took, against
+// these, up to (us): FP32 compact k = 8, 40^3, 77 / 55, k = 7, 36^3, 50 / 34, k = 5, 64^3, 60 / 44;
+// float-float k = 8, 20^3, 70 / 57, k = 5, 28^3, 39 / 26; FP64 k = 4, 25^3, 50 / 36, k = 1, 40^3, 27 / 14,
+// 2D, k = 7, 300^2, 38 / 17.
+struct TileRule {
+  int32_t upto[3];   // faces up to which the first, the second and the third shape run
+  Tiles shape[4];
+};
+constexpr TileRule tiles_at(Tiles a) { return {{0, 0, 0}, {a, a, a, a}}; }
+constexpr TileRule tiles_at(Tiles a, int n, Tiles b) { return {{n, n, n}, {a, b, b, b}}; }
+constexpr TileRule tiles_at(Tiles a, int n, Tiles b, int m, Tiles c) { return {{n, m, m}, {a, b, c, c}}; }
+constexpr TileRule tiles_at(Tiles a, int n, Tiles b, int m, Tiles c, int l, Tiles d) { return {{n, m, l}, {a, b, c, d}}; }
+typedef TileRule TileRules[2][8];   // [dimension - 2][degree - 1]
+constexpr TileRules kTilesF64 = {
+    {tiles_at({96, 256, 256}, 1000, {160, 256, 512}), tiles_at({42, 256, 512}), tiles_at({16, 16, 64}),
+     tiles_at({19, 128, 512}, 1000, {6, 32, 256}), tiles_at({10, 24, 256}), tiles_at({4, 32, 256}),
+     tiles_at({4, 16, 256}), tiles_at({3, 32, 512})},
+    {tiles_at({128, 256, 512}), tiles_at({14, 128, 512}, 2500, {10, 64, 512}, 24000, {21, 32, 256}),
+     tiles_at({2, 16, 256}, 6000, {8, 32, 512}), tiles_at({6, 32, 512}, 19000, {20, 32, 512}),
+     tiles_at({4, 8, 256}, 6000, {7, 16, 512}), tiles_at({3, 3, 256}, 3000, {5, 14, 512}), tiles_at({2, 8, 512}),
+     tiles_at({3, 4, 256})}};
+constexpr TileRules kTilesFF = {
+    {tiles_at({128, 256, 512}), tiles_at({42, 128, 256}), tiles_at({24, 32, 128}), tiles_at({19, 32, 256}),
+     tiles_at({10, 24, 256}), tiles_at({9, 32, 256}), tiles_at({8, 16, 256}), tiles_at({14, 32, 512})},
+    {tiles_at({128, 256, 512}), tiles_at({10, 64, 256}, 15000, {14, 64, 512}, 35000, {14, 128, 512}),
+     tiles_at({4, 16, 256}, 12000, {8, 28, 256}, 21000, {8, 24, 128}),
+     tiles_at({5, 32, 512}, 12000, {5, 32, 256}),
+     tiles_at({3, 16, 512}, 6000, {7, 24, 512}, 19000, {7, 32, 256}),
+     tiles_at({2, 14, 512}, 2500, {3, 32, 512}, 6000, {3, 64, 512}),
+     tiles_at({2, 8, 512}, 1400, {2, 16, 512}, 2800, {2, 24, 512}, 9700, {4, 32, 256}),
+     tiles_at({3, 4, 256}, 2500, {3, 32, 512}, 6000, {3, 32, 256})}};
+// FP32 that stores W_F: the degrees and sizes that store_compact leaves
+constexpr TileRules kTilesF32 = {
+    {tiles_at({192, 128, 256}), tiles_at({85, 128, 256}), tiles_at({48, 32, 128}), tiles_at({25, 64, 512}),
+     tiles_at({21, 16, 128}), tiles_at({18, 32, 256}), tiles_at({12, 16, 256}), tiles_at({10, 32, 512})},
+    {tiles_at({48, 64, 128}, 50000, {64, 128, 128}), tiles_at({21, 64, 512}, 21000, {14, 64, 512}),
+     tiles_at({8, 16, 256}), tiles_at({5, 32, 512}), tiles_at({3, 8, 256}),
+     tiles_at({2, 1, 64}, 2500, {3, 4, 256}), tiles_at({1, 4, 256}), tiles_at({1, 4, 256})}};
+constexpr TileRules kTilesF32Compact = {
+    {tiles_at({48, 64, 128}), tiles_at({85, 128, 256}), tiles_at({64, 64, 256}), tiles_at({51, 32, 128}),
+     tiles_at({21, 24, 128}), tiles_at({18, 32, 256}), tiles_at({12, 32, 256}), tiles_at({14, 32, 256})},
+    {tiles_at({64, 64, 128}), tiles_at({14, 64, 256}), tiles_at({6, 28, 256}, 50000, {8, 32, 128}),
+     tiles_at({5, 32, 512}, 35000, {5, 32, 256}),
+     tiles_at({3, 8, 256}, 3600, {3, 20, 256}, 35000, {3, 24, 256}),
+     tiles_at({3, 7, 128}, 21000, {3, 14, 128}),
+     tiles_at({2, 4, 256}, 2500, {1, 10, 256}, 7700, {2, 8, 128}),
+     tiles_at({1, 4, 256}, 2800, {1, 6, 128}, 9700, {1, 8, 128})}};
+
+// The model system's face kernel runs beside its cell kernel: CTAs of 130 to 260 threads are within 2 % of the
+// fastest at every size (12 meshes per degree), and small ones cost up to 30 us (FP64, k = 2, 16^3 ball, 7 / 10 / 21
+// faces: 56 / 25 / 24 us).  FP32, FP64, float-float in 3D; in 2D about 256 threads.
+constexpr int kSystemFaces[3][8] = {{64, 17, 8, 5, 3, 3, 2, 1}, {64, 21, 16, 20, 7, 5, 4, 3}, {64, 21, 16, 5, 7, 5, 4, 3}};
+
 template <int D, int K, typename V>
-Tiles default_tiles_t(const int form) {
-  const bool CO = (form & FORM_COMPACT) && StoreCompact<V>::value && D == 3;
-  const bool few = (form & FORM_FEW) != 0;
-  Tiles t;
-  constexpr bool F32 = std::is_same<V, float>::value && D == 3;
-  t.fb = F32 ? (130 / Shape<D, K>::L > 0 ? 130 / Shape<D, K>::L : 1) : Shape<D, K>::FB;
-  t.lcb = LiftShape<D, K>::CB;
-  t.lnt = LiftShape<D, K>::NT;
-  // W_F outputs in 3D: with 32 (or 16) owners per CTA every row type fills whole warps, which then take
-  // one path (128^3 gyroid, k = 4, lift with 16 / 32 owners: float-float 283 / 216 us, FP64, whose
-  // warps skip missing faces, 259 / 214 us at one row per thread; 96^3 ball, k = 5: float-float
-  // 118 / 91 us, FP64 112 / 92 us with 16)
-  constexpr bool FF = sizeof(V) == 8 && !std::is_same<V, double>::value && D == 3;
-  constexpr bool F64 = std::is_same<V, double>::value && D == 3;
-  // face CTAs at k = 4 (128^3 gyroid, face kernel): float-float 5 faces 355 us, 10 faces 367 us; FP64
-  // 20 faces 992 us, 10 faces 1010 us
-  if (FF && K == 4) t.fb = 5;
-  if (F64 && K == 4) t.fb = 20;
-  if (FF && K == 3 && !few) {
-    t.lcb = 24;
-    t.lnt = 128;
-  }
-  if (FF && (K == 4 || (K > 4 && !few))) t.lcb = 32;
-  if (F64 && K == 3) t.lcb = 16;
-  if (F64 && (K == 4 || K == 5)) {
-    t.lcb = K == 4 ? 32 : 16;
-    t.lnt = 512;
-  }
-  if (CO && K == 4) {
-    t.lcb = 32;
-    if (few) t.lnt = 512;
-  }
-  if (CO && few && (K == 5 || K == 7)) t.lcb = K == 5 ? 8 : 4;
-  if (CO && K >= 5 && !few) {
-    t.lcb = K <= 6 ? 16 : 8;
-    t.lnt = 128;
-  }
+Tiles default_tiles_t(const LaunchForm& form) {
+  constexpr bool F32 = std::is_same<V, float>::value, F64 = std::is_same<V, double>::value;
+  const TileRules& all = F32 ? (form.compact ? kTilesF32Compact : kTilesF32) : F64 ? kTilesF64 : kTilesFF;
+  const TileRule& r = all[D - 2][K - 1];
+  Tiles t = r.shape[form.faces <= r.upto[0] ? 0 : form.faces <= r.upto[1] ? 1 : form.faces <= r.upto[2] ? 2 : 3];
+  if (form.system) t.fb = D == 3 ? (F32 ? kSystemFaces[0] : F64 ? kSystemFaces[1] : kSystemFaces[2])[K - 1] : Shape<D, K>::FB;
   return t;
 }
 
@@ -117,7 +141,7 @@ Tiles default_tiles_t(const int form) {
 // (threads per CTA <= MAX_CTA_THREADS, lift threads a multiple of 32, dynamic
 // shared memory <= MAX_DYN_SMEM).  Returns false if t is out of range.
 template <int D, int K, typename V>
-bool resolve_tiles(Tiles& t, const int form) {
+bool resolve_tiles(Tiles& t, const LaunchForm& form) {
   const Tiles d = default_tiles_t<D, K, V>(form);
   if (t.fb == 0) t.fb = d.fb;
   if (t.lcb == 0) t.lcb = d.lcb;
@@ -130,8 +154,8 @@ bool resolve_tiles(Tiles& t, const int form) {
 
 // Per (arithmetic, dimension): default tiles and range check for degree k.
 struct TileOps {
-  Tiles (*defaults)(int k, int form);
-  bool (*resolve)(int k, Tiles& t, int form);
+  Tiles (*defaults)(int k, const LaunchForm& form);
+  bool (*resolve)(int k, Tiles& t, const LaunchForm& form);
 };
 TileOps tile_ops_f64_d2();
 TileOps tile_ops_f64_d3();
@@ -144,19 +168,19 @@ TileOps tile_ops_ff_d3();
   case K: return resolve_tiles<D, K, typename A::V>(t, form);
 #define GP_TILE_OPS(D, A)                                                                     \
   TileOps ops;                                                                                \
-  ops.defaults = [](int k, int form) -> Tiles {                                            \
+  ops.defaults = [](int k, const LaunchForm& form) -> Tiles {                                 \
     switch (k) {                                                                              \
-      case 1: return default_tiles_t<D, 1, typename A::V>(form);                                                 \
-      case 2: return default_tiles_t<D, 2, typename A::V>(form);                                                 \
-      case 3: return default_tiles_t<D, 3, typename A::V>(form);                                                 \
-      case 4: return default_tiles_t<D, 4, typename A::V>(form);                                                 \
-      case 5: return default_tiles_t<D, 5, typename A::V>(form);                                                 \
-      case 6: return default_tiles_t<D, 6, typename A::V>(form);                                                 \
-      case 7: return default_tiles_t<D, 7, typename A::V>(form);                                                 \
-      default: return default_tiles_t<D, 8, typename A::V>(form);                                                \
+      case 1: return default_tiles_t<D, 1, typename A::V>(form);                              \
+      case 2: return default_tiles_t<D, 2, typename A::V>(form);                              \
+      case 3: return default_tiles_t<D, 3, typename A::V>(form);                              \
+      case 4: return default_tiles_t<D, 4, typename A::V>(form);                              \
+      case 5: return default_tiles_t<D, 5, typename A::V>(form);                              \
+      case 6: return default_tiles_t<D, 6, typename A::V>(form);                              \
+      case 7: return default_tiles_t<D, 7, typename A::V>(form);                              \
+      default: return default_tiles_t<D, 8, typename A::V>(form);                             \
     }                                                                                         \
   };                                                                                          \
-  ops.resolve = [](int k, Tiles& t, int form) -> bool {                                    \
+  ops.resolve = [](int k, Tiles& t, const LaunchForm& form) -> bool {                         \
     switch (k) {                                                                              \
       GP_TILE_CASE(D, A, 1) GP_TILE_CASE(D, A, 2) GP_TILE_CASE(D, A, 3) GP_TILE_CASE(D, A, 4) \
       GP_TILE_CASE(D, A, 5) GP_TILE_CASE(D, A, 6) GP_TILE_CASE(D, A, 7) GP_TILE_CASE(D, A, 8) \
@@ -341,7 +365,7 @@ cudaError_t run_slabs(const ApplyArgs& Ar, const Consts<typename A::V, K>& c, co
       if (e != cudaSuccess) return e;
     }
     if (nb > 0) {
-      const auto face = pick_face<D, K, A>(ldl, (Ar.form & FORM_COMPACT) != 0);
+      const auto face = pick_face<D, K, A>(ldl, Ar.form.compact);
       const cudaError_t e =
           (s == 0 || Ar.slab_events)
               ? (face<<<nb, t.fb * S::L, face_smem<D, K, V>(t.fb), st>>>((const IO*)Ar.x, (V*)Ar.tp, (IO*)Ar.y, fa, t.fb, c),
@@ -358,7 +382,7 @@ cudaError_t run_slabs(const ApplyArgs& Ar, const Consts<typename A::V, K>& c, co
     if (la.nlift > 0) {
       // programmatic dependent of this slab's face launch (a plain launch after an event)
       const cudaError_t e =
-          launch_lift<D, K, A>(nb > 0 || !Ar.slab_events, (Ar.form & FORM_COMPACT) != 0, t, (const V*)Ar.tp, (IO*)Ar.y, Ar.add, la, c, st);
+          launch_lift<D, K, A>(nb > 0 || !Ar.slab_events, Ar.form.compact, t, (const V*)Ar.tp, (IO*)Ar.y, Ar.add, la, c, st);
       if (e != cudaSuccess) return e;
     }
     if (Ar.slab_events) {
@@ -415,13 +439,13 @@ cudaError_t run_apply(const ApplyArgs& Ar, cudaStream_t st) {
   const bool faces = Ar.fstart[D] > 0;
   if (Ar.ev) cudaEventRecord(Ar.ev[0], st);
   if (nb > 0 && (Ar.which & 1)) {
-    const auto face = pick_face<D, K, A>(ldl, (Ar.form & FORM_COMPACT) != 0 && !Ar.full_outputs);
+    const auto face = pick_face<D, K, A>(ldl, Ar.form.compact && !Ar.form.system);
     face<<<nb, t.fb * S::L, face_smem<D, K, V>(t.fb), st>>>((const IO*)Ar.x, (V*)Ar.tp, (IO*)Ar.y, fa, t.fb, c);
   }
   if (Ar.ev) cudaEventRecord(Ar.ev[1], st);
   if (Ar.la.nlift > 0 && faces && (Ar.which & 2)) {
     // programmatic dependent launch: the lift's CTAs start while the face grid drains
-    const cudaError_t e = launch_lift<D, K, A>(!Ar.ev && (Ar.which & 1), (Ar.form & FORM_COMPACT) != 0, t, (const V*)Ar.tp, (IO*)Ar.y, Ar.add,
+    const cudaError_t e = launch_lift<D, K, A>(!Ar.ev && (Ar.which & 1), Ar.form.compact, t, (const V*)Ar.tp, (IO*)Ar.y, Ar.add,
                                                Ar.la, c, st);
     if (e != cudaSuccess) return e;
   }
@@ -442,10 +466,11 @@ struct SegSpec {
 // Packs the segments of one (d, k, arithmetic) group into the device layouts of
 // FaceSeg<V, K> and LiftSeg, with the CTA offsets of both launches.
 template <int D, int K, class A>
-bool pack_batch(const std::vector<SegSpec>& in, const bool compact, Tiles& t, std::vector<unsigned char>& fsegs,
+bool pack_batch(const std::vector<SegSpec>& in, const LaunchForm& form, Tiles& t, std::vector<unsigned char>& fsegs,
                 std::vector<unsigned char>& lsegs, int& face_blocks, int& lift_blocks) {
   using V = typename A::V;
-  if (!resolve_tiles<D, K, V>(t, compact)) return false;
+  const bool compact = form.compact;
+  if (!resolve_tiles<D, K, V>(t, form)) return false;
   fsegs.assign(in.size() * sizeof(FaceSeg<V, K>), 0);
   lsegs.assign(in.size() * sizeof(LiftSeg), 0);
   int fb = 0, lb = 0;
@@ -475,12 +500,13 @@ bool pack_batch(const std::vector<SegSpec>& in, const bool compact, Tiles& t, st
 
 template <int D, int K, class A>
 cudaError_t run_batch(const void* fsegs, const void* lsegs, const void* ptrs, int nseg, int face_blocks,
-                      int lift_blocks, const double* g, const double* m, bool ldl, bool compact, Tiles t,
-                      cudaStream_t st) {
+                      int lift_blocks, const double* g, const double* m, bool ldl, const LaunchForm& form,
+                      Tiles t, cudaStream_t st) {
   using V = typename A::V;
   using IO = typename A::IO;
   using S = Shape<D, K>;
-  if (!resolve_tiles<D, K, V>(t, compact)) return cudaErrorInvalidConfiguration;
+  const bool compact = form.compact;
+  if (!resolve_tiles<D, K, V>(t, form)) return cudaErrorInvalidConfiguration;
   Consts<V, K> c;
   for (int j = 0; j < K; ++j)
     for (int b = 0; b < 2 * K + 1; ++b) c.g[j][b] = from_host<V>(g[j * (2 * K + 1) + b]);
@@ -530,11 +556,11 @@ void scaled_jumps(int k, const double* g, const double* s, std::vector<unsigned 
 
 // Per translation unit: batch packing and launch for one (arithmetic, dimension).
 struct BatchOps {
-  bool (*pack)(int k, const std::vector<SegSpec>&, bool, Tiles&, std::vector<unsigned char>&,
+  bool (*pack)(int k, const std::vector<SegSpec>&, const LaunchForm&, Tiles&, std::vector<unsigned char>&,
                std::vector<unsigned char>&, int&, int&);
   void (*jumps)(int k, const double* g, const double* s, std::vector<unsigned char>& out);
   cudaError_t (*run)(int k, const void*, const void*, const void*, int, int, int, const double*, const double*,
-                     bool, bool, Tiles, cudaStream_t);
+                     bool, const LaunchForm&, Tiles, cudaStream_t);
 };
 BatchOps batch_ops_f64_d2();
 BatchOps batch_ops_f64_d3();
@@ -546,32 +572,33 @@ BatchOps batch_ops_ff_d3();
 #define GP_BATCH_OPS(D, A)                                                                              \
   BatchOps ops;                                                                                         \
   ops.jumps = scaled_jumps<A>;                                                                          \
-  ops.pack = [](int k, const std::vector<SegSpec>& in, bool co, Tiles& t, std::vector<unsigned char>& fs,       \
+  ops.pack = [](int k, const std::vector<SegSpec>& in, const LaunchForm& form, Tiles& t,               \
+                std::vector<unsigned char>& fs,                                                         \
                 std::vector<unsigned char>& ls, int& fb, int& lb) -> bool {                             \
     switch (k) {                                                                                        \
-      case 1: return pack_batch<D, 1, A>(in, co, t, fs, ls, fb, lb);                                        \
-      case 2: return pack_batch<D, 2, A>(in, co, t, fs, ls, fb, lb);                                        \
-      case 3: return pack_batch<D, 3, A>(in, co, t, fs, ls, fb, lb);                                        \
-      case 4: return pack_batch<D, 4, A>(in, co, t, fs, ls, fb, lb);                                        \
-      case 5: return pack_batch<D, 5, A>(in, co, t, fs, ls, fb, lb);                                        \
-      case 6: return pack_batch<D, 6, A>(in, co, t, fs, ls, fb, lb);                                        \
-      case 7: return pack_batch<D, 7, A>(in, co, t, fs, ls, fb, lb);                                        \
-      case 8: return pack_batch<D, 8, A>(in, co, t, fs, ls, fb, lb);                                        \
+      case 1: return pack_batch<D, 1, A>(in, form, t, fs, ls, fb, lb);                                        \
+      case 2: return pack_batch<D, 2, A>(in, form, t, fs, ls, fb, lb);                                        \
+      case 3: return pack_batch<D, 3, A>(in, form, t, fs, ls, fb, lb);                                        \
+      case 4: return pack_batch<D, 4, A>(in, form, t, fs, ls, fb, lb);                                        \
+      case 5: return pack_batch<D, 5, A>(in, form, t, fs, ls, fb, lb);                                        \
+      case 6: return pack_batch<D, 6, A>(in, form, t, fs, ls, fb, lb);                                        \
+      case 7: return pack_batch<D, 7, A>(in, form, t, fs, ls, fb, lb);                                        \
+      case 8: return pack_batch<D, 8, A>(in, form, t, fs, ls, fb, lb);                                        \
       default: return false;                                                                            \
     }                                                                                                   \
   };                                                                                                    \
   ops.run = [](int k, const void* fs, const void* ls, const void* pt, int ns, int fb, int lb,          \
-               const double* g, const double* m, bool l, bool co, Tiles t,                           \
+               const double* g, const double* m, bool l, const LaunchForm& form, Tiles t,              \
                cudaStream_t st) -> cudaError_t {                                                        \
     switch (k) {                                                                                        \
-      case 1: return run_batch<D, 1, A>(fs, ls, pt, ns, fb, lb, g, m, l, co, t, st);                        \
-      case 2: return run_batch<D, 2, A>(fs, ls, pt, ns, fb, lb, g, m, l, co, t, st);                        \
-      case 3: return run_batch<D, 3, A>(fs, ls, pt, ns, fb, lb, g, m, l, co, t, st);                        \
-      case 4: return run_batch<D, 4, A>(fs, ls, pt, ns, fb, lb, g, m, l, co, t, st);                        \
-      case 5: return run_batch<D, 5, A>(fs, ls, pt, ns, fb, lb, g, m, l, co, t, st);                        \
-      case 6: return run_batch<D, 6, A>(fs, ls, pt, ns, fb, lb, g, m, l, co, t, st);                        \
-      case 7: return run_batch<D, 7, A>(fs, ls, pt, ns, fb, lb, g, m, l, co, t, st);                        \
-      case 8: return run_batch<D, 8, A>(fs, ls, pt, ns, fb, lb, g, m, l, co, t, st);                        \
+      case 1: return run_batch<D, 1, A>(fs, ls, pt, ns, fb, lb, g, m, l, form, t, st);                        \
+      case 2: return run_batch<D, 2, A>(fs, ls, pt, ns, fb, lb, g, m, l, form, t, st);                        \
+      case 3: return run_batch<D, 3, A>(fs, ls, pt, ns, fb, lb, g, m, l, form, t, st);                        \
+      case 4: return run_batch<D, 4, A>(fs, ls, pt, ns, fb, lb, g, m, l, form, t, st);                        \
+      case 5: return run_batch<D, 5, A>(fs, ls, pt, ns, fb, lb, g, m, l, form, t, st);                        \
+      case 6: return run_batch<D, 6, A>(fs, ls, pt, ns, fb, lb, g, m, l, form, t, st);                        \
+      case 7: return run_batch<D, 7, A>(fs, ls, pt, ns, fb, lb, g, m, l, form, t, st);                        \
+      case 8: return run_batch<D, 8, A>(fs, ls, pt, ns, fb, lb, g, m, l, form, t, st);                        \
       default: return cudaErrorInvalidValue;                                                            \
     }                                                                                                   \
   };                                                                                                    \

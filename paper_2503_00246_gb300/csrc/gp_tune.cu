@@ -85,7 +85,7 @@ int64_t ipow(int64_t b, int e) {
 
 // Candidate shapes: face CTAs of about 64..512 threads; lift CTAs of 64..512 threads
 // with one or two rows per thread.
-void candidates(const gp::Plan& p, const int form, const gp::TileOps& ops, std::vector<gp::Tiles>& face,
+void candidates(const gp::Plan& p, const gp::LaunchForm& form, const gp::TileOps& ops, std::vector<gp::Tiles>& face,
                 std::vector<gp::Tiles>& lift) {
   const gp::Tiles d = ops.defaults(p.k, form);
   const int L = p.L, KR = (int)ipow(p.k, p.dim - 1);
@@ -137,7 +137,7 @@ gp_status gp_tiles_record(int device, int dim, int degree, int precision, const 
       (precision != GP_FP64 && precision != GP_FP32 && precision != GP_FP64_FF))
     return fail(nullptr, GP_EINVAL, "bad (dim, degree, precision)");
   gp::Tiles t = from_abi(*tiles);
-  if (!gpi::tile_ops(dim, precision).resolve(degree, t, 0)) return fail(nullptr, GP_EINVAL, "tile shape out of range");
+  if (!gpi::tile_ops(dim, precision).resolve(degree, t, gp::LaunchForm{})) return fail(nullptr, GP_EINVAL, "tile shape out of range");
   gpi::tiles_record(device, dim, degree, precision, from_abi(*tiles));
   return GP_OK;
 }
