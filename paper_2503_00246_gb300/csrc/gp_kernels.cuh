@@ -54,13 +54,16 @@ template <int D, int K, typename V>
 __host__ __device__ constexpr size_t face_planes(int fb) {
   return (size_t)((D == 3) ? 2 : 1) * fb * K * Shape<D, K>::L * sizeof(V);
 }
-template <typename V>
+// (without compact outputs only up to k = 4: with the expansion's registers the staging spills, 128^2 disc at
+// k = 5 8.2 / 7.4 us, and in the model system, where the face kernel shares the SMs with the cell kernel, it was
+// slower than the plain gather at every size, 28^3 ball at k = 6 31.9 / 29.6 us, 24^3 at k = 8 45.5 / 43.7)
+template <typename V, int K, bool COMPACT>
 struct StagePatch {
-    static constexpr bool value = std::is_same<V, float>::value;
+  static constexpr bool value = std::is_same<V, float>::value && (COMPACT || K <= 4);
 };
 template <int D, int K, typename V>
 __host__ __device__ constexpr size_t face_smem(int fb) {
-  const size_t stage = StagePatch<V>::value ? (size_t)fb * Shape<D, K>::P * sizeof(V) : 0;
+  const size_t stage = StagePatch<V, K, true>::value ? (size_t)fb * Shape<D, K>::P * sizeof(V) : 0;
   const size_t planes = face_planes<D, K, V>(fb);
   // the padded planes and sums in use with the line factors of the triangular basis (FP64) behind them
   constexpr int N = K + 1, LP = (D == 3) ? (N | 1) * N : N;
@@ -501,12 +504,12 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
 
   // ---- gather this thread's normal line (2k+1 values)
   V v[NN];
-  if (StagePatch<V>::value && axis == 0) {
+  if (StagePatch<V, K, COMPACT>::value && axis == 0) {
     // Normal x: a line is 2k+1 consecutive values, and a lane per line would touch a cache line per
     // lane in each of its 2k+1 loads (FP32's kernel is bound by L1 wavefronts).  The CTA loads the
     // patches value by value, lanes along the lines, and passes them on through shared memory (an
     // odd pitch of 2k+1: no bank conflicts).  128^3 gyroid, k = 4: face kernel 132.5 -> 127 us.
-    if constexpr (StagePatch<V>::value) {
+    if constexpr (StagePatch<V, K, COMPACT>::value) {
       V* st = reinterpret_cast<V*>(dsm);
       const int32_t* rows = fa.frows + rbase + (int64_t)(f0 - fbase) * L;
       const int items = min(fb, fend - f0) * S::P;
