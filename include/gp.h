@@ -226,8 +226,9 @@ gp_status gp_partition_slabs(const gp_mesh* mesh, const gp_levelset* ls, const g
  *
  * The face kernel runs faces_per_cta faces per CTA (faces_per_cta * (k+1)^(d-1)
  * threads, one per normal line); the lift kernel runs lift_threads threads per CTA
- * over the rows of lift_cells_per_cta owner cells.  A field 0 means the default
- * (about 256 threads, one row per thread).  Limits: at most 512 threads per CTA,
+ * over the rows of lift_cells_per_cta owner cells.  A field 0 means the default,
+ * which depends on the number of ghost faces (in a batch: of the faces of all the vectors
+ * that share a launch).  Limits: at most 512 threads per CTA,
  * lift_threads a multiple of 32, and at most 46 KB of dynamic shared memory per CTA
  * (GP_EINVAL otherwise).  The shape changes the speed, never the result: every
  * DoF is summed in the same fixed order. */
@@ -242,21 +243,32 @@ gp_status gp_get_tiles(const gp_ctx* ctx, gp_tiles* out);
 /* Sets the context's shape (checked against the limits above). */
 gp_status gp_set_tiles(gp_ctx* ctx, const gp_tiles* tiles);
 
-/* Times every candidate shape of the face kernel (about 64 to 512 threads per
- * CTA) and of the lift kernel (64 to 512 threads, one or two rows per thread)
+/* Times the default and every candidate shape of the face kernel (about 64 to 512 threads per
+ * CTA) and of the lift kernel (64 to 512 threads, half a row to four rows per thread, 4 to 64 owner cells)
  * on this context's own tables: reps launches each, L2 flushed before every
  * timed launch, CUDA events on a private stream.  Keeps the fastest face shape
- * and the fastest lift shape in the context and records them in a
- * process-wide table keyed by (device, d, k, precision), which gp_setup reads
+ * and the fastest lift shape in the context, or the default where the whole apply is not faster with
+ * them (flushed and back to back), and records the choice in a
+ * process-wide table keyed by (device, d, k, precision) and the context's kind (gp_kernel_form: form[0] and
+ * form[2]), which gp_setup reads
  * for every new context.  best (may be NULL) receives the shape, ms (may be
  * NULL, 2 doubles) the mean face and lift kernel times in milliseconds.
  * Allocates and frees two vectors and a 256 MB flush buffer; synchronises. */
 gp_status gp_autotune(gp_ctx* ctx, int reps, gp_tiles* best, double* ms);
 
-/* The process-wide table: record a shape (e.g. one read back from a cache
- * file) or look one up (GP_EINVAL if absent). */
+/* The process-wide table: record a shape for contexts of every kind, or look up the shape recorded last
+ * (GP_EINVAL if absent).  gp_tiles_keep records the context's own shape (e.g. one read back from a
+ * cache file and set with gp_set_tiles) for contexts of its kind, as gp_autotune does. */
 gp_status gp_tiles_record(int device, int dim, int degree, int precision, const gp_tiles* tiles);
 gp_status gp_tiles_lookup(int device, int dim, int degree, int precision, gp_tiles* out);
+gp_status gp_tiles_keep(gp_ctx* ctx);
+
+/* The kernels behind gp_apply of this context, 4 int32: form[0] 1 if the face kernel stores compact outputs
+ * (FP32), form[1] 1 if it runs the triangular normal basis (FP64), form[2] the size class of the
+ * default tile shape (0..3), form[3] the version of the kernels that tuned shapes are for (a shape stored by
+ * another version is better tuned again).  Contexts with equal (d, k, precision), form[0] and form[2]
+ * are of one kind. */
+gp_status gp_kernel_form(const gp_ctx* ctx, int32_t* form);
 
 /* The FP64 1D reference matrices of this context (Sec. 2.4, M^1 and G^1_k):
  *   mass  (k+1)^2 doubles, M^[a][b] = integral_0^1 phi_a phi_b;

@@ -382,6 +382,9 @@ gp_status gp_setup(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* op
       }
     }
   }
+  // face outputs W_F of the face + lift path: float, double, or a (hi, lo) float pair per value
+  const size_t tp_bytes = (size_t)c->plan.num_faces() * c->plan.L * (2 * c->plan.k + 1) * (c->plan.precision == GP_FP32 ? 4 : 8);
+  c->form = gp::launch_form(c->plan.precision == GP_FP32, c->plan.dim, c->plan.k, (int64_t)tp_bytes, c->plan.num_faces());
   if (opts->device >= 0) {
     int ndev = 0;
     if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev == 0) {
@@ -400,10 +403,6 @@ gp_status gp_setup(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* op
     if (e == cudaSuccess) e = upload(&c->d_frows, p.frows);
     if (e == cudaSuccess) e = upload(&c->d_lwin, p.lwin);
     if (e == cudaSuccess) e = upload(&c->d_lrow, p.lrow);
-    const size_t vbytes = p.precision == GP_FP32 ? 4 : 8;
-    // face outputs W_F of the face + lift path: float, double, or a (hi, lo) float pair per value
-    const size_t tp_bytes = (size_t)p.num_faces() * p.L * (2 * p.k + 1) * vbytes;
-    c->form = gp::launch_form(p.precision == GP_FP32, p.dim, p.k, (int64_t)tp_bytes, p.num_faces());
     if (e == cudaSuccess && c->form.compact) e = upload(&c->d_lmask, p.lmask);
     if (e == cudaSuccess) e = upload(&c->d_zruns, zruns);
     if (c->use_brick) {
@@ -426,8 +425,7 @@ gp_status gp_setup(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* op
       return fail(nullptr, e == cudaErrorMemoryAllocation ? GP_ENOMEM : GP_ECUDA, m);
     }
     c->on_device = true;
-    if (c->use_brick) gpi::brick_tiles_lookup(c->device, c->plan.dim, c->plan.k, c->plan.precision, &c->tiles);
-    else gpi::tiles_lookup(c->device, c->plan.dim, c->plan.k, c->plan.precision, &c->tiles);
+    gpi::tiles_start(c);
   }
   *out = c;
   return GP_OK;

@@ -122,11 +122,7 @@ gp_status ensure_face_outputs(gp_ctx* c);
 // Tile-shape helpers for the context's (dimension, arithmetic).
 gp::TileOps tile_ops(int dim, int precision);
 
-// Process-wide table of tuned tile shapes, keyed by (device, dimension, degree, precision);
-// gp_setup starts every context from the entry of its key, if there is one.
-bool tiles_lookup(int device, int dim, int k, int precision, gp::Tiles* out);
-void tiles_record(int device, int dim, int k, int precision, const gp::Tiles& t);
-// The same for brick-path contexts (faces per chunk), filled by gp_autotune.
-bool brick_tiles_lookup(int device, int dim, int k, int precision, gp::Tiles* out);
+// Starts a new context from the process-wide table of tuned tile shapes, if that has a shape for its kind.
+void tiles_start(gp_ctx* c);
 
 }  // namespace gpi

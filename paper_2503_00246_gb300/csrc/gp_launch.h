@@ -128,11 +128,20 @@ constexpr TileRules kTilesF32Compact = {
 constexpr int kSystemFaces[3][8] = {{64, 17, 8, 5, 3, 3, 2, 1}, {64, 21, 16, 20, 7, 5, 4, 3}, {64, 21, 16, 5, 7, 5, 4, 3}};
 
 template <int D, int K, typename V>
+const TileRule& tile_rule(const LaunchForm& form) {
+  constexpr bool F32 = std::is_same<V, float>::value, F64 = std::is_same<V, double>::value;
+  return (F32 ? (form.compact ? kTilesF32Compact : kTilesF32) : F64 ? kTilesF64 : kTilesFF)[D - 2][K - 1];
+}
+inline int tile_class(const TileRule& r, const LaunchForm& form) {
+  int c = 0;
+  while (c < 3 && form.faces > r.upto[c]) ++c;
+  return c;
+}
+template <int D, int K, typename V>
 Tiles default_tiles_t(const LaunchForm& form) {
   constexpr bool F32 = std::is_same<V, float>::value, F64 = std::is_same<V, double>::value;
-  const TileRules& all = F32 ? (form.compact ? kTilesF32Compact : kTilesF32) : F64 ? kTilesF64 : kTilesFF;
-  const TileRule& r = all[D - 2][K - 1];
-  Tiles t = r.shape[form.faces <= r.upto[0] ? 0 : form.faces <= r.upto[1] ? 1 : form.faces <= r.upto[2] ? 2 : 3];
+  const TileRule& r = tile_rule<D, K, V>(form);
+  Tiles t = r.shape[tile_class(r, form)];
   if (form.system) t.fb = D == 3 ? (F32 ? kSystemFaces[0] : F64 ? kSystemFaces[1] : kSystemFaces[2])[K - 1] : Shape<D, K>::FB;
   return t;
 }
@@ -155,6 +164,7 @@ bool resolve_tiles(Tiles& t, const LaunchForm& form) {
 // Per (arithmetic, dimension): default tiles and range check for degree k.
 struct TileOps {
   Tiles (*defaults)(int k, const LaunchForm& form);
+  int (*size_class)(int k, const LaunchForm& form);   // which of the rule's shapes is the default
   bool (*resolve)(int k, Tiles& t, const LaunchForm& form);
 };
 TileOps tile_ops_f64_d2();
@@ -166,8 +176,17 @@ TileOps tile_ops_ff_d3();
 
 #define GP_TILE_CASE(D, A, K) \
   case K: return resolve_tiles<D, K, typename A::V>(t, form);
+#define GP_CLASS_CASE(D, A, K) \
+  case K: return tile_class(tile_rule<D, K, typename A::V>(form), form);
 #define GP_TILE_OPS(D, A)                                                                     \
   TileOps ops;                                                                                \
+  ops.size_class = [](int k, const LaunchForm& form) -> int {                                 \
+    switch (k) {                                                                              \
+      GP_CLASS_CASE(D, A, 1) GP_CLASS_CASE(D, A, 2) GP_CLASS_CASE(D, A, 3) GP_CLASS_CASE(D, A, 4) \
+      GP_CLASS_CASE(D, A, 5) GP_CLASS_CASE(D, A, 6) GP_CLASS_CASE(D, A, 7) GP_CLASS_CASE(D, A, 8) \
+      default: return 0;                                                                      \
+    }                                                                                         \
+  };                                                                                          \
   ops.defaults = [](int k, const LaunchForm& form) -> Tiles {                                 \
     switch (k) {                                                                              \
       case 1: return default_tiles_t<D, 1, typename A::V>(form);                              \

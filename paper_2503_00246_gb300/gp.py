@@ -95,6 +95,8 @@ def _load():
         "gp_set_tiles": ([P, C.POINTER(gp_tiles)], C.c_int),
         "gp_autotune": ([P, C.c_int, C.POINTER(gp_tiles), C.POINTER(C.c_double)], C.c_int),
         "gp_tiles_record": ([C.c_int, C.c_int, C.c_int, C.c_int, C.POINTER(gp_tiles)], C.c_int),
+        "gp_tiles_keep": ([P], C.c_int),
+        "gp_kernel_form": ([P, C.POINTER(C.c_int32)], C.c_int),
         "gp_tiles_lookup": ([C.c_int, C.c_int, C.c_int, C.c_int, C.POINTER(gp_tiles)], C.c_int),
         "gp_partition_info": ([P, C.POINTER(gp_partition)], C.c_int),
         "gp_partition_slabs": ([C.POINTER(gp_mesh), C.POINTER(gp_levelset), C.POINTER(gp_opts), C.c_int,
@@ -139,8 +141,8 @@ ABI_SYMBOLS = ("gp_setup", "gp_destroy", "gp_num_active_dofs", "gp_num_ghost_fac
                "gp_version", "gp_apply_noalloc", "gp_batch_create", "gp_batch_apply", "gp_batch_info",
                "gp_batch_destroy", "gp_system_create", "gp_system_apply", "gp_system_solve",
                "gp_system_destroy", "gp_partition_info", "gp_partition_slabs", "gp_get_tiles",
-               "gp_set_tiles", "gp_autotune", "gp_tiles_record", "gp_tiles_lookup", "gp_system_cells",
-               "gp_apply_batched_info", "gp_kernel_path", "gp_apply_host_bytes")
+               "gp_set_tiles", "gp_autotune", "gp_tiles_record", "gp_tiles_lookup", "gp_tiles_keep", "gp_system_cells",
+               "gp_apply_batched_info", "gp_kernel_path", "gp_kernel_form", "gp_apply_host_bytes")
 NOALLOC_SCRATCH_BYTES = 32 << 20
 
 
@@ -467,6 +469,11 @@ def gp_tiles_lookup(device: int, dim: int, degree: int, precision: int):
     return _tiles_dict(t)
 
 
+def gp_tiles_keep(ctx: Context):
+    """Records the context's tile shape for new contexts of its kind."""
+    _check(lib.gp_tiles_keep(ctx.handle), ctx)
+
+
 def tiles_cache_path() -> str:
     """The autotuner's cache file: $GP_TILES_CACHE, else ~/.cache/gp_gb300/tiles.json."""
     return os.environ.get("GP_TILES_CACHE") or os.path.join(os.path.expanduser("~"), ".cache", "gp_gb300",
@@ -474,14 +481,17 @@ def tiles_cache_path() -> str:
 
 
 def autotune_cached(ctx: Context, reps: int = 10, path: str | None = None) -> dict:
-    """Tile shapes for ctx from the cache file, keyed by (GPU name, d, k, precision, path); on a miss
+    """Tile shapes for ctx from the cache file, keyed by (GPU name, d, k, precision, path), the context's kind
+    and the version of the kernels; on a miss
     gp_autotune times the candidates and the result is written back.  Either way the shape is
-    set on ctx and recorded in the library's table for new contexts."""
+    set on ctx and recorded in the library's table for new contexts of its kind."""
     import json
     import torch
     path = path or tiles_cache_path()
     kpath = gp_kernel_path(ctx)["path"]
-    key = f"{torch.cuda.get_device_name(ctx.device)}|d{ctx.dim}|k{ctx.degree}|p{ctx.precision}|path{kpath}"
+    form = gp_kernel_form(ctx)
+    key = (f"{torch.cuda.get_device_name(ctx.device)}|d{ctx.dim}|k{ctx.degree}|p{ctx.precision}|path{kpath}"
+           f"|c{int(form['compact'])}|s{form['size_class']}|v{form['version']}")
     cache = {}
     if os.path.exists(path):
         with open(path) as fh:
@@ -490,7 +500,7 @@ def autotune_cached(ctx: Context, reps: int = 10, path: str | None = None) -> di
         tiles = cache[key]
         gp_set_tiles(ctx, tiles)
         if kpath == GP_PATH_FACE_LIFT:
-            gp_tiles_record(ctx.device, ctx.dim, ctx.degree, ctx.precision, tiles)
+            gp_tiles_keep(ctx)
         return tiles
     tiles, _ = gp_autotune(ctx, reps)
     cache[key] = tiles
@@ -515,6 +525,14 @@ def gp_partition_slabs(mesh: gp_mesh, levelset: gp_levelset, opts: gp_opts, npar
     _check(lib.gp_partition_slabs(C.byref(mesh), C.byref(levelset), C.byref(opts), int(nparts),
                                   b.ctypes.data_as(C.POINTER(C.c_int32))))
     return b
+
+
+def gp_kernel_form(ctx: Context) -> dict:
+    """{"compact": FP32 stores compact face outputs, "triangular": FP64 runs the triangular normal basis,
+    "size_class": of the default tile shape, "version": of the kernels that tuned shapes are for}."""
+    f = (C.c_int32 * 4)()
+    _check(lib.gp_kernel_form(ctx.handle, f), ctx)
+    return {"compact": bool(f[0]), "triangular": bool(f[1]), "size_class": f[2], "version": f[3]}
 
 
 def gp_kernel_path(ctx: Context) -> dict:

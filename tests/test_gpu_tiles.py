@@ -117,3 +117,27 @@ def test_autotune_cache_file(gplib, cuda, tmp_path):
     ctx2 = gplib.setup_problem(pr, precision=1, path=gplib.GP_PATH_FACE_LIFT)
     assert gplib.autotune_cached(ctx2, path=path) == {"faces_per_cta": 5, "lift_cells_per_cta": 7, "lift_threads": 96}
     assert gplib.gp_get_tiles(ctx2) == {"faces_per_cta": 5, "lift_cells_per_cta": 7, "lift_threads": 96}
+
+
+def test_tuned_shapes_stay_with_their_kind(gplib, cuda):
+    """A shape tuned on a large FP32 mesh (compact face outputs) is not put on a small one, which runs another
+    lift kernel, nor on a mesh of another size class; a shape recorded by hand is for every mesh."""
+    def ctx(n, k, prec):
+        return gplib.setup_problem(W.small_ball(3, n, k, seed=5), precision=prec, path=gplib.GP_PATH_FACE_LIFT)
+    odd = {"faces_per_cta": 4, "lift_cells_per_cta": 7, "lift_threads": 96}
+    for prec, k, large, small in ((1, 4, 60, 8), (0, 2, 50, 8)):
+        a, b = ctx(large, k, prec), ctx(small, k, prec)
+        fa, fb = gplib.gp_kernel_form(a), gplib.gp_kernel_form(b)
+        assert (fa["compact"], fa["size_class"]) != (fb["compact"], fb["size_class"])
+        da, db = gplib.gp_get_tiles(a), gplib.gp_get_tiles(b)
+        try:
+            gplib.gp_set_tiles(a, odd)
+            gplib.gp_tiles_keep(a)
+            assert gplib.gp_tiles_lookup(0, 3, k, prec) == odd
+            assert gplib.gp_get_tiles(ctx(large, k, prec)) == odd
+            assert gplib.gp_get_tiles(ctx(small, k, prec)) == db
+            gplib.gp_tiles_record(0, 3, k, prec, odd)
+            assert gplib.gp_get_tiles(ctx(small, k, prec)) == odd
+        finally:
+            gplib.gp_tiles_record(0, 3, k, prec, {})
+        assert gplib.gp_get_tiles(ctx(large, k, prec)) == da
