@@ -192,13 +192,13 @@ _PIVOTS = {1: (1,), 2: (2, 1), 3: (2, 2, 1), 4: (3, 2, 2, 3), 5: (3, 3, 1, 4, 5)
            7: (5, 4, 2, 6, 7, 2, 4), 8: (5, 4, 2, 7, 8, 1, 6, 6)}
 
 
-def _flops_executed(d, k, nf, prec="fp64"):
-    """Flops the face kernel executes, counted as in _flops_face: the even / odd split, the jump values
-    and the expansion of a normal line (FP64: triangular basis, unit and zero entries free; FP32
-    stores compact outputs and does not expand), the lumped masses with their rank-one term
-    line by line, and the scaling."""
+def _flops_executed(d, k, nf, prec, form):
+    """Flops the face kernel (or the brick kernel) executes, counted as in _flops_face: the even / odd split, the
+    jump values and the expansion of a normal line (form, from gp_kernel_form: the triangular basis, whose unit and
+    zero entries are free, or the jump vectors; compact outputs are not expanded), the lumped masses with
+    their rank-one term line by line, and the scaling."""
     N, L = k + 1, (k + 1) ** (d - 1)
-    if prec == "fp64":
+    if form["triangular"]:
         piv = _PIVOTS[k]
         jumps = expand = 0
         for par in (0, 1):
@@ -216,7 +216,7 @@ def _flops_executed(d, k, nf, prec="fp64"):
     else:
         n_odd, n_even = (k + 1) // 2, k // 2
         normal = 2 * k + n_odd * (2 * (k + 1) - 1) + n_even * (2 * k - 1)
-        if prec != "fp32":
+        if not form["compact"]:
             normal += (k + 1) * (2 * n_odd - 1)
             if k > 1:
                 normal += k * ((2 * n_even - 1) + 2)
@@ -367,7 +367,7 @@ def run_sweep(args):
             tf = ms_face / calls * 1e-3
             nf = ctx.n_faces
             w = 4 if prec == gp.GP_FP32 else 8
-            fl_exec = _flops_executed(pr.dim, k, nf, tags[prec].replace("ff64", "ff"))
+            fl_exec = _flops_executed(pr.dim, k, nf, tags[prec].replace("ff64", "ff"), gp.gp_kernel_form(ctx))
             fl_paper = _flops_paper(pr.dim, k, nf)
             r = {"gdofs": ctx.n_active / t / 1e9, "ms": t * 1e3, "face_ms": tf * 1e3, "lift_ms": ms_lift / calls,
                  "gfaces_per_s": nf / t / 1e9,
@@ -569,6 +569,7 @@ def measure_form(gp, W, torch, pr, prec, dev, args, flush, o=None, e2e=True, tun
     gp.gp_profile_enable(ctx, False)
     err = _sampled_error(o, x_np, y, prec, args.check_rows) if (o is not None and args.check) else None
     rec = {"ctx_sizes": (ctx.n_active, ctx.n_faces, ctx.n_touched), "t_step": t_step, "kernel_path": kp,
+           "kernel_form": gp.gp_kernel_form(ctx),
            "wall_ms_per_step": wall * 1e3 / steps, "face_ms": ms_face / calls, "lift_ms": ms_lift / calls,
            "tiles": tiles, "rel_err_vs_oracle": err}
     if e2e:
@@ -606,9 +607,10 @@ def form_summary(rec, pr, prec, gp, hbm, peak_src, ws=1):
     peak = {gp.GP_FP64: fp64_peak, gp.GP_FP32: fp32_peak, gp.GP_FP64_FF: fp32_peak / FF_OPS_PER_FMA}[prec]
     kname = {gp.GP_FP64: "double", gp.GP_FP32: "float", gp.GP_FP64_FF: "ff64"}[prec]
     form = {gp.GP_FP64: "fp64", gp.GP_FP32: "fp32", gp.GP_FP64_FF: "ff"}[prec]
-    flop_face = _flops_executed(d, k, nf, form)
+    flop_face = _flops_executed(d, k, nf, form, rec["kernel_form"])
     brick = rec["kernel_path"]["path"] == gp.GP_PATH_BRICK
-    kernels = ("brick_kernel", "plane_fixup_kernel") if brick else ("face_kernel", "lift_kernel")
+    lift = "lift_lines_kernel" if rec["kernel_form"]["compact"] else "lift_kernel"
+    kernels = ("brick_kernel", "plane_fixup_kernel") if brick else ("face_kernel", lift)
     roof = {"bound": "alu", "kernel": f"{kernels[0]}<{d},{k},{kname}>",
             "achieved": flop_face / (rec["face_ms"] * 1e-3) / 1e12 if rec["face_ms"] > 0 else None,
             "unit": "TFLOP/s", "peak": peak,

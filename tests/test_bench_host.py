@@ -32,6 +32,27 @@ def test_executed_flop_count_below_paper_count():
         assert bench._flops_face(3, k, 1) < bench._flops_face(3, k, 1, per_output=True)
 
 
+def test_executed_flops_follow_the_kernel_form():
+    wf, compact = {"compact": False, "triangular": False}, {"compact": True, "triangular": False}
+    triangular = {"compact": False, "triangular": True}
+    # d = 2, k = 1, FP32: per line 2 adds, a 2-term dot product (3), the expansion of 2 nodes (1 flop each), the
+    # scaling (1), the product with mw (1); per face one tangential line: a 2-term dot product and 2 multiply-adds
+    assert bench._flops_executed(2, 1, 1, "fp32", wf) == 2 * (2 + 3 + 2 + 1) + 3 + 4 + 2
+    assert bench._flops_executed(2, 1, 1, "fp32", compact) == bench._flops_executed(2, 1, 1, "fp32", wf) - 2 * 2
+    for d in (2, 3):
+        for k in range(1, 9):
+            L = (k + 1) ** (d - 1)
+            n_odd, n_even = (k + 1) // 2, k // 2
+            expand = (k + 1) * (2 * n_odd - 1) + (k * (2 * n_even + 1) if k > 1 else 0)
+            full = bench._flops_executed(d, k, 1, "fp32", wf)
+            assert full - bench._flops_executed(d, k, 1, "fp32", compact) == L * expand
+            # no scaling in FP64, fewer flops with the triangular basis
+            general = bench._flops_executed(d, k, 1, "fp64", wf)
+            assert general == bench._flops_executed(d, k, 1, "ff", wf)
+            assert bench._flops_executed(d, k, 1, "fp64", triangular) < general
+            assert bench._flops_executed(d, k, 3, "fp64", triangular) == 3 * bench._flops_executed(d, k, 1, "fp64", triangular)
+
+
 def test_traffic_lookup_follows_the_committed_counters(tmp_path, monkeypatch):
     """bench.py reads DRAM traffic per launch from profiles/traffic.json, and only while the
     kernel sources hash to the value recorded beside the counters."""
