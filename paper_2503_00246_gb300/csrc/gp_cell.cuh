@@ -121,8 +121,6 @@ struct CellTabs {
   const int32_t* own2lift = nullptr;
 };
 
-constexpr int GATHER_THREADS = 512;   // most threads of a gather CTA (gather_threads)
-
 // the two fields of a pass kept side by side in shared memory, so that one access
 // moves both (half the shared-memory instructions)
 template <typename V>
@@ -415,6 +413,8 @@ __global__ void __launch_bounds__(gather_threads(D, K))
 cell_gather(const typename A::V* __restrict__ wc, typename A::IO* __restrict__ y, const int add, const CellTabs ct) {
   using S = CellShape<D, K>;
   constexpr int KR = S::KR;
+  static_assert(gather_owners_per_cta(D, K) * KR <= gather_threads(D, K) && gather_threads(D, K) % 32 == 0,
+                "every row of the CTA's owners needs a thread");
   int o = 0, q = 0, r = 0;
   const bool slot = gather_slot<D, K>((int)threadIdx.x, o, q, r);
   const int own = (int)blockIdx.x * gather_owners_per_cta(D, K) + o;

@@ -25,7 +25,9 @@ int check() {
   constexpr int KR = CellShape<D, K>::KR;
   std::set<std::tuple<int, int, int>> seen;
   int bad = 0, last_type = -1;
-  for (int u = 0; u < GATHER_THREADS; ++u) {
+  constexpr int NT = gather_threads(D, K);
+  if (OPC * KR > NT || NT % 32 != 0 || NT > 1024) ++bad;
+  for (int u = 0; u < NT; ++u) {
     int o = -1, q = -1, r = -1;
     const bool live = gather_slot<D, K>(u, o, q, r);
     if (u >= OPC * KR) { bad += live; continue; }
