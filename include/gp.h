@@ -324,14 +324,16 @@ gp_status gp_kernel_path(const gp_ctx* ctx, int* path, int32_t* bdim, int64_t* c
  * pin_memory) is read by a gather kernel on the DoFs some face patch touches only (the only
  * entries the face kernel reads); other host memory is copied whole.  y is computed in a device
  * buffer owned by the context; a page-locked y comes back in chunks on a second stream while the
- * apply runs as a pipeline of up to 16 slabs (more for a larger y; each chunk as soon as the slabs that write it are
- * done; x is then gathered slab by slab on a third stream, each slab's face launch waiting for
- * its part), any other y in one copy at the end.  The device buffers, streams and events belong
+ * apply runs as a pipeline of slabs (1 for a y below 9 MB, up to 16 for larger ones; each chunk as soon as the
+ * slabs that write it are done; x is then gathered slab by slab on a third stream, each slab's face launch
+ * waiting for its part), any other y in one copy at the end.  The device buffers, streams and events belong
  * to ctx: calls on one context must not overlap. */
 gp_status gp_apply_host(gp_ctx* ctx, const void* x_host, void* y_host, void* stream);
 
 /* Bytes the last gp_apply_host of ctx moved from host to device and from device to host. */
 gp_status gp_apply_host_bytes(const gp_ctx* ctx, int64_t* h2d, int64_t* d2h);
+/* Slabs the last gp_apply_host of ctx ran as (1: one face and one lift launch; 0: nothing to do). */
+gp_status gp_apply_host_slabs(const gp_ctx* ctx, int32_t* slabs);
 
 /* Several independent problems, nrhs right-hand sides each (the batched workload
  * of many meshes of uneven n, k and geometry): x[p] and y[p] point to nrhs

@@ -619,6 +619,7 @@ gp_status gp_apply_host(gp_ctx* ctx, const void* x_host, void* y_host, void* str
   if (!ctx->on_device) return fail(ctx, GP_EDEVICE, "context was built host-only (device = -1)");
   const int64_t n = ctx->plan.n_active;
   ctx->host_bytes[0] = ctx->host_bytes[1] = 0;
+  ctx->host_slabs = n > 0 ? 1 : 0;
   if (n == 0) return GP_OK;
   if (!x_host || !y_host) return fail(ctx, GP_EINVAL, "null x or y");
   DeviceGuard g(ctx->device);
@@ -644,6 +645,7 @@ gp_status gp_apply_host(gp_ctx* ctx, const void* x_host, void* y_host, void* str
     GP_CUDA(ctx, gpi::ensure_host_pipeline(ctx));
     const int ns = (int)(ctx->hslabs.size() / gp::SLAB);
     if (ns > 1) {
+      ctx->host_slabs = ns;
       gpi::SlabRun run;
       run.table = ctx->hslabs.data();
       run.n = ns;
@@ -686,6 +688,12 @@ gp_status gp_apply_host_bytes(const gp_ctx* ctx, int64_t* h2d, int64_t* d2h) {
   if (!ctx || !h2d || !d2h) return fail(ctx, GP_EINVAL, "null argument");
   *h2d = ctx->host_bytes[0];
   *d2h = ctx->host_bytes[1];
+  return GP_OK;
+}
+
+gp_status gp_apply_host_slabs(const gp_ctx* ctx, int32_t* slabs) {
+  if (!ctx || !slabs) return fail(ctx, GP_EINVAL, "null argument");
+  *slabs = ctx->host_slabs;
   return GP_OK;
 }
 

@@ -38,6 +38,7 @@ struct gp_ctx {
   void* d_yh = nullptr;
   int2* d_truns = nullptr;       // gp_apply_host: runs (c0, len) of the touched DoFs
   int32_t ntruns = -1;           // -1: not built yet
+  int host_slabs = 0;              // slabs of the last gp_apply_host
   int64_t host_bytes[2] = {0, 0};  // bytes the last gp_apply_host moved host -> device, device -> host
   // gp_apply_host with a page-locked y: a slab pipeline whose finished parts of y go back on a
   // second stream while later slabs compute (built on first use)

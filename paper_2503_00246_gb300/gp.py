@@ -109,6 +109,7 @@ def _load():
         "gp_apply_host_bytes": ([P, i64p, i64p], C.c_int),
         "gp_apply_batched": ([C.POINTER(P), C.c_int, C.c_int, C.POINTER(P), C.POINTER(P), P], C.c_int),
         "gp_apply_batched_info": ([C.POINTER(P), C.c_int, C.c_int, i64p], C.c_int),
+        "gp_apply_host_slabs": ([P, C.POINTER(C.c_int32)], C.c_int),
         "gp_kernel_path": ([P, C.POINTER(C.c_int), C.POINTER(C.c_int32), i64p], C.c_int),
         "gp_batch_create": ([C.POINTER(P), C.c_int, C.c_int, C.POINTER(P)], C.c_int),
         "gp_batch_apply": ([P, C.POINTER(P), C.POINTER(P), P], C.c_int),
@@ -142,7 +143,8 @@ ABI_SYMBOLS = ("gp_setup", "gp_destroy", "gp_num_active_dofs", "gp_num_ghost_fac
                "gp_batch_destroy", "gp_system_create", "gp_system_apply", "gp_system_solve",
                "gp_system_destroy", "gp_partition_info", "gp_partition_slabs", "gp_get_tiles",
                "gp_set_tiles", "gp_autotune", "gp_tiles_record", "gp_tiles_lookup", "gp_tiles_keep", "gp_system_cells",
-               "gp_apply_batched_info", "gp_kernel_path", "gp_kernel_form", "gp_apply_host_bytes")
+               "gp_apply_batched_info", "gp_kernel_path", "gp_kernel_form", "gp_apply_host_bytes",
+               "gp_apply_host_slabs")
 NOALLOC_SCRATCH_BYTES = 32 << 20
 
 
@@ -263,6 +265,13 @@ def gp_apply_host_bytes(ctx: Context):
     a, b = C.c_int64(), C.c_int64()
     _check(lib.gp_apply_host_bytes(ctx.handle, C.byref(a), C.byref(b)), ctx)
     return a.value, b.value
+
+
+def gp_apply_host_slabs(ctx: Context) -> int:
+    """Slabs the last gp_apply_host of ctx ran as (1: one face and one lift launch)."""
+    n = C.c_int32()
+    _check(lib.gp_apply_host_slabs(ctx.handle, C.byref(n)), ctx)
+    return n.value
 
 
 def gp_apply_batched(ctxs, nrhs, xs, ys, stream=None):

@@ -187,12 +187,14 @@ def test_host_buffers_end_to_end(gplib, cuda):
 @pytest.mark.parametrize("prec", PRECS)
 def test_host_buffers_page_locked(gplib, cuda, prec):
     """Page-locked host buffers: the GPU gathers x on the touched DoFs only, and y comes back in
-    slab chunks while later slabs compute (the third problem has 8 slabs; y starts as NaN, so
-    every entry must come back); bitwise equal to the device apply and to the copy path of
+    slab chunks while later slabs compute (the last two problems run as at least three slabs; y starts as NaN,
+    so every entry must come back); bitwise equal to the device apply and to the copy path of
     pageable buffers, with the bytes each path moves."""
     dt = cuda.float32 if prec == 1 else cuda.float64
-    for pr in (W.small_ball(3, 12, 2, seed=9), W.small_ball(2, 30, 3, seed=10), W.small_ball(3, 24, 3, seed=12)):
+    for pr in (W.small_ball(3, 12, 2, seed=9), W.small_ball(2, 30, 3, seed=10), W.small_ball(3, 24, 3, seed=12),
+               W.small_ball(3, 96, 4, seed=13), W.small_ball(2, 1100, 4, seed=14)):
         ctx = gplib.setup_problem(pr, precision=prec)
+        pipeline = pr.n > 30
         x = W.x_vectors(pr, ctx.n_active)[0]
         y_dev = _apply(gplib, cuda, ctx, x, prec)
         xh = cuda.tensor(x, dtype=dt).pin_memory()
@@ -201,6 +203,7 @@ def test_host_buffers_page_locked(gplib, cuda, prec):
         assert np.array_equal(yh.double().numpy(), y_dev)
         w = xh.element_size()
         assert gplib.gp_apply_host_bytes(ctx) == (ctx.n_touched * w, ctx.n_active * w)
+        assert (gplib.gp_apply_host_slabs(ctx) >= 3) == pipeline
         yh.fill_(float("nan"))
         gplib.gp_apply_host(ctx, xh, yh)                   # again: the pipeline's second use
         assert np.array_equal(yh.double().numpy(), y_dev)
@@ -210,11 +213,13 @@ def test_host_buffers_page_locked(gplib, cuda, prec):
         # mixed: page-locked x with pageable y, and pageable x with page-locked y
         yp = cuda.full((ctx.n_active,), float("nan"), dtype=dt)
         gplib.gp_apply_host(ctx, xh, yp)
+        assert gplib.gp_apply_host_slabs(ctx) == 1
         assert np.array_equal(yp.double().numpy(), y_dev)
         assert gplib.gp_apply_host_bytes(ctx) == (ctx.n_touched * w, ctx.n_active * w)
         xp = cuda.tensor(x, dtype=dt)                     # pageable
         yh.fill_(float("nan"))
         gplib.gp_apply_host(ctx, xp, yh)
+        assert (gplib.gp_apply_host_slabs(ctx) >= 3) == pipeline
         assert np.array_equal(yh.double().numpy(), y_dev)
         assert gplib.gp_apply_host_bytes(ctx) == (ctx.n_active * w, ctx.n_active * w)
     # no ghost faces: nothing to gather, y is all zeros
