@@ -221,7 +221,7 @@ __device__ __forceinline__ void line_jumps(const V (&v)[2 * K + 1], const V (*g)
 // non-negative, so x^T G x stays a sum of squares.  The pivot orders are those whose elimination
 // grows least (entries below 1.2 for the default and for the factorial weights).  Native FP64 only,
 // whose kernel is bound by the FP64 pipe: apply of the 128^3 gyroid at k = 4 1450 -> 1263 us, of the
-// 64^3 ball at k = 3 68.9 -> 62.1 us.  Weights below 0 run the jump vectors themselves.
+// 64^3 ball at k = 3 68.9 -> 63.5 us.  Weights below 0 run the jump vectors themselves.
 template <int K>
 struct Pivots {
   // pivot node of row j in hexadecimal digit j
@@ -314,15 +314,15 @@ struct TanShape {
 
 // The factors a line's thread needs at its own tangential index (lane-dependent, so not in the
 // constant bank): mw of the line (the product of both directions) and mc.
-template <int D, int K, typename V>
+template <int D, int K, typename V, bool W = true>
 struct TanTable {
-  V w[Shape<D, K>::L];
+  V w[W ? Shape<D, K>::L : 1];
   V c[K + 1];
 };
-template <int D, int K, typename V>
-__device__ __forceinline__ void fill_tan_table(TanTable<D, K, V>& tab, const Consts<V, K>& c, const int t) {
+template <int D, int K, typename V, bool W>
+__device__ __forceinline__ void fill_tan_table(TanTable<D, K, V, W>& tab, const Consts<V, K>& c, const int t) {
   constexpr int N = K + 1;
-  if (t < Shape<D, K>::L) tab.w[t] = (D == 3) ? vmul(c.mw[t % N], c.mw[t / N]) : c.mw[t];
+  if (W && t < Shape<D, K>::L) tab.w[t] = (D == 3) ? vmul(c.mw[t % N], c.mw[t / N]) : c.mw[t];
   if (t < N) tab.c[t] = c.mc[t];
 }
 
@@ -423,8 +423,10 @@ __device__ __forceinline__ void line_expand(const Consts<V, K>& c, const V (&sj)
 // k = 4 and one vector access per line instead of 2k + 1.
 template <int K, typename V>
 struct Compact {
+  static_assert(sizeof(V) == 4, "FP32 only (StoreCompact)");
   static constexpr int KP = (K == 3) ? 4 : (K == 5) ? 6 : (K == 7) ? 8 : K;
-  static constexpr int VW = (sizeof(V) == 4 && KP % 4 == 0) ? 4 : (KP % 2 == 0) ? 2 : 1;   // values per access
+  static constexpr int VW = KP % 4 == 0 ? 4 : 2;   // values per access
+  static_assert(KP % VW == 0, "whole accesses");
   static_assert(KP <= 2 * K + 1, "compact outputs must fit the face-output buffer");
 };
 template <int VW, typename V>
@@ -433,12 +435,14 @@ struct alignas(VW * sizeof(V)) Chunk {
 };
 // FP32 stores T_F where W_F would not stay in L2 (store_compact): both of its kernels were bound by L1
 // wavefronts (68% and 65% of their peak) and moved 1.11 GB per apply of the 128^3 gyroid at k = 4, 0.79 GB
-// so: apply 306 -> 256 us (face kernel 187 -> 158 us, lift 117 -> 104 us).  FP64 stores W_F: the
+// so: apply 306 -> 261 us (face kernel 187 -> 158 us, lift 117 -> 104 us).  FP64 stores W_F: the
 // expansion and its FP64 adds cost the same operations either way, and W_F hides under the FP64 pipe;
 // so does float-float (a lift of compact outputs took 385 us there against 283 us).
-template <typename V>
+// value: some meshes of this dimension and degree store T_F; always: all do (store_compact has the sizes).
+template <int D, int K, typename V>
 struct StoreCompact {
-  static constexpr bool value = std::is_same<V, float>::value;
+  static constexpr bool value = std::is_same<V, float>::value && (D == 2 ? K >= 6 : K >= 3);
+  static constexpr bool always = value && (D == 2 || K == 5 || K >= 7);
 };
 
 // ----------------------------------------------------------------- face --
@@ -462,7 +466,7 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
   typedef V Dots[K][K1];
   Plane* buf = reinterpret_cast<Plane*>(dsm);            // [fb][K][LP]
   Dots* dots = reinterpret_cast<Dots*>(buf + fb);         // [fb][K][N], 3D only
-  __shared__ TanTable<D, K, V> tab;
+  __shared__ TanTable<D, K, V, !LDL> tab;   // LDL: the line factors are in wj
   V* wj = reinterpret_cast<V*>(dots + ((D == 3) ? fb : 0));   // LDL: [K][L] line factors D_j mw
   const int nt = (int)blockDim.x;
   // the lift may start its prologue as soon as every face CTA is running (programmatic
@@ -497,10 +501,8 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
 #pragma unroll
       for (int j = 0; j < K; ++j) wj[j * L + t] = sc[j] * w;
     }
-    if (t < K1) tab.c[t] = c.mc[t];
-  } else {
-    fill_tan_table<D, K, V>(tab, c, t);
   }
+  fill_tan_table<D, K, V>(tab, c, t);
 
   // ---- gather this thread's normal line (2k+1 values)
   V v[NN];
@@ -529,7 +531,7 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
       __syncthreads();
     }
   } else if (valid) {
-    if (axis == 0) {
+    if (!StagePatch<V, K, COMPACT>::value && axis == 0) {
       const int32_t base = __ldg(fa.frows + rbase + (int64_t)(f - fbase) * L + tau);
 #pragma unroll
       for (int b = 0; b < NN; ++b) v[b] = from_io(__ldg(x + base + b), (V*)nullptr);

@@ -105,7 +105,8 @@ constexpr TileRules kTilesFF = {
      tiles_at({2, 14, 512}, 2500, {3, 32, 512}, 6000, {3, 64, 512}),
      tiles_at({2, 8, 512}, 1400, {2, 16, 512}, 2800, {2, 24, 512}, 9700, {4, 32, 256}),
      tiles_at({3, 4, 256}, 2500, {3, 32, 512}, 6000, {3, 32, 256})}};
-// FP32 that stores W_F: the degrees and sizes that store_compact leaves
+// FP32 that stores W_F, and compact outputs (a row that store_compact leaves out only serves checks of shapes
+// given by hand)
 constexpr TileRules kTilesF32 = {
     {tiles_at({192, 128, 256}), tiles_at({85, 128, 256}), tiles_at({48, 32, 128}), tiles_at({25, 64, 512}),
      tiles_at({21, 16, 128}), tiles_at({18, 32, 256}), tiles_at({12, 16, 256}), tiles_at({10, 32, 512})},
@@ -299,13 +300,13 @@ cudaError_t launch_pdl(void (*kernel)(P...), int grid, int threads, size_t smem,
 // Owner cells per lift CTA and dynamic shared memory of the lift kernel.
 template <int D, int K, typename V>
 int lift_cells(const Tiles& t, const bool compact) {
-  if constexpr (StoreCompact<V>::value)
+  if constexpr (StoreCompact<D, K, V>::value)
     if (compact) return lift_lines_cells<D, K, V>(t.lcb);
   return t.lcb;
 }
 template <int D, int K, typename V>
 size_t lift_dyn_smem(int cb, const bool compact) {
-  if constexpr (StoreCompact<V>::value)
+  if constexpr (StoreCompact<D, K, V>::value)
     if (compact) return lift_lines_smem<D, K, V>(cb);
   return lift_smem<D, K>(cb);
 }
@@ -319,16 +320,19 @@ cudaError_t launch_lift(bool pdl, const bool compact, const Tiles& t, const type
   const int cb = lift_cells<D, K, V>(t, compact);
   const int nlb = (la.nlift + cb - 1) / cb;
   const size_t smem = lift_dyn_smem<D, K, V>(cb, compact);
-  if constexpr (StoreCompact<V>::value) {
+  if constexpr (StoreCompact<D, K, V>::value) {
     if (compact) {
       if (pdl) return launch_pdl(lift_lines_kernel<D, K, A>, nlb, t.lnt, smem, st, w, y, add, la, cb, c);
       lift_lines_kernel<D, K, A><<<nlb, t.lnt, smem, st>>>(w, y, add, la, cb, c);
       return cudaGetLastError();
     }
   }
-  if (pdl) return launch_pdl(lift_kernel<D, K, A>, nlb, t.lnt, smem, st, w, y, add, la, cb);
-  lift_kernel<D, K, A><<<nlb, t.lnt, smem, st>>>(w, y, add, la, cb);
-  return cudaGetLastError();
+  if constexpr (!StoreCompact<D, K, V>::always) {
+    if (pdl) return launch_pdl(lift_kernel<D, K, A>, nlb, t.lnt, smem, st, w, y, add, la, cb);
+    lift_kernel<D, K, A><<<nlb, t.lnt, smem, st>>>(w, y, add, la, cb);
+    return cudaGetLastError();
+  }
+  return cudaErrorInvalidConfiguration;   // (launch_form gives such a context compact outputs)
 }
 
 // The face kernel of this arithmetic: with the triangular normal basis or the jump vectors, storing its
@@ -336,7 +340,7 @@ cudaError_t launch_lift(bool pdl, const bool compact, const Tiles& t, const type
 template <int D, int K, class A>
 auto pick_face(const bool ldl, const bool compact) {
   using V = typename A::V;
-  constexpr bool CO = StoreCompact<V>::value, LD = std::is_same<V, double>::value;
+  constexpr bool CO = StoreCompact<D, K, V>::value, LD = std::is_same<V, double>::value;
   static_assert(!(CO && LD), "compact outputs are expanded with the jump vectors");
   auto f = face_kernel<D, K, A, false, false>;
   if constexpr (CO) {
@@ -534,11 +538,13 @@ cudaError_t run_batch(const void* fsegs, const void* lsegs, const void* ptrs, in
     c.s[j] = vzero<V>();                                          // per segment: FaceSeg::s
     for (int b = 0; b < 2 * K + 1; ++b) c.gs[j][b] = vzero<V>();  // per segment: FaceSeg::gs
   }
-  auto face = face_kernel_batched<D, K, A, false, false>;
+  using CO = StoreCompact<D, K, V>;
+  if (CO::always && !compact) return cudaErrorInvalidConfiguration;   // (launch_form gives it compact outputs)
+  auto face = face_kernel_batched<D, K, A, CO::always, false>;
   if constexpr (UseLdl<V>::value) {
     if (ldl) face = face_kernel_batched<D, K, A, false, true>;
   }
-  if constexpr (StoreCompact<V>::value) {
+  if constexpr (CO::value) {
     if (compact) face = face_kernel_batched<D, K, A, true, false>;
   }
   if (face_blocks > 0)
@@ -547,17 +553,16 @@ cudaError_t run_batch(const void* fsegs, const void* lsegs, const void* ptrs, in
   if (lift_blocks > 0) {
     const int cb = lift_cells<D, K, V>(t, compact);
     const size_t smem = lift_dyn_smem<D, K, V>(cb, compact);
-    bool done = false;
-    if constexpr (StoreCompact<V>::value) {
-      if (compact) {
+    if constexpr (CO::value) {
+      if (compact)
         lift_lines_kernel_batched<D, K, A><<<lift_blocks, t.lnt, smem, st>>>(
             (const LiftSeg*)lsegs, (const FaceSeg<V, K>*)fsegs, nseg, (const SegPtrs<IO>*)ptrs, cb, c);
-        done = true;
-      }
     }
-    if (!done)
-      lift_kernel_batched<D, K, A><<<lift_blocks, t.lnt, smem, st>>>(
-          (const LiftSeg*)lsegs, (const FaceSeg<V, K>*)fsegs, nseg, (const SegPtrs<IO>*)ptrs, cb);
+    if constexpr (!CO::always) {
+      if (!compact)
+        lift_kernel_batched<D, K, A><<<lift_blocks, t.lnt, smem, st>>>(
+            (const LiftSeg*)lsegs, (const FaceSeg<V, K>*)fsegs, nseg, (const SegPtrs<IO>*)ptrs, cb);
+    }
   }
   return cudaGetLastError();
 }

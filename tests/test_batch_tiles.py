@@ -50,8 +50,22 @@ void check(const char* name) {
 }
 template <int D, class A, int... Ks>
 void all(const char* name, std::integer_sequence<int, Ks...>) { (check<D, Ks + 1, A>(name), ...); }
+// the instances of the compact form cover what store_compact asks for, at every size
+template <int D, int K>
+void check_form() {
+  for (int mb = 0; mb <= 1 << 16; mb = mb ? 2 * mb : 1) {
+    const bool c = store_compact(D, K, (int64_t)mb << 20);
+    if ((c && !StoreCompact<D, K, float>::value) || (!c && StoreCompact<D, K, float>::always)) {
+      std::printf("FAIL compact d=%d k=%d %d MB\n", D, K, mb);
+      ++bad;
+    }
+  }
+}
+template <int D, int... Ks>
+void all_forms(std::integer_sequence<int, Ks...>) { (check_form<D, Ks + 1>(), ...); }
 int main() {
   const auto ks = std::make_integer_sequence<int, 8>{};
+  all_forms<2>(ks); all_forms<3>(ks);
   all<2, ArF32>("f32", ks); all<3, ArF32>("f32", ks);
   all<2, ArF64>("f64", ks); all<3, ArF64>("f64", ks);
   all<2, ArFF>("ff", ks); all<3, ArFF>("ff", ks);

@@ -1,4 +1,4 @@
-"""GPU: the FP32 lift over compact face outputs at the sizes where it can go wrong: every degree,
+"""GPU: the FP32 lift over compact face outputs at the sizes where it can go wrong: every degree that has them,
 owner cells with every candidate face (a full box) and with few (a ball), lift tiles of one owner,
 of more lines than threads, and larger than the shared memory (the kernel then takes fewer owners).
 Against the oracle at the FP32 bound of the library (1e-5), and bitwise equal over the tiles."""
@@ -15,7 +15,7 @@ BALL = {3: 100, 4: 84, 5: 54, 6: 44, 7: 34, 8: 28}   # cells per direction of th
 
 
 # 3D meshes with more than 24 MB of W_F, above which FP32 stores compact outputs at every k >= 3, and
-# small ones of the degrees that always do, as 2D does
+# small ones of the degrees that always do, as 2D does from k = 6 on (and W_F below)
 @pytest.mark.parametrize("box", [False, True])
 @pytest.mark.parametrize("dim,n,k", [(2, 9, k) for k in range(1, 9)] + [(3, 28, 3), (3, 22, 4), (3, 18, 5), (3, 16, 6),
                                                                        (3, 14, 7), (3, 13, 8), (3, 5, 5), (3, 3, 7),
@@ -25,6 +25,7 @@ def test_compact_lift(gplib, cuda, dim, n, k, box):
     ctx = gplib.setup_problem(pr, precision=1)
     if dim == 3 and n > 5:
         assert ctx.n_faces * (2 * k + 1) * (k + 1) ** 2 * 4 > 24 << 20
+    assert gplib.gp_kernel_form(ctx)["compact"] == (dim == 3 or k >= 6)
     x = W.x_vectors(pr, ctx.n_active)[0].astype(np.float32)
     o = Oracle(pr)
     rows = np.arange(ctx.n_active) if dim == 2 else np.unique(np.random.default_rng(k).integers(0, ctx.n_active, 1500))
