@@ -210,7 +210,10 @@ def _stream(stream):
         import torch
         if torch.cuda.is_initialized():
             # the handle alone: current_stream() builds a Stream object, 3.0 us of a 10.2 us apply
-            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+            try:
+                return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+            except AttributeError:      # private names, which a torch release may drop
+                pass
         return torch.cuda.current_stream().cuda_stream
     return stream if isinstance(stream, int) else stream.cuda_stream
 

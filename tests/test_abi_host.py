@@ -290,3 +290,18 @@ def test_ff_setup_refuses_extreme_scale_factors(gplib):
         gplib.setup_problem(pr, precision=2, device=-1)
     assert e.value.status == gplib.GP_EINVAL and "2^90" in str(e.value)
     gplib.setup_problem(pr, precision=0, device=-1).close()    # native FP64 accepts it
+
+
+def test_current_stream_without_private_torch_functions(gplib, monkeypatch):
+    # the handle of torch's current stream, by its private functions or without them
+    import sys
+    import types
+    stream = types.SimpleNamespace(cuda_stream=1234)
+    cuda = types.SimpleNamespace(is_initialized=lambda: True, current_stream=lambda: stream)
+    raw = types.SimpleNamespace(_cuda_getCurrentRawStream=lambda dev: 5678 + dev, _cuda_getDevice=lambda: 1)
+    monkeypatch.setitem(sys.modules, "torch", types.SimpleNamespace(cuda=cuda, _C=raw))
+    assert gplib._stream(None) == 5679
+    monkeypatch.setitem(sys.modules, "torch", types.SimpleNamespace(cuda=cuda, _C=types.SimpleNamespace()))
+    assert gplib._stream(None) == 1234
+    cuda.is_initialized = lambda: False
+    assert gplib._stream(None) == 1234 and gplib._stream(stream) == 1234 and gplib._stream(7) == 7
