@@ -92,7 +92,7 @@ constexpr TileRules kTilesF64 = {
      tiles_at({19, 128, 512}, 1000, {6, 32, 256}), tiles_at({10, 24, 256}), tiles_at({4, 32, 256}),
      tiles_at({4, 16, 256}), tiles_at({3, 32, 512})},
     {tiles_at({128, 256, 512}), tiles_at({14, 128, 512}, 2500, {10, 64, 512}, 24000, {21, 32, 256}),
-     tiles_at({2, 16, 256}, 6000, {8, 32, 512}), tiles_at({6, 32, 512}, 19000, {20, 32, 512}),
+     tiles_at({2, 16, 256}, 6000, {8, 16, 256}, 70000, {24, 32, 512}), tiles_at({6, 32, 512}, 19000, {20, 32, 512}),
      tiles_at({4, 8, 256}, 6000, {7, 16, 512}), tiles_at({3, 3, 256}, 3000, {5, 14, 512}), tiles_at({2, 8, 512}),
      tiles_at({3, 4, 256})}};
 constexpr TileRules kTilesFF = {
