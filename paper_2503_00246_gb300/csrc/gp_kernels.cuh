@@ -953,9 +953,15 @@ __device__ __forceinline__ void lift_line(const V* __restrict__ line, const int*
   auto expand = [&](const int sa) {
     if (!any[sa]) return;
 #pragma unroll
-    for (int j = 0; j < K; ++j)
+    for (int p = 0; p < (sa == 0 ? 1 : K); ++p) {
+      // each expansion is summed before it joins the node's sum: added term by term it rounded at the
+      // size of that sum (error against 64 bits, k = 5, 7, 8: 1.16 to 1.21 times that of the lift of W_F, 0.91 to
+      // 0.95 so, at the same speed)
+      V w = vmul(c.g[0][p + (2 - sa) * K], s[sa][0]);
 #pragma unroll
-      for (int p = 0; p < (sa == 0 ? 1 : K); ++p) dot_fma(acc[p], c.g[j][p + (2 - sa) * K], s[sa][j]);
+      for (int j = 1; j < K; ++j) w = vfma(c.g[j][p + (2 - sa) * K], s[sa][j], w);
+      sum_add(acc[p], w);
+    }
   };
 #pragma unroll
   for (int sa = 2; sa >= 0; --sa) {
