@@ -180,13 +180,16 @@ cudaError_t upload(T** dst, const std::vector<T>& src) {
   return cudaMemcpy(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice);
 }
 
+gp::BatchOps ops_for(int prec, int dim);
+
 void free_device(gp_ctx* c) {
-  void* ptrs[] = {c->d_frows, c->d_lwin, c->d_lrow, c->d_lmask, c->d_zruns, c->d_tp, c->d_xh, c->d_yh, c->d_truns,
+  void* ptrs[] = {c->d_frows, c->d_lwin, c->d_lrow, c->d_lmask, c->d_fac, c->d_zruns, c->d_tp, c->d_xh, c->d_yh, c->d_truns,
                   c->d_bdesc, c->d_bcell, c->d_bccoord, c->d_bface, c->d_rowtab,
                   c->d_pnode, c->d_poff, c->d_pslot, c->d_part};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   c->d_frows = c->d_lwin = c->d_lrow = c->d_lmask = nullptr;
+  c->d_fac = nullptr;
   c->d_zruns = nullptr;
   c->d_tp = c->d_xh = c->d_yh = nullptr;
   c->d_truns = nullptr;
@@ -244,6 +247,7 @@ gp_status gpi::launch(gp_ctx* c, const void* x, void* y, int add, cudaStream_t s
   a.nzruns = add ? 0 : (int32_t)p.num_zero_runs();
   a.g = p.jumps.data();
   a.m = p.lump.data();
+  a.fac = c->d_fac;
   a.s = p.scale.data();
   a.ldl = p.ldl.empty() ? nullptr : p.ldl.data();
   cudaEvent_t* ev = nullptr;
@@ -400,6 +404,9 @@ gp_status gp_setup(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* op
     const gp::Plan& p = c->plan;
     std::vector<int2> zruns(p.zruns.size() / 2);
     std::memcpy(zruns.data(), p.zruns.data(), p.zruns.size() * sizeof(int32_t));
+    std::vector<unsigned char> fac;
+    ops_for(p.precision, p.dim).values(p.fac.data(), p.fac.size(), fac);
+    if (e == cudaSuccess) e = upload(reinterpret_cast<unsigned char**>(&c->d_fac), fac);
     if (e == cudaSuccess) e = upload(&c->d_frows, p.frows);
     if (e == cudaSuccess) e = upload(&c->d_lwin, p.lwin);
     if (e == cudaSuccess) e = upload(&c->d_lrow, p.lrow);
@@ -851,12 +858,12 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
   for (size_t gi = 0; gi < b->groups.size() && e == cudaSuccess; ++gi) {
     auto& g = b->groups[gi];
     std::vector<gp::SegSpec> specs(g.prob.size());
-    const size_t nb = (size_t)g.k * (g.k + 1);   // the entries of B; D follows
     for (size_t i = 0; i < g.prob.size(); ++i) {
       const gp_ctx* c = ctxs[g.prob[i]];
       const gp::Plan& pl = c->plan;
       gp::SegSpec& sp = specs[i];
       sp.fa.frows = c->d_frows;
+      sp.fa.fac = c->d_fac;
       for (int a = 0; a < 4; ++a) {
         sp.fa.rbase[a] = pl.rbase[a];
         sp.fa.fstart[a] = pl.fstart[a];
@@ -870,7 +877,7 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
       sp.la.n_active = (int32_t)pl.n_active;
       sp.wp = (char*)b->d_w + woff[gi][i];
       sp.gs = (const char*)b->d_gs + gs_off[g.prob[i]];
-      for (int j = 0; j < pl.k; ++j) sp.s[j] = g.ldl ? pl.ldl[nb + j] : pl.scale[j];
+      for (int j = 0; j < pl.k; ++j) sp.s[j] = pl.scale[j];
     }
     std::vector<unsigned char> fs, ls;
     if (!g.ops.pack(g.k, specs, g.form, g.tiles, fs, ls, g.face_blocks, g.lift_blocks)) {

@@ -68,6 +68,11 @@ __device__ __forceinline__ ff64 vadd(ff64 a, ff64 b) {
   return ff64{hi, __fsub_rn(lo, __fsub_rn(hi, s))};
 }
 
+// ------------------------------------------- a times a power of two: exact --
+__device__ __forceinline__ float vscale(float a, float c) { return a * c; }
+__device__ __forceinline__ double vscale(double a, float c) { return a * (double)c; }
+__device__ __forceinline__ ff64 vscale(ff64 a, float c) { return ff64{__fmul_rn(a.hi, c), __fmul_rn(a.lo, c)}; }
+
 // ---------------------------------------------------------------- a - b --
 __device__ __forceinline__ float vsub(float a, float b) { return a - b; }
 __device__ __forceinline__ double vsub(double a, double b) { return a - b; }

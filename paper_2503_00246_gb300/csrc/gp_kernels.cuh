@@ -87,25 +87,24 @@ struct Consts {
   V g[K][2 * K + 1];   // jump of the j-th derivative of patch basis b (row j-1)
   V gs[K][2 * K + 1];  // s_j g_j[b], the jump vectors of the first step (FP64, float-float)
   V s[K];              // s_j (FP32)
-  // reference mass M^ = diag(mw) (I + mc ma^T) (see tangential_mass)
+  // reference mass M^ = diag(mw) (I + mc ma^T) (see tangential_mass; mw: LineFactors)
   V ma[K + 1];
   V mc[K + 1];
-  V mw[K + 1];
 };
 
-// Fills the lumped form of the reference mass from p = (ma, mc, mw), 3 (k+1) values.
+// Fills the lumped form of the reference mass from p = (ma, mc), 2 (k+1) values.
 template <typename V, int K>
 void mass_consts(const double* p, Consts<V, K>& c) {
   constexpr int N = K + 1;
   for (int i = 0; i < N; ++i) {
     c.ma[i] = from_host<V>(p[i]);
     c.mc[i] = from_host<V>(p[N + i]);
-    c.mw[i] = from_host<V>(p[2 * N + i]);
   }
 }
 
 struct FaceArgs {
   const int32_t* frows;   // per-face row starts of the patch (see rbase)
+  const void* fac;        // factors of the normal lines, V values (see Plan::fac)
   int64_t rbase[4];       // row entry of face fstart[a] of each axis
   int32_t fstart[4];      // first face of each axis in this launch
   int32_t fend[4];        // one past the last face of each axis in this launch
@@ -216,7 +215,8 @@ __device__ __forceinline__ void line_jumps(const V (&v)[2 * K + 1], const V (*g)
 // orders of that parity: G^ = sum_j s_j g_j g_j^T = B diag(D) B^T, row j of B with a 1 at its pivot
 // node and 0 at the pivots of the earlier rows of its parity (rows j = 0, 2, .. even in b, 1, 3, ..
 // odd).  Those entries cost nothing in the jumps (t_j = B_j . v) or in the expansion: 12 + 12
-// multiply-adds per line instead of 18 + 18 at k = 4, 48 + 48 instead of 68 + 68 at k = 8; D_j goes into the line factors mw (a table per CTA).  The host eliminates
+// multiply-adds per line instead of 18 + 18 at k = 4, 48 + 48 instead of 68 + 68 at k = 8; D_j goes into the line factors mw (Plan::fac, rounded
+// once: products of rounded D_j and mw had errors up to 1.25 times those of the jump vectors).  The host eliminates
 // in 113-bit arithmetic (Plan::ldl), from the largest direction to the smallest: D is graded and
 // non-negative, so x^T G x stays a sum of squares.  The pivot orders are those whose elimination
 // grows least (entries below 1.2 for the default and for the factorial weights).  Native FP64 only,
@@ -312,38 +312,52 @@ struct TanShape {
   __host__ __device__ static constexpr int at(int tau) { return (D == 3) ? tau % N + PITCH * (tau / N) : tau; }
 };
 
-// The factors a line's thread needs at its own tangential index (lane-dependent, so not in the
-// constant bank): mw of the line (the product of both directions) and mc.
-template <int D, int K, typename V, bool W = true>
-struct TanTable {
-  V w[W ? Shape<D, K>::L : 1];
-  V c[K + 1];
-};
-template <int D, int K, typename V, bool W>
-__device__ __forceinline__ void fill_tan_table(TanTable<D, K, V, W>& tab, const Consts<V, K>& c, const int t) {
-  constexpr int N = K + 1;
-  if (W && t < Shape<D, K>::L) tab.w[t] = (D == 3) ? vmul(c.mw[t % N], c.mw[t / N]) : c.mw[t];
-  if (t < N) tab.c[t] = c.mc[t];
+// mc by tangential index in shared memory (a thread's index is lane-dependent: not for the constant bank)
+template <int K, typename V>
+__device__ __forceinline__ void fill_mc(V (&mc)[K + 1], const Consts<V, K>& c, const int t) {
+  if (t <= K) mc[t] = c.mc[t];
+}
+
+// u -> (I + mc ma^T) u of one tangential line.  k = 1: (2 u_0 + u_1, u_0 + 2 u_1), one rounding each.  (The integer
+// form of k = 2, 1/30 (4 2 -1; 2 16 2; -1 2 4), was no more accurate and in FP64 4 % slower.)
+template <int K, typename V>
+__device__ __forceinline__ V line_dot(const Consts<V, K>& c, const V (&u)[K + 1]) {
+  Dot<V> acc = dot_first(c.ma[0], u[0]);
+#pragma unroll
+  for (int q = 1; q <= K; ++q) dot_fma(acc, c.ma[q], u[q]);
+  return dot_value(acc);
+}
+template <int K, typename V>
+__device__ __forceinline__ void line_mass(const Consts<V, K>& c, V (&u)[K + 1]) {
+  if constexpr (K == 1) {
+    const V a = u[0], b = u[1];
+    u[0] = vadd(vscale(a, 2.f), b);
+    u[1] = vadd(vscale(b, 2.f), a);
+  } else {
+    const V s = line_dot<K, V>(c, u);
+#pragma unroll
+    for (int q = 0; q <= K; ++q) u[q] = vfma(c.mc[q], s, u[q]);
+  }
 }
 
 // out[j] = ((M^ x M^) u_j)(tau) for the k jump values u_j of every line in `plane`.  A task is one
 // (face, order j, tangential line of N values); the tasks of the CTA's fb faces are packed onto its
 // first threads.  3D: pass 1 along t2 (neighbouring lanes on neighbouring t1) in place; pass 2
 // along t1 only takes the dot product ma . u of each line, and every line's thread adds its own
-// mc and multiplies by mw (FP32, bound by shared-memory accesses and not by arithmetic: pass 2 in
-// place too, one access less per value).  2D: pass 1 in place.  wl[tau + WS j] is the factor of
-// order j and line tau (WS = 0: one for every order), mc[t] the correction of tangential index t, both
-// in shared memory.  Every thread of the CTA calls it (it synchronises, also before its first read:
-// the caller has only written plane, wl and mc).
+// mc and multiplies by mw (FP32, bound by shared-memory accesses and not by arithmetic, and k = 1: pass 2 in
+// place too, one access less per value).  2D: pass 1 in place.  wt is the
+// factor of the thread's line or, with the triangular basis, wl[tau + WS j] that of order j and line tau, mc[t]
+// the correction of tangential index t, both in shared memory.  Every thread of the CTA calls it (it
+// synchronises, also before its first read: the caller has only written plane, wl and mc).
 template <int D, int K, typename V, int WS = 0>
 __device__ __forceinline__ void tangential_mass(V (*plane)[K][TanShape<D, K>::LP], V (*dots)[K][K + 1], const int fb,
-                                                const Consts<V, K>& c, const V* wl, const V* mc, const int fl,
+                                                const Consts<V, K>& c, const V wt, const V* wl, const V* mc, const int fl,
                                                 const int tau, V (&out)[K]) {
   using T = TanShape<D, K>;
   constexpr int N = K + 1;
   constexpr int TASKS = (D == 3) ? K * N : K;     // per face and pass
   constexpr int ST = (D == 3) ? T::PITCH : 1;     // stride of pass 1
-  constexpr bool DOTS = D == 3 && !std::is_same<V, float>::value;
+  constexpr bool DOTS = D == 3 && K > 1 && !std::is_same<V, float>::value;
   const int u = threadIdx.x;
   const bool task = u < fb * TASKS;
   const int tf = u / TASKS, w = u - tf * TASKS;
@@ -354,12 +368,9 @@ __device__ __forceinline__ void tangential_mass(V (*plane)[K][TanShape<D, K>::LP
     V uu[N];
 #pragma unroll
     for (int q = 0; q < N; ++q) uu[q] = p[ST * q];
-    Dot<V> acc = dot_first(c.ma[0], uu[0]);
+    line_mass<K, V>(c, uu);
 #pragma unroll
-    for (int q = 1; q < N; ++q) dot_fma(acc, c.ma[q], uu[q]);
-    const V s = dot_value(acc);
-#pragma unroll
-    for (int q = 0; q < N; ++q) p[ST * q] = vfma(c.mc[q], s, uu[q]);
+    for (int q = 0; q < N; ++q) p[ST * q] = uu[q];
   }
   __syncthreads();
   if constexpr (D == 3) {
@@ -368,20 +379,16 @@ __device__ __forceinline__ void tangential_mass(V (*plane)[K][TanShape<D, K>::LP
       V uu[N];
 #pragma unroll
       for (int q = 0; q < N; ++q) uu[q] = p[q];
-      Dot<V> acc = dot_first(c.ma[0], uu[0]);
-#pragma unroll
-      for (int q = 1; q < N; ++q) dot_fma(acc, c.ma[q], uu[q]);
-      const V s = dot_value(acc);
       if constexpr (DOTS) {
-        dots[tf][j][tr] = s;
+        dots[tf][j][tr] = line_dot<K, V>(c, uu);
       } else {
+        line_mass<K, V>(c, uu);
 #pragma unroll
-        for (int q = 0; q < N; ++q) p[q] = vfma(c.mc[q], s, uu[q]);
+        for (int q = 0; q < N; ++q) p[q] = uu[q];
       }
     }
     __syncthreads();
   }
-  const V wt = wl[tau];
   const V ct = DOTS ? mc[tau % N] : vzero<V>();
 #pragma unroll
   for (int jj = 0; jj < K; ++jj) {
@@ -451,7 +458,7 @@ struct StoreCompact {
 // (FP64, float-float: the scaled s_j g_j, c.gs or a batch segment's copy in shared memory;
 // FP32: the plain c.g) and `sc` the k factors s_j (FP32 only); `dsm` is the
 // face_smem<D, K, V>(fb) bytes of dynamic shared memory.  COMPACT: store T_F instead of W_F.  LDL: gs
-// holds the rows of B and sc the k factors D_j.
+// holds the rows of B.
 template <int D, int K, class A, bool COMPACT, bool LDL>
 __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, typename A::V* __restrict__ wp,
                                           typename A::IO* __restrict__ y, const FaceArgs& fa,
@@ -466,7 +473,7 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
   typedef V Dots[K][K1];
   Plane* buf = reinterpret_cast<Plane*>(dsm);            // [fb][K][LP]
   Dots* dots = reinterpret_cast<Dots*>(buf + fb);         // [fb][K][N], 3D only
-  __shared__ TanTable<D, K, V, !LDL> tab;   // LDL: the line factors are in wj
+  __shared__ V mc[K1];
   V* wj = reinterpret_cast<V*>(dots + ((D == 3) ? fb : 0));   // LDL: [K][L] line factors D_j mw
   const int nt = (int)blockDim.x;
   // the lift may start its prologue as soon as every face CTA is running (programmatic
@@ -495,15 +502,13 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
   const int fl = t / L, tau = t - fl * L;
   const int f = f0 + fl;
   const bool valid = f < fend;
+  const V* fac = static_cast<const V*>(fa.fac);
   if constexpr (LDL) {
-    if (t < L) {
-      const V w = (D == 3) ? c.mw[t % K1] * c.mw[t / K1] : c.mw[t];
-#pragma unroll
-      for (int j = 0; j < K; ++j) wj[j * L + t] = sc[j] * w;
-    }
+    // the factors of the triangular basis on their way to shared memory while the gather runs
+    for (int i = t; i < K * L; i += nt)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(wj + i)),
+                   "l"(fac + L + i) : "memory");
   }
-  fill_tan_table<D, K, V>(tab, c, t);
-
   // ---- gather this thread's normal line (2k+1 values)
   V v[NN];
   if (StagePatch<V, K, COMPACT>::value && axis == 0) {
@@ -558,6 +563,8 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
 #pragma unroll
     for (int b = 0; b < NN; ++b) v[b] = vzero<V>();
   }
+  if constexpr (LDL) asm volatile("cp.async.wait_all;" ::: "memory");
+  fill_mc<K, V>(mc, c, t);
   // ---- contract with the k jump vectors, then the tangential reference masses
   {
     V t[K];
@@ -567,7 +574,8 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
     for (int j = 0; j < K; ++j) buf[fl][j][T::at(tau)] = t[j];
   }
   V out[K];
-  tangential_mass<D, K, V, LDL ? L : 0>(buf, dots, fb, c, LDL ? wj : tab.w, tab.c, fl, tau, out);
+  // (the factor is used behind three barriers: its load is hidden)
+  tangential_mass<D, K, V, LDL ? L : 0>(buf, dots, fb, c, LDL ? vzero<V>() : fac[tau], wj, mc, fl, tau, out);
 
   if (!valid) return;
   if constexpr (!FoldScale<V>::value) {
@@ -629,7 +637,7 @@ struct FaceSeg {
   V* wp;           // this segment's face outputs
   const V* gs;     // FP64, float-float: K x (2K+1) scaled jump vectors s_j g_j of the problem, or the rows
                    // of its triangular basis B
-  V s[K];          // FP32: s_j of the problem; triangular basis: D_j
+  V s[K];          // FP32: s_j of the problem
   int32_t block0;  // first CTA of the segment in the group's face launch
 };
 

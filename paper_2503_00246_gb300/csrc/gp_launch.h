@@ -34,7 +34,8 @@ struct ApplyArgs {
   const int2* zruns = nullptr;
   int32_t nzruns = 0;        // zero runs to fill (0 for the add form)
   const double* g = nullptr; // host FP64: k x (2k+1)
-  const double* m = nullptr; // host FP64: the lumped mass, 3 (k+1) values (Plan::lump)
+  const double* m = nullptr; // host FP64: the lumped mass, 2 (k+1) values (Plan::lump)
+  const void* fac = nullptr; // device: factors of the normal lines, V values (Plan::fac)
   const double* s = nullptr; // host FP64: k
   const double* ldl = nullptr;  // host FP64: the triangular normal basis (Plan::ldl); nullptr: g and s as they are
   cudaEvent_t* ev = nullptr;  // optional: 3 events recorded around the two kernels
@@ -93,7 +94,7 @@ constexpr TileRules kTilesF64 = {
      tiles_at({4, 16, 256}), tiles_at({3, 32, 512})},
     {tiles_at({128, 256, 512}), tiles_at({14, 128, 512}, 2500, {10, 64, 512}, 24000, {21, 32, 256}),
      tiles_at({2, 16, 256}, 6000, {8, 16, 256}, 70000, {24, 32, 512}), tiles_at({6, 32, 512}, 19000, {20, 32, 512}),
-     tiles_at({4, 8, 256}, 6000, {7, 16, 512}), tiles_at({3, 3, 256}, 3000, {5, 14, 512}), tiles_at({2, 8, 512}),
+     tiles_at({4, 8, 256}, 6000, {7, 16, 512}), tiles_at({3, 3, 256}, 3000, {5, 4, 256}, 5000, {5, 14, 512}), tiles_at({2, 8, 512}),
      tiles_at({3, 4, 256})}};
 constexpr TileRules kTilesFF = {
     {tiles_at({128, 256, 512}), tiles_at({42, 128, 256}), tiles_at({24, 32, 128}), tiles_at({19, 32, 256}),
@@ -123,10 +124,10 @@ constexpr TileRules kTilesF32Compact = {
      tiles_at({2, 4, 256}, 2500, {1, 10, 256}, 7700, {2, 8, 128}),
      tiles_at({1, 4, 256}, 2800, {1, 6, 128}, 9700, {1, 8, 128})}};
 
-// The model system's face kernel runs beside its cell kernel: CTAs of 130 to 260 threads are within 2 % of the
+// The model system's face kernel runs beside its cell kernel: CTAs of 110 to 260 threads are within 2 % of the
 // fastest at every size (12 meshes per degree), and small ones cost up to 30 us (FP64, k = 2, 16^3 ball, 7 / 10 / 21
 // faces: 56 / 25 / 24 us).  FP32, FP64, float-float in 3D; in 2D about 256 threads.
-constexpr int kSystemFaces[3][8] = {{64, 17, 8, 5, 3, 3, 2, 1}, {64, 21, 16, 20, 7, 5, 4, 3}, {64, 21, 16, 5, 7, 5, 4, 3}};
+constexpr int kSystemFaces[3][8] = {{64, 14, 8, 5, 3, 3, 2, 1}, {64, 21, 16, 20, 7, 5, 4, 3}, {64, 21, 16, 5, 7, 5, 4, 3}};
 
 template <int D, int K, typename V>
 const TileRule& tile_rule(const LaunchForm& form) {
@@ -236,6 +237,7 @@ cudaError_t run_brick(const ApplyArgs& Ar, const Consts<typename A::V, K>& c, cu
   constexpr int L = Shape<D, K>::L;
   const int fb = brick_fb<D, K>(Ar.tiles);
   BrickArgs ba = Ar.ba;
+  ba.fac = Ar.fac;
   ba.zruns = Ar.zruns;
   ba.nzruns = Ar.nzruns;
   ba.nzblocks = (Ar.nzruns + ZGROUP - 1) / ZGROUP;
@@ -373,6 +375,7 @@ cudaError_t run_slabs(const ApplyArgs& Ar, const Consts<typename A::V, K>& c, co
     const int32_t* sl = Ar.slabs + (size_t)s * SLAB_INTS;
     FaceArgs fa;
     fa.frows = Ar.frows;
+    fa.fac = Ar.fac;
     fa.zruns = Ar.zruns;
     fa.nzruns = s == 0 ? Ar.nzruns : 0;
     fa.tail_wait = s > 0 && !Ar.slab_events;
@@ -423,10 +426,8 @@ struct UseLdl {
 };
 template <typename V, int K>
 void ldl_consts(const double* p, Consts<V, K>& c) {
-  for (int j = 0; j < K; ++j) {
+  for (int j = 0; j < K; ++j)
     for (int b = 0; b <= K; ++b) c.g[j][b] = from_host<V>(p[j * (K + 1) + b]);
-    c.s[j] = from_host<V>(p[K * (K + 1) + j]);
-  }
 }
 
 template <int D, int K, class A>
@@ -452,6 +453,7 @@ cudaError_t run_apply(const ApplyArgs& Ar, cudaStream_t st) {
   if (Ar.nslab > 1 && !Ar.ev && Ar.which == 3) return run_slabs<D, K, A>(Ar, c, t, ldl, st);
   FaceArgs fa;
   fa.frows = Ar.frows;
+  fa.fac = Ar.fac;
   for (int a = 0; a < 4; ++a) fa.rbase[a] = Ar.rbase[a];
   fa.zruns = Ar.zruns;
   fa.nzruns = Ar.nzruns;
@@ -483,7 +485,7 @@ struct SegSpec {
   LiftArgs la;
   void* wp = nullptr;   // the segment's face-output buffer
   const void* gs = nullptr;   // device: K x (2K+1) scaled jump vectors of the segment's problem, or its B
-  double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};   // the problem's s_j (triangular basis: D_j)
+  double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};   // the problem's s_j
 };
 
 // Packs the segments of one (d, k, arithmetic) group into the device layouts of
@@ -578,8 +580,18 @@ void scaled_jumps(int k, const double* g, const double* s, std::vector<unsigned 
     for (int b = 0; b < 2 * k + 1; ++b) o[j * (2 * k + 1) + b] = from_host<V>(s[j] * g[j * (2 * k + 1) + b]);
 }
 
+// n host values in the value type of the arithmetic.
+template <class A>
+void to_values(const double* v, size_t n, std::vector<unsigned char>& out) {
+  using V = typename A::V;
+  out.resize(n * sizeof(V));
+  V* o = reinterpret_cast<V*>(out.data());
+  for (size_t i = 0; i < n; ++i) o[i] = from_host<V>(v[i]);
+}
+
 // Per translation unit: batch packing and launch for one (arithmetic, dimension).
 struct BatchOps {
+  void (*values)(const double* v, size_t n, std::vector<unsigned char>& out);
   bool (*pack)(int k, const std::vector<SegSpec>&, const LaunchForm&, Tiles&, std::vector<unsigned char>&,
                std::vector<unsigned char>&, int&, int&);
   void (*jumps)(int k, const double* g, const double* s, std::vector<unsigned char>& out);
@@ -595,6 +607,7 @@ BatchOps batch_ops_ff_d3();
 
 #define GP_BATCH_OPS(D, A)                                                                              \
   BatchOps ops;                                                                                         \
+  ops.values = to_values<A>;                                                                            \
   ops.jumps = scaled_jumps<A>;                                                                          \
   ops.pack = [](int k, const std::vector<SegSpec>& in, const LaunchForm& form, Tiles& t,               \
                 std::vector<unsigned char>& fs,                                                         \

@@ -164,10 +164,11 @@ void reference_1d(int k, const std::vector<double>& /*gl*/, std::vector<double>&
 // 2/k for the integral of P_k^2 and the integral is 2/(2k+1), and P_k has the leading coefficient
 // c = (2k)! / (2^k k!^2), so E = (2/k - 2/(2k+1)) / c^2 / 2 / 4^k.  k = 1 has the equal form
 // diag(1/6) (I + 1 1^T), whose terms are all positive.
-bool lumped_mass(int k, const std::vector<double>& mass, std::vector<double>& lump) {
+bool lumped_mass(int k, const std::vector<double>& mass, std::vector<double>& lump, std::vector<R>& w) {
   const int N = k + 1;
-  std::vector<R> gl, a(N, R(1)), w(N);
+  std::vector<R> gl, a(N, R(1));
   gauss_lobatto_01_r(k, gl);
+  w.assign(N, R(0));
   R E = 0, amax = 0;
   if (k == 1) {
     w[0] = w[1] = R(1) / 6;
@@ -187,11 +188,10 @@ bool lumped_mass(int k, const std::vector<double>& mass, std::vector<double>& lu
       amax = std::max(amax, std::fabs(a[i]));
     }
   }
-  lump.assign(3 * N, 0.0);
+  lump.assign(2 * N, 0.0);
   for (int i = 0; i < N; ++i) {
     lump[i] = (double)(a[i] / amax);
     lump[N + i] = (double)(-E * a[i] * amax / w[i]);
-    lump[2 * N + i] = (double)w[i];
   }
   R dev = 0;
   for (int i = 0; i < N; ++i)
@@ -213,10 +213,11 @@ static const int kPivot[8][8] = {{1}, {2, 1}, {2, 2, 1}, {3, 2, 2, 3}, {3, 3, 1,
                                  {5, 4, 2, 6, 7, 2, 4}, {5, 4, 2, 7, 8, 1, 6, 6}};
 
 void normal_basis(int k, const std::vector<double>& jumps, const std::vector<double>& c, double hd,
-                  std::vector<double>& ldl) {
+                  std::vector<double>& ldl, std::vector<R>& factors) {
   const int N = k + 1, NN = 2 * k + 1;
+  factors.assign(k, R(0));
   auto absq = [](Q v) { return v < 0 ? -v : v; };
-  ldl.assign((size_t)k * N + k, 0.0);
+  ldl.assign((size_t)k * N, 0.0);
   for (double v : c)
     if (!(v >= 0.0) || std::isinf(v)) {
       ldl.clear();
@@ -253,7 +254,7 @@ void normal_basis(int k, const std::vector<double>& jumps, const std::vector<dou
         ldl.clear();
         return;
       }
-      ldl[(size_t)k * N + j] = D;
+      factors[j] = (R)(d * Q(hd));
       for (int a = 0; a < n; ++a)
         for (int e = 0; e < n; ++e) A[a * n + e] -= d * b[a] * b[e];
     }
@@ -262,6 +263,18 @@ void normal_basis(int k, const std::vector<double>& jumps, const std::vector<dou
         ldl.clear();
         return;
       }
+  }
+}
+
+// Plan::fac from the lumped weights and the factors of the triangular basis, in extended precision: products of
+// values already rounded to double cost FP64 applies up to a quarter of their accuracy.
+static void line_factors(Plan& p, const std::vector<R>& mw, const std::vector<R>& D) {
+  const int N = p.k + 1;
+  p.fac.assign((size_t)p.L * (p.ldl.empty() ? 1 : p.k + 1), 0.0);
+  for (int t = 0; t < p.L; ++t) {
+    const R w = p.dim == 3 ? mw[t % N] * mw[t / N] : mw[t];
+    p.fac[t] = (double)w;
+    for (int j = 0; j < p.k && !p.ldl.empty(); ++j) p.fac[(size_t)p.L * (j + 1) + t] = (double)(D[j] * w);
   }
 }
 
@@ -1239,7 +1252,8 @@ gp_status build_plan(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* 
   // ---- 1D reference data and the per-order scale c_j h^(d-2)
   gauss_lobatto_01(k, p.gl);
   reference_1d(k, p.gl, p.mass, p.jumps);
-  if (!lumped_mass(k, p.mass, p.lump)) { err = "internal: the lumped form misses the reference mass"; return GP_EINVAL; }
+  std::vector<R> mw, D;
+  if (!lumped_mass(k, p.mass, p.lump, mw)) { err = "internal: the lumped form misses the reference mass"; return GP_EINVAL; }
   reference_stiffness(k, p.stiff);
   p.scale.resize(k);
   p.stabilization = opts->stabilization;
@@ -1257,7 +1271,8 @@ gp_status build_plan(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* 
       }
     }
     for (double& v : lam) v *= opts->gamma;
-    if (opts->precision == GP_FP64) normal_basis(k, p.jumps, lam, hv, p.ldl);
+    if (opts->precision == GP_FP64) normal_basis(k, p.jumps, lam, hv, p.ldl, D);
+    line_factors(p, mw, D);
     return GP_OK;
   }
   if (opts->stabilization != GP_STAB_GHOST) { err = "unknown stabilization"; return GP_EINVAL; }
@@ -1275,7 +1290,8 @@ gp_status build_plan(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* 
       return GP_EINVAL;
     }
   }
-  if (opts->precision == GP_FP64) normal_basis(k, p.jumps, cw, hd, p.ldl);
+  if (opts->precision == GP_FP64) normal_basis(k, p.jumps, cw, hd, p.ldl, D);
+  line_factors(p, mw, D);
   return GP_OK;
 }
 

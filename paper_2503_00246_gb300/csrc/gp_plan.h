@@ -119,10 +119,13 @@ struct Plan {
   std::vector<double> gl;         // k+1 Gauss-Lobatto points on [0,1]
   std::vector<double> stiff;      // (k+1)^2: int_0^1 l_a' l_b' 
   std::vector<double> mass;       // (k+1)^2
-  std::vector<double> lump;       // 3 (k+1): ma, mc, mw with mass = diag(mw) (I + mc ma^T)
+  std::vector<double> lump;       // 2 (k+1): ma, mc with mass = diag(mw) (I + mc ma^T)
+  // factors of a face's L normal lines, each rounded once: mw (3D: the product of both directions'), then, with
+  // a triangular basis, D_j mw for the k rows of ldl
+  std::vector<double> fac;
   std::vector<double> jumps;      // k x (2k+1)
-  // triangular normal basis: k rows of k+1 entries of B, then k factors D_j, with sum_j scale_j g_j g_j^T
-  // = B diag(D) B^T (see gp_kernels.cuh); empty if the weights have none
+  // triangular normal basis: k rows of k+1 entries of B, with sum_j scale_j g_j g_j^T = B diag(D) B^T
+  // (see gp_kernels.cuh; D is in fac); empty if the weights have none
   std::vector<double> ldl;
   std::vector<double> scale;      // k: c_j h^(dim-2) (macro patch: gamma lambda_j h^dim)
   int stabilization = GP_STAB_GHOST;
@@ -150,12 +153,12 @@ void gauss_lobatto_01(int k, std::vector<double>& x);
 void reference_1d(int k, const std::vector<double>& gl, std::vector<double>& mass,
                   std::vector<double>& jumps);
 // The lumped form of the mass matrix (see Plan::lump); false if it does not reproduce `mass`.
-bool lumped_mass(int k, const std::vector<double>& mass, std::vector<double>& lump);
+bool lumped_mass(int k, const std::vector<double>& mass, std::vector<double>& lump, std::vector<long double>& mw);
 // The triangular normal basis of the weights c (per order, without the factor hd of the mesh
 // size, so that problems of one degree and one set of weights have equal B); empty for weights that are
 // negative, infinite or NaN, an elimination that grows, or factors D outside 2^-900 .. 2^900.
 void normal_basis(int k, const std::vector<double>& jumps, const std::vector<double>& c, double hd,
-                  std::vector<double>& ldl);
+                  std::vector<double>& ldl, std::vector<long double>& D);
 void reference_stiffness(int k, std::vector<double>& stiff);
 // Macro-patch 1D data: k mirror-(anti)symmetric vectors (k x (2k+1)) and weights lambda_j;
 // false if the matrix is not of rank k with the expected parities.

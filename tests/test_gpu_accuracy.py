@@ -1,5 +1,6 @@
 """GPU: the error of y = G x against an extended-precision reference stays at the size of the rounding of each
-arithmetic: the expansions of compact face outputs are summed before they join a node's sum.  The reference takes the 1D data to
+arithmetic: products of constants are rounded once (line factors of the tangential masses) and the
+expansions of compact face outputs are summed before they join a node's sum.  The reference takes the 1D data to
 40 digits and applies it in long double (64 bits of mantissa or more).  Inputs are single-precision numbers,
 so that every arithmetic sees the same x; the bounds are 2-norm errors in units of 2^-53, 2^-48 and 2^-24."""
 import functools
@@ -89,8 +90,9 @@ def _reference(dim, n, k):
 BOUND = {0: 1.8 * 2.0 ** -53, 1: 1.7 * 2.0 ** -24, 2: 2.3 * 2.0 ** -48}
 
 
-@pytest.mark.parametrize("prec", [1])
-@pytest.mark.parametrize("dim,n,k", [(2, 20, k) for k in range(1, 9)] + [(3, 7, 5), (3, 5, 7), (3, 4, 8)])
+@pytest.mark.parametrize("prec", [0, 1, 2])
+@pytest.mark.parametrize("dim,n,k", [(3, 7, k) for k in (1, 2, 3, 4, 5)] + [(2, 20, k) for k in range(1, 9)]
+                         + [(3, 5, 7), (3, 4, 8)])
 def test_error_at_the_rounding_of_the_arithmetic(gplib, cuda, prec, dim, n, k):
     pr, x, ref = _reference(dim, n, k)
     ctx = gplib.setup_problem(pr, precision=prec, path=gplib.GP_PATH_FACE_LIFT)

@@ -29,6 +29,7 @@ template <int K>
 void check() {
   constexpr int N = K + 1, NN = 2 * K + 1;
   std::vector<double> gl, mass, g, ldl;
+  std::vector<long double> D;
   gp::gauss_lobatto_01(K, gl);
   gp::reference_1d(K, gl, mass, g);
   const double inf = std::numeric_limits<double>::infinity(), nan = std::numeric_limits<double>::quiet_NaN();
@@ -43,8 +44,8 @@ void check() {
       if (kind == 4) c[j] = 0.0;
     }
     const double hd = 0.03125;
-    gp::normal_basis(K, g, c, hd, ldl);
-    if (ldl.size() != (size_t)(K * N + K)) { fail("no basis", K, kind); continue; }
+    gp::normal_basis(K, g, c, hd, ldl, D);
+    if (ldl.size() != (size_t)(K * N) || D.size() != (size_t)K) { fail("no basis", K, kind); continue; }
     auto B = [&](int j, int b) -> double {          // row j on the folded line, mirrored with its parity
       return b <= K ? ldl[j * N + b] : (j & 1 ? -1.0 : 1.0) * ldl[j * N + NN - 1 - b];
     };
@@ -59,7 +60,7 @@ void check() {
         long double s = 0, t = 0;
         for (int j = 0; j < K; ++j) {
           s += (long double)hd * c[j] * g[j * NN + a] * g[j * NN + b];
-          t += (long double)ldl[K * N + j] * B(j, a) * B(j, b);
+          t += D[j] * B(j, a) * B(j, b);
         }
         // every entry and every factor is rounded once: a few units in the last place of the largest entry
         if (!(std::fabs((double)(s - t)) <= 4 * K * 1.2e-16L * top)) { fail("B D B^T", K, kind); a = b = NN; }
@@ -69,7 +70,7 @@ void check() {
       for (int b = 0; b <= K; ++b)
         if (gp::Pivots<K>::zero(j, b) && B(j, b) != 0.0) fail("zero entry", K, kind);
       if ((j & 1) && B(j, K) != 0.0) fail("odd row at the face", K, kind);
-      if (!(ldl[K * N + j] >= 0.0)) fail("factor", K, kind);
+      if (!(D[j] >= 0.0)) fail("factor", K, kind);
     }
   }
   const double none[] = {inf, nan, -0.5, -inf, 1e300, 1e-305};
@@ -77,7 +78,7 @@ void check() {
     for (int j = 0; j < K; ++j) {
       std::vector<double> c(K, kind >= 4 ? none[kind] : 0.5);
       c[j] = none[kind];
-      gp::normal_basis(K, g, c, 0.03125, ldl);
+      gp::normal_basis(K, g, c, 0.03125, ldl, D);
       if (!ldl.empty()) fail("basis of unusable weights", K, 10 + kind);
     }
   std::printf("%d:", K);
