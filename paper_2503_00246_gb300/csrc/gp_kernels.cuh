@@ -611,7 +611,8 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
 extern __shared__ __align__(16) unsigned char gp_dyn_smem[];
 
 // resident CTAs of MAX_CTA_THREADS threads to compile for: FP32 is held to 32 registers, every warp
-// slot of the SM (128^3 gyroid, k = 4, with 38 registers: 154 against 135 us); 0: the compiler's choice
+// slot of the SM (128^3 gyroid, k = 4, with 38 registers: 154 against 135 us; the compiler's choice at other degrees:
+// applies of the 80^3 ball at k = 5 66.9 / 65.7 us, of the 600^2 disc at k = 7 12.1 / 11.0 us); 0: that choice
 template <typename V>
 struct FaceCtas {
   static constexpr int value = std::is_same<V, float>::value ? 4 : 0;
