@@ -180,8 +180,6 @@ cudaError_t upload(T** dst, const std::vector<T>& src) {
   return cudaMemcpy(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice);
 }
 
-gp::BatchOps ops_for(int prec, int dim);
-
 void free_device(gp_ctx* c) {
   void* ptrs[] = {c->d_frows, c->d_lwin, c->d_lrow, c->d_lmask, c->d_fac, c->d_zruns, c->d_tp, c->d_xh, c->d_yh, c->d_truns,
                   c->d_bdesc, c->d_bcell, c->d_bccoord, c->d_bface, c->d_rowtab,
@@ -247,6 +245,7 @@ gp_status gpi::launch(gp_ctx* c, const void* x, void* y, int add, cudaStream_t s
   a.nzruns = add ? 0 : (int32_t)p.num_zero_runs();
   a.g = p.jumps.data();
   a.m = p.lump.data();
+  a.w = p.fac.data();
   a.fac = c->d_fac;
   a.s = p.scale.data();
   a.ldl = p.ldl.empty() ? nullptr : p.ldl.data();
@@ -404,9 +403,10 @@ gp_status gp_setup(const gp_mesh* mesh, const gp_levelset* ls, const gp_opts* op
     const gp::Plan& p = c->plan;
     std::vector<int2> zruns(p.zruns.size() / 2);
     std::memcpy(zruns.data(), p.zruns.data(), p.zruns.size() * sizeof(int32_t));
-    std::vector<unsigned char> fac;
-    ops_for(p.precision, p.dim).values(p.fac.data(), p.fac.size(), fac);
-    if (e == cudaSuccess) e = upload(reinterpret_cast<unsigned char**>(&c->d_fac), fac);
+    if (e == cudaSuccess && p.precision == GP_FP32)
+      e = upload(reinterpret_cast<float**>(&c->d_fac), std::vector<float>(p.fac.begin(), p.fac.begin() + p.L));
+    if (e == cudaSuccess && p.precision == GP_FP64)
+      e = upload(reinterpret_cast<double**>(&c->d_fac), std::vector<double>(p.fac.begin() + p.L, p.fac.end()));
     if (e == cudaSuccess) e = upload(&c->d_frows, p.frows);
     if (e == cudaSuccess) e = upload(&c->d_lwin, p.lwin);
     if (e == cudaSuccess) e = upload(&c->d_lrow, p.lrow);
@@ -904,7 +904,7 @@ gp_status gp_batch_create(gp_ctx* const* ctxs, int nprob, int nrhs, gp_batch** o
                           b->cap);
       if (e == cudaSuccess)
         e = g.ops.run(g.k, g.d_fsegs, g.d_lsegs, g.d_ptrs[i], (int)g.prob.size(), g.face_blocks, g.lift_blocks,
-                      pl0.jumps.data(), pl0.lump.data(), g.ldl, g.form, g.tiles, b->cap);
+                      pl0.jumps.data(), pl0.lump.data(), pl0.fac.data(), g.ldl, g.form, g.tiles, b->cap);
     }
     cudaGraph_t graph = nullptr;
     const cudaError_t e2 = cudaStreamEndCapture(b->cap, &graph);

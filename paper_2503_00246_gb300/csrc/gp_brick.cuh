@@ -45,7 +45,6 @@ struct BrickArgs {
   const int32_t* bccoord;  // packed local coords cx | cy << 8 | cz << 16 of the own cells
   const uint32_t* bface;   // packed faces: axis | K- << 2 | K+ << 12 | K- own << 22 | K+ own << 23
   const int32_t* rowtab;   // per involved cell: compact index of node (ci k, row t), t < L
-  const void* fac;         // factors of the normal lines, V values (see Plan::fac)
   void* part;              // partial grids, V values
   const int2* zruns;       // zero runs (overwrite form)
   int32_t nzruns, nzblocks;
@@ -128,7 +127,7 @@ __device__ __forceinline__ void brick_chunk(const uint32_t* __restrict__ bface, 
                                             Sum<typename A::V>* ys,
                                             typename A::V (*buf)[K][TanShape<D, K>::LP],
                                             typename A::V (*dots)[K][K + 1],
-                                            const typename A::V* __restrict__ fac, const typename A::V* mc,
+                                            const typename A::V* wl, const typename A::V* mc,
                                             const Consts<typename A::V, K>& c) {
   using V = typename A::V;
   constexpr int L = Shape<D, K>::L, NN = 2 * K + 1, K1 = K + 1;
@@ -155,7 +154,7 @@ __device__ __forceinline__ void brick_chunk(const uint32_t* __restrict__ bface, 
     for (int j = 0; j < K; ++j) buf[fl][j][TanShape<D, K>::at(tau)] = tj[j];
   }
   V out[K];
-  tangential_mass<D, K, V>(buf, dots, fb, c, fac[tau], static_cast<const V*>(nullptr), mc, fl, tau, out);
+  tangential_mass<D, K, V>(buf, dots, fb, c, wl, mc, fl, tau, out);
   V w[NN];
   if (valid) {
     if constexpr (!FoldScale<V>::value) {
@@ -186,7 +185,7 @@ brick_kernel(const typename A::IO* __restrict__ x, typename A::IO* __restrict__ 
   constexpr int NB = (D == 3) ? K1 * K1 * K1 : K1 * K1;
   typedef V Plane[K][TanShape<D, K>::LP];
   typedef V Dots[K][K1];
-  __shared__ V mc[K1];
+  __shared__ V mc[K1], wl[L];
   const int t = threadIdx.x, nt = (int)blockDim.x;
   // the plane fixup may take its prologue while the bricks run (it waits for this grid)
   asm volatile("griddepcontrol.launch_dependents;");
@@ -217,7 +216,7 @@ brick_kernel(const typename A::IO* __restrict__ x, typename A::IO* __restrict__ 
   Dots* dots = reinterpret_cast<Dots*>(buf + fb);
 
   fill_mc<K, V>(mc, c, t);
-  const V* fac = static_cast<const V*>(ba.fac);
+  if (t < L) wl[t] = c.w[t];
   // ---- own-cell map and coordinates, zero accumulators, row starts, staged x blocks
   for (int i = t; i < nown; i += nt) {
     const int cc = __ldg(ba.bccoord + cell_off + i);
@@ -253,11 +252,11 @@ brick_kernel(const typename A::IO* __restrict__ x, typename A::IO* __restrict__ 
     const int fl = t / L, tau = t - fl * L;
     const uint32_t* bf = ba.bface + face_off;
     const int a1 = sd[8], a2 = (D == 3) ? sd[9] : nface;
-    for (int f0 = 0; f0 < a1; f0 += fb) brick_chunk<D, K, A, 0>(bf, f0, a1, fl, tau, fb, xs, ys, buf, dots, fac, mc, c);
-    for (int f0 = a1; f0 < a2; f0 += fb) brick_chunk<D, K, A, 1>(bf, f0, a2, fl, tau, fb, xs, ys, buf, dots, fac, mc, c);
+    for (int f0 = 0; f0 < a1; f0 += fb) brick_chunk<D, K, A, 0>(bf, f0, a1, fl, tau, fb, xs, ys, buf, dots, wl, mc, c);
+    for (int f0 = a1; f0 < a2; f0 += fb) brick_chunk<D, K, A, 1>(bf, f0, a2, fl, tau, fb, xs, ys, buf, dots, wl, mc, c);
     if constexpr (D == 3) {
       for (int f0 = a2; f0 < nface; f0 += fb)
-        brick_chunk<D, K, A, 2>(bf, f0, nface, fl, tau, fb, xs, ys, buf, dots, fac, mc, c);
+        brick_chunk<D, K, A, 2>(bf, f0, nface, fl, tau, fb, xs, ys, buf, dots, wl, mc, c);
     }
   }
 

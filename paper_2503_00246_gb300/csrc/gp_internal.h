@@ -19,7 +19,7 @@ struct gp_ctx {
   int32_t* d_lwin = nullptr;
   int32_t* d_lrow = nullptr;
   int32_t* d_lmask = nullptr;
-  void* d_fac = nullptr;         // Plan::fac in the context's arithmetic
+  void* d_fac = nullptr;         // line factors (Plan::fac): FP32 mw, FP64 those of the triangular basis
   gp::LaunchForm form{};         // gp::launch_form
   int2* d_zruns = nullptr;
   void* d_tp = nullptr;          // per-face outputs W_F (scratch of the face + lift path)

@@ -87,15 +87,19 @@ struct Consts {
   V g[K][2 * K + 1];   // jump of the j-th derivative of patch basis b (row j-1)
   V gs[K][2 * K + 1];  // s_j g_j[b], the jump vectors of the first step (FP64, float-float)
   V s[K];              // s_j (FP32)
-  // reference mass M^ = diag(mw) (I + mc ma^T) (see tangential_mass; mw: LineFactors)
+  // reference mass M^ = diag(mw) (I + mc ma^T) (see tangential_mass), and the factors mw of a face's lines (3D: the
+  // product of both directions')
   V ma[K + 1];
   V mc[K + 1];
+  V w[(K + 1) * (K + 1)];   // 2D: the first K + 1
 };
 
-// Fills the lumped form of the reference mass from p = (ma, mc), 2 (k+1) values.
-template <typename V, int K>
-void mass_consts(const double* p, Consts<V, K>& c) {
+// Fills the lumped form of the reference mass from p = (ma, mc), 2 (k+1) values, and the line factors from
+// fac (Plan::fac).
+template <int D, int K, typename V>
+void mass_consts(const double* p, const double* fac, Consts<V, K>& c) {
   constexpr int N = K + 1;
+  for (int i = 0; i < N * N; ++i) c.w[i] = i < Shape<D, K>::L ? from_host<V>(fac[i]) : vzero<V>();
   for (int i = 0; i < N; ++i) {
     c.ma[i] = from_host<V>(p[i]);
     c.mc[i] = from_host<V>(p[N + i]);
@@ -104,7 +108,7 @@ void mass_consts(const double* p, Consts<V, K>& c) {
 
 struct FaceArgs {
   const int32_t* frows;   // per-face row starts of the patch (see rbase)
-  const void* fac;        // factors of the normal lines, V values (see Plan::fac)
+  const void* fac;        // FP32: mw of a face's L lines; triangular basis: D_j mw, K rows of L (see Plan::fac)
   int64_t rbase[4];       // row entry of face fstart[a] of each axis
   int32_t fstart[4];      // first face of each axis in this launch
   int32_t fend[4];        // one past the last face of each axis in this launch
@@ -318,8 +322,7 @@ __device__ __forceinline__ void fill_mc(V (&mc)[K + 1], const Consts<V, K>& c, c
   if (t <= K) mc[t] = c.mc[t];
 }
 
-// u -> (I + mc ma^T) u of one tangential line.  k = 1: (2 u_0 + u_1, u_0 + 2 u_1), one rounding each.  (The integer
-// form of k = 2, 1/30 (4 2 -1; 2 16 2; -1 2 4), was no more accurate and in FP64 4 % slower.)
+// ma . u of one tangential line
 template <int K, typename V>
 __device__ __forceinline__ V line_dot(const Consts<V, K>& c, const V (&u)[K + 1]) {
   Dot<V> acc = dot_first(c.ma[0], u[0]);
@@ -327,16 +330,17 @@ __device__ __forceinline__ V line_dot(const Consts<V, K>& c, const V (&u)[K + 1]
   for (int q = 1; q <= K; ++q) dot_fma(acc, c.ma[q], u[q]);
   return dot_value(acc);
 }
+// u -> (I + mc ma^T) u of the line at p with stride st.  k = 1: (2 u_0 + u_1, u_0 + 2 u_1), one rounding each.  (The
+// integer form of k = 2, 1/30 (4 2 -1; 2 16 2; -1 2 4), was no more accurate and in FP64 4 % slower.)
 template <int K, typename V>
-__device__ __forceinline__ void line_mass(const Consts<V, K>& c, V (&u)[K + 1]) {
+__device__ __forceinline__ void line_mass(const Consts<V, K>& c, const V (&u)[K + 1], V* p, const int st) {
   if constexpr (K == 1) {
-    const V a = u[0], b = u[1];
-    u[0] = vadd(vscale(a, 2.f), b);
-    u[1] = vadd(vscale(b, 2.f), a);
+    p[0] = vadd(vscale(u[0], 2.f), u[1]);
+    p[st] = vadd(vscale(u[1], 2.f), u[0]);
   } else {
     const V s = line_dot<K, V>(c, u);
 #pragma unroll
-    for (int q = 0; q <= K; ++q) u[q] = vfma(c.mc[q], s, u[q]);
+    for (int q = 0; q <= K; ++q) p[st * q] = vfma(c.mc[q], s, u[q]);
   }
 }
 
@@ -345,14 +349,14 @@ __device__ __forceinline__ void line_mass(const Consts<V, K>& c, V (&u)[K + 1]) 
 // first threads.  3D: pass 1 along t2 (neighbouring lanes on neighbouring t1) in place; pass 2
 // along t1 only takes the dot product ma . u of each line, and every line's thread adds its own
 // mc and multiplies by mw (FP32, bound by shared-memory accesses and not by arithmetic, and k = 1: pass 2 in
-// place too, one access less per value).  2D: pass 1 in place.  wt is the
-// factor of the thread's line or, with the triangular basis, wl[tau + WS j] that of order j and line tau, mc[t]
-// the correction of tangential index t, both in shared memory.  Every thread of the CTA calls it (it
-// synchronises, also before its first read: the caller has only written plane, wl and mc).
+// place too, one access less per value).  2D: pass 1 in place.  wl[tau + WS j] is the factor of
+// order j and line tau (WS = 0: one for every order; WS < 0: wt, of the thread's line), mc[t] the correction of
+// tangential index t, both in shared memory.  Every thread of the CTA calls it (it synchronises, also before its first read:
+// the caller has only written plane, wl and mc).
 template <int D, int K, typename V, int WS = 0>
 __device__ __forceinline__ void tangential_mass(V (*plane)[K][TanShape<D, K>::LP], V (*dots)[K][K + 1], const int fb,
-                                                const Consts<V, K>& c, const V wt, const V* wl, const V* mc, const int fl,
-                                                const int tau, V (&out)[K]) {
+                                                const Consts<V, K>& c, const V* wl, const V* mc, const int fl,
+                                                const int tau, V (&out)[K], const V wt = vzero<V>()) {
   using T = TanShape<D, K>;
   constexpr int N = K + 1;
   constexpr int TASKS = (D == 3) ? K * N : K;     // per face and pass
@@ -368,9 +372,7 @@ __device__ __forceinline__ void tangential_mass(V (*plane)[K][TanShape<D, K>::LP
     V uu[N];
 #pragma unroll
     for (int q = 0; q < N; ++q) uu[q] = p[ST * q];
-    line_mass<K, V>(c, uu);
-#pragma unroll
-    for (int q = 0; q < N; ++q) p[ST * q] = uu[q];
+    line_mass<K, V>(c, uu, p, ST);
   }
   __syncthreads();
   if constexpr (D == 3) {
@@ -382,19 +384,18 @@ __device__ __forceinline__ void tangential_mass(V (*plane)[K][TanShape<D, K>::LP
       if constexpr (DOTS) {
         dots[tf][j][tr] = line_dot<K, V>(c, uu);
       } else {
-        line_mass<K, V>(c, uu);
-#pragma unroll
-        for (int q = 0; q < N; ++q) p[q] = uu[q];
+        line_mass<K, V>(c, uu, p, 1);
       }
     }
     __syncthreads();
   }
+  const V f = WS == 0 ? wl[tau] : wt;
   const V ct = DOTS ? mc[tau % N] : vzero<V>();
 #pragma unroll
   for (int jj = 0; jj < K; ++jj) {
     V v = plane[fl][jj][T::at(tau)];
     if constexpr (DOTS) v = vfma(ct, dots[fl][jj][tau / N], v);
-    out[jj] = vmul(WS ? wl[WS * jj + tau] : wt, v);
+    out[jj] = vmul(WS > 0 ? wl[WS * jj + tau] : f, v);
   }
 }
 
@@ -474,7 +475,13 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
   Plane* buf = reinterpret_cast<Plane*>(dsm);            // [fb][K][LP]
   Dots* dots = reinterpret_cast<Dots*>(buf + fb);         // [fb][K][N], 3D only
   __shared__ V mc[K1];
-  V* wj = reinterpret_cast<V*>(dots + ((D == 3) ? fb : 0));   // LDL: [K][L] line factors D_j mw
+  // The lines' factors.  FP32: loaded into the thread of the line, to be used behind three barriers; the triangular
+  // basis: D_j mw [K][L] behind the planes, copied there while the gather runs; else mw [L] from the constant bank.
+  // (FP32 from the constant bank, 25 to 81 values for each warp in turn: 128^3 gyroid at k = 4 229.9 / 227.1 us, 49^3
+  // ball at k = 8 85.3 / 83.7; float-float in registers: 50^3 ball at k = 6 123.8 / 119.7.)
+  constexpr bool REG = std::is_same<V, float>::value;
+  __shared__ V tw[LDL || REG ? 1 : L];
+  V* wl = LDL ? reinterpret_cast<V*>(dots + ((D == 3) ? fb : 0)) : tw;
   const int nt = (int)blockDim.x;
   // the lift may start its prologue as soon as every face CTA is running (programmatic
   // dependent launch; it waits for this grid's completion before it reads W)
@@ -502,13 +509,14 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
   const int fl = t / L, tau = t - fl * L;
   const int f = f0 + fl;
   const bool valid = f < fend;
-  const V* fac = static_cast<const V*>(fa.fac);
   if constexpr (LDL) {
-    // the factors of the triangular basis on their way to shared memory while the gather runs
     for (int i = t; i < K * L; i += nt)
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(wj + i)),
-                   "l"(fac + L + i) : "memory");
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((unsigned)__cvta_generic_to_shared(wl + i)),
+                   "l"(static_cast<const V*>(fa.fac) + i) : "memory");
+  } else if (!REG && t < L) {
+    wl[t] = c.w[t];
   }
+  fill_mc<K, V>(mc, c, t);
   // ---- gather this thread's normal line (2k+1 values)
   V v[NN];
   if (StagePatch<V, K, COMPACT>::value && axis == 0) {
@@ -564,7 +572,6 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
     for (int b = 0; b < NN; ++b) v[b] = vzero<V>();
   }
   if constexpr (LDL) asm volatile("cp.async.wait_all;" ::: "memory");
-  fill_mc<K, V>(mc, c, t);
   // ---- contract with the k jump vectors, then the tangential reference masses
   {
     V t[K];
@@ -574,8 +581,8 @@ __device__ __forceinline__ void face_body(const typename A::IO* __restrict__ x, 
     for (int j = 0; j < K; ++j) buf[fl][j][T::at(tau)] = t[j];
   }
   V out[K];
-  // (the factor is used behind three barriers: its load is hidden)
-  tangential_mass<D, K, V, LDL ? L : 0>(buf, dots, fb, c, LDL ? vzero<V>() : fac[tau], wj, mc, fl, tau, out);
+  tangential_mass<D, K, V, LDL ? L : REG ? -1 : 0>(buf, dots, fb, c, wl, mc, fl, tau, out,
+                                                   REG ? static_cast<const V*>(fa.fac)[tau] : vzero<V>());
 
   if (!valid) return;
   if constexpr (!FoldScale<V>::value) {
@@ -613,13 +620,13 @@ extern __shared__ __align__(16) unsigned char gp_dyn_smem[];
 // resident CTAs of MAX_CTA_THREADS threads to compile for: FP32 is held to 32 registers, every warp
 // slot of the SM (128^3 gyroid, k = 4, with 38 registers: 154 against 135 us; the compiler's choice at other degrees:
 // applies of the 80^3 ball at k = 5 66.9 / 65.7 us, of the 600^2 disc at k = 7 12.1 / 11.0 us); 0: that choice
-template <typename V>
+template <typename V, int K>
 struct FaceCtas {
-  static constexpr int value = std::is_same<V, float>::value ? 4 : 0;
+  static constexpr int value = std::is_same<V, float>::value || (std::is_same<V, ff64>::value && K == 4) ? 4 : 0;
 };
 
 template <int D, int K, class A, bool COMPACT, bool LDL>
-__global__ void __launch_bounds__(MAX_CTA_THREADS, FaceCtas<typename A::V>::value)
+__global__ void __launch_bounds__(MAX_CTA_THREADS, FaceCtas<typename A::V, K>::value)
 face_kernel(const typename A::IO* __restrict__ x, typename A::V* __restrict__ wp,
             typename A::IO* __restrict__ y, const FaceArgs fa, const int fb,
             const __grid_constant__ Consts<typename A::V, K> c) {
@@ -669,7 +676,7 @@ __device__ __forceinline__ int find_segment(const Seg* segs, const int nseg, con
 // problems of any weights share one launch: 64 FP64 balls, 24^3, k = 3, with 1, 16 or 64 sets of weights 421 us;
 // with B in the constant bank and a launch per set 434, 835 and 2351 us.
 template <int D, int K, class A, bool COMPACT, bool LDL>
-__global__ void __launch_bounds__(MAX_CTA_THREADS, FaceCtas<typename A::V>::value)
+__global__ void __launch_bounds__(MAX_CTA_THREADS, FaceCtas<typename A::V, K>::value)
 face_kernel_batched(const FaceSeg<typename A::V, K>* __restrict__ segs, const int nseg,
                     const SegPtrs<typename A::IO>* __restrict__ ptrs, const int fb,
                     const __grid_constant__ Consts<typename A::V, K> c) {

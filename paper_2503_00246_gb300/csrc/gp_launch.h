@@ -35,7 +35,8 @@ struct ApplyArgs {
   int32_t nzruns = 0;        // zero runs to fill (0 for the add form)
   const double* g = nullptr; // host FP64: k x (2k+1)
   const double* m = nullptr; // host FP64: the lumped mass, 2 (k+1) values (Plan::lump)
-  const void* fac = nullptr; // device: factors of the normal lines, V values (Plan::fac)
+  const double* w = nullptr; // host FP64: factors of the normal lines (Plan::fac)
+  const void* fac = nullptr; // device: those of FP32, or of the triangular basis
   const double* s = nullptr; // host FP64: k
   const double* ldl = nullptr;  // host FP64: the triangular normal basis (Plan::ldl); nullptr: g and s as they are
   cudaEvent_t* ev = nullptr;  // optional: 3 events recorded around the two kernels
@@ -237,7 +238,6 @@ cudaError_t run_brick(const ApplyArgs& Ar, const Consts<typename A::V, K>& c, cu
   constexpr int L = Shape<D, K>::L;
   const int fb = brick_fb<D, K>(Ar.tiles);
   BrickArgs ba = Ar.ba;
-  ba.fac = Ar.fac;
   ba.zruns = Ar.zruns;
   ba.nzruns = Ar.nzruns;
   ba.nzblocks = (Ar.nzruns + ZGROUP - 1) / ZGROUP;
@@ -442,7 +442,7 @@ cudaError_t run_apply(const ApplyArgs& Ar, cudaStream_t st) {
     c.s[j] = from_host<V>(Ar.s[j]);
     for (int b = 0; b < 2 * K + 1; ++b) c.gs[j][b] = from_host<V>(Ar.s[j] * Ar.g[j * (2 * K + 1) + b]);
   }
-  mass_consts<V, K>(Ar.m, c);
+  mass_consts<D, K, V>(Ar.m, Ar.w, c);
   // the triangular basis takes the place of g and s (the brick path runs the general form)
   constexpr bool HAS_LDL = UseLdl<V>::value;
   const bool ldl = HAS_LDL && Ar.ldl && !Ar.brick;
@@ -525,8 +525,8 @@ bool pack_batch(const std::vector<SegSpec>& in, const LaunchForm& form, Tiles& t
 
 template <int D, int K, class A>
 cudaError_t run_batch(const void* fsegs, const void* lsegs, const void* ptrs, int nseg, int face_blocks,
-                      int lift_blocks, const double* g, const double* m, bool ldl, const LaunchForm& form,
-                      Tiles t, cudaStream_t st) {
+                      int lift_blocks, const double* g, const double* m, const double* w, bool ldl,
+                      const LaunchForm& form, Tiles t, cudaStream_t st) {
   using V = typename A::V;
   using IO = typename A::IO;
   using S = Shape<D, K>;
@@ -535,7 +535,7 @@ cudaError_t run_batch(const void* fsegs, const void* lsegs, const void* ptrs, in
   Consts<V, K> c;
   for (int j = 0; j < K; ++j)
     for (int b = 0; b < 2 * K + 1; ++b) c.g[j][b] = from_host<V>(g[j * (2 * K + 1) + b]);
-  mass_consts<V, K>(m, c);
+  mass_consts<D, K, V>(m, w, c);
   for (int j = 0; j < K; ++j) {
     c.s[j] = vzero<V>();                                          // per segment: FaceSeg::s
     for (int b = 0; b < 2 * K + 1; ++b) c.gs[j][b] = vzero<V>();  // per segment: FaceSeg::gs
@@ -580,23 +580,13 @@ void scaled_jumps(int k, const double* g, const double* s, std::vector<unsigned 
     for (int b = 0; b < 2 * k + 1; ++b) o[j * (2 * k + 1) + b] = from_host<V>(s[j] * g[j * (2 * k + 1) + b]);
 }
 
-// n host values in the value type of the arithmetic.
-template <class A>
-void to_values(const double* v, size_t n, std::vector<unsigned char>& out) {
-  using V = typename A::V;
-  out.resize(n * sizeof(V));
-  V* o = reinterpret_cast<V*>(out.data());
-  for (size_t i = 0; i < n; ++i) o[i] = from_host<V>(v[i]);
-}
-
 // Per translation unit: batch packing and launch for one (arithmetic, dimension).
 struct BatchOps {
-  void (*values)(const double* v, size_t n, std::vector<unsigned char>& out);
   bool (*pack)(int k, const std::vector<SegSpec>&, const LaunchForm&, Tiles&, std::vector<unsigned char>&,
                std::vector<unsigned char>&, int&, int&);
   void (*jumps)(int k, const double* g, const double* s, std::vector<unsigned char>& out);
   cudaError_t (*run)(int k, const void*, const void*, const void*, int, int, int, const double*, const double*,
-                     bool, const LaunchForm&, Tiles, cudaStream_t);
+                     const double*, bool, const LaunchForm&, Tiles, cudaStream_t);
 };
 BatchOps batch_ops_f64_d2();
 BatchOps batch_ops_f64_d3();
@@ -607,7 +597,6 @@ BatchOps batch_ops_ff_d3();
 
 #define GP_BATCH_OPS(D, A)                                                                              \
   BatchOps ops;                                                                                         \
-  ops.values = to_values<A>;                                                                            \
   ops.jumps = scaled_jumps<A>;                                                                          \
   ops.pack = [](int k, const std::vector<SegSpec>& in, const LaunchForm& form, Tiles& t,               \
                 std::vector<unsigned char>& fs,                                                         \
@@ -625,17 +614,17 @@ BatchOps batch_ops_ff_d3();
     }                                                                                                   \
   };                                                                                                    \
   ops.run = [](int k, const void* fs, const void* ls, const void* pt, int ns, int fb, int lb,          \
-               const double* g, const double* m, bool l, const LaunchForm& form, Tiles t,              \
+               const double* g, const double* m, const double* w, bool l, const LaunchForm& form, Tiles t,    \
                cudaStream_t st) -> cudaError_t {                                                        \
     switch (k) {                                                                                        \
-      case 1: return run_batch<D, 1, A>(fs, ls, pt, ns, fb, lb, g, m, l, form, t, st);                        \
-      case 2: return run_batch<D, 2, A>(fs, ls, pt, ns, fb, lb, g, m, l, form, t, st);                        \
-      case 3: return run_batch<D, 3, A>(fs, ls, pt, ns, fb, lb, g, m, l, form, t, st);                        \
-      case 4: return run_batch<D, 4, A>(fs, ls, pt, ns, fb, lb, g, m, l, form, t, st);                        \
-      case 5: return run_batch<D, 5, A>(fs, ls, pt, ns, fb, lb, g, m, l, form, t, st);                        \
-      case 6: return run_batch<D, 6, A>(fs, ls, pt, ns, fb, lb, g, m, l, form, t, st);                        \
-      case 7: return run_batch<D, 7, A>(fs, ls, pt, ns, fb, lb, g, m, l, form, t, st);                        \
-      case 8: return run_batch<D, 8, A>(fs, ls, pt, ns, fb, lb, g, m, l, form, t, st);                        \
+      case 1: return run_batch<D, 1, A>(fs, ls, pt, ns, fb, lb, g, m, w, l, form, t, st);                        \
+      case 2: return run_batch<D, 2, A>(fs, ls, pt, ns, fb, lb, g, m, w, l, form, t, st);                        \
+      case 3: return run_batch<D, 3, A>(fs, ls, pt, ns, fb, lb, g, m, w, l, form, t, st);                        \
+      case 4: return run_batch<D, 4, A>(fs, ls, pt, ns, fb, lb, g, m, w, l, form, t, st);                        \
+      case 5: return run_batch<D, 5, A>(fs, ls, pt, ns, fb, lb, g, m, w, l, form, t, st);                        \
+      case 6: return run_batch<D, 6, A>(fs, ls, pt, ns, fb, lb, g, m, w, l, form, t, st);                        \
+      case 7: return run_batch<D, 7, A>(fs, ls, pt, ns, fb, lb, g, m, w, l, form, t, st);                        \
+      case 8: return run_batch<D, 8, A>(fs, ls, pt, ns, fb, lb, g, m, w, l, form, t, st);                        \
       default: return cudaErrorInvalidValue;                                                            \
     }                                                                                                   \
   };                                                                                                    \
