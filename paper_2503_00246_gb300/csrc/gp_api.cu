@@ -262,6 +262,7 @@ gp_status gpi::launch(gp_ctx* c, const void* x, void* y, int add, cudaStream_t s
   }
   a.ev = ev;
   a.tiles = tiles ? *tiles : c->tiles;
+  if (full_outputs && c->tuned) a.tiles.fb = 0;
   a.which = which;
   a.form = c->form;
   a.form.system = full_outputs;

@@ -53,6 +53,7 @@ struct gp_ctx {
   std::vector<cudaEvent_t> hgev; // one per slab, recorded after its gather
   cudaStream_t hin = nullptr;    // the gather stream
   gp::Tiles tiles{};             // tile shape of the face and lift launches (0: defaults)
+  bool tuned = false;            // tiles was measured for the apply (the model system's face kernel keeps its default)
   std::string err;
   // tracing: one event triple per traced apply
   bool prof = false;

@@ -61,7 +61,8 @@ void tiles_start(gp_ctx* c) {
   auto it = g_tiles.find(key_of(c));
   if (it == g_tiles.end()) return;
   auto own = it->second.kind.find(kind_of(c));
-  if (own != it->second.kind.end()) c->tiles = own->second;
+  c->tuned = own != it->second.kind.end();
+  if (c->tuned) c->tiles = own->second;
   else if (it->second.any) c->tiles = it->second.all;
 }
 
@@ -143,6 +144,7 @@ gp_status gp_set_tiles(gp_ctx* ctx, const gp_tiles* tiles) {
   if (!gpi::tile_ops(ctx->plan.dim, ctx->plan.precision).resolve(ctx->plan.k, t, ctx->form))
     return fail(ctx, GP_EINVAL, "tile shape out of range (threads per CTA, shared memory or lift threads)");
   ctx->tiles = from_abi(*tiles);
+  ctx->tuned = false;
   return GP_OK;
 }
 
@@ -305,6 +307,7 @@ gp_status gp_autotune(gp_ctx* ctx, int reps, gp_tiles* best, double* ms) {
   chosen.lcb = bl.lcb;
   chosen.lnt = bl.lnt;
   ctx->tiles = chosen;
+  ctx->tuned = true;
   gp_tiles_keep(ctx);
   if (best) *best = to_abi(chosen);
   if (ms) {
