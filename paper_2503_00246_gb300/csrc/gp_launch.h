@@ -95,7 +95,8 @@ constexpr TileRules kTilesF64 = {
      tiles_at({4, 16, 256}), tiles_at({3, 32, 512})},
     {tiles_at({128, 256, 512}), tiles_at({14, 128, 512}, 2500, {10, 64, 512}, 24000, {21, 32, 256}),
      tiles_at({2, 16, 256}, 6000, {8, 16, 256}, 70000, {24, 32, 512}), tiles_at({6, 32, 512}, 19000, {20, 32, 512}),
-     tiles_at({4, 8, 256}, 6000, {7, 16, 512}), tiles_at({3, 3, 256}, 3000, {5, 4, 256}, 5000, {5, 14, 512}), tiles_at({2, 8, 512}),
+     tiles_at({4, 8, 256}, 6000, {7, 16, 512}),
+     tiles_at({5, 1, 128}, 700, {3, 3, 256}, 3000, {7, 4, 256}, 3600, {5, 14, 512}), tiles_at({2, 8, 512}),
      tiles_at({3, 4, 256})}};
 constexpr TileRules kTilesFF = {
     {tiles_at({128, 256, 512}), tiles_at({42, 128, 256}), tiles_at({24, 32, 128}), tiles_at({19, 32, 256}),
@@ -104,7 +105,7 @@ constexpr TileRules kTilesFF = {
      tiles_at({4, 16, 256}, 12000, {8, 28, 256}, 21000, {8, 24, 128}),
      tiles_at({5, 32, 512}, 12000, {5, 32, 256}),
      tiles_at({3, 16, 512}, 6000, {7, 24, 512}, 19000, {7, 32, 256}),
-     tiles_at({2, 14, 512}, 2500, {3, 32, 512}, 6000, {3, 64, 512}),
+     tiles_at({2, 14, 512}, 1000, {2, 3, 128}, 2600, {3, 4, 128}, 3500, {3, 32, 512}),
      tiles_at({2, 8, 512}, 1400, {2, 16, 512}, 2800, {2, 24, 512}, 9700, {4, 32, 256}),
      tiles_at({3, 4, 256}, 2500, {3, 32, 512}, 6000, {3, 32, 256})}};
 // FP32 that stores W_F, and compact outputs (a row that store_compact leaves out only serves checks of shapes
